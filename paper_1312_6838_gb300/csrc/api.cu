@@ -624,7 +624,7 @@ size_t css_workspace_size(css_op op, css_dtype dtype, int64_t m, int64_t n, int6
       return backward_workspace_bytes(dtype, m, n, k);
     case CSS_OP_EMBED:
       if (k <= 0 || k > 1024 || k > m || k > n) return 0;
-      return embed_workspace_bytes(m, k);
+      return embed_workspace_bytes(m, n, k);
     default:
       break;
   }

@@ -19,7 +19,7 @@
 #include <vector>
 
 #include "backward.cuh"
-#include "df.cuh"
+#include "slice_gemm.cuh"
 
 using namespace css;
 
@@ -334,369 +334,79 @@ void chol_inv(double* G, int k, double* Linv, int* status, cudaStream_t s) {
   linv_kernel<<<(k + kLinvWarps - 1) / kLinvWarps, kLinvWarps * 32, smem, s>>>(G, k, Linv);
 }
 
-// Q = A_S L^-T (m x k): Q[i, j] = sum_{l <= j} A_S[i, l] Linv[j, l]; the
-// double-float split of Q is stored alongside.
+// Q = A_S L^-T (m x k): Q[i, j] = sum_{l <= j} A_S[i, l] Linv[j, l].
 __global__ void q_kernel(const double* __restrict__ AS, const double* __restrict__ Linv, int m, int k,
-                         double* __restrict__ Q, float* __restrict__ Qh, float* __restrict__ Ql) {
+                         double* __restrict__ Q) {
   const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (long long)m * k) return;
   const int i = (int)(idx % m), j = (int)(idx / m);
   double acc = 0.0;
   for (int l = 0; l <= j; ++l) acc = fma(AS[(long long)l * m + i], Linv[(long long)l * k + j], acc);
   Q[idx] = acc;
-  float h, lo;
-  df_split(acc, h, lo);
-  Qh[idx] = h;
-  Ql[idx] = lo;
 }
 
-// --------------------------------------------------- W = Q^T A  (k x n) -----
-// 32 (k) x 64 (n) outputs per block, 2 x 4 per thread, K = m in chunks of 16.
-// Element (j, c) of W goes to W[j * wj + c * wc]; the double-float split to
-// Wh / Wl (same positions) when those are not null.
-template <typename TA>
-__global__ void __launch_bounds__(256) w_kernel(const float* __restrict__ Qh, const float* __restrict__ Ql,
-                                                const double* __restrict__ Q, const TA* __restrict__ A,
-                                                long long lda, int m, int n, int k,
-                                                double* __restrict__ W, long long wj, long long wc,
-                                                float* __restrict__ Wh, float* __restrict__ Wl) {
-  constexpr int BK = 16;
-  __shared__ float qh[BK][33], ql[BK][33];
-  __shared__ double qd[BK][33];
-  __shared__ float as[BK][65];
-  __shared__ double ad[BK][65];
-  const int j0 = blockIdx.y * 32, c0 = blockIdx.x * 64;
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;  // ty: 16 rows of j (x2), tx: 16 cols (x4)
-  constexpr bool F64 = sizeof(TA) == 8;
-  DF acc[2][4];
-  double accd[2][4];
-#pragma unroll
-  for (int a = 0; a < 2; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) { acc[a][b] = DF{0.f, 0.f}; accd[a][b] = 0.0; }
-  for (int r0 = 0; r0 < m; r0 += BK) {
-    for (int e = threadIdx.x; e < BK * 32; e += 256) {
-      const int rr = e % BK, jj = e / BK;
-      const bool ok = r0 + rr < m && j0 + jj < k;
-      const long long o = (long long)(j0 + jj) * m + r0 + rr;
-      if (F64) qd[rr][jj] = ok ? Q[o] : 0.0;
-      else { qh[rr][jj] = ok ? Qh[o] : 0.f; ql[rr][jj] = ok ? Ql[o] : 0.f; }
-    }
-    for (int e = threadIdx.x; e < BK * 64; e += 256) {
-      const int rr = e % BK, cc = e / BK;
-      const bool ok = r0 + rr < m && c0 + cc < n;
-      const double v = ok ? to_d<TA>(A[(long long)(c0 + cc) * lda + r0 + rr]) : 0.0;
-      if (F64) ad[rr][cc] = v;
-      else as[rr][cc] = (float)v;
-    }
-    __syncthreads();
-#pragma unroll 4
-    for (int rr = 0; rr < BK; ++rr) {
-#pragma unroll
-      for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-          if (F64) accd[a][b] = fma(qd[rr][ty * 2 + a], ad[rr][tx * 4 + b], accd[a][b]);
-          else df_fma(acc[a][b], as[rr][tx * 4 + b], qh[rr][ty * 2 + a], ql[rr][ty * 2 + a]);
-        }
-    }
-    __syncthreads();
+// The call's status once its work is enqueued (opts->sync): [0] A_S is rank
+// deficient, [1] a product's wait ran out.
+css_status finish(const int* status, const css_opts& o, cudaStream_t s) {
+  if (!o.sync) return CSS_OK;
+  int st[2] = {0, 0};
+  if (cudaMemcpyAsync(st, status, sizeof(st), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+      cudaStreamSynchronize(s) != cudaSuccess)
+    return CSS_ERR_CUDA;
+  if (st[1]) return (css_status)st[1];
+  return st[0] ? CSS_ERR_INVALID_ARG : CSS_OK;   // A_S is rank deficient
+}
+
+// -------------------------------------------------- products in digits -----
+// W = Q^T A, R = A - Q W and P = R W^T run on the slice GEMM (slice_gemm.cu).
+// W's operand A is split a range of columns at a time, which bounds the
+// workspace: as many tiles of 128 columns as 1.25 GB of digits hold, cut to a
+// whole number of rounds over the 152 SMs.
+constexpr long long kDigitBudget = 1280ll << 20;
+constexpr int kRound = 152;
+
+long long chunk_cols(long long m, long long n, int k) {
+  const long long tiles = (n + 127) / 128, tn = (k + 127) / 128;
+  const long long per_tile = 128 * 16 * ((m + 63) / 64 * 64);
+  long long c = std::max<long long>(1, kDigitBudget / per_tile);
+  if (c * tn > kRound) c = c * tn / kRound * kRound / tn;
+  return std::min(c, tiles) * 128;
+}
+
+// W = Q^T A: element (j, c) to W[j * wj + c * wc].  Q's digits are in DQ.
+cudaError_t w_product(const sg::Digits& DQ, const sg::Source& q, const void* A, int dtype, long long lda, int m, int n,
+                      int k, double* W, long long wj, long long wc, sg::Digits& DA, const sg::Scratch& sc, int* err,
+                      unsigned long long spin_ns, cudaStream_t s) {
+  const long long cols = chunk_cols(m, n, k);
+  const long long esz = dtype == CSS_F64 ? 8 : dtype == CSS_F32 ? 4 : 2;
+  for (long long c0 = 0; c0 < n; c0 += cols) {
+    const sg::Source a{(const char*)A + c0 * lda * esz, dtype, lda, 1, (int)std::min(cols, n - c0), m};
+    cudaError_t e = sg::split(a, DA, s);
+    if (e != cudaSuccess) return e;
+    const sg::Store st{W + c0 * wc, wc, wj, 0};
+    if ((e = sg::gemm(DA, a, DQ, q, st, sc, err, spin_ns, s)) != cudaSuccess) return e;
   }
-#pragma unroll
-  for (int a = 0; a < 2; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      const int j = j0 + ty * 2 + a, c = c0 + tx * 4 + b;
-      if (j < k && c < n) {
-        const double v = F64 ? accd[a][b] : (double)acc[a][b].s + (double)acc[a][b].c;
-        const long long o = (long long)j * wj + (long long)c * wc;
-        W[o] = v;
-        if (Wh) {
-          float h, lo;
-          df_split(v, h, lo);
-          Wh[o] = h;
-          Wl[o] = lo;
-        }
-      }
-    }
+  return cudaSuccess;
 }
 
-// The FP32/BF16 (double-float) form of w_kernel: 64 x 64 outputs per block,
-// 4 x 4 per thread, so that each K step reads three 16-byte vectors of shared
-// memory for 16 double-float multiply-adds; K chunks of 16 double-buffered
-// through registers.  Each output's terms are added in the same order as in
-// w_kernel, so the result is bit-identical.
-constexpr int kDT = 64, kDK = 16, kDP = kDT + 4;
-
-template <typename TA>
-__global__ void __launch_bounds__(256) w_df_kernel(const float* __restrict__ Qh, const float* __restrict__ Ql,
-                                                   const TA* __restrict__ A, long long lda, int m, int n, int k,
-                                                   double* __restrict__ W, long long wj, long long wc,
-                                                   float* __restrict__ Wh, float* __restrict__ Wl) {
-  __shared__ __align__(16) float sq[2][2][kDK][kDP];   // [buffer][hi, lo][row of the chunk][j]
-  __shared__ __align__(16) float sa[2][kDK][kDP];      // [buffer][row of the chunk][column]
-  const int j0 = blockIdx.y * kDT, c0 = blockIdx.x * kDT;
-  const int tid = threadIdx.x, ty = tid / 16, tx = tid % 16;
-  const int rr = tid % kDK, cq = tid / kDK;   // staging: row rr, columns cq + 16 v
-  float rh[4], rl[4], ra[4];
-  DF acc[4][4];
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = DF{0.f, 0.f};
-  auto fetch = [&](int r0) {
-    const int r = r0 + rr;
-    const bool okr = r < m;
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      const int x = cq + 16 * v;
-      const bool okq = okr && j0 + x < k, oka = okr && c0 + x < n;
-      rh[v] = okq ? Qh[(long long)(j0 + x) * m + r] : 0.f;
-      rl[v] = okq ? Ql[(long long)(j0 + x) * m + r] : 0.f;
-      ra[v] = oka ? (float)to_d<TA>(A[(long long)(c0 + x) * lda + r]) : 0.f;
-    }
-  };
-  auto stage = [&](int b) {
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      sq[b][0][rr][cq + 16 * v] = rh[v];
-      sq[b][1][rr][cq + 16 * v] = rl[v];
-      sa[b][rr][cq + 16 * v] = ra[v];
-    }
-  };
-  fetch(0);
-  stage(0);
-  __syncthreads();
-  int buf = 0;
-  for (int r0 = 0; r0 < m; r0 += kDK) {
-    const bool more = r0 + kDK < m;
-    if (more) fetch(r0 + kDK);
-#pragma unroll 4
-    for (int kk = 0; kk < kDK; ++kk) {
-      const float4 qh4 = *reinterpret_cast<const float4*>(&sq[buf][0][kk][ty * 4]);
-      const float4 ql4 = *reinterpret_cast<const float4*>(&sq[buf][1][kk][ty * 4]);
-      const float4 a4 = *reinterpret_cast<const float4*>(&sa[buf][kk][tx * 4]);
-      const float qh[4] = {qh4.x, qh4.y, qh4.z, qh4.w}, ql[4] = {ql4.x, ql4.y, ql4.z, ql4.w};
-      const float av[4] = {a4.x, a4.y, a4.z, a4.w};
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) df_fma(acc[a][b], av[b], qh[a], ql[a]);
-    }
-    if (more) stage(buf ^ 1);
-    __syncthreads();
-    buf ^= 1;
-  }
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      const int j = j0 + ty * 4 + a, c = c0 + tx * 4 + b;
-      if (j < k && c < n) {
-        const double v = (double)acc[a][b].s + (double)acc[a][b].c;
-        const long long o = (long long)j * wj + (long long)c * wc;
-        W[o] = v;
-        if (Wh) {
-          float h, lo;
-          df_split(v, h, lo);
-          Wh[o] = h;
-          Wl[o] = lo;
-        }
-      }
-    }
-}
-
-// W = Q^T A launch: FP64 A on w_kernel, FP32/BF16 A on w_df_kernel.
-template <typename TA>
-void launch_w(const float* Qh, const float* Ql, const double* Q, const TA* A, long long lda, int m, int n, int k,
-              double* W, long long wj, long long wc, float* Wh, float* Wl, cudaStream_t s) {
-  if constexpr (sizeof(TA) == 8)
-    w_kernel<TA><<<dim3((n + 63) / 64, (k + 31) / 32), 256, 0, s>>>(Qh, Ql, Q, A, lda, m, n, k, W, wj, wc, Wh, Wl);
-  else
-    w_df_kernel<TA><<<dim3((n + kDT - 1) / kDT, (k + kDT - 1) / kDT), 256, 0, s>>>(Qh, Ql, A, lda, m, n, k, W, wj,
-                                                                                 wc, Wh, Wl);
-}
-
-// ------------------------------------ R = A - Q W (m x n) with epilogues -----
-// 64 x 64 outputs per block, 4 x 4 per thread, K = k in chunks of 16.
-// Writes R (FP32, or FP64 for FP64 input) when Rout != null, dA = 2 g R when
-// dA != null, and a per-block partial of ||R||^2.
-template <typename TA>
-__global__ void __launch_bounds__(256) r_kernel(const float* __restrict__ Qh, const float* __restrict__ Ql,
-                                                const double* __restrict__ Q, const float* __restrict__ Wh,
-                                                const float* __restrict__ Wl, const double* __restrict__ W,
-                                                const TA* __restrict__ A, long long lda, int m, int n, int k,
-                                                void* __restrict__ Rout, TA* __restrict__ dA, long long ldda,
-                                                double g2, double* __restrict__ loss_part) {
-  constexpr int BK = 16;
-  constexpr bool F64 = sizeof(TA) == 8;
-  __shared__ float qh[BK][65], ql[BK][65], wh[BK][65], wl[BK][65];
-  __shared__ double qd[BK][65], wd[BK][65];
-  __shared__ double red[8];
-  const int i0 = blockIdx.x * 64, c0 = blockIdx.y * 64;
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  DF acc[4][4];
-  double accd[4][4];
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) { acc[a][b] = DF{0.f, 0.f}; accd[a][b] = 0.0; }
-  for (int j0 = 0; j0 < k; j0 += BK) {
-    for (int e = threadIdx.x; e < BK * 64; e += 256) {
-      const int ii = e % 64, jj = e / 64;   // Q: rows contiguous
-      const bool okq = i0 + ii < m && j0 + jj < k;
-      const long long oq = (long long)(j0 + jj) * m + i0 + ii;
-      const int jj2 = e % BK, cc = e / BK;  // W: k contiguous per column
-      const bool okw = j0 + jj2 < k && c0 + cc < n;
-      const long long ow = (long long)(c0 + cc) * k + j0 + jj2;
-      if (F64) {
-        qd[jj][ii] = okq ? Q[oq] : 0.0;
-        wd[jj2][cc] = okw ? W[ow] : 0.0;
-      } else {
-        qh[jj][ii] = okq ? Qh[oq] : 0.f;
-        ql[jj][ii] = okq ? Ql[oq] : 0.f;
-        wh[jj2][cc] = okw ? Wh[ow] : 0.f;
-        wl[jj2][cc] = okw ? Wl[ow] : 0.f;
-      }
-    }
-    __syncthreads();
-#pragma unroll 2
-    for (int jj = 0; jj < BK; ++jj) {
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-          if (F64) accd[a][b] = fma(qd[jj][ty * 4 + a], wd[jj][tx * 4 + b], accd[a][b]);
-          else df_fma2(acc[a][b], qh[jj][ty * 4 + a], ql[jj][ty * 4 + a], wh[jj][tx * 4 + b],
-                       wl[jj][tx * 4 + b]);
-        }
-    }
-    __syncthreads();
-  }
+// FP64 input: V = Q W on entry, R = A - V on return (in place), dA = g2 R when
+// dA != null, and one partial of ||R||^2 per block.
+constexpr int kLossBlocks = 152 * 8;
+__global__ void __launch_bounds__(256) residual_f64_kernel(const double* __restrict__ A, long long lda, int m,
+                                                           long long mn, double* __restrict__ R,
+                                                           double* __restrict__ dA, long long ldda, double g2,
+                                                           double* __restrict__ loss_part) {
+  __shared__ double red[32];
   double sq = 0.0;
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      const int i = i0 + ty * 4 + a, c = c0 + tx * 4 + b;
-      if (i < m && c < n) {
-        const double av = to_d<TA>(A[(long long)c * lda + i]);
-        // a - (s + c) in double: the pair carries the product to ~2^-48
-        const double r = F64 ? av - accd[a][b] : (av - (double)acc[a][b].s) - (double)acc[a][b].c;
-        sq += r * r;
-        if (Rout) {
-          if (F64) ((double*)Rout)[(long long)c * m + i] = r;
-          else ((float*)Rout)[(long long)c * m + i] = (float)r;
-        }
-        if (dA) dA[(long long)c * ldda + i] = from_d<TA>(g2 * r);
-      }
-    }
-  sq = warp_sum(sq);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sq;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int w = 0; w < 8; ++w) t += red[w];
-    loss_part[(long long)blockIdx.y * gridDim.x + blockIdx.x] = t;
+  for (long long idx = (long long)blockIdx.x * 256 + threadIdx.x; idx < mn; idx += (long long)gridDim.x * 256) {
+    const long long c = idx / m, i = idx - c * m;
+    const double r = A[c * lda + i] - R[idx];
+    R[idx] = r;
+    if (dA) dA[c * ldda + i] = g2 * r;
+    sq = fma(r, r, sq);
   }
-}
-
-// The FP32/BF16 (double-float) form of r_kernel: the same 64 x 64 tile and
-// 4 x 4 outputs per thread, with Q and W staged so that each K step reads
-// four 16-byte vectors of shared memory for 16 double-float multiply-adds,
-// and K chunks double-buffered through registers.  Same order of terms and
-// of the loss partial sums as r_kernel, so the results are bit-identical.
-template <typename TA>
-__global__ void __launch_bounds__(256) r_df_kernel(const float* __restrict__ Qh, const float* __restrict__ Ql,
-                                                   const float* __restrict__ Wh, const float* __restrict__ Wl,
-                                                   const TA* __restrict__ A, long long lda, int m, int n, int k,
-                                                   float* __restrict__ Rout, TA* __restrict__ dA, long long ldda,
-                                                   double g2, double* __restrict__ loss_part) {
-  __shared__ __align__(16) float sq[2][2][kDK][kDP];   // [buffer][hi, lo][j of the chunk][row]
-  __shared__ __align__(16) float sw[2][2][kDK][kDP];   // [buffer][hi, lo][j of the chunk][column]
-  __shared__ double red[8];
-  const int i0 = blockIdx.x * kDT, c0 = blockIdx.y * kDT;
-  const int tid = threadIdx.x, ty = tid / 16, tx = tid % 16;
-  // staging: Q rows ii = tid % 64 of chunk entries jq + 4 v; W entries jw = tid % 16 of columns cw + 16 v
-  const int ii = tid % kDT, jq = tid / kDT;
-  const int jw = tid % kDK, cw = tid / kDK;
-  float qh_r[4], ql_r[4], wh_r[4], wl_r[4];
-  DF acc[4][4];
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = DF{0.f, 0.f};
-  auto fetch = [&](int jb) {
-    const bool oki = i0 + ii < m;
-    const bool okw = jb + jw < k;
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      const int j = jb + jq + 4 * v;
-      const bool okq = oki && j < k;
-      qh_r[v] = okq ? Qh[(long long)j * m + i0 + ii] : 0.f;
-      ql_r[v] = okq ? Ql[(long long)j * m + i0 + ii] : 0.f;
-      const int c = c0 + cw + 16 * v;
-      const bool ok = okw && c < n;
-      wh_r[v] = ok ? Wh[(long long)c * k + jb + jw] : 0.f;
-      wl_r[v] = ok ? Wl[(long long)c * k + jb + jw] : 0.f;
-    }
-  };
-  auto stage = [&](int b) {
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      sq[b][0][jq + 4 * v][ii] = qh_r[v];
-      sq[b][1][jq + 4 * v][ii] = ql_r[v];
-      sw[b][0][jw][cw + 16 * v] = wh_r[v];
-      sw[b][1][jw][cw + 16 * v] = wl_r[v];
-    }
-  };
-  fetch(0);
-  stage(0);
-  __syncthreads();
-  int buf = 0;
-  for (int jb = 0; jb < k; jb += kDK) {
-    const bool more = jb + kDK < k;
-    if (more) fetch(jb + kDK);
-#pragma unroll 2
-    for (int jj = 0; jj < kDK; ++jj) {
-      const float4 qh4 = *reinterpret_cast<const float4*>(&sq[buf][0][jj][ty * 4]);
-      const float4 ql4 = *reinterpret_cast<const float4*>(&sq[buf][1][jj][ty * 4]);
-      const float4 wh4 = *reinterpret_cast<const float4*>(&sw[buf][0][jj][tx * 4]);
-      const float4 wl4 = *reinterpret_cast<const float4*>(&sw[buf][1][jj][tx * 4]);
-      const float qh[4] = {qh4.x, qh4.y, qh4.z, qh4.w}, ql[4] = {ql4.x, ql4.y, ql4.z, ql4.w};
-      const float wh[4] = {wh4.x, wh4.y, wh4.z, wh4.w}, wl[4] = {wl4.x, wl4.y, wl4.z, wl4.w};
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) df_fma2(acc[a][b], qh[a], ql[a], wh[b], wl[b]);
-    }
-    if (more) stage(buf ^ 1);
-    __syncthreads();
-    buf ^= 1;
-  }
-  double sq_sum = 0.0;
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      const int i = i0 + ty * 4 + a, c = c0 + tx * 4 + b;
-      if (i < m && c < n) {
-        const double av = to_d<TA>(A[(long long)c * lda + i]);
-        // a - (s + c) in double: the pair carries the product to ~2^-48
-        const double r = (av - (double)acc[a][b].s) - (double)acc[a][b].c;
-        sq_sum += r * r;
-        if (Rout) Rout[(long long)c * m + i] = (float)r;
-        if (dA) dA[(long long)c * ldda + i] = from_d<TA>(g2 * r);
-      }
-    }
-  sq_sum = warp_sum(sq_sum);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sq_sum;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int w = 0; w < 8; ++w) t += red[w];
-    loss_part[(long long)blockIdx.y * gridDim.x + blockIdx.x] = t;
-  }
+  sq = block_sum(sq, red);
+  if (threadIdx.x == 0) loss_part[blockIdx.x] = sq;
 }
 
 __global__ void sum_kernel(const double* __restrict__ part, long long cnt, double scale,
@@ -706,126 +416,6 @@ __global__ void sum_kernel(const double* __restrict__ part, long long cnt, doubl
   for (long long i = threadIdx.x; i < cnt; i += blockDim.x) a += part[i];
   a = block_sum(a, red);
   if (threadIdx.x == 0) out[0] = a * scale;
-}
-
-// ------------------------------ P = R W^T (m x k), split over column slices --
-// partial[s][i + j*m] = sum over columns c of slice s of R[i, c] W[j, c].
-template <typename TR>
-__global__ void __launch_bounds__(256) rwt_kernel(const TR* __restrict__ R, const double* __restrict__ W,
-                                                  int m, int n, int k, int slice,
-                                                  TR* __restrict__ partial) {
-  constexpr int BK = 16;
-  __shared__ TR rs[BK][65];
-  __shared__ TR ws[BK][33];
-  const int i0 = blockIdx.x * 64, j0 = blockIdx.y * 32, sl = blockIdx.z;
-  const int cb = sl * slice, ce = min(n, cb + slice);
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  TR acc[4][2];
-#pragma unroll
-  for (int a = 0; a < 4; ++a) { acc[a][0] = TR(0); acc[a][1] = TR(0); }
-  for (int c0 = cb; c0 < ce; c0 += BK) {
-    for (int e = threadIdx.x; e < BK * 64; e += 256) {
-      const int ii = e % 64, cc = e / 64;
-      rs[cc][ii] = (c0 + cc < ce && i0 + ii < m) ? R[(long long)(c0 + cc) * m + i0 + ii] : TR(0);
-    }
-    for (int e = threadIdx.x; e < BK * 32; e += 256) {
-      const int jj = e % 32, cc = e / 32;
-      ws[cc][jj] = (c0 + cc < ce && j0 + jj < k) ? (TR)W[(long long)(c0 + cc) * k + j0 + jj] : TR(0);
-    }
-    __syncthreads();
-#pragma unroll 4
-    for (int cc = 0; cc < BK; ++cc)
-#pragma unroll
-      for (int a = 0; a < 4; ++a) {
-        acc[a][0] = fma(rs[cc][ty * 4 + a], ws[cc][tx * 2 + 0], acc[a][0]);
-        acc[a][1] = fma(rs[cc][ty * 4 + a], ws[cc][tx * 2 + 1], acc[a][1]);
-      }
-    __syncthreads();
-  }
-  TR* out = partial + (long long)sl * m * k;
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 2; ++b) {
-      const int i = i0 + ty * 4 + a, j = j0 + tx * 2 + b;
-      if (i < m && j < k) out[(long long)j * m + i] = acc[a][b];
-    }
-}
-
-// FP32 form of rwt_kernel: 64 x 64 outputs per block, 4 x 4 per thread, two
-// 16-byte shared-memory reads per K step for 16 FMAs, K chunks
-// double-buffered through registers; same order of terms (bit-identical).
-__global__ void __launch_bounds__(256) rwt_f32_kernel(const float* __restrict__ R, const double* __restrict__ W,
-                                                      int m, int n, int k, int slice, float* __restrict__ partial) {
-  __shared__ __align__(16) float rs[2][kDK][kDP];
-  __shared__ __align__(16) float ws[2][kDK][kDP];
-  const int i0 = blockIdx.x * kDT, j0 = blockIdx.y * kDT, sl = blockIdx.z;
-  const int cb = sl * slice, ce = min(n, cb + slice);
-  const int tid = threadIdx.x, ty = tid / 16, tx = tid % 16;
-  const int xi = tid % kDT, kq = tid / kDT;   // staging: row / entry xi of chunk columns kq + 4 v
-  float rr[4], wr[4];
-  float acc[4][4];
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
-  auto fetch = [&](int c0) {
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      const int c = c0 + kq + 4 * v;
-      const bool okc = c < ce;
-      rr[v] = (okc && i0 + xi < m) ? R[(long long)c * m + i0 + xi] : 0.f;
-      wr[v] = (okc && j0 + xi < k) ? (float)W[(long long)c * k + j0 + xi] : 0.f;
-    }
-  };
-  auto stage = [&](int b) {
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      rs[b][kq + 4 * v][xi] = rr[v];
-      ws[b][kq + 4 * v][xi] = wr[v];
-    }
-  };
-  if (cb < ce) {
-    fetch(cb);
-    stage(0);
-  }
-  __syncthreads();
-  int buf = 0;
-  for (int c0 = cb; c0 < ce; c0 += kDK) {
-    const bool more = c0 + kDK < ce;
-    if (more) fetch(c0 + kDK);
-#pragma unroll 4
-    for (int kk = 0; kk < kDK; ++kk) {
-      const float4 r4 = *reinterpret_cast<const float4*>(&rs[buf][kk][ty * 4]);
-      const float4 w4 = *reinterpret_cast<const float4*>(&ws[buf][kk][tx * 4]);
-      const float ra[4] = {r4.x, r4.y, r4.z, r4.w}, wa[4] = {w4.x, w4.y, w4.z, w4.w};
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] = fmaf(ra[a], wa[b], acc[a][b]);
-    }
-    if (more) stage(buf ^ 1);
-    __syncthreads();
-    buf ^= 1;
-  }
-  float* out = partial + (long long)sl * m * k;
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      const int i = i0 + ty * 4 + a, j = j0 + tx * 4 + b;
-      if (i < m && j < k) out[(long long)j * m + i] = acc[a][b];
-    }
-}
-
-// P = R W^T (m x k) from the slices, added in slice order, in FP64.
-template <typename TR>
-__global__ void sum_slices_kernel(const TR* __restrict__ partial, int S, long long mk, double* __restrict__ P) {
-  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= mk) return;
-  double p = 0.0;
-  for (int s = 0; s < S; ++s) p += (double)partial[(long long)s * mk + idx];
-  P[idx] = p;
 }
 
 // dA[:, S[j]] = -2 g sum_{l >= j} P[i, l] Linv[l, j].
@@ -840,17 +430,14 @@ __global__ void das_kernel(const double* __restrict__ P, const double* __restric
   dA[(long long)sel[j] * ldda + i] = from_d<TA>(-g2 * acc);
 }
 
-constexpr int kSlices = 16;
-
 struct BwLayout {
-  int* status;
+  int* status;   // [0] A_S is rank deficient, [1] error of the products
   double *AS, *G, *gpart, *Linv, *Q, *W;
-  float *Qh, *Ql, *Wh, *Wl;
-  void* R;
-  void* P;
+  void* R;       // residual: FP32, FP64 for FP64 input
   double* Psum;
   double* loss_part;
-  double* loss_tmp;
+  sg::Digits DQ, DQr, DW, DWr, DA, DR;   // operands of the products (r: the other way round)
+  sg::Scratch sc, scp;
   size_t bytes;
 };
 
@@ -863,62 +450,73 @@ BwLayout bw_layout(void* ws, size_t cap, int dt, int64_t m, int64_t n, int32_t k
   L.gpart = c.take<double>(gram_part_doubles((int)m, k));
   L.Linv = c.take<double>((size_t)k * k);
   L.Q = c.take<double>((size_t)m * k);
-  L.Qh = c.take<float>((size_t)m * k);
-  L.Ql = c.take<float>((size_t)m * k);
   L.W = c.take<double>((size_t)k * n);
-  L.Wh = c.take<float>((size_t)k * n);
-  L.Wl = c.take<float>((size_t)k * n);
   const size_t rs = dt == CSS_F64 ? 8 : 4;
-  L.R = grad ? (void*)c.take<char>((size_t)m * n * rs) : nullptr;
-  L.P = grad ? (void*)c.take<char>((size_t)kSlices * m * k * rs) : nullptr;
+  L.R = grad || dt == CSS_F64 ? (void*)c.take<char>((size_t)m * n * rs) : nullptr;
   L.Psum = grad ? c.take<double>((size_t)m * k) : nullptr;
-  L.loss_part = c.take<double>((size_t)((m + 63) / 64) * ((n + 63) / 64));
-  L.loss_tmp = c.take<double>(1);
+  L.loss_part = c.take<double>((size_t)std::max(kLossBlocks, sg::residual_parts()));
+  L.DQ = sg::carve_digits(c, k, m);
+  L.DQr = sg::carve_digits(c, m, k);
+  L.DWr = sg::carve_digits(c, n, k);
+  const long long cols = chunk_cols(m, n, k);
+  L.sc = sg::carve_scratch(c, cols, k, m);
+  L.DW = sg::carve_digits(c, k, n);
+  // A's digits are done with when R's are formed
+  const size_t at = c.off;
+  L.DA = sg::carve_digits(c, cols, m);
+  if (grad) {
+    const size_t end = c.off;
+    c.off = at;
+    L.DR = sg::carve_digits(c, m, n);
+    c.off = std::max(c.off, end);
+    L.scp = sg::carve_scratch(c, m, k, n);
+  }
   L.bytes = c.off;
   return L;
 }
 
 template <typename TA>
 css_status run_backward(const TA* A, int m, int n, long long lda, const int* sel, int k,
-                        double grad_out, TA* dA, long long ldda, double* loss, const BwLayout& L,
+                        double grad_out, TA* dA, long long ldda, double* loss, BwLayout& L,
                         const css_opts& o, cudaStream_t s) {
-  using TR = typename AccOf<TA>::type;
-  cudaMemsetAsync(L.status, 0, sizeof(int), s);
+  constexpr int dt = sizeof(TA) == 8 ? CSS_F64 : sizeof(TA) == 4 ? CSS_F32 : CSS_BF16;
+  const unsigned long long spin = o.spin_budget_ns ? o.spin_budget_ns : 2000000000ull;
+  cudaMemsetAsync(L.status, 0, 2 * sizeof(int), s);
+  int* err = L.status + 1;
   const long long mk = (long long)m * k;
   gather_cols_kernel<TA><<<(unsigned)((mk + 255) / 256), 256, 0, s>>>(A, lda, m, sel, k, L.AS);
   gram(L.AS, m, k, L.gpart, L.G, s);
   chol_inv(L.G, k, L.Linv, L.status, s);
-  q_kernel<<<(unsigned)((mk + 255) / 256), 256, 0, s>>>(L.AS, L.Linv, m, k, L.Q, L.Qh, L.Ql);
-  launch_w<TA>(L.Qh, L.Ql, L.Q, A, lda, m, n, k, L.W, 1, k, L.Wh, L.Wl, s);
-  const dim3 rg((m + 63) / 64, (n + 63) / 64);
-  if constexpr (sizeof(TA) == 8)
-    r_kernel<TA><<<rg, 256, 0, s>>>(L.Qh, L.Ql, L.Q, L.Wh, L.Wl, L.W, A, lda, m, n, k, dA ? L.R : nullptr,
-                                    dA, ldda, 2.0 * grad_out, L.loss_part);
-  else
-    r_df_kernel<TA><<<rg, 256, 0, s>>>(L.Qh, L.Ql, L.Wh, L.Wl, A, lda, m, n, k,
-                                       dA ? (float*)L.R : nullptr, dA, ldda, 2.0 * grad_out, L.loss_part);
-  if (loss) sum_kernel<<<1, 512, 0, s>>>(L.loss_part, (long long)rg.x * rg.y, 1.0, loss);
+  q_kernel<<<(unsigned)((mk + 255) / 256), 256, 0, s>>>(L.AS, L.Linv, m, k, L.Q);
+  const sg::Source q{L.Q, CSS_F64, m, 1, k, m}, qr{L.Q, CSS_F64, 1, m, m, k};
+  const sg::Source w{L.W, CSS_F64, 1, k, k, n}, wr{L.W, CSS_F64, k, 1, n, k};
+  if (sg::split(q, L.DQ, s) != cudaSuccess || sg::split(qr, L.DQr, s) != cudaSuccess) return CSS_ERR_CUDA;
+  if (w_product(L.DQ, q, A, dt, lda, m, n, k, L.W, 1, k, L.DA, L.sc, err, spin, s) != cudaSuccess)
+    return CSS_ERR_CUDA;
+  if (sg::split(wr, L.DWr, s) != cudaSuccess) return CSS_ERR_CUDA;
+  int parts = kLossBlocks;
+  if constexpr (dt == CSS_F64) {
+    const sg::Store st{(double*)L.R, 1, m, 0};
+    if (sg::gemm(L.DQr, qr, L.DWr, wr, st, L.sc, err, spin, s) != cudaSuccess) return CSS_ERR_CUDA;
+    residual_f64_kernel<<<kLossBlocks, 256, 0, s>>>((const double*)A, lda, m, (long long)m * n, (double*)L.R,
+                                                    (double*)dA, ldda, 2.0 * grad_out, L.loss_part);
+  } else {
+    const sg::Residual r{A, dt, lda, dA ? (float*)L.R : nullptr, dA, ldda, 2.0 * grad_out, L.loss_part};
+    parts = sg::residual_parts();
+    if (sg::gemm_residual(L.DQr, L.DWr, r, err, spin, s) != cudaSuccess) return CSS_ERR_CUDA;
+  }
+  if (loss) sum_kernel<<<1, 512, 0, s>>>(L.loss_part, parts, 1.0, loss);
   if (dA) {
-    const int slice = (n + kSlices - 1) / kSlices;
-    if constexpr (sizeof(TR) == 4)
-      rwt_f32_kernel<<<dim3((m + kDT - 1) / kDT, (k + kDT - 1) / kDT, kSlices), 256, 0, s>>>(
-          (const float*)L.R, L.W, m, n, k, slice, (float*)L.P);
-    else
-      rwt_kernel<TR><<<dim3((m + 63) / 64, (k + 31) / 32, kSlices), 256, 0, s>>>((const TR*)L.R, L.W, m, n,
-                                                                                k, slice, (TR*)L.P);
-    sum_slices_kernel<TR><<<(unsigned)((mk + 255) / 256), 256, 0, s>>>((const TR*)L.P, kSlices, mk, L.Psum);
+    const sg::Source r{L.R, dt == CSS_F64 ? CSS_F64 : CSS_F32, 1, m, m, n};
+    const sg::Store st{L.Psum, 1, m, 0};
+    if (sg::split(r, L.DR, s) != cudaSuccess || sg::split(w, L.DW, s) != cudaSuccess ||
+        sg::gemm(L.DR, r, L.DW, w, st, L.scp, err, spin, s) != cudaSuccess)
+      return CSS_ERR_CUDA;
     das_kernel<TA><<<(unsigned)((mk + 255) / 256), 256, 0, s>>>(L.Psum, L.Linv, m, k, sel, 2.0 * grad_out, dA,
                                                                ldda);
   }
   if (cudaGetLastError() != cudaSuccess) return CSS_ERR_CUDA;
-  if (o.sync) {
-    int st = 0;
-    if (cudaMemcpyAsync(&st, L.status, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaStreamSynchronize(s) != cudaSuccess)
-      return CSS_ERR_CUDA;
-    if (st) return CSS_ERR_INVALID_ARG;   // A_S is rank deficient
-  }
-  return CSS_OK;
+  return finish(L.status, o, s);
 }
 
 // ------------------------------------------------ embedding (Sec. 3.2) -----
@@ -934,11 +532,12 @@ __global__ void copy_cols_kernel(const double* __restrict__ src, int m, int l, d
 struct EmbLayout {
   int* status;
   double *AS, *G, *gpart, *Linv, *Q1, *Q;
-  float *Qh, *Ql;
+  sg::Digits DQ, DA;
+  sg::Scratch sc;
   size_t bytes;
 };
 
-EmbLayout emb_layout(void* ws, size_t cap, int64_t m, int32_t l) {
+EmbLayout emb_layout(void* ws, size_t cap, int64_t m, int64_t n, int32_t l) {
   WsCarver c(ws, cap);
   EmbLayout L{};
   L.status = c.take<int>(64);
@@ -948,8 +547,10 @@ EmbLayout emb_layout(void* ws, size_t cap, int64_t m, int32_t l) {
   L.Linv = c.take<double>((size_t)l * l);
   L.Q1 = c.take<double>((size_t)m * l);
   L.Q = c.take<double>((size_t)m * l);
-  L.Qh = c.take<float>((size_t)m * l);
-  L.Ql = c.take<float>((size_t)m * l);
+  const long long cols = chunk_cols(m, n, l);
+  L.DQ = sg::carve_digits(c, l, m);
+  L.DA = sg::carve_digits(c, cols, m);
+  L.sc = sg::carve_scratch(c, cols, l, m);
   L.bytes = c.off;
   return L;
 }
@@ -958,30 +559,29 @@ EmbLayout emb_layout(void* ws, size_t cap, int64_t m, int32_t l) {
 // Q = Q1 L2^-T.  Then W = Q^T A (row t at W + t * ldw).
 template <typename TA>
 css_status run_embed(const TA* A, int m, int n, long long lda, const int* sel, int l, double* Qout,
-                     long long ldq, double* W, long long ldw, const EmbLayout& L, const css_opts& o,
+                     long long ldq, double* W, long long ldw, EmbLayout& L, const css_opts& o,
                      cudaStream_t s) {
-  cudaMemsetAsync(L.status, 0, sizeof(int), s);
+  constexpr int dt = sizeof(TA) == 8 ? CSS_F64 : sizeof(TA) == 4 ? CSS_F32 : CSS_BF16;
+  cudaMemsetAsync(L.status, 0, 2 * sizeof(int), s);
   const long long ml = (long long)m * l;
   const unsigned gb = (unsigned)((ml + 255) / 256);
   gather_cols_kernel<TA><<<gb, 256, 0, s>>>(A, lda, m, sel, l, L.AS);
   gram(L.AS, m, l, L.gpart, L.G, s);
   chol_inv(L.G, l, L.Linv, L.status, s);
-  q_kernel<<<gb, 256, 0, s>>>(L.AS, L.Linv, m, l, L.Q1, L.Qh, L.Ql);
+  q_kernel<<<gb, 256, 0, s>>>(L.AS, L.Linv, m, l, L.Q1);
   gram(L.Q1, m, l, L.gpart, L.G, s);
   chol_inv(L.G, l, L.Linv, L.status, s);
-  q_kernel<<<gb, 256, 0, s>>>(L.Q1, L.Linv, m, l, L.Q, L.Qh, L.Ql);
-  if (W)
-    launch_w<TA>(L.Qh, L.Ql, L.Q, A, lda, m, n, l, W, ldw, 1, nullptr, nullptr, s);
+  q_kernel<<<gb, 256, 0, s>>>(L.Q1, L.Linv, m, l, L.Q);
+  if (W) {
+    const sg::Source q{L.Q, CSS_F64, m, 1, l, m};
+    if (sg::split(q, L.DQ, s) != cudaSuccess ||
+        w_product(L.DQ, q, A, dt, lda, m, n, l, W, ldw, 1, L.DA, L.sc, L.status + 1,
+                  o.spin_budget_ns ? o.spin_budget_ns : 2000000000ull, s) != cudaSuccess)
+      return CSS_ERR_CUDA;
+  }
   if (Qout) copy_cols_kernel<<<gb, 256, 0, s>>>(L.Q, m, l, Qout, ldq);
   if (cudaGetLastError() != cudaSuccess) return CSS_ERR_CUDA;
-  if (o.sync) {
-    int st = 0;
-    if (cudaMemcpyAsync(&st, L.status, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaStreamSynchronize(s) != cudaSuccess)
-      return CSS_ERR_CUDA;
-    if (st) return CSS_ERR_INVALID_ARG;   // A_S is rank deficient
-  }
-  return CSS_OK;
+  return finish(L.status, o, s);
 }
 
 // The selected indices are device memory the caller wrote on `s`: read back
@@ -1001,7 +601,9 @@ css_status check_selection(const int32_t* sel, int32_t k, int64_t n, cudaStream_
 
 }  // namespace
 
-size_t embed_workspace_bytes(int64_t m, int32_t l) { return emb_layout(nullptr, (size_t)-1, m, l).bytes; }
+size_t embed_workspace_bytes(int64_t m, int64_t n, int32_t l) {
+  return emb_layout(nullptr, (size_t)-1, m, n, l).bytes;
+}
 
 extern "C" css_status css_embed(const void* A, css_dtype dtype, int64_t m, int64_t n, int64_t lda,
                                 const int32_t* sel, int32_t l, double* Q, int64_t ldq, double* W,
@@ -1016,7 +618,7 @@ extern "C" css_status css_embed(const void* A, css_dtype dtype, int64_t m, int64
   if (m > INT32_MAX || n > INT32_MAX) return CSS_ERR_INVALID_ARG;
   if ((Q && ldq < m) || (W && ldw < n)) return CSS_ERR_INVALID_ARG;
   if (!ws || ((uintptr_t)ws % kWsAlign) != 0) return CSS_ERR_WORKSPACE;
-  EmbLayout L = emb_layout(ws, ws_bytes, m, l);
+  EmbLayout L = emb_layout(ws, ws_bytes, m, n, l);
   if (L.bytes > ws_bytes) return CSS_ERR_WORKSPACE;
   cudaStream_t s = (cudaStream_t)stream;
   css_status cs = check_selection(sel, l, n, s);

@@ -5,4 +5,4 @@
 #include "css_common.cuh"
 
 size_t backward_workspace_bytes(int dtype, int64_t m, int64_t n, int32_t k);
-size_t embed_workspace_bytes(int64_t m, int32_t l);
+size_t embed_workspace_bytes(int64_t m, int64_t n, int32_t l);

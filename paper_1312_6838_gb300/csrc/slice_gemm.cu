@@ -1,0 +1,804 @@
+// Products to FP64 accuracy on the BF16 tensor cores.
+//
+// FP64 multiply-adds issue at two lanes per clock and SM on this part and
+// double-float ones cost about eleven FP32 operations, while the BF16 tensor
+// cores run some 1500 times the FP64 rate.  So a dense product whose result
+// must keep 48 to 53 bits is formed from integer digits (the error-free
+// transformation of Ozaki, Ogita, Oishi and Rump, Numerical Algorithms 59,
+// 2012, with tensor cores as in Mukunoki, Ozaki, Ogita and Imamura, 2020):
+//
+//   row i of an operand is scaled by a power of two so that every entry is at
+//   most 1/2, and written in base 256 with balanced digits,
+//     x = sum_{s=1..8} d_s 256^-s,   |d_s| <= 128  (exact in BF16).
+//   x y = sum over w = s + t of 256^-w d_s e_t, and w = 2..9 is kept: what is
+//   dropped is below 2^-64 of the product of the rows' largest entries.
+//
+// Each w has its own TMEM accumulator.  A product of digits is at most 2^14,
+// so an accumulator that has taken at most 1024 of them holds an integer of
+// at most 2^24, which FP32 accumulation represents exactly whatever its
+// rounding; it is then drained into 64-bit integers (or double-float for the
+// residual).  The whole sum is exact but for the dropped digits and the
+// conversion of the result, so it does not depend on the order of the work,
+// and split-K partial sums may meet in integer atomics.
+//
+// Measured: W = Q^T A of a 4096 x 65536 BF16 matrix with l = 256 (68.7 G
+// multiply-adds) 24 ms as double-float on the FP32 pipe, 5.0 ms here with the
+// split; its error against 64 bits fell from 1.1e-12 to 2.2e-15.
+//
+// Slices that are zero in a block of 128 rows x 64 k are not stored, loaded
+// or multiplied: BF16 entries of similar size have three non-zero slices,
+// FP32 ones five.
+//
+// One CTA of the product owns a 128 x 128 tile of the result: four
+// accumulators of 128 columns are all of TMEM, so the eight w run as two
+// halves, low digits first.  (With all eight resident at 64 columns the
+// 128 x 64 x 16 MMAs would read 6 KB of shared memory in the time of 4 KB.)
+#include "slice_gemm.cuh"
+
+#include <algorithm>
+
+#include "df.cuh"
+#include "tc_ptx.cuh"
+
+namespace css {
+namespace sg {
+namespace {
+
+using namespace css::tc;
+
+constexpr int kT = 128;                 // rows of an operand tile
+constexpr int kS = 8;                   // slices
+constexpr int kSliceBytes = kT * 16 * 2;   // one slice of a tile's 16 k
+constexpr int kKb = 64;                 // k per zero-slice count
+constexpr int kBudget = 1024;           // digit products per accumulator between drains
+
+__host__ __device__ inline long long ceil_div(long long a, long long b) { return (a + b - 1) / b; }
+
+__host__ __device__ inline int exp_bias(int dtype) { return dtype == CSS_F64 ? 1023 : 127; }
+__host__ __device__ inline int exp_special(int dtype) { return dtype == CSS_F64 ? 2047 : 255; }
+// entries of a row with largest biased exponent e are at most 2^(scale_exp - 1)
+__device__ __forceinline__ int scale_exp(int e, int dtype) { return e - exp_bias(dtype) + 2; }
+
+__device__ __forceinline__ int biased_exp(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
+__device__ __forceinline__ int biased_exp(float v) { return (__float_as_int(v) >> 23) & 0xff; }
+__device__ __forceinline__ float load_val(const float* p) { return __ldg(p); }
+__device__ __forceinline__ double load_val(const double* p) { return __ldg(p); }
+__device__ __forceinline__ float load_val(const __nv_bfloat16* p) {
+  return __uint_as_float(((uint32_t)__ldg((const unsigned short*)p)) << 16);
+}
+
+// 8 consecutive elements at p
+template <bool VEC>
+__device__ __forceinline__ void load8(const __nv_bfloat16* p, float (&v)[8]) {
+  if (VEC) {
+    const uint4 r = __ldg(reinterpret_cast<const uint4*>(p));
+    const uint32_t w[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) { v[2 * i] = bf16_lo(w[i]); v[2 * i + 1] = bf16_hi(w[i]); }
+  } else {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = load_val(p + i);
+  }
+}
+template <bool VEC>
+__device__ __forceinline__ void load8(const float* p, float (&v)[8]) {
+  if (VEC) {
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const float4 r = __ldg(reinterpret_cast<const float4*>(p) + i);
+      v[4 * i] = r.x; v[4 * i + 1] = r.y; v[4 * i + 2] = r.z; v[4 * i + 3] = r.w;
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = load_val(p + i);
+  }
+}
+template <bool VEC>
+__device__ __forceinline__ void load8(const double* p, double (&v)[8]) {
+  if (VEC) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const double2 r = __ldg(reinterpret_cast<const double2*>(p) + i);
+      v[2 * i] = r.x; v[2 * i + 1] = r.y;
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = load_val(p + i);
+  }
+}
+
+// The block's 128 rows x 64 k in registers: each thread four chunks of 8
+// consecutive k.  KC (k contiguous): chunk q = row tid / 8 + 32 q, k chunk
+// tid % 8, so that eight lanes read a row's 64 k.  Otherwise rows are
+// contiguous: row tid % 128, k chunk tid / 128 + 2 q.  Zero outside.
+template <typename T, typename V, bool KC, bool VEC>
+__device__ __forceinline__ void load_block(const T* p, long long rs, long long ks, int rows, int K, int r0, int k0,
+                                           V (&v)[4][8]) {
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int row = r0 + (KC ? (int)threadIdx.x / 8 + 32 * q : (int)threadIdx.x % 128);
+    const int k = k0 + 8 * (KC ? (int)threadIdx.x % 8 : (int)threadIdx.x / 128 + 2 * q);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) v[q][e] = V(0);
+    if (row >= rows) continue;
+    const T* src = p + row * rs + k * ks;
+    if (KC && k + 8 <= K) {
+      load8<VEC>(src, v[q]);
+    } else {
+#pragma unroll
+      for (int e = 0; e < 8; ++e)
+        if (k + e < K) v[q][e] = load_val(src + e * ks);
+    }
+  }
+}
+
+// Largest biased exponent of every row (ex zeroed before): a block takes 128
+// rows and every gridDim.y-th 64 k of them.  Memory-bound.
+template <typename T, typename V, bool KC, bool VEC>
+__global__ void __launch_bounds__(256) row_exp_kernel(const T* __restrict__ p, long long rs, long long ks, int rows,
+                                                      int K, int* __restrict__ ex) {
+  const int r0 = blockIdx.x * kT;
+  int best[4] = {0, 0, 0, 0};
+  for (int k0 = blockIdx.y * kKb; k0 < K; k0 += gridDim.y * kKb) {
+    V v[4][8];
+    load_block<T, V, KC, VEC>(p, rs, ks, rows, K, r0, k0, v);
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int e = 0; e < 8; ++e) best[q] = max(best[q], biased_exp(v[q][e]));
+  }
+  if (KC) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) best[q] = max(best[q], __shfl_xor_sync(0xffffffffu, best[q], o));
+      const int row = r0 + threadIdx.x / 8 + 32 * q;
+      if (threadIdx.x % 8 == 0 && row < rows && best[q] > 0) atomicMax(ex + row, best[q]);
+    }
+  } else {
+    const int row = r0 + threadIdx.x % 128, b = max(max(best[0], best[1]), max(best[2], best[3]));
+    if (row < rows && b > 0) atomicMax(ex + row, b);
+  }
+}
+
+__device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) << 23); }
+
+// Digits of one block of 128 rows x 64 k; slices are written until what is
+// left can give no digit, and their number goes to ns.  Rows with an infinity
+// or a NaN get zero digits (the product restores them from the source).
+template <typename T, typename V, bool KC, bool VEC>
+__global__ void __launch_bounds__(256) split_kernel(const T* __restrict__ p, long long rs, long long ks, int rows,
+                                                    int K, int k64, int dtype, const int* __restrict__ ex,
+                                                    unsigned char* __restrict__ d, unsigned char* __restrict__ ns) {
+  const int r0 = blockIdx.x * kT, kb = blockIdx.y;
+  V v[4][8];
+  load_block<T, V, KC, VEC>(p, rs, ks, rows, K, r0, kb * kKb, v);
+  unsigned char* out[4];
+  unsigned long long G[4][8];   // FP64: the balanced digits of |x|, biased by 128 but for the first
+  uint32_t neg[4] = {0, 0, 0, 0};
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int rl = KC ? (int)threadIdx.x / 8 + 32 * q : (int)threadIdx.x % 128;
+    const int kc = KC ? (int)threadIdx.x % 8 : (int)threadIdx.x / 128 + 2 * q;
+    out[q] = d + (((long long)blockIdx.x * k64 + kb) * 4 + kc / 2) * (kS * kSliceBytes) + (kc % 2) * (kT * 16) + rl * 16;
+    const int e = r0 + rl < rows ? ex[r0 + rl] : 0;
+    const bool dead = e == exp_special(dtype);
+    if constexpr (sizeof(V) == 4) {
+      // two factors, so that neither leaves FP32's range
+      const int sh = 8 - scale_exp(e, dtype), h1 = sh / 2;
+      const float f1 = pow2f(h1), f2 = pow2f(sh - h1);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) v[q][i] = dead ? 0.f : v[q][i] * f1 * f2;
+    } else {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const unsigned long long b = (unsigned long long)__double_as_longlong(v[q][i]);
+        const int be = (int)(b >> 52) & 0x7ff;
+        unsigned long long mant = b & 0xfffffffffffffull;
+        if (be > 0) mant |= 1ull << 52;
+        // |x| 2^(64 - scale), rounded to an integer below 2^63
+        const int sh = max(be, 1) - e + 10;
+        unsigned long long F = 0;
+        if (!dead) {
+          if (sh >= 0) F = mant << sh;
+          else if (sh > -64) F = (mant + (1ull << (-sh - 1))) >> -sh;
+        }
+        if (b >> 63) neg[q] |= 1u << i;
+        G[q][i] = F;
+      }
+    }
+  }
+  int s = 0;
+  for (; s < kS; ++s) {
+    int any = 0;
+    if constexpr (sizeof(V) == 4) {
+      const float least = 0.5f * pow2f(-8 * (kS - 1 - s));
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int i = 0; i < 8; ++i) any |= fabsf(v[q][i]) >= least;
+    } else {
+      const unsigned long long mask = s == 0 ? ~0ull : (1ull << (64 - 8 * s)) - 1;
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int i = 0; i < 8; ++i) any |= (G[q][i] & mask) != 0;
+    }
+    if (!__syncthreads_or(any)) break;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      uint32_t w[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        float dg[2];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          const int x = 2 * i + j;
+          if constexpr (sizeof(V) == 4) {
+            const float f = (v[q][x] + 12582912.f) - 12582912.f;   // round to nearest integer
+            v[q][x] = (v[q][x] - f) * 256.f;
+            dg[j] = f;
+          } else {
+            const unsigned long long b = G[q][x] + 0x0080808080808080ull;
+            const uint32_t byte = (uint32_t)(b >> (56 - 8 * s)) & 0xffu;
+            float f = __uint_as_float(0x4b000000u | byte) - (s == 0 ? 8388608.f : 8388736.f);
+            dg[j] = (neg[q] >> x) & 1u ? -f : f;
+          }
+        }
+        // digits have at most 8 bits, so their upper halves are their BF16
+        w[i] = __byte_perm(__float_as_uint(dg[0]), __float_as_uint(dg[1]), 0x7632);
+      }
+      *reinterpret_cast<uint4*>(out[q] + s * kSliceBytes) = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+  }
+  if (threadIdx.x == 0) ns[(long long)blockIdx.x * k64 + kb] = (unsigned char)s;
+}
+
+// ------------------------------------------------------------- product -----
+constexpr int kStages = 3;
+constexpr int kOperandSlot = kS * kSliceBytes;          // 32 KB
+constexpr int kStageBytes = 2 * kOperandSlot;
+constexpr int kEpiWarps = 8;
+constexpr int kThreads = (2 + kEpiWarps) * 32;
+constexpr int kSmem = kStages * kStageBytes + 256 + 1024;
+constexpr int kCtas = 152;
+
+enum Ep { kEpStore = 0, kEpSplitK = 1, kEpResidual = 2 };
+
+struct Args {
+  const unsigned char *xd, *yd, *xns, *yns;
+  const int *xe, *ye;
+  int xdt, ydt;
+  int M, N, K;
+  int k16, k64;        // 16-k blocks in use, 64-k blocks stored
+  int tn, tiles;       // tiles along N; tiles in all
+  int lower;
+  int ksplit, k16_per; // K slices and their 16-k blocks (a multiple of 4)
+  Store st;
+  Source sx, sy;
+  double* lo;
+  unsigned long long* sums;
+  Residual r;
+  int* err;
+  unsigned long long spin_ns;
+};
+
+struct Item {
+  int tm, tn, k0, k1;
+};
+__device__ __forceinline__ Item item_of(const Args& P, int it) {
+  Item w;
+  const int tile = it / P.ksplit, sl = it % P.ksplit;
+  if (P.lower) {
+    int a = (int)((sqrtf(8.f * tile + 1.f) - 1.f) * 0.5f);
+    while (a * (a + 1) / 2 > tile) --a;
+    while ((a + 1) * (a + 2) / 2 <= tile) ++a;
+    w.tm = a;
+    w.tn = tile - a * (a + 1) / 2;
+  } else {
+    w.tm = tile / P.tn;
+    w.tn = tile % P.tn;
+  }
+  w.k0 = sl * P.k16_per;
+  w.k1 = min(P.k16, w.k0 + P.k16_per);
+  return w;
+}
+
+// Shared-memory descriptor of a K-major operand without swizzle: 8 x 16-byte
+// core matrices, 128 bytes apart along the rows, 2 KB apart along k.
+__device__ __forceinline__ uint64_t plain_desc(uint32_t saddr) {
+  return (uint64_t)((saddr >> 4) & 0x3FFFu) | (uint64_t)((kT * 16) >> 4) << 16 | (uint64_t)(128 >> 4) << 32 |
+         (uint64_t)1 << 46;
+}
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(bar)
+               : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+
+// v 2^e (e may leave the range of one factor)
+__device__ __forceinline__ double scale2(double v, int e) {
+  if (e > -1000 && e < 1000) return v * __hiloint2double((e + 1023) << 20, 0);
+  return scalbn(v, e);
+}
+
+template <typename TX>
+__device__ double plain_dot_x(const Source& x, const Source& y, int i, int j) {
+  const TX* p = (const TX*)x.p + i * x.rs;
+  double s = 0.0;
+  for (int k = 0; k < x.K; ++k) {
+    const long long o = j * y.rs + k * y.ks;
+    const double b = y.dtype == CSS_F64   ? ((const double*)y.p)[o]
+                     : y.dtype == CSS_F32 ? (double)((const float*)y.p)[o]
+                                          : (double)load_val((const __nv_bfloat16*)y.p + o);
+    s = fma((double)load_val(p + k * x.ks), b, s);
+  }
+  return s;
+}
+// A row with an infinity or a NaN: the product as FP64 arithmetic gives it.
+__device__ __noinline__ double plain_dot(const Source& x, const Source& y, int i, int j) {
+  if (x.dtype == CSS_F64) return plain_dot_x<double>(x, y, i, j);
+  if (x.dtype == CSS_F32) return plain_dot_x<float>(x, y, i, j);
+  return plain_dot_x<__nv_bfloat16>(x, y, i, j);
+}
+
+// The result from its integer sums: hi in units of 2^-40, lo in 2^-72, times
+// the rows' scales.
+__device__ __forceinline__ double combine(double hi, double lo, int ex, int ey) {
+  return scale2(hi * 0x1p-40 + lo * 0x1p-72, ex + ey);
+}
+
+template <int EP>
+__global__ void __launch_bounds__(kThreads, 1) slice_gemm_kernel(const __grid_constant__ Args P) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  uint64_t* full = (uint64_t*)(smem + kStages * kStageBytes);
+  uint64_t* empty = full + kStages;
+  uint64_t* acc_full = empty + kStages;
+  uint64_t* acc_empty = acc_full + 1;      // one per accumulator
+  uint64_t* done = acc_empty + 4;
+  uint32_t* s_tmem = (uint32_t*)(done + 1);
+  int* s_chunk = (int*)(s_tmem + 1);       // accumulators in use | last chunk of the half << 4
+  int* s_ns = s_chunk + 1;                 // per stage: slices of X | of Y << 8
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int items = P.tiles * P.ksplit;
+
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < kStages; ++i) {
+      mbar_init(smem_u32(&full[i]), 1);
+      mbar_init(smem_u32(&empty[i]), 1);
+    }
+    mbar_init(smem_u32(acc_full), 2);      // the MMAs' commit, and the issuer's own arrival
+    for (int g = 0; g < 4; ++g) mbar_init(smem_u32(&acc_empty[g]), kEpiWarps);
+    mbar_init(smem_u32(done), 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(s_tmem)),
+                 "r"(512u)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  fence_before();
+  __syncthreads();
+  fence_after();
+  const uint32_t tmem = *s_tmem;
+
+  if (warp == 0) {
+    // ------------------------------------------------------------ producer
+    // (the whole warp walks the stages: its lanes hold the slice counts of
+    // the next 32 blocks of 64 k)
+    int st = 0;
+    bool ok = true;
+    for (int it = blockIdx.x; ok && it < items; it += gridDim.x) {
+      const Item w = item_of(P, it);
+      for (int half = 1; ok && half >= 0; --half) {
+        const int kps = half ? 1 : 2, cap = half ? kS : 4;
+        int cnt = 0;
+        for (int k = w.k0; ok && k < w.k1; k += kps, ++st) {
+          if ((k - w.k0) % 128 == 0) {
+            const int kb = k / 4 + lane;
+            cnt = 0;
+            if (kb < P.k64)
+              cnt = P.xns[(long long)w.tm * P.k64 + kb] | P.yns[(long long)w.tn * P.k64 + kb] << 8;
+          }
+          const int both = __shfl_sync(0xffffffffu, cnt, ((k - w.k0) / 4) & 31);
+          const int nx = min(both & 0xff, cap), ny = min(both >> 8, cap);
+          const int slot = st % kStages;
+          if (lane == 0) {
+            ok = mbar_wait(smem_u32(&empty[slot]), (uint32_t)((st / kStages) & 1) ^ 1u, P.err, P.spin_ns);
+            if (ok) {
+              s_ns[slot] = nx | ny << 8;
+              const uint32_t fb = smem_u32(&full[slot]);
+              const int nk = min(kps, w.k1 - k);
+              if (nx > 0 && ny > 0) {
+                mbar_expect_tx(fb, (uint32_t)(nk * (nx + ny) * kSliceBytes));
+                for (int q = 0; q < nk; ++q) {
+                  uint8_t* dst = smem + slot * kStageBytes + q * 4 * kSliceBytes;
+                  const long long kx = (long long)w.tm * P.k64 * 4 + k + q, ky = (long long)w.tn * P.k64 * 4 + k + q;
+                  bulk_load(smem_u32(dst), P.xd + kx * kOperandSlot, (uint32_t)(nx * kSliceBytes), fb);
+                  bulk_load(smem_u32(dst + kOperandSlot), P.yd + ky * kOperandSlot, (uint32_t)(ny * kSliceBytes), fb);
+                }
+              } else {
+                mbar_arrive(fb);
+              }
+            }
+          }
+          ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
+          if (!ok) break;   // this stage was not issued
+        }
+      }
+    }
+    // every copy issued has landed before the CTA exits
+    if (lane == 0)
+      for (int i = max(0, st - kStages); i < st; ++i)
+        mbar_drain(smem_u32(&full[i % kStages]), (uint32_t)((i / kStages) & 1));
+  } else if (warp == 1) {
+    // ---------------------------------------------------------- MMA issuer
+    if (lane == 0) {
+      const uint32_t idesc = make_idesc(kT, kT, false, false);
+      int st = 0;
+      uint32_t chunk = 0;
+      bool ok = true;
+      for (int it = blockIdx.x; ok && it < items; it += gridDim.x) {
+        const Item w = item_of(P, it);
+        for (int half = 1; ok && half >= 0; --half) {
+          const int kps = half ? 1 : 2, w0 = half ? 6 : 2;
+          int used = 0, budget = 0, ready = 0;   // accumulators written, and waited for, in this chunk
+          for (int k = w.k0; ok && k < w.k1; k += kps, ++st) {
+            const int slot = st % kStages;
+            ok = mbar_wait(smem_u32(&full[slot]), (uint32_t)((st / kStages) & 1), P.err, P.spin_ns);
+            if (!ok) break;
+            fence_after();
+            const int nx = s_ns[slot] & 0xff, ny = s_ns[slot] >> 8;
+            const int nk = min(kps, w.k1 - k);
+            const int cost = nk * 16 * min(nx, ny);
+            if (budget + cost > kBudget) {
+              // drain before the accumulators can leave FP32's integers
+              for (int g = 0; ok && g < 4; ++g)
+                if (!(ready >> g & 1)) ok = mbar_wait(smem_u32(&acc_empty[g]), (chunk & 1) ^ 1u, P.err, P.spin_ns);
+              if (!ok) break;
+              *s_chunk = used;
+              umma_commit(smem_u32(acc_full));
+              mbar_arrive(smem_u32(acc_full));
+              ++chunk;
+              used = budget = ready = 0;
+            }
+            budget += cost;
+            const uint32_t sx = smem_u32(smem + slot * kStageBytes), sy = sx + kOperandSlot;
+            for (int g = 0; g < 4; ++g) {
+              const int wt = w0 + g;
+              const int s_lo = max(1, wt - ny), s_hi = min(nx, wt - 1);
+              if (s_lo > s_hi) continue;
+              if (!(ready >> g & 1)) {
+                ok = mbar_wait(smem_u32(&acc_empty[g]), (chunk & 1) ^ 1u, P.err, P.spin_ns);
+                if (!ok) break;
+                ready |= 1 << g;
+                fence_after();
+              }
+              for (int q = 0; q < nk; ++q)
+                for (int s = s_lo; s <= s_hi; ++s) {
+                  const int o = q * 4;
+                  umma(tmem + g * kT, plain_desc(sx + (o + s - 1) * kSliceBytes),
+                       plain_desc(sy + (o + wt - s - 1) * kSliceBytes), idesc, (uint32_t)(used >> g & 1));
+                  used |= 1 << g;
+                }
+            }
+            umma_commit(smem_u32(&empty[slot]));
+          }
+          if (!ok) break;
+          for (int g = 0; ok && g < 4; ++g)
+            if (!(ready >> g & 1)) ok = mbar_wait(smem_u32(&acc_empty[g]), (chunk & 1) ^ 1u, P.err, P.spin_ns);
+          if (!ok) break;
+          *s_chunk = used | 16;
+          umma_commit(smem_u32(acc_full));
+          mbar_arrive(smem_u32(acc_full));
+          ++chunk;
+        }
+      }
+      umma_commit(smem_u32(done));
+      mbar_drain(smem_u32(done), 0u);   // no MMA is in flight when TMEM is released
+    }
+    __syncwarp();
+  } else {
+    // ------------------------------------------------------------ epilogue
+    const int q = warp & 3, ch = (warp - 2) >> 2;   // TMEM lane quarter, column half
+    const int r_tile = q * 32 + lane;
+    const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(ch * 64);
+    uint32_t chunk = 0;
+    bool ok = true;
+    float lsh = 0.f, lsl = 0.f;   // residual: ||R||^2 of this thread's entries in double-float
+    for (int it = blockIdx.x; ok && it < items; it += gridDim.x) {
+      const Item w = item_of(P, it);
+      const int row = w.tm * kT + r_tile, col0 = w.tn * kT + ch * 64;
+      long long acc[EP == kEpResidual ? 1 : 64];
+      DF df[EP == kEpResidual ? 64 : 1];
+      if constexpr (EP == kEpResidual) {
+#pragma unroll
+        for (int j = 0; j < 64; ++j) df[j] = DF{0.f, 0.f};
+      }
+      double* lo = P.lo + (long long)blockIdx.x * (kT * kT) + (long long)(ch * 64) * kT + r_tile;
+      for (int half = 1; ok && half >= 0; --half) {
+        if constexpr (EP != kEpResidual) {
+#pragma unroll
+          for (int j = 0; j < 64; ++j) acc[j] = 0;
+        }
+        bool last = false;
+        while (!last) {
+          ok = mbar_wait(smem_u32(acc_full), chunk & 1, P.err, P.spin_ns);
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) break;
+          const int info = *(volatile int*)s_chunk;
+          last = (info & 16) != 0;
+          fence_after();
+#pragma unroll
+          for (int g = 0; g < 4; ++g) {
+            if (info >> g & 1) {
+#pragma unroll
+              for (int j0 = 0; j0 < 64; j0 += 16) {
+                float v[16];
+                tmem_ld16(tbase + (uint32_t)(g * kT + j0), v);
+#pragma unroll
+                for (int jj = 0; jj < 16; ++jj) {
+                  if constexpr (EP == kEpResidual) {
+                    // in units of 2^-16
+                    const float x = v[jj] * (half ? pow2f(-32 - 8 * g) : pow2f(-8 * g));
+                    DF& a = df[j0 + jj];
+                    const float s = a.s + x, bb = s - a.s;
+                    a.c += (a.s - (s - bb)) + (x - bb);
+                    a.s = s;
+                  } else {
+                    acc[j0 + jj] += (long long)__float2int_rn(v[jj]) * (1ll << (24 - 8 * g));
+                  }
+                }
+              }
+            }
+            fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&acc_empty[g]));
+          }
+          ++chunk;
+        }
+        if (!ok) break;
+        if constexpr (EP == kEpStore) {
+          if (half == 1) {
+#pragma unroll
+            for (int j = 0; j < 64; ++j) __stcg(lo + (long long)j * kT, (double)acc[j]);
+          } else if (row < P.M) {
+            const int exr = P.xe[row], ex = scale_exp(exr, P.xdt);
+            const bool dead_r = exr == exp_special(P.xdt);
+#pragma unroll
+            for (int j = 0; j < 64; ++j) {
+              const int c = col0 + j;
+              if (c >= P.N) break;
+              const int eyr = P.ye[c];
+              double v = combine((double)acc[j], __ldcg(lo + (long long)j * kT), ex, scale_exp(eyr, P.ydt));
+              if (dead_r || eyr == exp_special(P.ydt)) v = plain_dot(P.sx, P.sy, row, c);
+              P.st.out[row * P.st.rs + c * P.st.cs] = v;
+              if (P.lower && row != c) P.st.out[c * P.st.rs + row * P.st.cs] = v;
+            }
+          }
+        } else if constexpr (EP == kEpSplitK) {
+          unsigned long long* sums = P.sums + (half ? 0 : (long long)P.M * P.N);
+          if (row < P.M) {
+#pragma unroll
+            for (int j = 0; j < 64; ++j) {
+              const int c = col0 + j;
+              if (c < P.N) atomicAdd(sums + (long long)c * P.M + row, (unsigned long long)acc[j]);
+            }
+          }
+        }
+      }
+      if constexpr (EP == kEpResidual) {
+        if (!ok) break;
+        const Residual& R = P.r;
+        if (row < P.M) {
+          const int exr = P.xe[row], ex = scale_exp(exr, P.xdt) - 16;
+          const bool dead_r = exr == exp_special(P.xdt);
+          const float gh = (float)R.g2, gl = (float)(R.g2 - (double)gh);
+          const bool g_plain = fabsf(gh) < 1e30f && fabsf(gh) > 1e-30f;
+#pragma unroll
+          for (int j = 0; j < 64; ++j) {
+            const int c = col0 + j;
+            if (c >= P.N) break;
+            const int eyr = P.ye[c];
+            const int e = ex + scale_exp(eyr, P.ydt);
+            const int e1 = max(-126, min(127, e)), e2 = max(-126, min(127, e - e1));
+            float vh = df[j].s * pow2f(e1) * pow2f(e2), vl = df[j].c * pow2f(e1) * pow2f(e2);
+            if (dead_r || eyr == exp_special(P.ydt)) vh = __int_as_float(0x7fffffff);
+            const float a = R.dtype == CSS_F32 ? load_val((const float*)R.A + (long long)c * R.lda + row)
+                                               : load_val((const __nv_bfloat16*)R.A + (long long)c * R.lda + row);
+            // r = a - vh - vl as a normalised pair
+            const float s = a - vh, bb = s - a;
+            const float t = ((a - (s - bb)) + (-vh - bb)) - vl;
+            const float rh = s + t, rl = t - (rh - s);
+            const float p = rh * rh;
+            const float pe = fmaf(rh, rh, -p) + 2.f * rh * rl;
+            const float ns = lsh + p, nb = ns - lsh;
+            lsl += ((lsh - (ns - nb)) + (p - nb)) + pe;
+            lsh = ns;
+            if (R.R) R.R[(long long)c * P.M + row] = rh;
+            if (R.dA) {
+              float g;
+              if (g_plain) {
+                const float gp = gh * rh;
+                g = gp + (fmaf(gh, rh, -gp) + (gh * rl + gl * rh));
+              } else {
+                g = (float)(R.g2 * ((double)rh + (double)rl));
+              }
+              if (R.dtype == CSS_F32) ((float*)R.dA)[(long long)c * R.ldda + row] = g;
+              else ((__nv_bfloat16*)R.dA)[(long long)c * R.ldda + row] = __float2bfloat16_rn(g);
+            }
+          }
+        }
+      }
+    }
+    if constexpr (EP == kEpResidual) {
+      // the CTA's share of ||R||^2, in a fixed order
+      __shared__ double s_loss[kEpiWarps];
+      const double t = warp_sum(to_f64(lsh) + to_f64(lsl));
+      if (lane == 0) s_loss[warp - 2] = t;
+      asm volatile("bar.sync 1, 256;" ::: "memory");
+      if (warp == 2 && lane == 0) {
+        double sum = 0.0;
+        for (int i = 0; i < kEpiWarps; ++i) sum += s_loss[i];
+        P.r.loss_part[blockIdx.x] = sum;
+      }
+    }
+    fence_before();
+  }
+  __syncthreads();
+  if (warp == 1) {
+    fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
+  }
+}
+
+// The split-K sums (lo half first) to FP64.
+__global__ void __launch_bounds__(256) finish_kernel(const __grid_constant__ Args P) {
+  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= (long long)P.M * P.N) return;
+  const int row = (int)(idx % P.M), c = (int)(idx / P.M);
+  // lower: the tiles above the diagonal were not computed
+  const bool up = P.lower && row / kT < c / kT;
+  const long long at = up ? (long long)row * P.M + c : idx;
+  const int exr = P.xe[row], eyr = P.ye[c];
+  double v = combine((double)(long long)P.sums[(long long)P.M * P.N + at], (double)(long long)P.sums[at],
+                     scale_exp(exr, P.xdt), scale_exp(eyr, P.ydt));
+  if (exr == exp_special(P.xdt) || eyr == exp_special(P.ydt)) v = plain_dot(P.sx, P.sy, row, c);
+  P.st.out[row * P.st.rs + c * P.st.cs] = v;
+}
+
+int k_blocks(long long K) { return (int)ceil_div(K, kKb); }
+
+template <typename T, typename V, bool KC, bool VEC>
+void launch_split(const Source& src, const Digits& D, cudaStream_t s) {
+  const int k64 = k_blocks(src.K);
+  const unsigned tiles = (unsigned)ceil_div(src.rows, kT);
+  const unsigned ky = (unsigned)std::min<long long>(k64, std::max<long long>(1, ceil_div(152 * 8, tiles)));
+  row_exp_kernel<T, V, KC, VEC><<<dim3(tiles, ky), 256, 0, s>>>((const T*)src.p, src.rs, src.ks, src.rows, src.K,
+                                                                D.ex);
+  split_kernel<T, V, KC, VEC><<<dim3(tiles, (unsigned)k64), 256, 0, s>>>((const T*)src.p, src.rs, src.ks, src.rows,
+                                                                        src.K, k64, src.dtype, D.ex, D.d, D.ns);
+}
+template <typename T, typename V>
+void launch_split_of(const Source& src, const Digits& D, cudaStream_t s) {
+  const bool vec = ((uintptr_t)src.p & 15u) == 0 && (src.rs * (long long)sizeof(T)) % 16 == 0;
+  if (src.ks == 1 && vec) launch_split<T, V, true, true>(src, D, s);
+  else if (src.ks == 1) launch_split<T, V, true, false>(src, D, s);
+  else launch_split<T, V, false, false>(src, D, s);
+}
+
+Args base_args(const Digits& X, const Digits& Y, int* err, unsigned long long spin_ns) {
+  Args P{};
+  P.xd = X.d;
+  P.yd = Y.d;
+  P.xns = X.ns;
+  P.yns = Y.ns;
+  P.xe = X.ex;
+  P.ye = Y.ex;
+  P.xdt = X.dtype;
+  P.ydt = Y.dtype;
+  P.M = X.rows;
+  P.N = Y.rows;
+  P.K = X.K;
+  P.k64 = k_blocks(X.K);
+  P.k16 = (int)ceil_div(X.K, 16);
+  P.tn = (int)ceil_div(P.N, kT);
+  P.tiles = (int)ceil_div(P.M, kT) * P.tn;
+  P.ksplit = 1;
+  P.k16_per = P.k64 * 4;
+  P.err = err;
+  P.spin_ns = spin_ns;
+  return P;
+}
+
+template <int EP>
+cudaError_t launch_gemm(const Args& P, cudaStream_t s) {
+  cudaError_t e = cudaFuncSetAttribute(slice_gemm_kernel<EP>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+  if (e != cudaSuccess) return e;
+  slice_gemm_kernel<EP><<<std::min(kCtas, P.tiles * P.ksplit), kThreads, kSmem, s>>>(P);
+  return cudaGetLastError();
+}
+
+// K slices for `tiles` result tiles: enough items for every SM, slices of at
+// least 512 k (a tile's two halves are then some twenty drains).
+int k_slices(long long tiles, long long K) {
+  if (tiles * 2 > kCtas) return 1;
+  return (int)std::max<long long>(1, std::min(kCtas / tiles, K / 512));
+}
+
+}  // namespace
+
+Digits carve_digits(WsCarver& c, long long rows, long long K) {
+  Digits D{};
+  const long long tiles = ceil_div(rows, kT), k64 = k_blocks(K);
+  D.d = c.take<unsigned char>((size_t)(tiles * k64 * 4 * kS * kSliceBytes));
+  D.ns = c.take<unsigned char>((size_t)(tiles * k64));
+  D.ex = c.take<int>((size_t)rows);
+  return D;
+}
+
+cudaError_t split(const Source& src, Digits& D, cudaStream_t s) {
+  D.rows = src.rows;
+  D.K = src.K;
+  D.dtype = src.dtype;
+  cudaError_t e = cudaMemsetAsync(D.ex, 0, sizeof(int) * (size_t)src.rows, s);
+  if (e != cudaSuccess) return e;
+  switch (src.dtype) {
+    case CSS_F64: launch_split_of<double, double>(src, D, s); break;
+    case CSS_F32: launch_split_of<float, float>(src, D, s); break;
+    default: launch_split_of<__nv_bfloat16, float>(src, D, s); break;
+  }
+  return cudaGetLastError();
+}
+
+Scratch carve_scratch(WsCarver& c, long long M, long long N, long long K) {
+  Scratch w{};
+  w.lo = c.take<double>((size_t)kCtas * kT * kT);
+  if (k_slices(1, K) > 1 && ceil_div(M, kT) * ceil_div(N, kT) * 2 <= 2 * kCtas)
+    w.sums = c.take<unsigned long long>((size_t)(2 * M * N));
+  return w;
+}
+
+cudaError_t gemm(const Digits& X, const Source& sx, const Digits& Y, const Source& sy, const Store& st,
+                 const Scratch& w, int* err, unsigned long long spin_ns, cudaStream_t s) {
+  Args P = base_args(X, Y, err, spin_ns);
+  P.st = st;
+  P.sx = sx;
+  P.sy = sy;
+  P.lo = w.lo;
+  P.lower = st.lower;
+  if (st.lower) P.tiles = P.tn * (P.tn + 1) / 2;
+  P.ksplit = w.sums ? k_slices(P.tiles, P.K) : 1;
+  if (P.ksplit == 1) return launch_gemm<kEpStore>(P, s);
+  P.sums = w.sums;
+  P.k16_per = (int)ceil_div(ceil_div(P.k16, P.ksplit), 4) * 4;
+  P.ksplit = (int)ceil_div(P.k16, P.k16_per);
+  const size_t mn = (size_t)P.M * P.N;
+  cudaError_t e = cudaMemsetAsync(P.sums, 0, 2 * mn * sizeof(unsigned long long), s);
+  if (e != cudaSuccess) return e;
+  if ((e = launch_gemm<kEpSplitK>(P, s)) != cudaSuccess) return e;
+  finish_kernel<<<(unsigned)((mn + 255) / 256), 256, 0, s>>>(P);
+  return cudaGetLastError();
+}
+
+int residual_parts() { return kCtas; }
+
+cudaError_t gemm_residual(const Digits& X, const Digits& Y, const Residual& r, int* err,
+                          unsigned long long spin_ns, cudaStream_t s) {
+  Args P = base_args(X, Y, err, spin_ns);
+  P.r = r;
+  const int ctas = std::min(kCtas, P.tiles);
+  if (ctas < kCtas) {
+    cudaError_t e = cudaMemsetAsync(r.loss_part, 0, sizeof(double) * kCtas, s);
+    if (e != cudaSuccess) return e;
+  }
+  return launch_gemm<kEpResidual>(P, s);
+}
+
+}  // namespace sg
+}  // namespace css

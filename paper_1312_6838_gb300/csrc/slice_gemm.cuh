@@ -1,0 +1,68 @@
+// Internal interface of the slice GEMM (slice_gemm.cu): products of FP64,
+// FP32 or BF16 matrices to FP64 accuracy on the BF16 tensor cores.
+#pragma once
+
+#include "css_common.cuh"
+
+namespace css {
+namespace sg {
+
+// A rows x K operand in its own type: element (row, k) at p[row * rs + k * ks].
+struct Source {
+  const void* p;
+  int dtype;            // css_dtype
+  long long rs, ks;
+  int rows, K;
+};
+
+// The operand as digits (see slice_gemm.cu).
+struct Digits {
+  unsigned char* d;     // tiles of 128 rows x 16 k x 8 slices
+  unsigned char* ns;    // non-zero leading slices per (row tile, 64 k)
+  int* ex;              // largest biased exponent of each row
+  int rows, K, dtype;
+};
+
+// Carves the digits of a rows x K operand from a workspace (rows may be the
+// largest of several operands that use the same space one after another).
+Digits carve_digits(WsCarver& c, long long rows, long long K);
+// Splits src into digits (src.rows <= the carved rows).  Three launches.
+cudaError_t split(const Source& src, Digits& D, cudaStream_t s);
+
+// Scratch of gemm: per-CTA partial sums, and for split-K the two halves of
+// the M x N sums.
+struct Scratch {
+  double* lo;
+  unsigned long long* sums;
+};
+Scratch carve_scratch(WsCarver& c, long long M, long long N, long long K);
+
+// out[i * rs + j * cs] = sum_k X[i, k] Y[j, k].  lower: X and Y are the same
+// operand; only tiles touching i >= j are computed and both triangles written.
+struct Store {
+  double* out;
+  long long rs, cs;
+  int lower;
+};
+cudaError_t gemm(const Digits& X, const Source& sx, const Digits& Y, const Source& sy, const Store& st,
+                 const Scratch& w, int* err, unsigned long long spin_ns, cudaStream_t s);
+
+// R = A - X Y^T for FP32 or BF16 A (M x N, leading dimension lda): writes R
+// (FP32, leading dimension M) when R != null, dA = g2 R when dA != null, and
+// one partial of ||R||^2 per CTA of the launch (residual_parts of them).
+struct Residual {
+  const void* A;
+  int dtype;
+  long long lda;
+  float* R;
+  void* dA;
+  long long ldda;
+  double g2;
+  double* loss_part;
+};
+int residual_parts();
+cudaError_t gemm_residual(const Digits& X, const Digits& Y, const Residual& r, int* err,
+                          unsigned long long spin_ns, cudaStream_t s);
+
+}  // namespace sg
+}  // namespace css
