@@ -259,7 +259,11 @@ constexpr int kStages = 3;
 constexpr int kOperandSlot = kS * kSliceBytes;          // 32 KB
 constexpr int kStageBytes = 2 * kOperandSlot;
 constexpr int kEpiWarps = 8;
-constexpr int kThreads = (2 + kEpiWarps) * 32;
+constexpr int kThreads = (4 + kEpiWarps) * 32;
+// 168 registers a thread at launch; the epilogue's two warpgroups take those
+// that the first one (producer, MMA issuer, two idle warps) gives back
+constexpr int kRegsIssue = 56, kRegsEpi = 224;
+static_assert(4 * kRegsIssue + kEpiWarps * kRegsEpi <= (4 + kEpiWarps) * 168, "within the launch's registers");
 constexpr int kSmem = kStages * kStageBytes + 256 + 1024;
 constexpr int kCtas = 152;
 
@@ -304,11 +308,24 @@ __device__ __forceinline__ Item item_of(const Args& P, int it) {
   return w;
 }
 
-// Shared-memory descriptor of a K-major operand without swizzle: 8 x 16-byte
-// core matrices, 128 bytes apart along the rows, 2 KB apart along k.
-__device__ __forceinline__ uint64_t plain_desc(uint32_t saddr) {
-  return (uint64_t)((saddr >> 4) & 0x3FFFu) | (uint64_t)((kT * 16) >> 4) << 16 | (uint64_t)(128 >> 4) << 32 |
-         (uint64_t)1 << 46;
+// Shared-memory descriptors of a K-major operand without swizzle: 8 x 16-byte
+// core matrices, 128 bytes apart along the rows, 2 KB apart along k.  Only the
+// address field (16-byte units) changes from one MMA to the next.
+constexpr uint32_t kDescHi = (128u >> 4) | 1u << 14;
+__device__ __forceinline__ uint32_t desc_lo(uint32_t saddr) { return (saddr >> 4) | (uint32_t)((kT * 16) >> 4) << 16; }
+constexpr uint32_t kDescSlice = kSliceBytes >> 4;
+// The elected lane issues; the whole warp walks the loops around it with
+// warp-uniform values, so that addresses and descriptors live in uniform
+// registers: a 128 x 128 x 16 MMA takes 64 clocks, less than moving its
+// operands there from a divergent thread's registers.
+__device__ __forceinline__ void umma_slices(uint32_t elected, uint32_t tmem_d, uint32_t xlo, uint32_t ylo,
+                                            uint32_t idesc, uint32_t acc) {
+  asm volatile(
+      "{\n .reg .pred p, q;\n .reg .b64 da, db;\n setp.ne.b32 p, %5, 0;\n setp.ne.b32 q, %6, 0;\n"
+      " mov.b64 da, {%1, %4};\n mov.b64 db, {%2, %4};\n"
+      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, p;\n}" ::"r"(tmem_d),
+      "r"(xlo), "r"(ylo), "r"(idesc), "r"(kDescHi), "r"(acc), "r"(elected)
+      : "memory");
 }
 __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
@@ -351,6 +368,24 @@ __device__ __forceinline__ double combine(double hi, double lo, int ex, int ey) 
   return scale2(hi * 0x1p-40 + lo * 0x1p-72, ex + ey);
 }
 
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t e;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}" : "=r"(e));
+  return e;
+}
+// mbar_wait by the whole warp, with one answer
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, int* err, unsigned long long budget) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, err, budget));
+}
+
+// N columns of this warp's TMEM lanes
+template <int N>
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, float (&v)[N]) {
+  static_assert(N == 16, "one load");
+  tmem_ld16(taddr, v);
+}
+constexpr int kLd = 16;
+
 template <int EP>
 __global__ void __launch_bounds__(kThreads, 1) slice_gemm_kernel(const __grid_constant__ Args P) {
   extern __shared__ uint8_t smem_raw[];
@@ -387,6 +422,8 @@ __global__ void __launch_bounds__(kThreads, 1) slice_gemm_kernel(const __grid_co
   fence_after();
   const uint32_t tmem = *s_tmem;
 
+  if (warp < 4) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsIssue));
   if (warp == 0) {
     // ------------------------------------------------------------ producer
     // (the whole warp walks the stages: its lanes hold the slice counts of
@@ -438,74 +475,91 @@ __global__ void __launch_bounds__(kThreads, 1) slice_gemm_kernel(const __grid_co
         mbar_drain(smem_u32(&full[i % kStages]), (uint32_t)((i / kStages) & 1));
   } else if (warp == 1) {
     // ---------------------------------------------------------- MMA issuer
-    if (lane == 0) {
-      const uint32_t idesc = make_idesc(kT, kT, false, false);
-      int st = 0;
-      uint32_t chunk = 0;
-      bool ok = true;
-      for (int it = blockIdx.x; ok && it < items; it += gridDim.x) {
-        const Item w = item_of(P, it);
-        for (int half = 1; ok && half >= 0; --half) {
-          const int kps = half ? 1 : 2, w0 = half ? 6 : 2;
-          int used = 0, budget = 0, ready = 0;   // accumulators written, and waited for, in this chunk
-          for (int k = w.k0; ok && k < w.k1; k += kps, ++st) {
-            const int slot = st % kStages;
-            ok = mbar_wait(smem_u32(&full[slot]), (uint32_t)((st / kStages) & 1), P.err, P.spin_ns);
+    const uint32_t idesc = make_idesc(kT, kT, false, false);
+    const uint32_t elected = elect_one();
+    const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+    const uint32_t base = smem_u32(smem);
+    int st = 0, slot = 0;
+    uint32_t chunk = 0, ph = 0;
+    bool ok = true;
+    // the accumulators not yet waited for in this chunk, then its end
+    auto finish_chunk = [&](int used, int ready, int last) {
+      for (int g = 0; ok && g < 4; ++g)
+        if (!(ready >> g & 1)) ok = mbar_wait_warp(smem_u32(&acc_empty[g]), (chunk & 1) ^ 1u, P.err, P.spin_ns);
+      if (!ok) return;
+      if (elected) {
+        *s_chunk = used | last;
+        umma_commit(smem_u32(acc_full));
+        mbar_arrive(smem_u32(acc_full));
+      }
+      __syncwarp();
+      ++chunk;
+    };
+    for (int it = blockIdx.x; ok && it < items; it += gridDim.x) {
+      const Item w = item_of(P, it);
+      for (int half = 1; ok && half >= 0; --half) {
+        const int kps = half ? 1 : 2, w0 = half ? 6 : 2;
+        int used = 0, budget = 0, ready = 0;   // accumulators written, and waited for, in this chunk
+        for (int k = w.k0; k < w.k1; k += kps, ++st) {
+          ok = mbar_wait_warp(smem_u32(&full[slot]), ph, P.err, P.spin_ns);
+          if (!ok) break;
+          fence_after();
+          const int both = __shfl_sync(0xffffffffu, s_ns[slot], 0);
+          const int nx = both & 0xff, ny = both >> 8;
+          const int nk = min(kps, w.k1 - k);
+          const int cost = nk * 16 * min(nx, ny);
+          if (budget + cost > kBudget) {
+            // drain before the accumulators can leave FP32's integers
+            finish_chunk(used, ready, 0);
             if (!ok) break;
-            fence_after();
-            const int nx = s_ns[slot] & 0xff, ny = s_ns[slot] >> 8;
-            const int nk = min(kps, w.k1 - k);
-            const int cost = nk * 16 * min(nx, ny);
-            if (budget + cost > kBudget) {
-              // drain before the accumulators can leave FP32's integers
-              for (int g = 0; ok && g < 4; ++g)
-                if (!(ready >> g & 1)) ok = mbar_wait(smem_u32(&acc_empty[g]), (chunk & 1) ^ 1u, P.err, P.spin_ns);
+            used = budget = ready = 0;
+          }
+          budget += cost;
+          const uint32_t dx = desc_lo(base + slot * kStageBytes), dy = dx + (kOperandSlot >> 4);
+#pragma unroll
+          for (int g = 0; g < 4; ++g) {
+            const int wt = w0 + g;
+            const int s_lo = max(1, wt - ny), s_hi = min(nx, wt - 1);
+            if (s_lo > s_hi) continue;
+            if (!(ready >> g & 1)) {
+              ok = ok && mbar_wait_warp(smem_u32(&acc_empty[g]), (chunk & 1) ^ 1u, P.err, P.spin_ns);
               if (!ok) break;
-              *s_chunk = used;
-              umma_commit(smem_u32(acc_full));
-              mbar_arrive(smem_u32(acc_full));
-              ++chunk;
-              used = budget = ready = 0;
+              ready |= 1 << g;
+              fence_after();
             }
-            budget += cost;
-            const uint32_t sx = smem_u32(smem + slot * kStageBytes), sy = sx + kOperandSlot;
-            for (int g = 0; g < 4; ++g) {
-              const int wt = w0 + g;
-              const int s_lo = max(1, wt - ny), s_hi = min(nx, wt - 1);
-              if (s_lo > s_hi) continue;
-              if (!(ready >> g & 1)) {
-                ok = mbar_wait(smem_u32(&acc_empty[g]), (chunk & 1) ^ 1u, P.err, P.spin_ns);
-                if (!ok) break;
-                ready |= 1 << g;
-                fence_after();
+            uint32_t acc = used >> g & 1;
+            used |= 1 << g;
+            for (int q = 0; q < nk; ++q) {
+              uint32_t xl = dx + (q * 4 + s_lo - 1) * kDescSlice, yl = dy + (q * 4 + wt - s_lo - 1) * kDescSlice;
+              for (int s = s_lo; s <= s_hi; ++s) {
+                umma_slices(elected, tm + g * kT, xl, yl, idesc, acc);
+                acc = 1;
+                xl += kDescSlice;
+                yl -= kDescSlice;
               }
-              for (int q = 0; q < nk; ++q)
-                for (int s = s_lo; s <= s_hi; ++s) {
-                  const int o = q * 4;
-                  umma(tmem + g * kT, plain_desc(sx + (o + s - 1) * kSliceBytes),
-                       plain_desc(sy + (o + wt - s - 1) * kSliceBytes), idesc, (uint32_t)(used >> g & 1));
-                  used |= 1 << g;
-                }
             }
-            umma_commit(smem_u32(&empty[slot]));
           }
           if (!ok) break;
-          for (int g = 0; ok && g < 4; ++g)
-            if (!(ready >> g & 1)) ok = mbar_wait(smem_u32(&acc_empty[g]), (chunk & 1) ^ 1u, P.err, P.spin_ns);
-          if (!ok) break;
-          *s_chunk = used | 16;
-          umma_commit(smem_u32(acc_full));
-          mbar_arrive(smem_u32(acc_full));
-          ++chunk;
+          if (elected) umma_commit(smem_u32(&empty[slot]));
+          __syncwarp();
+          if (++slot == kStages) {
+            slot = 0;
+            ph ^= 1u;
+          }
         }
+        if (ok) finish_chunk(used, ready, 16);
       }
+    }
+    if (elected) {
       umma_commit(smem_u32(done));
       mbar_drain(smem_u32(done), 0u);   // no MMA is in flight when TMEM is released
     }
     __syncwarp();
+  }
   } else {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsEpi));
     // ------------------------------------------------------------ epilogue
-    const int q = warp & 3, ch = (warp - 2) >> 2;   // TMEM lane quarter, column half
+    const int q = warp & 3, ch = (warp - 4) >> 2;   // TMEM lane quarter, column half
     const int r_tile = q * 32 + lane;
     const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(ch * 64);
     uint32_t chunk = 0;
@@ -514,6 +568,15 @@ __global__ void __launch_bounds__(kThreads, 1) slice_gemm_kernel(const __grid_co
     for (int it = blockIdx.x; ok && it < items; it += gridDim.x) {
       const Item w = item_of(P, it);
       const int row = w.tm * kT + r_tile, col0 = w.tn * kT + ch * 64;
+      // exponents: this thread's row, and the 64 columns over the lanes
+      int exr = 0, ey2[2] = {0, 0};
+      if (EP != kEpSplitK) {
+        if (row < P.M) exr = __ldg(P.xe + row);
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+          if (col0 + 32 * i + lane < P.N) ey2[i] = __ldg(P.ye + col0 + 32 * i + lane);
+      }
+      const bool dead_r = exr == exp_special(P.xdt);
       long long acc[EP == kEpResidual ? 1 : 64];
       DF df[EP == kEpResidual ? 64 : 1];
       if constexpr (EP == kEpResidual) {
@@ -538,11 +601,11 @@ __global__ void __launch_bounds__(kThreads, 1) slice_gemm_kernel(const __grid_co
           for (int g = 0; g < 4; ++g) {
             if (info >> g & 1) {
 #pragma unroll
-              for (int j0 = 0; j0 < 64; j0 += 16) {
-                float v[16];
-                tmem_ld16(tbase + (uint32_t)(g * kT + j0), v);
+              for (int j0 = 0; j0 < 64; j0 += kLd) {
+                float v[kLd];
+                tmem_ld<kLd>(tbase + (uint32_t)(g * kT + j0), v);
 #pragma unroll
-                for (int jj = 0; jj < 16; ++jj) {
+                for (int jj = 0; jj < kLd; ++jj) {
                   if constexpr (EP == kEpResidual) {
                     // in units of 2^-16
                     const float x = v[jj] * (half ? pow2f(-32 - 8 * g) : pow2f(-8 * g));
@@ -567,18 +630,24 @@ __global__ void __launch_bounds__(kThreads, 1) slice_gemm_kernel(const __grid_co
           if (half == 1) {
 #pragma unroll
             for (int j = 0; j < 64; ++j) __stcg(lo + (long long)j * kT, (double)acc[j]);
-          } else if (row < P.M) {
-            const int exr = P.xe[row], ex = scale_exp(exr, P.xdt);
-            const bool dead_r = exr == exp_special(P.xdt);
+          } else {
+            // (loads of a batch before its stores, which they could alias)
+            const int ex = scale_exp(exr, P.xdt);
 #pragma unroll
-            for (int j = 0; j < 64; ++j) {
-              const int c = col0 + j;
-              if (c >= P.N) break;
-              const int eyr = P.ye[c];
-              double v = combine((double)acc[j], __ldcg(lo + (long long)j * kT), ex, scale_exp(eyr, P.ydt));
-              if (dead_r || eyr == exp_special(P.ydt)) v = plain_dot(P.sx, P.sy, row, c);
-              P.st.out[row * P.st.rs + c * P.st.cs] = v;
-              if (P.lower && row != c) P.st.out[c * P.st.rs + row * P.st.cs] = v;
+            for (int j0 = 0; j0 < 64; j0 += 16) {
+              double lv[16];
+#pragma unroll
+              for (int jj = 0; jj < 16; ++jj) lv[jj] = __ldcg(lo + (long long)(j0 + jj) * kT);
+#pragma unroll
+              for (int jj = 0; jj < 16; ++jj) {
+                const int c = col0 + j0 + jj;
+                const int eyr = __shfl_sync(0xffffffffu, ey2[j0 / 32], (j0 + jj) & 31);
+                if (row >= P.M || c >= P.N) continue;
+                double v = combine((double)acc[j0 + jj], lv[jj], ex, scale_exp(eyr, P.ydt));
+                if (dead_r || eyr == exp_special(P.ydt)) v = plain_dot(P.sx, P.sy, row, c);
+                P.st.out[row * P.st.rs + c * P.st.cs] = v;
+                if (P.lower && row != c) P.st.out[c * P.st.rs + row * P.st.cs] = v;
+              }
             }
           }
         } else if constexpr (EP == kEpSplitK) {
@@ -595,22 +664,32 @@ __global__ void __launch_bounds__(kThreads, 1) slice_gemm_kernel(const __grid_co
       if constexpr (EP == kEpResidual) {
         if (!ok) break;
         const Residual& R = P.r;
-        if (row < P.M) {
-          const int exr = P.xe[row], ex = scale_exp(exr, P.xdt) - 16;
-          const bool dead_r = exr == exp_special(P.xdt);
-          const float gh = (float)R.g2, gl = (float)(R.g2 - (double)gh);
-          const bool g_plain = fabsf(gh) < 1e30f && fabsf(gh) > 1e-30f;
+        const int ex = scale_exp(exr, P.xdt) - 16;
+        const float gh = (float)R.g2, gl = (float)(R.g2 - (double)gh);
+        const bool g_plain = fabsf(gh) < 1e30f && fabsf(gh) > 1e-30f;
+        const bool f32 = R.dtype == CSS_F32;
+        const bool row_ok = row < P.M;
 #pragma unroll
-          for (int j = 0; j < 64; ++j) {
-            const int c = col0 + j;
-            if (c >= P.N) break;
-            const int eyr = P.ye[c];
+        for (int j0 = 0; j0 < 64; j0 += 16) {
+          float av[16];
+#pragma unroll
+          for (int jj = 0; jj < 16; ++jj) {
+            const int c = col0 + j0 + jj;
+            av[jj] = 0.f;
+            if (row_ok && c < P.N)
+              av[jj] = f32 ? load_val((const float*)R.A + (long long)c * R.lda + row)
+                           : load_val((const __nv_bfloat16*)R.A + (long long)c * R.lda + row);
+          }
+#pragma unroll
+          for (int jj = 0; jj < 16; ++jj) {
+            const int c = col0 + j0 + jj;
+            const int eyr = __shfl_sync(0xffffffffu, ey2[j0 / 32], (j0 + jj) & 31);
+            if (!row_ok || c >= P.N) continue;
             const int e = ex + scale_exp(eyr, P.ydt);
             const int e1 = max(-126, min(127, e)), e2 = max(-126, min(127, e - e1));
-            float vh = df[j].s * pow2f(e1) * pow2f(e2), vl = df[j].c * pow2f(e1) * pow2f(e2);
+            float vh = df[j0 + jj].s * pow2f(e1) * pow2f(e2), vl = df[j0 + jj].c * pow2f(e1) * pow2f(e2);
             if (dead_r || eyr == exp_special(P.ydt)) vh = __int_as_float(0x7fffffff);
-            const float a = R.dtype == CSS_F32 ? load_val((const float*)R.A + (long long)c * R.lda + row)
-                                               : load_val((const __nv_bfloat16*)R.A + (long long)c * R.lda + row);
+            const float a = av[jj];
             // r = a - vh - vl as a normalised pair
             const float s = a - vh, bb = s - a;
             const float t = ((a - (s - bb)) + (-vh - bb)) - vl;
@@ -629,7 +708,7 @@ __global__ void __launch_bounds__(kThreads, 1) slice_gemm_kernel(const __grid_co
               } else {
                 g = (float)(R.g2 * ((double)rh + (double)rl));
               }
-              if (R.dtype == CSS_F32) ((float*)R.dA)[(long long)c * R.ldda + row] = g;
+              if (f32) ((float*)R.dA)[(long long)c * R.ldda + row] = g;
               else ((__nv_bfloat16*)R.dA)[(long long)c * R.ldda + row] = __float2bfloat16_rn(g);
             }
           }
@@ -640,9 +719,9 @@ __global__ void __launch_bounds__(kThreads, 1) slice_gemm_kernel(const __grid_co
       // the CTA's share of ||R||^2, in a fixed order
       __shared__ double s_loss[kEpiWarps];
       const double t = warp_sum(to_f64(lsh) + to_f64(lsl));
-      if (lane == 0) s_loss[warp - 2] = t;
+      if (lane == 0) s_loss[warp - 4] = t;
       asm volatile("bar.sync 1, 256;" ::: "memory");
-      if (warp == 2 && lane == 0) {
+      if (warp == 4 && lane == 0) {
         double sum = 0.0;
         for (int i = 0; i < kEpiWarps; ++i) sum += s_loss[i];
         P.r.loss_part[blockIdx.x] = sum;
