@@ -314,19 +314,6 @@ __device__ __forceinline__ Item item_of(const Args& P, int it) {
 constexpr uint32_t kDescHi = (128u >> 4) | 1u << 14;
 __device__ __forceinline__ uint32_t desc_lo(uint32_t saddr) { return (saddr >> 4) | (uint32_t)((kT * 16) >> 4) << 16; }
 constexpr uint32_t kDescSlice = kSliceBytes >> 4;
-// The elected lane issues; the whole warp walks the loops around it with
-// warp-uniform values, so that addresses and descriptors live in uniform
-// registers: a 128 x 128 x 16 MMA takes 64 clocks, less than moving its
-// operands there from a divergent thread's registers.
-__device__ __forceinline__ void umma_slices(uint32_t elected, uint32_t tmem_d, uint32_t xlo, uint32_t ylo,
-                                            uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n .reg .pred p, q;\n .reg .b64 da, db;\n setp.ne.b32 p, %5, 0;\n setp.ne.b32 q, %6, 0;\n"
-      " mov.b64 da, {%1, %4};\n mov.b64 db, {%2, %4};\n"
-      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, p;\n}" ::"r"(tmem_d),
-      "r"(xlo), "r"(ylo), "r"(idesc), "r"(kDescHi), "r"(acc), "r"(elected)
-      : "memory");
-}
 __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
                "l"(src), "r"(bytes), "r"(bar)
@@ -366,16 +353,6 @@ __device__ __noinline__ double plain_dot(const Source& x, const Source& y, int i
 // the rows' scales.
 __device__ __forceinline__ double combine(double hi, double lo, int ex, int ey) {
   return scale2(hi * 0x1p-40 + lo * 0x1p-72, ex + ey);
-}
-
-__device__ __forceinline__ uint32_t elect_one() {
-  uint32_t e;
-  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}" : "=r"(e));
-  return e;
-}
-// mbar_wait by the whole warp, with one answer
-__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, int* err, unsigned long long budget) {
-  return __all_sync(0xffffffffu, mbar_wait(bar, parity, err, budget));
 }
 
 // N columns of this warp's TMEM lanes
@@ -532,7 +509,7 @@ __global__ void __launch_bounds__(kThreads, 1) slice_gemm_kernel(const __grid_co
             for (int q = 0; q < nk; ++q) {
               uint32_t xl = dx + (q * 4 + s_lo - 1) * kDescSlice, yl = dy + (q * 4 + wt - s_lo - 1) * kDescSlice;
               for (int s = s_lo; s <= s_hi; ++s) {
-                umma_slices(elected, tm + g * kT, xl, yl, idesc, acc);
+                umma_elected(elected, tm + g * kT, xl, yl, kDescHi, idesc, acc);
                 acc = 1;
                 xl += kDescSlice;
                 yl -= kDescSlice;

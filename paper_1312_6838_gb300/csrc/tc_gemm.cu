@@ -50,8 +50,6 @@ constexpr int kTmemCols = 512;   // TMEM columns a CTA takes unless Params::tmem
 // The initial-score GEMMs of BF16 A take 256 TMEM columns and two 48 KB ring
 // stages per CTA, so that two CTAs share an SM and one's epilogue overlaps
 // the other's MMAs (instead of 512 columns and 96-112 KB stages, one CTA per SM)
-constexpr bool kSyrk2Cta = true;
-constexpr bool kDots2Cta = true;
 // FP32 A's column-dot GEMM: columns per CTA (its two accumulators take
 // twice that of TMEM; 128 lets two CTAs share an SM)
 constexpr int kDotsF32Cols = 128;
@@ -84,10 +82,6 @@ struct Params {
   // the lower triangle (rows >= columns); mode 3 multiplies by the upper
   // triangle U' of C (diagonal halved), so M-tile J starts at K = 128 J
   int tri;
-  // group: one ring stage holds the distinct tiles of every part for one K
-  // block (a tile shared by all parts is loaded once), and the parts' MMAs
-  // run back to back on it; otherwise each (K block, part) is its own stage
-  int group;
   int stages;        // ring depth (1..STAGES)
   int stall;         // test hook: the epilogue also waits on a phase nothing completes
   // modes 2 and 3: K blocks per blockIdx.z chunk.  The tensor cores' FP32
@@ -186,6 +180,9 @@ __device__ __forceinline__ void df_acc_prod(float& sh, float& sl, float a, float
   sl += err + e;
 }
 
+// a value that every lane of the warp holds, known to be uniform
+__device__ __forceinline__ int uni(int v) { return __shfl_sync(0xffffffffu, v, 0); }
+
 // v += the second accumulator's 16 columns at taddr (when acc2_col != 0),
 // rounded to nearest once
 __device__ __forceinline__ void add_acc2(uint32_t taddr, int acc2_col, float (&v)[16]) {
@@ -244,12 +241,9 @@ __device__ __forceinline__ void tc_body(const Params& P, const CUtensorMap* mapA
     }
   }
   const int parts = P.nparts;
-  // group mode: tiles per stage (a part stride of 0 means one shared tile)
-  const int nA = (P.group && P.a_part_stride != 0) ? parts : 1;
-  const int nB = (P.group && P.b_part_stride != 0) ? parts : 1;
   const int b_tile_bytes = P.halves * P.n_half * BK * 2;
-  // stages per K block: one (group), one per pair, or one per part
-  const int per_kb = P.group ? 1 : (P.npairs > 0 ? P.npairs : parts);
+  // stages per K block: one per pair, or one per part
+  const int per_kb = P.npairs > 0 ? P.npairs : parts;
   const int n_it = max(0, kb_end - kb_begin) * per_kb;
 
   if (threadIdx.x == 0) {
@@ -272,47 +266,51 @@ __device__ __forceinline__ void tc_body(const Params& P, const CUtensorMap* mapA
   fence_after();
   const uint32_t tmem = *s_tmem;
 
-  if (warp == 0 && lane == 0) {
+  if (warp == 0) {
     // ------------------------------------------------------------ producer
-    int issued = 0;
-    for (int it = 0; it < n_it; ++it) {
-      const int s = it % NSTG;
-      const uint32_t ph = (uint32_t)((it / NSTG) & 1);
-      if (!mbar_wait(smem_u32(&empty[s]), ph ^ 1u, P.err, P.spin_ns)) break;
-      const int kb = kb_begin + it / per_kb;
-      const int q_it = it % per_kb;
-      const int part_a0 = P.group ? 0 : (P.npairs > 0 ? P.pair_a[q_it] : q_it);
-      const int part_b0 = P.group ? 0 : (P.npairs > 0 ? P.pair_b[q_it] : q_it);
-      const int k0 = kb * BK;
-      uint8_t* sa = smem + s * P.stage_bytes;
-      uint8_t* sb = sa + nA * a_bytes;
-      const uint32_t fb = smem_u32(&full[s]);
-      mbar_expect_tx(fb, (uint32_t)(nA * a_bytes + nB * b_tile_bytes));
-      for (int pa = 0; pa < nA; ++pa) {
-        const int part = part_a0 + pa;
-        uint8_t* ta = sa + pa * a_bytes;
-        if (A_MN) {
-          const int ka = part * P.a_kpart + k0;
-          tma_load_2d(smem_u32(ta), &tmA, fb, tile0, ka);
-          tma_load_2d(smem_u32(ta + 64 * BK * 2), &tmA, fb, tile0 + 64, ka);
-        } else {
-          tma_load_2d(smem_u32(ta), &tmA, fb, k0, part * P.a_part_stride + tile0);
-        }
+    const uint32_t elected = elect_one();
+    const uint32_t sbase = smem_u32(smem);
+    const int u_per_kb = uni(per_kb), u_it = uni(n_it), nstg = uni(NSTG), stage_bytes = uni(P.stage_bytes);
+    const int row0 = uni(tile0), col0 = uni(ntile0), kb0 = uni(kb_begin);
+    const int npairs = uni(P.npairs), n_half = uni(P.n_half), halves = uni(P.halves);
+    const int a_kpart = uni(P.a_kpart), b_kpart = uni(P.b_kpart);
+    const int a_stride = uni(P.a_part_stride), b_stride = uni(P.b_part_stride);
+    const uint32_t tx = (uint32_t)(a_bytes + uni(b_tile_bytes));
+    int issued = 0, slot = 0, q = 0, k0 = kb0 * BK;
+    uint32_t ph = 1u;
+    for (int it = 0; it < u_it; ++it) {
+      if (!mbar_wait_warp(smem_u32(&empty[slot]), ph, P.err, P.spin_ns)) break;
+      const int part_a = npairs > 0 ? uni(P.pair_a[q]) : q;
+      const int part_b = npairs > 0 ? uni(P.pair_b[q]) : q;
+      const uint32_t sa = sbase + (uint32_t)(slot * stage_bytes), sb = sa + a_bytes;
+      const uint32_t fb = smem_u32(&full[slot]);
+      if (elected) mbar_expect_tx(fb, tx);
+      __syncwarp();
+      if (A_MN) {
+        const int ka = part_a * a_kpart + k0;
+        tma_load_2d_elected(elected, sa, &tmA, fb, row0, ka);
+        tma_load_2d_elected(elected, sa + 64 * BK * 2, &tmA, fb, row0 + 64, ka);
+      } else {
+        tma_load_2d_elected(elected, sa, &tmA, fb, k0, part_a * a_stride + row0);
       }
-      for (int pb = 0; pb < nB; ++pb) {
-        const int part = part_b0 + pb;
-        uint8_t* tb = sb + pb * b_tile_bytes;
-        if (B_MN) {
-          // N-major B: 64-row boxes stacked 8 KB apart (the descriptor's LBO)
-          for (int q = 0; q < P.halves * P.n_half / 64; ++q)
-            tma_load_2d(smem_u32(tb + q * 64 * BK * 2), &tmB, fb, ntile0 + 64 * q, part * P.b_kpart + k0);
-        } else {
-          for (int h = 0; h < P.halves; ++h)
-            tma_load_2d(smem_u32(tb + h * P.n_half * BK * 2), &tmB, fb, k0,
-                        ntile0 + part * P.b_part_stride + h * P.n_half);
-        }
+      if (B_MN) {
+        // N-major B: 64-row boxes stacked 8 KB apart (the descriptor's LBO)
+        const int kb = part_b * b_kpart + k0;
+        for (int x = 0; x < halves * n_half / 64; ++x)
+          tma_load_2d_elected(elected, sb + x * 64 * BK * 2, &tmB, fb, col0 + 64 * x, kb);
+      } else {
+        for (int h = 0; h < halves; ++h)
+          tma_load_2d_elected(elected, sb + h * n_half * BK * 2, &tmB, fb, k0, col0 + part_b * b_stride + h * n_half);
       }
       issued = it + 1;
+      if (++q == u_per_kb) {
+        q = 0;
+        k0 += BK;
+      }
+      if (++slot == nstg) {
+        slot = 0;
+        ph ^= 1u;
+      }
     }
     // the copies issued last (one per stage) have landed before the CTA
     // exits, also when a wait failed and the MMA issuer stopped consuming
@@ -320,49 +318,49 @@ __device__ __forceinline__ void tc_body(const Params& P, const CUtensorMap* mapA
       const int s = it % NSTG;
       mbar_drain(smem_u32(&full[s]), (uint32_t)((it / NSTG) & 1));
     }
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1) {
     // ---------------------------------------------------------- MMA issuer
-    const uint32_t idesc = make_idesc(P.n_half, BM, A_MN, B_MN);
-    // MMAs that share one stage: group mode runs every part on it; otherwise
-    // a stage is one part or one pair
-    const int pg = P.group ? parts : 1;
-    for (int it = 0; it < n_it; ++it) {
-      const int s = it % NSTG;
-      const uint32_t ph = (uint32_t)((it / NSTG) & 1);
-      if (!mbar_wait(smem_u32(&full[s]), ph, P.err, P.spin_ns)) break;
+    const uint32_t elected = elect_one();
+    const uint32_t sbase = smem_u32(smem);
+    const int u_per_kb = uni(per_kb), u_it = uni(n_it), nstg = uni(NSTG), stage_bytes = uni(P.stage_bytes);
+    const int npairs = uni(P.npairs), n_half = uni(P.n_half), halves = uni(P.halves), acc2 = uni(P.acc2_col);
+    const uint32_t tm = (uint32_t)uni((int)tmem);
+    const uint32_t idesc = make_idesc(n_half, BM, A_MN, B_MN);
+    // M/N-major: 16 K rows of 128 bytes per step, 64-row boxes 8 KB apart;
+    // K-major: 32 bytes per step
+    constexpr uint32_t lbo_a = A_MN ? 64 * BK * 2 : 16, lbo_b = B_MN ? 64 * BK * 2 : 16;
+    constexpr uint32_t step_a = (A_MN ? 2048 : 32) >> 4, step_b = (B_MN ? 2048 : 32) >> 4;
+    const uint32_t step_h = (uint32_t)(n_half * BK * 2) >> 4;
+    uint32_t used = 0;   // accumulators already written (the first MMA ignores its input)
+    int slot = 0, q = 0;
+    uint32_t ph = 0u;
+    for (int it = 0; it < u_it; ++it) {
+      if (!mbar_wait_warp(smem_u32(&full[slot]), ph, P.err, P.spin_ns)) break;
       fence_after();
-      const uint32_t sa0 = smem_u32(smem + s * P.stage_bytes);
-      const uint32_t sb0 = sa0 + nA * a_bytes;
+      const uint32_t sa = sbase + (uint32_t)(slot * stage_bytes);
+      const uint32_t da = sw128_desc_lo(sa, lbo_a), db = sw128_desc_lo(sa + a_bytes, lbo_b);
+      const uint32_t which = npairs > 0 ? (uint32_t)uni(P.pair_acc[q]) : 0u;
+      const uint32_t d = tm + which * (uint32_t)acc2;
+      uint32_t acc = used >> which & 1u;
+      used |= 1u << which;
 #pragma unroll
       for (int ks = 0; ks < BK / 16; ++ks) {
-        for (int pp = 0; pp < pg; ++pp) {
-          // the stage's tiles, its accumulator, and whether this MMA is the
-          // first into that accumulator (its input is then ignored)
-          const int ia = nA > 1 ? pp : 0, ib = nB > 1 ? pp : 0;
-          uint32_t acc = 0;
-          bool first = it == 0 && ks == 0 && pp == 0;
-          if (P.npairs > 0) {
-            const int q = it % per_kb;
-            acc = (uint32_t)(P.pair_acc[q] * P.acc2_col);
-            first = it / per_kb == 0 && ks == 0;
-            for (int q2 = 0; q2 < q; ++q2)
-              if (P.pair_acc[q2] == P.pair_acc[q]) first = false;
-          }
-          const uint32_t sa = sa0 + ia * a_bytes;
-          const uint32_t sb = sb0 + ib * b_tile_bytes;
-          // A: M-major -> 16 K rows of 128 bytes per step; K-major -> 32 bytes
-          const uint64_t ad = A_MN ? make_desc(sa + ks * 2048, 64 * BK * 2, 1024)
-                                   : make_desc(sa + ks * 32, 16, 1024);
-          for (int h = 0; h < P.halves; ++h) {
-            const uint64_t bd = B_MN ? make_desc(sb + h * P.n_half * BK * 2 + ks * 2048, 64 * BK * 2, 1024)
-                                     : make_desc(sb + h * P.n_half * BK * 2 + ks * 32, 16, 1024);
-            umma(tmem + acc + h * P.n_half, ad, bd, idesc, first ? 0u : 1u);
-          }
-        }
+        umma_elected(elected, d, da + ks * step_a, db + ks * step_b, sw128_desc_hi(1024), idesc, acc);
+        if (halves > 1)
+          umma_elected(elected, d + n_half, da + ks * step_a, db + step_h + ks * step_b, sw128_desc_hi(1024), idesc,
+                       acc);
+        acc = 1u;
       }
-      umma_commit(smem_u32(&empty[s]));
+      if (elected) umma_commit(smem_u32(&empty[slot]));
+      __syncwarp();
+      if (++q == u_per_kb) q = 0;
+      if (++slot == nstg) {
+        slot = 0;
+        ph ^= 1u;
+      }
     }
-    umma_commit(smem_u32(done));
+    if (elected) umma_commit(smem_u32(done));
+    __syncwarp();
     // every MMA issued has finished before TMEM is released at the end
     mbar_drain(smem_u32(done), 0u);
   } else if (warp >= 2) {
@@ -891,7 +889,7 @@ void set_pairs(Params& P) {
 }
 
 // Columns of D per CTA of the column-dot GEMM.
-int dots_n_tile(bool f32) { return f32 ? kDotsF32Cols : kDots2Cta ? 256 : 512; }
+int dots_n_tile(bool f32) { return f32 ? kDotsF32Cols : 256; }
 
 // Tensor maps of the two GEMMs: C = A A^T (both operands A, or its parts,
 // row-major in K = the column index), and U' A (U' parts K-major; A, or its
@@ -937,7 +935,7 @@ Params f0_params_syrk(const F0Layout& L, int m, int n, int src, int* err, unsign
   }
   P.stage_bytes = BM * BK * 2 + L.tw * BK * 2;
   P.stages = fit_stages(P.stage_bytes, STAGES);
-  if (kSyrk2Cta && !f32) {
+  if (!f32) {
     P.stages = 2;
     P.tmem_cols = 256;
   }
@@ -975,7 +973,6 @@ Params f0_params_dots(const F0Layout& L, const void* A, long long lda, int m, in
     // U' parts times A parts, one stage per (K block, pair), 256 columns
     // per CTA (the cross products take the other half of TMEM): 48 KB per
     // stage
-    P.group = 0;
     P.nparts = 1;
     set_pairs(P);
     P.acc2_col = P.n_tile;
@@ -983,28 +980,16 @@ Params f0_params_dots(const F0Layout& L, const void* A, long long lda, int m, in
     P.b_part_stride = L.npad;
     P.stage_bytes = BM * BK * 2 + P.n_tile * BK * 2;
     P.stages = P.n_tile < 256 ? 3 : fit_stages(P.stage_bytes, STAGES);
-  } else if (kDots2Cta) {
+  } else {
     // 256 columns per CTA, one stage per (K block, U' part) holding that
     // part's tile and the A tile (48 KB), two stages: two CTAs per SM
-    P.group = 0;
     P.nparts = kParts;
     P.b_part_stride = 0;
     P.stage_bytes = BM * BK * 2 + 256 * BK * 2;
     P.stages = 2;
     P.tmem_cols = 256;
-  } else {
-    // 512 columns per CTA (two MMAs of N = 256, the whole TMEM) and one
-    // stage per K block holding the U' parts and the single shared A tile:
-    // 112 KB per stage
-    P.group = 1;
-    P.nparts = kParts;
-    P.b_part_stride = 0;
-    P.stage_bytes = kParts * BM * BK * 2 + 512 * BK * 2;
-    P.stages = 2;
   }
   // the epilogue stages the tile's Acol (BM x n_tile, BF16 or FP32) in the ring
-  static_assert(BM * 512 * 2 <= 2 * (kParts * BM * BK * 2 + 512 * BK * 2), "BF16 ring holds the Acol tile");
-  static_assert(2 * (kParts * BM * BK * 2 + 512 * BK * 2) + 256 + 1024 <= kSmemMax, "BF16 ring fits");
   static_assert(BM * 256 * 4 <= 3 * (BM * BK * 2 + 256 * BK * 2), "FP32 ring holds the Acol tile");
   static_assert(BM * 256 * 2 <= 2 * (BM * BK * 2 + 256 * BK * 2), "two-stage BF16 ring holds the Acol tile");
   P.f = L.partial;

@@ -61,35 +61,47 @@ __device__ __forceinline__ void mbar_drain(uint32_t bar, uint32_t parity) {
   while (!mbar_try_wait(bar, parity))
     if (gtimer() - t0 > 1000000000ull) return;
 }
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0,
-                                            int c1) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], "
-      "[%2];" ::"r"(dst),
-      "l"((uint64_t)map), "r"(bar), "r"(c0), "r"(c1)
-      : "memory");
+// Shared-memory matrix descriptor, 128-byte swizzle (sm_100 format), as halves.
+__device__ __forceinline__ uint32_t sw128_desc_lo(uint32_t saddr, uint32_t lbo) {
+  return ((saddr >> 4) & 0x3FFFu) | ((lbo >> 4) & 0x3FFFu) << 16;
 }
-// Shared-memory matrix descriptor, 128-byte swizzle (sm_100 format).
-__device__ __forceinline__ uint64_t make_desc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
-  d |= (uint64_t)((lbo >> 4) & 0x3FFFu) << 16;
-  d |= (uint64_t)((sbo >> 4) & 0x3FFFu) << 32;
-  d |= (uint64_t)1 << 46;
-  d |= (uint64_t)2 << 61;
-  return d;
-}
+__host__ __device__ constexpr uint32_t sw128_desc_hi(uint32_t sbo) { return (sbo >> 4) | 1u << 14 | 2u << 29; }
 // Instruction descriptor: kind::f16, BF16 x BF16 -> FP32.
 __device__ __forceinline__ uint32_t make_idesc(int N, int M, bool a_mn, bool b_mn) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)a_mn << 15) | ((uint32_t)b_mn << 16) |
          ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
-__device__ __forceinline__ void umma(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                     uint32_t accumulate) {
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t e;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}" : "=r"(e));
+  return e;
+}
+// mbar_wait by the whole warp, with one answer
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, int* err, unsigned long long budget) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, err, budget));
+}
+// Issue by one elected lane of a warp that walks its loops as a whole, with
+// warp-uniform values, so that addresses and descriptors live in uniform
+// registers.  From a divergent thread each MMA cost about 150 clocks of moves
+// into them, more than a 128 x 128 x 16 (64 clocks) or 128 x 256 x 16 (128)
+// MMA takes.  Descriptors come as 32-bit halves; only the address field of the
+// low one changes from one MMA to the next.
+__device__ __forceinline__ void umma_elected(uint32_t elected, uint32_t tmem_d, uint32_t a_lo, uint32_t b_lo,
+                                             uint32_t desc_hi, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem_d),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      "{\n .reg .pred p, q;\n .reg .b64 da, db;\n setp.ne.b32 p, %5, 0;\n setp.ne.b32 q, %6, 0;\n"
+      " mov.b64 da, {%1, %4};\n mov.b64 db, {%2, %4};\n"
+      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, p;\n}" ::"r"(tmem_d),
+      "r"(a_lo), "r"(b_lo), "r"(idesc), "r"(desc_hi), "r"(accumulate), "r"(elected)
+      : "memory");
+}
+__device__ __forceinline__ void tma_load_2d_elected(uint32_t elected, uint32_t dst, const CUtensorMap* map,
+                                                    uint32_t bar, int c0, int c1) {
+  asm volatile(
+      "{\n .reg .pred q;\n setp.ne.b32 q, %5, 0;\n"
+      " @q cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], "
+      "[%2];\n}" ::"r"(dst),
+      "l"((uint64_t)map), "r"(bar), "r"(c0), "r"(c1), "r"(elected)
       : "memory");
 }
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
