@@ -131,207 +131,155 @@ void gram(const double* AS, int m, int k, double* part, double* G, cudaStream_t 
   gram_fin_kernel<<<(unsigned)(((long long)k * k + 255) / 256), 256, 0, s>>>(part, g.nslices, g.npairs, k, G);
 }
 
-// Cholesky G = L L^T in place (lower triangle of the column-major k x k G).
-// For k > kCholSmemK (G too large for one block's shared memory) it runs
-// blocked right-looking, kCb columns a panel, as stream-ordered launches:
-//   chol_block_kernel: one warp factors the panel's diagonal block D in
-//     shared memory and writes it back;
-//   chol_rows_kernel: each CTA solves kCb of the rows below it, L_i = G_i D^-T;
-//   chol_update_kernel: one CTA per 32 x 32 tile of the trailing lower
-//     triangle subtracts the panel's outer product, G_IJ -= L_I L_J^T.
-// FP64 runs at two lanes per clock per SM on this part, so the k^3 / 6
-// multiply-adds are spread over many SMs instead of one.  A pivot at or below
-// 1e-12 of its column's initial squared norm (diag0, saved first) means the
-// selected columns are linearly dependent to working precision: the pivot
-// is replaced by 1 and status[0] = 1.
+// Cholesky G = L L^T in place (lower triangle of the column-major k x k G) and
+// X = L^-1 together, blocked and right-looking, kCb columns a panel, as
+// stream-ordered launches.  With D the panel's diagonal block of L:
+//   chol_diag_kernel: one block forms D and D^-1 in shared memory, a column of
+//     one and a row of the other a step (the steps depend on one another, so
+//     they are short loops: unrolled into registers of one warp, the code's
+//     own fetches took 69 us a panel);
+//   chol_rows_kernel: below the panel L_i = G_i D^-T, left of it X_j = D^-1 X_j;
+//   chol_update_kernel: G_IJ -= L_I L_J^T and X_I -= L_I X_j below the panel.
+// FP64 runs at two lanes per clock per SM on this part, so the products are
+// cut into CTAs of 256 outputs, 32 multiply-adds each (2 us), and D is applied
+// as an inverse instead of by substitution.  A pivot at or below 1e-12 of its
+// column's initial squared norm (diag0, saved first) means the selected
+// columns are linearly dependent to working precision: the pivot is replaced
+// by 1 and status[0] = 1.  Factor and inverse together, measured: k = 128
+// 472 -> 172 us (one block in shared memory, then a substitution per
+// column), k = 256 656 -> 346 us (blocked with substitutions).
 constexpr int kCb = 32;
 
-__global__ void chol_diag_kernel(const double* __restrict__ G, int k, double* __restrict__ diag0) {
+__global__ void chol_save_kernel(const double* __restrict__ G, int k, double* __restrict__ diag0) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j < k) diag0[j] = G[(long long)j * k + j];
 }
 
-__global__ void __launch_bounds__(32) chol_block_kernel(double* __restrict__ G, int k, int j0,
+__global__ void __launch_bounds__(256) chol_diag_kernel(double* __restrict__ G, double* __restrict__ X, int k, int j0,
                                                         const double* __restrict__ diag0,
                                                         int* __restrict__ status) {
-  __shared__ double D[kCb][kCb + 1];   // rows x columns of the diagonal block
-  const int lane = threadIdx.x;
-  const int b = min(kCb, k - j0);
-  for (int c = 0; c < b; ++c)
-    if (lane >= c && lane < b) D[lane][c] = G[(long long)(j0 + c) * k + j0 + lane];
-  __syncwarp();
+  __shared__ double D[kCb][kCb + 1], V[kCb][kCb + 1];   // the block, and D^-1 as it forms
+  const int t = threadIdx.x, b = min(kCb, k - j0);
+  for (int e = t; e < kCb * kCb; e += 256) {
+    const int r = e % kCb, c = e / kCb;
+    D[r][c] = r < b && c <= r ? G[(long long)(j0 + c) * k + j0 + r] : 0.0;
+    V[r][c] = r == c ? 1.0 : 0.0;
+  }
+  const double least = t < b ? 1e-12 * diag0[j0 + t] : 0.0;
+  __syncthreads();
   bool bad = false;
   for (int c = 0; c < b; ++c) {
-    const double dd = D[c][c];
-    const bool ok = dd > 1e-12 * diag0[j0 + c];
-    const double d = ok ? sqrt(dd) : 1.0;
-    bad |= !ok;
-    __syncwarp();
-    if (lane == c) D[c][c] = d;
-    if (lane > c && lane < b) D[lane][c] /= d;
-    __syncwarp();
-    if (lane > c && lane < b) {
-      const double lrc = D[lane][c];
-      for (int q = c + 1; q <= lane; ++q) D[lane][q] -= lrc * D[q][c];
+    if (t < kCb) {
+      // column c of L and row c of D^-1 are done but for the pivot
+      const double d = D[c][c];
+      const bool ok = d > __shfl_sync(0xffffffffu, least, c);
+      bad |= !ok;
+      const double r = ok ? rsqrt(d) : 1.0;
+      __syncwarp();
+      if (t == c) D[c][c] = ok ? d * r : 1.0;
+      else if (t > c) D[t][c] *= r;
+      if (t <= c) V[c][t] *= r;
     }
-    __syncwarp();
+    __syncthreads();
+    // rows below: column c out of the block's trailing part and of D^-1
+    const int q = t / 8;
+    if (q > c && q < b) {
+      const double l = D[q][c];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int x = t % 8 + 8 * i;
+        if (x <= c) V[q][x] = fma(-l, V[c][x], V[q][x]);
+        else if (x <= q) D[q][x] = fma(-l, D[x][c], D[q][x]);
+      }
+    }
+    __syncthreads();
   }
-  for (int c = 0; c < b; ++c)
-    if (lane >= c && lane < b) G[(long long)(j0 + c) * k + j0 + lane] = D[lane][c];
-  if (lane == 0 && bad) status[0] = 1;
-}
-
-// The rows below the factored diagonal block (kCb rows a CTA): row i of L
-// solves x D^T = g by forward substitution over the block's columns.
-__global__ void __launch_bounds__(32) chol_rows_kernel(double* __restrict__ G, int k, int j0) {
-  __shared__ double D[kCb][kCb + 1];
-  __shared__ double dinv[kCb];
-  const int lane = threadIdx.x;
-  const int b = min(kCb, k - j0);
-  for (int c = 0; c < b; ++c)
-    if (lane >= c && lane < b) D[lane][c] = G[(long long)(j0 + c) * k + j0 + lane];
-  __syncwarp();
-  if (lane < b) dinv[lane] = 1.0 / D[lane][lane];
-  __syncwarp();
-  const int i = j0 + b + blockIdx.x * kCb + lane;
-  if (i >= k) return;
-  double x[kCb];
-#pragma unroll
-  for (int c = 0; c < kCb; ++c) x[c] = c < b ? G[(long long)(j0 + c) * k + i] : 0.0;
-#pragma unroll
-  for (int c = 0; c < kCb; ++c) {
-    if (c < b) {
-      double v = x[c];
-#pragma unroll
-      for (int q = 0; q < c; ++q) v = fma(-x[q], D[c][q], v);
-      x[c] = v * dinv[c];
+  if (t == 0 && bad) status[0] = 1;
+  for (int e = t; e < kCb * kCb; e += 256) {
+    const int r = e % kCb, c = e / kCb;
+    if (r < b && c <= r) {
+      G[(long long)(j0 + c) * k + j0 + r] = D[r][c];
+      X[(long long)(j0 + c) * k + j0 + r] = V[r][c];
     }
   }
-#pragma unroll
-  for (int c = 0; c < kCb; ++c)
-    if (c < b) G[(long long)(j0 + c) * k + i] = x[c];
 }
 
-// Trailing update after the panel at j0 (width b): rows and columns from
-// t0 = j0 + b on, lower tiles (ti >= tj) of 32 x 32, four outputs a thread.
-__global__ void __launch_bounds__(256) chol_update_kernel(double* __restrict__ G, int k, int j0, int b) {
-  __shared__ double PI[32][kCb + 1], PJ[32][kCb + 1];
-  const int t0 = j0 + b;
-  int ti = (int)((sqrtf(8.f * blockIdx.x + 1.f) - 1.f) * 0.5f);
-  while (ti * (ti + 1) / 2 > (int)blockIdx.x) --ti;
-  while ((ti + 1) * (ti + 2) / 2 <= (int)blockIdx.x) ++ti;
-  const int tj = blockIdx.x - ti * (ti + 1) / 2;
-  const int r0 = t0 + ti * 32, c0 = t0 + tj * 32;
-  for (int e = threadIdx.x; e < 32 * kCb; e += 256) {
-    const int r = e % 32, c = e / 32;
-    const bool okc = c < b;
-    PI[r][c] = (okc && r0 + r < k) ? G[(long long)(j0 + c) * k + r0 + r] : 0.0;
-    PJ[r][c] = (okc && c0 + r < k) ? G[(long long)(j0 + c) * k + c0 + r] : 0.0;
+// Blocks 0 .. nlow - 1: eight rows of L below the panel; the others: eight
+// columns of X's panel rows.
+__global__ void __launch_bounds__(256) chol_rows_kernel(double* __restrict__ G, double* __restrict__ X, int k, int j0,
+                                                        int nlow) {
+  __shared__ double D[kCb][kCb + 1], V[8][kCb + 1];
+  const int b = min(kCb, k - j0), t = threadIdx.x;
+  const bool low = (int)blockIdx.x < nlow;
+  for (int e = t; e < kCb * kCb; e += 256) {
+    const int r = e % kCb, c = e / kCb;
+    D[r][c] = r < b && c <= r ? X[(long long)(j0 + c) * k + j0 + r] : 0.0;
   }
+  const int at = low ? j0 + b + blockIdx.x * 8 : ((int)blockIdx.x - nlow) * 8;   // first row of L, or column of X
+  const int v = low ? t % 8 : t / kCb, q = low ? t / 8 : t % kCb;
+  const bool in = q < b && at + v < (low ? k : j0);
+  double* p = low ? G + (long long)(j0 + q) * k + at + v : X + (long long)(at + v) * k + j0 + q;
+  V[v][q] = in ? *p : 0.0;
   __syncthreads();
-  const int r = threadIdx.x % 32;
-  const int i = r0 + r;
-  if (i >= k) return;
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int cl = threadIdx.x / 32 + 8 * q;
-    const int l = c0 + cl;
-    if (l >= k || l > i) continue;
-    double acc = 0.0;
+  double acc = 0.0;
 #pragma unroll 8
-    for (int c = 0; c < b; ++c) acc = fma(PI[r][c], PJ[cl][c], acc);
-    G[(long long)l * k + i] -= acc;
-  }
+  for (int e = 0; e < kCb; ++e) acc = fma(V[v][e], D[q][e], acc);
+  if (in) *p = acc;
 }
 
-// Linv = L^-1 by forward substitution L x = e_j, one warp per column j: the
-// sum over the already known x_l is split across the lanes and the column
-// is kept in shared memory.
-constexpr int kLinvWarps = 8;
-__global__ void __launch_bounds__(kLinvWarps * 32) linv_kernel(const double* __restrict__ G, int k,
-                                                                double* __restrict__ Linv) {
-  extern __shared__ double xs[];   // kLinvWarps x k
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int j = blockIdx.x * kLinvWarps + w;
-  if (j >= k) return;
-  double* x = xs + (size_t)w * k;
-  for (int i = lane; i < j; i += 32) Linv[(long long)j * k + i] = 0.0;
-  for (int i = j; i < k; ++i) {
-    double part = 0.0;
-    for (int l = j + lane; l < i; l += 32) part = fma(G[(long long)l * k + i], x[l], part);
-    part = warp_sum(part);
-    if (lane == 0) {
-      const double v = ((i == j) ? 1.0 : 0.0) - part;
-      x[i] = v / G[(long long)i * k + i];
-    }
-    __syncwarp();
+// 16 x 16 outputs a block: lower tiles of G's trailing part, then the tiles
+// of X's rows below the panel (columns up to the panel's last).
+__global__ void __launch_bounds__(256) chol_update_kernel(double* __restrict__ G, double* __restrict__ X, int k,
+                                                          int j0, int ntri, int xcols) {
+  __shared__ double P[16][kCb + 1], Q[16][kCb + 1];
+  const int t0 = j0 + kCb, t = threadIdx.x, bid = blockIdx.x;   // (a panel with rows below it is full)
+  const bool tri = bid < ntri;
+  int ti, tj;
+  if (tri) {
+    ti = (int)((sqrtf(8.f * bid + 1.f) - 1.f) * 0.5f);
+    while (ti * (ti + 1) / 2 > bid) --ti;
+    while ((ti + 1) * (ti + 2) / 2 <= bid) ++ti;
+    tj = bid - ti * (ti + 1) / 2;
+  } else {
+    ti = (bid - ntri) / xcols;
+    tj = (bid - ntri) % xcols;
   }
-  for (int i = j + lane; i < k; i += 32) Linv[(long long)j * k + i] = x[i];
-}
-
-// For k <= kCholSmemK one block factors G held in shared memory (one launch;
-// faster than the blocked form at these sizes): the k steps of the unblocked
-// right-looking update read shared memory; L is written back over G.
-constexpr int kCholSmemK = 128;
-__global__ void __launch_bounds__(1024) chol_smem_kernel(double* __restrict__ Gg, int k, int* __restrict__ status) {
-  extern __shared__ double G[];   // k x k, column-major
-  __shared__ int bad;
-  __shared__ double diag0[kCholSmemK];
-  if (threadIdx.x == 0) bad = 0;
-  for (int e = threadIdx.x; e < k * k; e += blockDim.x) G[e] = Gg[e];
-  __syncthreads();
-  for (int j = threadIdx.x; j < k; j += blockDim.x) diag0[j] = G[j * k + j];
-  __syncthreads();
-  for (int j = 0; j < k; ++j) {
-    if (threadIdx.x == 0) {
-      // a pivot at or below 1e-12 of its column's squared norm: the selected
-      // columns are linearly dependent to working precision
-      const double d = G[j * k + j];
-      const bool ok = d > 1e-12 * diag0[j];
-      if (!ok) bad = 1;
-      G[j * k + j] = ok ? sqrt(d) : 1.0;
-    }
-    __syncthreads();
-    const double d = G[j * k + j];
-    for (int i = j + 1 + threadIdx.x; i < k; i += blockDim.x) G[j * k + i] /= d;
-    __syncthreads();
-    const int rem = k - j - 1;
-    for (int e = threadIdx.x; e < rem * rem; e += blockDim.x) {
-      const int i = j + 1 + e % rem, l = j + 1 + e / rem;
-      if (l <= i) G[l * k + i] -= G[j * k + i] * G[j * k + l];
-    }
-    __syncthreads();
+  const int r0 = t0 + ti * 16, c0 = (tri ? t0 : 0) + tj * 16;
+  for (int e = t; e < 16 * kCb; e += 256) {
+    const int r = e % 16, q = e / 16;
+    P[r][q] = r0 + r < k ? G[(long long)(j0 + q) * k + r0 + r] : 0.0;
+    if (tri) Q[r][q] = c0 + r < k ? G[(long long)(j0 + q) * k + c0 + r] : 0.0;
   }
-  for (int e = threadIdx.x; e < k * k; e += blockDim.x) Gg[e] = G[e];
-  if (threadIdx.x == 0 && bad) status[0] = 1;
+  if (!tri)
+    for (int e = t; e < 16 * kCb; e += 256) {
+      const int q = e % kCb, c = e / kCb;
+      Q[c][q] = X[(long long)(c0 + c) * k + j0 + q];
+    }
+  __syncthreads();
+  const int r = t % 16, c = t / 16;
+  const int i = r0 + r, l = c0 + c;
+  if (i >= k || (tri && l > i)) return;
+  double acc = 0.0;
+#pragma unroll 8
+  for (int q = 0; q < kCb; ++q) acc = fma(P[r][q], Q[c][q], acc);
+  (tri ? G : X)[(long long)l * k + i] -= acc;
 }
 
 // Cholesky of the k x k matrix in G (overwritten by L) and L^-1 into Linv
-// (status[0] = 1 for a rank-deficient G).
-void chol_inv(double* G, int k, double* Linv, int* status, cudaStream_t s) {
-  if (k <= kCholSmemK) {
-    const size_t smem = (size_t)k * k * sizeof(double);
-    if (smem > 48 * 1024)
-      cudaFuncSetAttribute(chol_smem_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    chol_smem_kernel<<<1, 1024, smem, s>>>(G, k, status);
-  } else {
-    // the initial diagonal is kept in Linv, which is written only afterwards
-    double* diag0 = Linv;
-    chol_diag_kernel<<<(k + 255) / 256, 256, 0, s>>>(G, k, diag0);
-    for (int j0 = 0; j0 < k; j0 += kCb) {
-      const int b = std::min(kCb, k - j0);
-      const int below = k - j0 - b;
-      chol_block_kernel<<<1, 32, 0, s>>>(G, k, j0, diag0, status);
-      if (below > 0) {
-        chol_rows_kernel<<<(below + kCb - 1) / kCb, 32, 0, s>>>(G, k, j0);
-        const int T = (below + 31) / 32;
-        chol_update_kernel<<<T * (T + 1) / 2, 256, 0, s>>>(G, k, j0, b);
-      }
+// (status[0] = 1 for a rank-deficient G).  diag0: k doubles of scratch.
+void chol_inv(double* G, int k, double* Linv, double* diag0, int* status, cudaStream_t s) {
+  cudaMemsetAsync(Linv, 0, (size_t)k * k * sizeof(double), s);
+  chol_save_kernel<<<(k + 255) / 256, 256, 0, s>>>(G, k, diag0);
+  for (int j0 = 0; j0 < k; j0 += kCb) {
+    const int below = std::max(0, k - j0 - kCb);
+    chol_diag_kernel<<<1, 256, 0, s>>>(G, Linv, k, j0, diag0, status);
+    const int nlow = (below + 7) / 8, nx = j0 / 8;
+    if (nlow + nx > 0) chol_rows_kernel<<<nlow + nx, 256, 0, s>>>(G, Linv, k, j0, nlow);
+    if (below > 0) {
+      const int T = (below + 15) / 16, ntri = T * (T + 1) / 2, xcols = (j0 + kCb) / 16;
+      chol_update_kernel<<<ntri + T * xcols, 256, 0, s>>>(G, Linv, k, j0, ntri, xcols);
     }
   }
-  const size_t smem = (size_t)kLinvWarps * k * sizeof(double);
-  if (smem > 48 * 1024) cudaFuncSetAttribute(linv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  linv_kernel<<<(k + kLinvWarps - 1) / kLinvWarps, kLinvWarps * 32, smem, s>>>(G, k, Linv);
 }
 
 // Q = A_S L^-T (m x k): Q[i, j] = sum_{l <= j} A_S[i, l] Linv[j, l].
@@ -343,6 +291,51 @@ __global__ void q_kernel(const double* __restrict__ AS, const double* __restrict
   double acc = 0.0;
   for (int l = 0; l <= j; ++l) acc = fma(AS[(long long)l * m + i], Linv[(long long)l * k + j], acc);
   Q[idx] = acc;
+}
+
+// Above this many columns G = A_S^T A_S and Q = A_S L^-T run on the slice GEMM.
+// css_embed at m = 4096, n = 256 (two rounds of both, us): l = 65 582 with the FP64
+// kernels and 667 with slices, l = 128 853 and 848; at l = 256 the FP64 kernels
+// take 600 us a round, the slice products with their splits about 200.
+constexpr int kSliceK = 128;
+
+// A_S's orthonormal basis by Cholesky: G = A_S^T A_S = L L^T, Q = A_S L^-T.
+struct OrthSpace {
+  double *G, *gpart, *Linv;
+  sg::Digits DS, DSr, DL;   // A_S both ways, L^-1
+  sg::Scratch sc;
+  int* status;              // [0] rank deficient, [1] error of the products
+};
+OrthSpace carve_orth(WsCarver& c, int* status, long long m, int k) {
+  OrthSpace w{};
+  w.status = status;
+  w.G = c.take<double>((size_t)k * k);
+  w.gpart = c.take<double>(gram_part_doubles((int)m, k));
+  w.Linv = c.take<double>((size_t)k * k);
+  if (k > kSliceK) {
+    w.DS = sg::carve_digits(c, k, m);
+    w.DSr = sg::carve_digits(c, m, k);
+    w.DL = sg::carve_digits(c, k, k);
+    w.sc = sg::carve_scratch(c, std::max(sg::sum_words(k, k, m, 1), sg::sum_words(m, k, k, 0)));
+  }
+  return w;
+}
+cudaError_t orth(const double* AS, int m, int k, double* Q, OrthSpace& w, unsigned long long spin_ns,
+                 cudaStream_t s) {
+  cudaError_t e;
+  const long long mk = (long long)m * k;
+  if (k <= kSliceK) {
+    gram(AS, m, k, w.gpart, w.G, s);
+    chol_inv(w.G, k, w.Linv, w.gpart, w.status, s);
+    q_kernel<<<(unsigned)((mk + 255) / 256), 256, 0, s>>>(AS, w.Linv, m, k, Q);
+    return cudaGetLastError();
+  }
+  const sg::Source a{AS, CSS_F64, m, 1, k, m}, ar{AS, CSS_F64, 1, m, m, k}, li{w.Linv, CSS_F64, 1, k, k, k};
+  if ((e = sg::split(a, w.DS, s)) != cudaSuccess || (e = sg::split(ar, w.DSr, s)) != cudaSuccess) return e;
+  if ((e = sg::gemm(w.DS, a, w.DS, a, sg::Store{w.G, 1, k, 1}, w.sc, w.status + 1, spin_ns, s)) != cudaSuccess) return e;
+  chol_inv(w.G, k, w.Linv, w.gpart, w.status, s);
+  if ((e = sg::split(li, w.DL, s)) != cudaSuccess) return e;
+  return sg::gemm(w.DSr, ar, w.DL, li, sg::Store{Q, 1, m, 0}, w.sc, w.status + 1, spin_ns, s);
 }
 
 // The call's status once its work is enqueued (opts->sync): [0] A_S is rank
@@ -432,7 +425,8 @@ __global__ void das_kernel(const double* __restrict__ P, const double* __restric
 
 struct BwLayout {
   int* status;   // [0] A_S is rank deficient, [1] error of the products
-  double *AS, *G, *gpart, *Linv, *Q, *W;
+  double *AS, *Q, *W;
+  OrthSpace o;
   void* R;       // residual: FP32, FP64 for FP64 input
   double* Psum;
   double* loss_part;
@@ -446,9 +440,7 @@ BwLayout bw_layout(void* ws, size_t cap, int dt, int64_t m, int64_t n, int32_t k
   BwLayout L{};
   L.status = c.take<int>(64);
   L.AS = c.take<double>((size_t)m * k);
-  L.G = c.take<double>((size_t)k * k);
-  L.gpart = c.take<double>(gram_part_doubles((int)m, k));
-  L.Linv = c.take<double>((size_t)k * k);
+  L.o = carve_orth(c, L.status, m, k);
   L.Q = c.take<double>((size_t)m * k);
   L.W = c.take<double>((size_t)k * n);
   const size_t rs = dt == CSS_F64 ? 8 : 4;
@@ -459,7 +451,7 @@ BwLayout bw_layout(void* ws, size_t cap, int dt, int64_t m, int64_t n, int32_t k
   L.DQr = sg::carve_digits(c, m, k);
   L.DWr = sg::carve_digits(c, n, k);
   const long long cols = chunk_cols(m, n, k);
-  L.sc = sg::carve_scratch(c, cols, k, m);
+  L.sc = sg::carve_scratch(c, std::max(sg::sum_words(cols, k, m, 0), sg::sum_words(128, k, m, 0)));
   L.DW = sg::carve_digits(c, k, n);
   // A's digits are done with when R's are formed
   const size_t at = c.off;
@@ -469,7 +461,7 @@ BwLayout bw_layout(void* ws, size_t cap, int dt, int64_t m, int64_t n, int32_t k
     c.off = at;
     L.DR = sg::carve_digits(c, m, n);
     c.off = std::max(c.off, end);
-    L.scp = sg::carve_scratch(c, m, k, n);
+    L.scp = sg::carve_scratch(c, sg::sum_words(m, k, n, 0));
   }
   L.bytes = c.off;
   return L;
@@ -485,9 +477,7 @@ css_status run_backward(const TA* A, int m, int n, long long lda, const int* sel
   int* err = L.status + 1;
   const long long mk = (long long)m * k;
   gather_cols_kernel<TA><<<(unsigned)((mk + 255) / 256), 256, 0, s>>>(A, lda, m, sel, k, L.AS);
-  gram(L.AS, m, k, L.gpart, L.G, s);
-  chol_inv(L.G, k, L.Linv, L.status, s);
-  q_kernel<<<(unsigned)((mk + 255) / 256), 256, 0, s>>>(L.AS, L.Linv, m, k, L.Q);
+  if (orth(L.AS, m, k, L.Q, L.o, spin, s) != cudaSuccess) return CSS_ERR_CUDA;
   const sg::Source q{L.Q, CSS_F64, m, 1, k, m}, qr{L.Q, CSS_F64, 1, m, m, k};
   const sg::Source w{L.W, CSS_F64, 1, k, k, n}, wr{L.W, CSS_F64, k, 1, n, k};
   if (sg::split(q, L.DQ, s) != cudaSuccess || sg::split(qr, L.DQr, s) != cudaSuccess) return CSS_ERR_CUDA;
@@ -503,16 +493,18 @@ css_status run_backward(const TA* A, int m, int n, long long lda, const int* sel
   } else {
     const sg::Residual r{A, dt, lda, dA ? (float*)L.R : nullptr, dA, ldda, 2.0 * grad_out, L.loss_part};
     parts = sg::residual_parts();
-    if (sg::gemm_residual(L.DQr, L.DWr, r, err, spin, s) != cudaSuccess) return CSS_ERR_CUDA;
+    if (sg::gemm_residual(L.DQr, L.DWr, r, L.sc, err, spin, s) != cudaSuccess) return CSS_ERR_CUDA;
   }
   if (loss) sum_kernel<<<1, 512, 0, s>>>(L.loss_part, parts, 1.0, loss);
   if (dA) {
     const sg::Source r{L.R, dt == CSS_F64 ? CSS_F64 : CSS_F32, 1, m, m, n};
     const sg::Store st{L.Psum, 1, m, 0};
-    if (sg::split(r, L.DR, s) != cudaSuccess || sg::split(w, L.DW, s) != cudaSuccess ||
-        sg::gemm(L.DR, r, L.DW, w, st, L.scp, err, spin, s) != cudaSuccess)
+    // (R is held in FP32 for FP32 and BF16 input)
+    const sg::Precision prec = dt == CSS_F64 ? sg::kFull : sg::kSingle;
+    if (sg::split(r, L.DR, s, prec) != cudaSuccess || sg::split(w, L.DW, s, prec) != cudaSuccess ||
+        sg::gemm(L.DR, r, L.DW, w, st, L.scp, err, spin, s, prec) != cudaSuccess)
       return CSS_ERR_CUDA;
-    das_kernel<TA><<<(unsigned)((mk + 255) / 256), 256, 0, s>>>(L.Psum, L.Linv, m, k, sel, 2.0 * grad_out, dA,
+    das_kernel<TA><<<(unsigned)((mk + 255) / 256), 256, 0, s>>>(L.Psum, L.o.Linv, m, k, sel, 2.0 * grad_out, dA,
                                                                ldda);
   }
   if (cudaGetLastError() != cudaSuccess) return CSS_ERR_CUDA;
@@ -531,7 +523,8 @@ __global__ void copy_cols_kernel(const double* __restrict__ src, int m, int l, d
 
 struct EmbLayout {
   int* status;
-  double *AS, *G, *gpart, *Linv, *Q1, *Q;
+  double *AS, *Q1, *Q;
+  OrthSpace o;
   sg::Digits DQ, DA;
   sg::Scratch sc;
   size_t bytes;
@@ -542,15 +535,13 @@ EmbLayout emb_layout(void* ws, size_t cap, int64_t m, int64_t n, int32_t l) {
   EmbLayout L{};
   L.status = c.take<int>(64);
   L.AS = c.take<double>((size_t)m * l);
-  L.G = c.take<double>((size_t)l * l);
-  L.gpart = c.take<double>(gram_part_doubles((int)m, l));
-  L.Linv = c.take<double>((size_t)l * l);
+  L.o = carve_orth(c, L.status, m, l);
   L.Q1 = c.take<double>((size_t)m * l);
   L.Q = c.take<double>((size_t)m * l);
   const long long cols = chunk_cols(m, n, l);
   L.DQ = sg::carve_digits(c, l, m);
   L.DA = sg::carve_digits(c, cols, m);
-  L.sc = sg::carve_scratch(c, cols, l, m);
+  L.sc = sg::carve_scratch(c, std::max(sg::sum_words(cols, l, m, 0), sg::sum_words(128, l, m, 0)));
   L.bytes = c.off;
   return L;
 }
@@ -566,17 +557,13 @@ css_status run_embed(const TA* A, int m, int n, long long lda, const int* sel, i
   const long long ml = (long long)m * l;
   const unsigned gb = (unsigned)((ml + 255) / 256);
   gather_cols_kernel<TA><<<gb, 256, 0, s>>>(A, lda, m, sel, l, L.AS);
-  gram(L.AS, m, l, L.gpart, L.G, s);
-  chol_inv(L.G, l, L.Linv, L.status, s);
-  q_kernel<<<gb, 256, 0, s>>>(L.AS, L.Linv, m, l, L.Q1);
-  gram(L.Q1, m, l, L.gpart, L.G, s);
-  chol_inv(L.G, l, L.Linv, L.status, s);
-  q_kernel<<<gb, 256, 0, s>>>(L.Q1, L.Linv, m, l, L.Q);
+  const unsigned long long spin = o.spin_budget_ns ? o.spin_budget_ns : 2000000000ull;
+  if (orth(L.AS, m, l, L.Q1, L.o, spin, s) != cudaSuccess || orth(L.Q1, m, l, L.Q, L.o, spin, s) != cudaSuccess)
+    return CSS_ERR_CUDA;
   if (W) {
     const sg::Source q{L.Q, CSS_F64, m, 1, l, m};
     if (sg::split(q, L.DQ, s) != cudaSuccess ||
-        w_product(L.DQ, q, A, dt, lda, m, n, l, W, ldw, 1, L.DA, L.sc, L.status + 1,
-                  o.spin_budget_ns ? o.spin_budget_ns : 2000000000ull, s) != cudaSuccess)
+        w_product(L.DQ, q, A, dt, lda, m, n, l, W, ldw, 1, L.DA, L.sc, L.status + 1, spin, s) != cudaSuccess)
       return CSS_ERR_CUDA;
   }
   if (Qout) copy_cols_kernel<<<gb, 256, 0, s>>>(L.Q, m, l, Qout, ldq);

@@ -5,9 +5,8 @@
 //
 // W is short and wide (l x n, l <= 1024), so its SVD goes through the l x l
 // Gram matrix G = W W^T = U^(W) (Sigma^(W))^2 U^(W)^T:
-//   1. gram_rows_kernel: G in FP64 over lower 32 x 32 tiles, the n columns cut
-//      into slices whose partial tiles gram_reduce_kernel adds in a fixed
-//      order (bitwise reproducible).
+//   1. G on the slice GEMM (slice_gemm.cu): exact digit products, so G is as
+//      accurate as an FP64 product, on the tensor cores.
 //   2. jacobi_kernel: the eigenvalues of G by two-sided cyclic Jacobi
 //      rotations (Golub and Van Loan, Matrix Computations, Sec. 8.5) in the
 //      parallel round-robin ordering of Brent and Luk (1985): each round
@@ -21,94 +20,34 @@
 //      the 1 / sigma scaling of V~; replay_columns_kernel forms only the k
 //      wanted eigenvectors from the rotation log, off the barrier-bound path,
 //      and signs them (U^(W)_k).
-//   4. gemm_nn_df_kernel: U~ = Q U^(W)_k and V~ = W^T U^(W)_k Sigma_k^-1,
-//      products in double-float (df.cuh) on the FP32 pipe.
+//   4. U~ = Q U^(W)_k and V~ = W^T U^(W)_k Sigma_k^-1 on the slice GEMM.
 //
-// Steps 1-3 are FP64: on this part FP64 runs at 1/64 of the FP32 rate, so
-// the Gram matrix (l^2 n / 2 multiply-adds) is bound by the FP64 pipe, and
-// each Jacobi round by latency: one dependent L2 trip, a short chain of FP64
-// arithmetic and a grid barrier.  The products of step 4 (l k (m + n)
-// multiply-adds) need no more than double-float's 48 bits: their results
-// are a singular basis, accurate to the Gram route's resolution anyway.
+// The Jacobi rounds are bound by latency: one dependent L2 trip, a short chain
+// of FP64 arithmetic (two lanes per clock and SM) and a grid barrier each.
 #include <algorithm>
 #include <cmath>
 #include <vector>
 
 #include "css_common.cuh"
 #include "lowrank.cuh"
-#include "df.cuh"
+#include "slice_gemm.cuh"
 
 using namespace css;
 
 namespace {
 
-constexpr int kGT = 32;          // Gram tile
-constexpr int kGK = 32;          // columns per staged chunk
 constexpr int kMaxL = 1024;
 constexpr int kMaxSweeps = 40;
 constexpr int kJacobiThreads = 256;
 constexpr int kMaxGridDim = 16;  // at most 16 * 17 / 2 = 136 CTAs (<= one per SM)
 
-// ----------------------------------------------------------- 1. G = W W^T --
-// Block (pair, slice): output tile (ti, tj), ti >= tj, over the columns of one
-// slice; 2 x 2 outputs per thread.
-__global__ void __launch_bounds__(256) gram_rows_kernel(const double* __restrict__ W, long long ldw, int l,
-                                                        int n, int slice, int npairs,
-                                                        double* __restrict__ part) {
-  __shared__ double xa[kGT][kGK + 1], xb[kGT][kGK + 1];
-  const int pidx = blockIdx.x, sl = blockIdx.y;
-  int ti = (int)((sqrtf(8.f * pidx + 1.f) - 1.f) * 0.5f);
-  while (ti * (ti + 1) / 2 > pidx) --ti;
-  while ((ti + 1) * (ti + 2) / 2 <= pidx) ++ti;
-  const int tj = pidx - ti * (ti + 1) / 2;
-  const int a0 = ti * kGT, b0 = tj * kGT;
-  const int cb = sl * slice, ce = min(n, cb + slice);
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  double acc00 = 0.0, acc01 = 0.0, acc10 = 0.0, acc11 = 0.0;
-  for (int c0 = cb; c0 < ce; c0 += kGK) {
-    for (int e = threadIdx.x; e < kGT * kGK; e += 256) {
-      const int row = e / kGK, col = e % kGK;
-      const bool okc = c0 + col < ce;
-      xa[row][col] = (okc && a0 + row < l) ? W[(long long)(a0 + row) * ldw + c0 + col] : 0.0;
-      xb[row][col] = (okc && b0 + row < l) ? W[(long long)(b0 + row) * ldw + c0 + col] : 0.0;
-    }
-    __syncthreads();
-#pragma unroll 8
-    for (int kk = 0; kk < kGK; ++kk) {
-      const double u0 = xa[ty * 2][kk], u1 = xa[ty * 2 + 1][kk];
-      const double v0 = xb[tx * 2][kk], v1 = xb[tx * 2 + 1][kk];
-      acc00 = fma(u0, v0, acc00);
-      acc01 = fma(u0, v1, acc01);
-      acc10 = fma(u1, v0, acc10);
-      acc11 = fma(u1, v1, acc11);
-    }
-    __syncthreads();
-  }
-  double* out = part + ((long long)sl * npairs + pidx) * (kGT * kGT);
-  out[(ty * 2) * kGT + tx * 2] = acc00;
-  out[(ty * 2) * kGT + tx * 2 + 1] = acc01;
-  out[(ty * 2 + 1) * kGT + tx * 2] = acc10;
-  out[(ty * 2 + 1) * kGT + tx * 2 + 1] = acc11;
-}
-
-// G (lp x lp, column-major, zero padding row/column when l is odd) from the
-// slices' partial tiles, added in slice order.
-__global__ void gram_reduce_kernel(const double* __restrict__ part, int nslices, int npairs, int l, int lp,
-                                   double* __restrict__ G) {
-  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (long long)lp * lp) return;
-  const int r = (int)(idx % lp), c = (int)(idx / lp);
-  if (r >= l || c >= l) {
-    G[idx] = 0.0;
-    return;
-  }
-  const int a = max(r, c), b = min(r, c);
-  const int ti = a / kGT, tj = b / kGT;
-  const int pidx = ti * (ti + 1) / 2 + tj;
-  const int off = (a % kGT) * kGT + (b % kGT);
-  double s = 0.0;
-  for (int q = 0; q < nslices; ++q) s += part[((long long)q * npairs + pidx) * (kGT * kGT) + off];
-  G[idx] = s;
+// A zero padding row and column when l is odd (the Gram matrix is written
+// with leading dimension lp).
+__global__ void pad_kernel(double* __restrict__ G, int l, int lp) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= lp) return;
+  G[(long long)l * lp + i] = 0.0;
+  G[(long long)i * lp + l] = 0.0;
 }
 
 // ------------------------------------------------------------- 2. Jacobi --
@@ -428,111 +367,28 @@ __global__ void __launch_bounds__(1024) order_kernel(const double* __restrict__ 
   }
 }
 
-// ----------------------------------- 4. C = A B diag(scale), double-float --
-// A: M x K (lda), B: K x N (ldb), C: M x N (ldc), all column-major FP64.
-// 64 x 64 outputs per block, 4 x 4 per thread (rows tx + 16 a, columns
-// ty + 16 b).  The operands are split into hi + lo floats as they are staged
-// and the products accumulate in double-float (df.cuh): about 2^-46 relative
-// per term against FP64's 2^-53, on the FP32 pipe.  When a_bound is given
-// (a device value >= every |A_ij|), A is first scaled by 2^-(e+1), where
-// 2^e <= a_bound < 2^(e+1), so its entries stay inside FP32's range; the
-// scaling is exact and is undone on the output.  B's entries must lie in
-// FP32's range (here: orthonormal columns, entries <= 1).
-__global__ void __launch_bounds__(256) gemm_nn_df_kernel(const double* __restrict__ A, long long lda,
-                                                         const double* __restrict__ B, long long ldb,
-                                                         const double* __restrict__ scale,
-                                                         const double* __restrict__ a_bound,
-                                                         double* __restrict__ C, long long ldc, long long M,
-                                                         int N, int K) {
-  constexpr int BK = 16;
-  __shared__ float2 as[BK][64], bs[BK][65];
-  const long long m0 = (long long)blockIdx.x * 64;
-  const int n0 = blockIdx.y * 64;
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  double sa = 1.0, inv_sa = 1.0;
-  if (a_bound) {
-    const double ab = *a_bound;
-    if (ab > 0.0 && isfinite(ab)) {
-      const int e = ilogb(ab) + 1;
-      sa = ldexp(1.0, -e);
-      inv_sa = ldexp(1.0, e);
-    }
-  }
-  DF acc[4][4];
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = DF{0.f, 0.f};
-  for (int k0 = 0; k0 < K; k0 += BK) {
-    for (int e = threadIdx.x; e < BK * 64; e += 256) {
-      const int i = e % 64, kk = e / 64;
-      float2 va = make_float2(0.f, 0.f), vb = make_float2(0.f, 0.f);
-      if (m0 + i < M && k0 + kk < K) df_split(A[(long long)(k0 + kk) * lda + m0 + i] * sa, va.x, va.y);
-      as[kk][i] = va;
-      const int kk2 = e % BK, j = e / BK;
-      if (n0 + j < N && k0 + kk2 < K) df_split(B[(long long)(n0 + j) * ldb + k0 + kk2], vb.x, vb.y);
-      bs[kk2][j] = vb;
-    }
-    __syncthreads();
-#pragma unroll 4
-    for (int kk = 0; kk < BK; ++kk) {
-      float2 av[4], bv[4];
-#pragma unroll
-      for (int a = 0; a < 4; ++a) av[a] = as[kk][tx + 16 * a];
-#pragma unroll
-      for (int b = 0; b < 4; ++b) bv[b] = bs[kk][ty + 16 * b];
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) df_fma2(acc[a][b], av[a].x, av[a].y, bv[b].x, bv[b].y);
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int b = 0; b < 4; ++b) {
-    const int j = n0 + ty + 16 * b;
-    if (j >= N) continue;
-    const double sc = (scale ? scale[j] : 1.0) * inv_sa;
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      const long long i = m0 + tx + 16 * a;
-      if (i < M) C[(long long)j * ldc + i] = ((double)acc[a][b].s + (double)acc[a][b].c) * sc;
-    }
-  }
-}
-
 // ------------------------------------------------------------ host side --
 struct LrLayout {
   DevStatus* st;
   int* info;
   int* flags;
   uint32_t* bar;
-  double *part, *G0, *G1, *Uw, *scale;
+  double *G0, *G1, *Uw, *scale;
   int* ord;
   double2* rotlog;
   long long max_rounds;
-  int nslices, npairs, slice;
+  sg::Digits DW, DUw;   // W (both ways, one after the other) or Q, and U^(W)_k
+  sg::Scratch sc;
   size_t bytes;
 };
 
-int gram_tiles(int l) { return (l + kGT - 1) / kGT; }
-
-LrLayout lr_layout(void* ws, size_t cap, int64_t n, int32_t l, int32_t k, int sms) {
+LrLayout lr_layout(void* ws, size_t cap, int64_t n, int32_t l, int32_t k) {
   WsCarver c(ws, cap);
   LrLayout L{};
   L.st = (DevStatus*)c.take<char>(kStatusBytes);   // first: css_read_status reads it
   L.info = c.take<int>(64);
   L.flags = c.take<int>(kMaxSweeps + 4);
   L.bar = c.take<uint32_t>(64);
-  const int t = gram_tiles(l);
-  L.npairs = t * (t + 1) / 2;
-  // about twelve (pair, slice) blocks per SM, so that the uneven last share
-  // of blocks costs little; slices of >= 256 columns
-  const int want = std::max(1, (12 * std::max(sms, 1) + L.npairs - 1) / L.npairs);
-  const int cap_slices = (int)std::max<int64_t>(1, (n + 255) / 256);
-  L.nslices = std::min({want, cap_slices, 256});
-  L.slice = (int)((n + L.nslices - 1) / L.nslices);
-  L.part = c.take<double>((size_t)L.nslices * L.npairs * kGT * kGT);
   const int lp = l + (l & 1);
   L.G0 = c.take<double>((size_t)lp * lp);
   L.G1 = c.take<double>((size_t)lp * lp);
@@ -541,6 +397,16 @@ LrLayout lr_layout(void* ws, size_t cap, int64_t n, int32_t l, int32_t k, int sm
   L.rotlog = c.take<double2>((size_t)L.max_rounds * (lp / 2));
   L.Uw = c.take<double>((size_t)l * k);
   L.scale = c.take<double>(k);
+  // the digits of W by rows, of W by columns and of Q (n rows at a time)
+  // share their space
+  const size_t at = c.off;
+  sg::carve_digits(c, l, n);
+  const size_t end = c.off;
+  c.off = at;
+  L.DW = sg::carve_digits(c, n, l);
+  c.off = std::max(c.off, end);
+  L.DUw = sg::carve_digits(c, k, l);
+  L.sc = sg::carve_scratch(c, sg::sum_words(l, l, n, 1));
   L.bytes = c.off;
   return L;
 }
@@ -552,14 +418,10 @@ int device_sms() {
   return n;
 }
 
-// The Gram slices are sized for 152 SMs whatever the device, so that
-// css_workspace_size needs no device and the launch carves the same layout.
-constexpr int kLayoutSms = 152;
-
 }  // namespace
 
 size_t lowrank_workspace_bytes(int64_t n, int32_t l, int32_t k) {
-  return lr_layout(nullptr, (size_t)-1, n, l, k, kLayoutSms).bytes;
+  return lr_layout(nullptr, (size_t)-1, n, l, k).bytes;
 }
 
 extern "C" css_status css_lowrank(const double* W, int64_t ldw, const double* Q, int64_t ldq, int64_t m,
@@ -574,7 +436,7 @@ extern "C" css_status css_lowrank(const double* W, int64_t ldw, const double* Q,
   if (U && (!Q || m < 1 || m > INT32_MAX || ldq < m || ldu < m)) return CSS_ERR_INVALID_ARG;
   if (V && ldv < n) return CSS_ERR_INVALID_ARG;
   if (!ws || ((uintptr_t)ws % kWsAlign) != 0) return CSS_ERR_WORKSPACE;
-  LrLayout L = lr_layout(ws, ws_bytes, n, l, k, kLayoutSms);
+  LrLayout L = lr_layout(ws, ws_bytes, n, l, k);
   if (L.bytes > ws_bytes) return CSS_ERR_WORKSPACE;
   int dev = 0, major = 0, minor = 0, coop = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return CSS_ERR_CUDA;
@@ -616,9 +478,18 @@ extern "C" css_status css_lowrank(const double* W, int64_t ldw, const double* Q,
     }
   } guard{ev};
   if (timed) cudaEventRecord(ev[0], s);
-  gram_rows_kernel<<<dim3(L.npairs, L.nslices), 256, 0, s>>>(W, ldw, l, (int)n, L.slice, L.npairs, L.part);
-  gram_reduce_kernel<<<(unsigned)(((long long)lp * lp + 255) / 256), 256, 0, s>>>(L.part, L.nslices, L.npairs,
-                                                                                   l, lp, L.G0);
+  int* err = &L.st->code;
+  const sg::Source w{W, CSS_F64, ldw, 1, l, (int)n}, wr{W, CSS_F64, 1, ldw, (int)n, l};
+  sg::Digits DG = L.DW;
+  {
+    // (the same space, carved for l rows of n)
+    WsCarver c(L.DW.d, (size_t)-1);
+    DG = sg::carve_digits(c, l, n);
+  }
+  e = sg::split(w, DG, s);
+  if (e == cudaSuccess) e = sg::gemm(DG, w, DG, w, sg::Store{L.G0, 1, lp, 1}, L.sc, err, hs.spin_budget_ns, s);
+  if (e != cudaSuccess) return CSS_ERR_CUDA;
+  if (lp > l) pad_kernel<<<(lp + 255) / 256, 256, 0, s>>>(L.G0, l, lp);
   if (cudaGetLastError() != cudaSuccess) return CSS_ERR_CUDA;
   if (timed) cudaEventRecord(ev[1], s);
   JacobiArgs ja{L.G0, L.G1, L.rotlog, L.max_rounds, lp, gdim, chunk, L.bar, L.flags, L.info, L.st};
@@ -630,13 +501,22 @@ extern "C" css_status css_lowrank(const double* W, int64_t ldw, const double* Q,
   order_kernel<<<1, 1024, 0, s>>>(L.G0, L.G1, L.info, l, lp, k, (long long)n, sigma, L.scale, tail, L.ord);
   replay_columns_kernel<<<k, (h + 31) / 32 * 32, lp * sizeof(double), s>>>(L.rotlog, L.info, L.ord, l, lp, uw);
   if (timed) cudaEventRecord(ev[2], s);
-  // |W_ij| <= ||W||_2 = sigma_1 bounds W's entries for the FP32 split
-  if (U)
-    gemm_nn_df_kernel<<<dim3((unsigned)((m + 63) / 64), (k + 63) / 64), 256, 0, s>>>(Q, ldq, uw, l, nullptr, nullptr,
-                                                                                      U, ldu, m, k, l);
-  if (V)
-    gemm_nn_df_kernel<<<dim3((unsigned)((n + 63) / 64), (k + 63) / 64), 256, 0, s>>>(W, ldw, uw, l, L.scale, sigma,
-                                                                                      V, ldv, n, k, l);
+  sg::Digits& DQ = L.DW;
+  const sg::Source us{uw, CSS_F64, l, 1, k, l};
+  e = U || V ? sg::split(us, L.DUw, s) : cudaSuccess;
+  const int rows = ((int)n + 127) / 128 * 128;   // the digits' space holds whole tiles
+  for (int64_t r0 = 0; U && e == cudaSuccess && r0 < m; r0 += rows) {
+    const sg::Source q{Q + r0, CSS_F64, 1, ldq, (int)std::min<int64_t>(rows, m - r0), l};
+    e = sg::split(q, DQ, s);
+    if (e == cudaSuccess)
+      e = sg::gemm(DQ, q, L.DUw, us, sg::Store{U + r0, 1, ldu, 0}, L.sc, err, hs.spin_budget_ns, s);
+  }
+  if (V && e == cudaSuccess) {
+    e = sg::split(wr, L.DW, s);
+    if (e == cudaSuccess)
+      e = sg::gemm(L.DW, wr, L.DUw, us, sg::Store{V, 1, ldv, 0, L.scale}, L.sc, err, hs.spin_budget_ns, s);
+  }
+  if (e != cudaSuccess) return CSS_ERR_CUDA;
   if (cudaGetLastError() != cudaSuccess) return CSS_ERR_CUDA;
   if (timed) cudaEventRecord(ev[3], s);
   if (!o.sync) return CSS_OK;

@@ -22,8 +22,11 @@
 // and split-K partial sums may meet in integer atomics.
 //
 // Measured: W = Q^T A of a 4096 x 65536 BF16 matrix with l = 256 (68.7 G
-// multiply-adds) 24 ms as double-float on the FP32 pipe, 5.0 ms here with the
-// split; its error against 64 bits fell from 1.1e-12 to 2.2e-15.
+// multiply-adds) 24 ms as double-float on the FP32 pipe; here 2.3 ms and 0.7 ms
+// for the split of A; its error against 64 bits fell from 1.1e-12 to 2.2e-15.
+// The tensor pipe is active 57 % of the time; the rest is the drains, during
+// which the accumulators cannot take products.  G = W W^T, 256 x 65536: 4.26 ms
+// in FP64 instructions, 0.17 ms here.
 //
 // Slices that are zero in a block of 128 rows x 64 k are not stored, loaded
 // or multiplied: BF16 entries of similar size have three non-zero slices,
@@ -168,8 +171,9 @@ __device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) 
 // or a NaN get zero digits (the product restores them from the source).
 template <typename T, typename V, bool KC, bool VEC>
 __global__ void __launch_bounds__(256) split_kernel(const T* __restrict__ p, long long rs, long long ks, int rows,
-                                                    int K, int k64, int dtype, const int* __restrict__ ex,
-                                                    unsigned char* __restrict__ d, unsigned char* __restrict__ ns) {
+                                                    int K, int k64, int dtype, int slices,
+                                                    const int* __restrict__ ex, unsigned char* __restrict__ d,
+                                                    unsigned char* __restrict__ ns) {
   const int r0 = blockIdx.x * kT, kb = blockIdx.y;
   V v[4][8];
   load_block<T, V, KC, VEC>(p, rs, ks, rows, K, r0, kb * kKb, v);
@@ -209,10 +213,10 @@ __global__ void __launch_bounds__(256) split_kernel(const T* __restrict__ p, lon
     }
   }
   int s = 0;
-  for (; s < kS; ++s) {
+  for (; s < slices; ++s) {
     int any = 0;
     if constexpr (sizeof(V) == 4) {
-      const float least = 0.5f * pow2f(-8 * (kS - 1 - s));
+      const float least = 0.5f * pow2f(-8 * (slices - 1 - s));
 #pragma unroll
       for (int q = 0; q < 4; ++q)
 #pragma unroll
@@ -278,9 +282,10 @@ struct Args {
   int tn, tiles;       // tiles along N; tiles in all
   int lower;
   int ksplit, k16_per; // K slices and their 16-k blocks (a multiple of 4)
+  int halves;          // 2, or 1: the high digits alone
   Store st;
   Source sx, sy;
-  double* lo;
+  long long* part;
   unsigned long long* sums;
   Residual r;
   int* err;
@@ -323,12 +328,6 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
-// v 2^e (e may leave the range of one factor)
-__device__ __forceinline__ double scale2(double v, int e) {
-  if (e > -1000 && e < 1000) return v * __hiloint2double((e + 1023) << 20, 0);
-  return scalbn(v, e);
-}
-
 template <typename TX>
 __device__ double plain_dot_x(const Source& x, const Source& y, int i, int j) {
   const TX* p = (const TX*)x.p + i * x.rs;
@@ -349,19 +348,70 @@ __device__ __noinline__ double plain_dot(const Source& x, const Source& y, int i
   return plain_dot_x<__nv_bfloat16>(x, y, i, j);
 }
 
-// The result from its integer sums: hi in units of 2^-40, lo in 2^-72, times
-// the rows' scales.
-__device__ __forceinline__ double combine(double hi, double lo, int ex, int ey) {
-  return scale2(hi * 0x1p-40 + lo * 0x1p-72, ex + ey);
+// The result from its integer sums, (hi 2^32 + lo) 2^(e - 72), rounded once to
+// nearest even.  In integer instructions: an FP64 instruction occupies the SM's
+// FP64 pipe for 16 clocks, and conversions, scaling and the sum would take
+// seven of them an entry.
+__device__ __forceinline__ double combine(long long hi, long long lo, int e) {
+  unsigned long long b = (unsigned long long)hi << 32;
+  long long t = hi >> 32;
+  const unsigned long long l = (unsigned long long)lo;
+  b += l;
+  t += (b < l) + (lo >> 63);
+  const bool neg = t < 0;
+  unsigned long long a = (unsigned long long)t;
+  if (neg) {
+    b = ~b + 1;
+    a = ~a + (b == 0);
+  }
+  if ((a | b) == 0) return 0.0;
+  // normalised: the leading bit at the top of a
+  int n = 0;
+  if (a == 0) {
+    a = b;
+    b = 0;
+    n = 64;
+  }
+  const int z = __clzll((long long)a);
+  if (z > 0) {
+    a = a << z | b >> (64 - z);
+    b <<= z;
+  }
+  n += z;
+  unsigned long long mant = a >> 11;
+  const unsigned int rest = (unsigned int)a & 0x7ffu;
+  mant += rest > 0x400u || (rest == 0x400u && (b != 0 || (mant & 1)));
+  const int ex = 127 - n - 72 + e;
+  double v;
+  if (ex > -1022 && ex < 1023)
+    v = __longlong_as_double((long long)((unsigned long long)(ex + 1022) << 52) + (long long)mant);
+  else
+    v = scalbn((double)mant, ex - 52);
+  return neg ? -v : v;
 }
 
-// N columns of this warp's TMEM lanes
-template <int N>
-__device__ __forceinline__ void tmem_ld(uint32_t taddr, float (&v)[N]) {
-  static_assert(N == 16, "one load");
-  tmem_ld16(taddr, v);
+__device__ __forceinline__ void store(const Store& st, int row, int c, double v) {
+  if (st.cscale) v *= __ldg(st.cscale + c);
+  if (st.out32) st.out32[row * st.rs + c * st.cs] = (float)v;
+  else st.out[row * st.rs + c * st.cs] = v;
 }
-constexpr int kLd = 16;
+
+// 32 columns of this warp's TMEM lanes
+constexpr int kLd = 32;
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, float (&v)[32]) {
+  uint32_t r[32];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,"
+      "%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+}
 
 template <int EP>
 __global__ void __launch_bounds__(kThreads, 1) slice_gemm_kernel(const __grid_constant__ Args P) {
@@ -409,7 +459,7 @@ __global__ void __launch_bounds__(kThreads, 1) slice_gemm_kernel(const __grid_co
     bool ok = true;
     for (int it = blockIdx.x; ok && it < items; it += gridDim.x) {
       const Item w = item_of(P, it);
-      for (int half = 1; ok && half >= 0; --half) {
+      for (int half = P.halves - 1; ok && half >= 0; --half) {
         const int kps = half ? 1 : 2, cap = half ? kS : 4;
         int cnt = 0;
         for (int k = w.k0; ok && k < w.k1; k += kps, ++st) {
@@ -474,7 +524,7 @@ __global__ void __launch_bounds__(kThreads, 1) slice_gemm_kernel(const __grid_co
     };
     for (int it = blockIdx.x; ok && it < items; it += gridDim.x) {
       const Item w = item_of(P, it);
-      for (int half = 1; ok && half >= 0; --half) {
+      for (int half = P.halves - 1; ok && half >= 0; --half) {
         const int kps = half ? 1 : 2, w0 = half ? 6 : 2;
         int used = 0, budget = 0, ready = 0;   // accumulators written, and waited for, in this chunk
         for (int k = w.k0; k < w.k1; k += kps, ++st) {
@@ -560,8 +610,11 @@ __global__ void __launch_bounds__(kThreads, 1) slice_gemm_kernel(const __grid_co
 #pragma unroll
         for (int j = 0; j < 64; ++j) df[j] = DF{0.f, 0.f};
       }
-      double* lo = P.lo + (long long)blockIdx.x * (kT * kT) + (long long)(ch * 64) * kT + r_tile;
-      for (int half = 1; ok && half >= 0; --half) {
+      // this thread's 64 entries in the CTA's scratch (hi, then lo halves): the
+      // results are formed from there in short loops, because 64 unrolled
+      // copies of that code do not stay in the instruction cache
+      long long* mine = P.part + (long long)blockIdx.x * (2 * kT * kT) + (long long)(ch * 64) * kT + r_tile;
+      for (int half = P.halves - 1; ok && half >= 0; --half) {
         if constexpr (EP != kEpResidual) {
 #pragma unroll
           for (int j = 0; j < 64; ++j) acc[j] = 0;
@@ -576,16 +629,16 @@ __global__ void __launch_bounds__(kThreads, 1) slice_gemm_kernel(const __grid_co
           fence_after();
 #pragma unroll
           for (int g = 0; g < 4; ++g) {
+            const float unit = half ? pow2f(-32 - 8 * g) : pow2f(-8 * g);   // residual: in units of 2^-16
             if (info >> g & 1) {
 #pragma unroll
               for (int j0 = 0; j0 < 64; j0 += kLd) {
                 float v[kLd];
-                tmem_ld<kLd>(tbase + (uint32_t)(g * kT + j0), v);
+                tmem_ld(tbase + (uint32_t)(g * kT + j0), v);
 #pragma unroll
                 for (int jj = 0; jj < kLd; ++jj) {
                   if constexpr (EP == kEpResidual) {
-                    // in units of 2^-16
-                    const float x = v[jj] * (half ? pow2f(-32 - 8 * g) : pow2f(-8 * g));
+                    const float x = v[jj] * unit;
                     DF& a = df[j0 + jj];
                     const float s = a.s + x, bb = s - a.s;
                     a.c += (a.s - (s - bb)) + (x - bb);
@@ -604,29 +657,9 @@ __global__ void __launch_bounds__(kThreads, 1) slice_gemm_kernel(const __grid_co
         }
         if (!ok) break;
         if constexpr (EP == kEpStore) {
-          if (half == 1) {
+          long long* part = mine + (half ? (long long)kT * kT : 0);
 #pragma unroll
-            for (int j = 0; j < 64; ++j) __stcg(lo + (long long)j * kT, (double)acc[j]);
-          } else {
-            // (loads of a batch before its stores, which they could alias)
-            const int ex = scale_exp(exr, P.xdt);
-#pragma unroll
-            for (int j0 = 0; j0 < 64; j0 += 16) {
-              double lv[16];
-#pragma unroll
-              for (int jj = 0; jj < 16; ++jj) lv[jj] = __ldcg(lo + (long long)(j0 + jj) * kT);
-#pragma unroll
-              for (int jj = 0; jj < 16; ++jj) {
-                const int c = col0 + j0 + jj;
-                const int eyr = __shfl_sync(0xffffffffu, ey2[j0 / 32], (j0 + jj) & 31);
-                if (row >= P.M || c >= P.N) continue;
-                double v = combine((double)acc[j0 + jj], lv[jj], ex, scale_exp(eyr, P.ydt));
-                if (dead_r || eyr == exp_special(P.ydt)) v = plain_dot(P.sx, P.sy, row, c);
-                P.st.out[row * P.st.rs + c * P.st.cs] = v;
-                if (P.lower && row != c) P.st.out[c * P.st.rs + row * P.st.cs] = v;
-              }
-            }
-          }
+          for (int j = 0; j < 64; ++j) __stcg(part + (long long)j * kT, acc[j]);
         } else if constexpr (EP == kEpSplitK) {
           unsigned long long* sums = P.sums + (half ? 0 : (long long)P.M * P.N);
           if (row < P.M) {
@@ -638,33 +671,65 @@ __global__ void __launch_bounds__(kThreads, 1) slice_gemm_kernel(const __grid_co
           }
         }
       }
+      if (!ok) break;
+      if constexpr (EP == kEpStore) {
+        const int ex = scale_exp(exr, P.xdt);
+        const bool two = P.halves > 1;
+#pragma unroll 1
+        for (int j0 = 0; j0 < 64; j0 += 8) {
+          long long hv[8], lv[8];
+#pragma unroll
+          for (int jj = 0; jj < 8; ++jj) {
+            hv[jj] = __ldcg(mine + (long long)(j0 + jj) * kT);
+            lv[jj] = two ? __ldcg(mine + (long long)(kT + j0 + jj) * kT) : 0;
+          }
+          const int ey = j0 < 32 ? ey2[0] : ey2[1];
+#pragma unroll
+          for (int jj = 0; jj < 8; ++jj) {
+            const int c = col0 + j0 + jj;
+            const int eyr = __shfl_sync(0xffffffffu, ey, (j0 + jj) & 31);
+            if (row >= P.M || c >= P.N) continue;
+            double v = combine(hv[jj], lv[jj], ex + scale_exp(eyr, P.ydt));
+            if (dead_r || eyr == exp_special(P.ydt)) v = plain_dot(P.sx, P.sy, row, c);
+            store(P.st, row, c, v);
+            if (P.lower && row != c) store(P.st, c, row, v);
+          }
+        }
+      }
       if constexpr (EP == kEpResidual) {
-        if (!ok) break;
+        float2* pairs = reinterpret_cast<float2*>(mine);
+#pragma unroll
+        for (int j = 0; j < 64; ++j) __stcg(pairs + (long long)j * kT, make_float2(df[j].s, df[j].c));
         const Residual& R = P.r;
         const int ex = scale_exp(exr, P.xdt) - 16;
         const float gh = (float)R.g2, gl = (float)(R.g2 - (double)gh);
         const bool g_plain = fabsf(gh) < 1e30f && fabsf(gh) > 1e-30f;
         const bool f32 = R.dtype == CSS_F32;
         const bool row_ok = row < P.M;
+#pragma unroll 1
+        for (int j0 = 0; j0 < 64; j0 += 8) {
+          float av[8];
+          float2 pv[8];
 #pragma unroll
-        for (int j0 = 0; j0 < 64; j0 += 16) {
-          float av[16];
-#pragma unroll
-          for (int jj = 0; jj < 16; ++jj) {
+          for (int jj = 0; jj < 8; ++jj) {
             const int c = col0 + j0 + jj;
+            pv[jj] = __ldcg(pairs + (long long)(j0 + jj) * kT);
             av[jj] = 0.f;
             if (row_ok && c < P.N)
               av[jj] = f32 ? load_val((const float*)R.A + (long long)c * R.lda + row)
                            : load_val((const __nv_bfloat16*)R.A + (long long)c * R.lda + row);
           }
+          const int ey = j0 < 32 ? ey2[0] : ey2[1];
 #pragma unroll
-          for (int jj = 0; jj < 16; ++jj) {
+          for (int jj = 0; jj < 8; ++jj) {
             const int c = col0 + j0 + jj;
-            const int eyr = __shfl_sync(0xffffffffu, ey2[j0 / 32], (j0 + jj) & 31);
+            const int eyr = __shfl_sync(0xffffffffu, ey, (j0 + jj) & 31);
             if (!row_ok || c >= P.N) continue;
             const int e = ex + scale_exp(eyr, P.ydt);
             const int e1 = max(-126, min(127, e)), e2 = max(-126, min(127, e - e1));
-            float vh = df[j0 + jj].s * pow2f(e1) * pow2f(e2), vl = df[j0 + jj].c * pow2f(e1) * pow2f(e2);
+            const float f1 = pow2f(e1), f2 = pow2f(e2);
+            float vh = pv[jj].x * f1 * f2;
+            const float vl = pv[jj].y * f1 * f2;
             if (dead_r || eyr == exp_special(P.ydt)) vh = __int_as_float(0x7fffffff);
             const float a = av[jj];
             // r = a - vh - vl as a normalised pair
@@ -722,30 +787,31 @@ __global__ void __launch_bounds__(256) finish_kernel(const __grid_constant__ Arg
   const bool up = P.lower && row / kT < c / kT;
   const long long at = up ? (long long)row * P.M + c : idx;
   const int exr = P.xe[row], eyr = P.ye[c];
-  double v = combine((double)(long long)P.sums[(long long)P.M * P.N + at], (double)(long long)P.sums[at],
-                     scale_exp(exr, P.xdt), scale_exp(eyr, P.ydt));
+  double v = combine((long long)P.sums[(long long)P.M * P.N + at], (long long)P.sums[at],
+                     scale_exp(exr, P.xdt) + scale_exp(eyr, P.ydt));
   if (exr == exp_special(P.xdt) || eyr == exp_special(P.ydt)) v = plain_dot(P.sx, P.sy, row, c);
-  P.st.out[row * P.st.rs + c * P.st.cs] = v;
+  store(P.st, row, c, v);
 }
 
 int k_blocks(long long K) { return (int)ceil_div(K, kKb); }
 
 template <typename T, typename V, bool KC, bool VEC>
-void launch_split(const Source& src, const Digits& D, cudaStream_t s) {
+void launch_split(const Source& src, const Digits& D, int slices, cudaStream_t s) {
   const int k64 = k_blocks(src.K);
   const unsigned tiles = (unsigned)ceil_div(src.rows, kT);
   const unsigned ky = (unsigned)std::min<long long>(k64, std::max<long long>(1, ceil_div(152 * 8, tiles)));
   row_exp_kernel<T, V, KC, VEC><<<dim3(tiles, ky), 256, 0, s>>>((const T*)src.p, src.rs, src.ks, src.rows, src.K,
                                                                 D.ex);
   split_kernel<T, V, KC, VEC><<<dim3(tiles, (unsigned)k64), 256, 0, s>>>((const T*)src.p, src.rs, src.ks, src.rows,
-                                                                        src.K, k64, src.dtype, D.ex, D.d, D.ns);
+                                                                        src.K, k64, src.dtype, slices, D.ex, D.d,
+                                                                        D.ns);
 }
 template <typename T, typename V>
-void launch_split_of(const Source& src, const Digits& D, cudaStream_t s) {
+void launch_split_of(const Source& src, const Digits& D, int slices, cudaStream_t s) {
   const bool vec = ((uintptr_t)src.p & 15u) == 0 && (src.rs * (long long)sizeof(T)) % 16 == 0;
-  if (src.ks == 1 && vec) launch_split<T, V, true, true>(src, D, s);
-  else if (src.ks == 1) launch_split<T, V, true, false>(src, D, s);
-  else launch_split<T, V, false, false>(src, D, s);
+  if (src.ks == 1 && vec) launch_split<T, V, true, true>(src, D, slices, s);
+  else if (src.ks == 1) launch_split<T, V, true, false>(src, D, slices, s);
+  else launch_split<T, V, false, false>(src, D, slices, s);
 }
 
 Args base_args(const Digits& X, const Digits& Y, int* err, unsigned long long spin_ns) {
@@ -766,6 +832,7 @@ Args base_args(const Digits& X, const Digits& Y, int* err, unsigned long long sp
   P.tn = (int)ceil_div(P.N, kT);
   P.tiles = (int)ceil_div(P.M, kT) * P.tn;
   P.ksplit = 1;
+  P.halves = 2;
   P.k16_per = P.k64 * 4;
   P.err = err;
   P.spin_ns = spin_ns;
@@ -781,10 +848,10 @@ cudaError_t launch_gemm(const Args& P, cudaStream_t s) {
 }
 
 // K slices for `tiles` result tiles: enough items for every SM, slices of at
-// least 512 k (a tile's two halves are then some twenty drains).
+// least 256 k (a few drains each; below that the atomics of the sums show).
 int k_slices(long long tiles, long long K) {
   if (tiles * 2 > kCtas) return 1;
-  return (int)std::max<long long>(1, std::min(kCtas / tiles, K / 512));
+  return (int)std::max<long long>(1, std::min(kCtas / tiles, K / 256));
 }
 
 }  // namespace
@@ -794,42 +861,49 @@ Digits carve_digits(WsCarver& c, long long rows, long long K) {
   const long long tiles = ceil_div(rows, kT), k64 = k_blocks(K);
   D.d = c.take<unsigned char>((size_t)(tiles * k64 * 4 * kS * kSliceBytes));
   D.ns = c.take<unsigned char>((size_t)(tiles * k64));
-  D.ex = c.take<int>((size_t)rows);
+  D.ex = c.take<int>((size_t)(tiles * kT));
   return D;
 }
 
-cudaError_t split(const Source& src, Digits& D, cudaStream_t s) {
+cudaError_t split(const Source& src, Digits& D, cudaStream_t s, Precision prec) {
   D.rows = src.rows;
   D.K = src.K;
   D.dtype = src.dtype;
   cudaError_t e = cudaMemsetAsync(D.ex, 0, sizeof(int) * (size_t)src.rows, s);
   if (e != cudaSuccess) return e;
   switch (src.dtype) {
-    case CSS_F64: launch_split_of<double, double>(src, D, s); break;
-    case CSS_F32: launch_split_of<float, float>(src, D, s); break;
-    default: launch_split_of<__nv_bfloat16, float>(src, D, s); break;
+    case CSS_F64: launch_split_of<double, double>(src, D, prec, s); break;
+    case CSS_F32: launch_split_of<float, float>(src, D, prec, s); break;
+    default: launch_split_of<__nv_bfloat16, float>(src, D, prec, s); break;
   }
   return cudaGetLastError();
 }
 
-Scratch carve_scratch(WsCarver& c, long long M, long long N, long long K) {
+size_t sum_words(long long M, long long N, long long K, int lower) {
+  const long long tm = ceil_div(M, kT), tiles = lower ? tm * (tm + 1) / 2 : tm * ceil_div(N, kT);
+  return k_slices(tiles, K) > 1 ? (size_t)(2 * M * N) : 0;
+}
+
+Scratch carve_scratch(WsCarver& c, size_t words) {
   Scratch w{};
-  w.lo = c.take<double>((size_t)kCtas * kT * kT);
-  if (k_slices(1, K) > 1 && ceil_div(M, kT) * ceil_div(N, kT) * 2 <= 2 * kCtas)
-    w.sums = c.take<unsigned long long>((size_t)(2 * M * N));
+  w.part = c.take<long long>((size_t)2 * kCtas * kT * kT);
+  w.sums = c.take<unsigned long long>(words);
+  w.cap = words;
   return w;
 }
 
 cudaError_t gemm(const Digits& X, const Source& sx, const Digits& Y, const Source& sy, const Store& st,
-                 const Scratch& w, int* err, unsigned long long spin_ns, cudaStream_t s) {
+                 const Scratch& w, int* err, unsigned long long spin_ns, cudaStream_t s, Precision prec) {
   Args P = base_args(X, Y, err, spin_ns);
+  P.halves = prec == kFull ? 2 : 1;
   P.st = st;
   P.sx = sx;
   P.sy = sy;
-  P.lo = w.lo;
+  P.part = w.part;
   P.lower = st.lower;
   if (st.lower) P.tiles = P.tn * (P.tn + 1) / 2;
-  P.ksplit = w.sums ? k_slices(P.tiles, P.K) : 1;
+  const size_t words = sum_words(P.M, P.N, P.K, P.lower);
+  P.ksplit = words && words <= w.cap ? k_slices(P.tiles, P.K) : 1;
   if (P.ksplit == 1) return launch_gemm<kEpStore>(P, s);
   P.sums = w.sums;
   P.k16_per = (int)ceil_div(ceil_div(P.k16, P.ksplit), 4) * 4;
@@ -844,9 +918,10 @@ cudaError_t gemm(const Digits& X, const Source& sx, const Digits& Y, const Sourc
 
 int residual_parts() { return kCtas; }
 
-cudaError_t gemm_residual(const Digits& X, const Digits& Y, const Residual& r, int* err,
+cudaError_t gemm_residual(const Digits& X, const Digits& Y, const Residual& r, const Scratch& w, int* err,
                           unsigned long long spin_ns, cudaStream_t s) {
   Args P = base_args(X, Y, err, spin_ns);
+  P.part = w.part;
   P.r = r;
   const int ctas = std::min(kCtas, P.tiles);
   if (ctas < kCtas) {

@@ -23,29 +23,41 @@ struct Digits {
   int rows, K, dtype;
 };
 
-// Carves the digits of a rows x K operand from a workspace (rows may be the
+// Accuracy of a product: kFull keeps all eight slices (what is dropped is
+// below 2^-64 of the rows' largest products), kSingle four and the digit
+// products down to 2^-33, for results that are held in FP32.
+enum Precision { kFull = 8, kSingle = 4 };
+
+// Carves the digits of a rows x K operand (whole tiles of 128 rows) from a
+// workspace (rows may be the
 // largest of several operands that use the same space one after another).
 Digits carve_digits(WsCarver& c, long long rows, long long K);
 // Splits src into digits (src.rows <= the carved rows).  Three launches.
-cudaError_t split(const Source& src, Digits& D, cudaStream_t s);
+cudaError_t split(const Source& src, Digits& D, cudaStream_t s, Precision prec = kFull);
 
-// Scratch of gemm: per-CTA partial sums, and for split-K the two halves of
-// the M x N sums.
+// Scratch of gemm: per-CTA partial sums, and the integer sums of a product
+// whose inner dimension is cut into slices (taken when they fit).
 struct Scratch {
-  double* lo;
+  long long* part;
   unsigned long long* sums;
+  size_t cap;           // 8-byte words of sums
 };
-Scratch carve_scratch(WsCarver& c, long long M, long long N, long long K);
+// Words of integer sums that an M x N product over K can use (0: none).
+size_t sum_words(long long M, long long N, long long K, int lower);
+Scratch carve_scratch(WsCarver& c, size_t words);
 
-// out[i * rs + j * cs] = sum_k X[i, k] Y[j, k].  lower: X and Y are the same
-// operand; only tiles touching i >= j are computed and both triangles written.
+// out[i * rs + j * cs] = cscale[j] sum_k X[i, k] Y[j, k] (FP64, or FP32 to
+// out32; cscale may be null).  lower: X and Y are the same operand; only tiles
+// touching i >= j are computed and both triangles written.
 struct Store {
   double* out;
   long long rs, cs;
   int lower;
+  const double* cscale;
+  float* out32;
 };
 cudaError_t gemm(const Digits& X, const Source& sx, const Digits& Y, const Source& sy, const Store& st,
-                 const Scratch& w, int* err, unsigned long long spin_ns, cudaStream_t s);
+                 const Scratch& w, int* err, unsigned long long spin_ns, cudaStream_t s, Precision prec = kFull);
 
 // R = A - X Y^T for FP32 or BF16 A (M x N, leading dimension lda): writes R
 // (FP32, leading dimension M) when R != null, dA = g2 R when dA != null, and
@@ -61,7 +73,7 @@ struct Residual {
   double* loss_part;
 };
 int residual_parts();
-cudaError_t gemm_residual(const Digits& X, const Digits& Y, const Residual& r, int* err,
+cudaError_t gemm_residual(const Digits& X, const Digits& Y, const Residual& r, const Scratch& w, int* err,
                           unsigned long long spin_ns, cudaStream_t s);
 
 }  // namespace sg
