@@ -249,13 +249,25 @@ css_status prepare_units(const Header& h, std::vector<UnitDesc>& units, const st
     k_max = std::max(k_max, u.k);
     r_max = std::max(r_max, u.r);
   }
-  const size_t smem = greedy_smem_bytes(dt, m_max, k_max, r_max, threads);
+  size_t smem = greedy_smem_bytes(dt, m_max, k_max, r_max, threads);
   if (smem > 227 * 1024) return CSS_ERR_UNSUPPORTED;
-  const int occ = greedy_occupancy(dt, tile_cols, smem, threads);
+  const int occ = greedy_occupancy(dt, tile_cols, kFeedRegs, smem, threads);
   const int sms = sm_count();
   if (occ <= 0 || sms <= 0) return CSS_ERR_CUDA;
   int grid = std::min(grid_max > 0 ? grid_max : sms * occ, sms * occ);
   grid = std::min(grid, kMaxCtas);
+  // the feed's slots take shared memory that as many CTAs per SM still have
+  double a_bytes = 0.0;
+  for (auto& u : units) a_bytes += (double)u.m * u.n * (dt == CSS_F64 ? 8 : dt == CSS_F32 ? 4 : 2);
+  const bool solo = (int)units.size() > grid;
+  const double on = std::min<double>(grid, (double)units.size());   // problems at a time
+  const size_t cta_bytes = (size_t)(a_bytes / (double)units.size() * (solo ? 1.0 : on / grid));
+  int feed = kFeedRegs, short_rows = 0;
+  const size_t smem_feed = greedy_feed(dt, tile_cols, smem, cta_bytes, solo, &feed, &short_rows, threads);
+  if (feed != kFeedRegs) {
+    if (greedy_occupancy(dt, tile_cols, feed, smem_feed, threads) >= occ) smem = smem_feed;
+    else feed = short_rows = 0;
+  }
   Plan P = make_plan(work, grid);
   int split_used = 0;
   for (size_t t = 0; t < P.teams.size(); ++t) {
@@ -298,6 +310,8 @@ css_status prepare_units(const Header& h, std::vector<UnitDesc>& units, const st
   L.r_max = r_max;
   L.grid = P.grid;
   L.threads = threads;
+  L.feed = feed;
+  L.short_rows = short_rows;
   L.smem = smem;
   info.L = L;
   info.split_used = split_used;

@@ -56,6 +56,10 @@ struct Ctx {
   double* scoef; // coefficients (FP64)
   Acc* sups;     // upsilon in Acc precision
   double* sred;  // NS * RB partials
+  uint32_t ring;   // this warp's slots of the fused step's copies (shared address)
+  uint32_t tails;  // this warp's column ends, kTailSlots of them
+  uint32_t cring;  // this warp's slots of the rows of C, or 0
+  uint32_t* sctr;  // single-CTA teams: the two tile counters, in shared memory
   uint32_t* epoch;  // thread 0: barriers of the team passed so far
 };
 
@@ -473,6 +477,29 @@ __device__ double team_sum(const Ctx<Acc>& x, int slot) {
   return v;
 }
 
+// Theorem 2 / Theorem 4 for one column: f - 2 omega o x + s (omega o omega),
+// g - omega o omega, the omega row, and the candidate.
+__device__ __forceinline__ void update_column(const UnitDesc& u, int t, int p, double s, int col, double w, double h,
+                                              long long& bv, int& bi) {
+  double fi = ld_cg(u.f + col), gi = ld_cg(u.g + col);
+  const double thr = ld_cg(u.thr + col);
+  bool selected = __ldcg(u.selmask + col) != 0;
+  fi = fi - 2.0 * w * h + s * (w * w);
+  gi = gi - w * w;
+  u.f[col] = fi;
+  u.g[col] = gi;
+  if (u.W) u.W[(long long)t * u.n + col] = w;
+  if (col == p) { u.selmask[col] = 1; selected = true; }
+  if (!selected && gi > thr) {
+    const double sc = u.score_mode ? gi : fmax(fi, 0.0) / gi;
+    const long long sk = score_key(sc);
+    if (better(sk, col, bv, bi)) { bv = sk; bi = col; }
+  }
+}
+
+// A warp's first unit of work in a fused step.
+__device__ __forceinline__ int first_unit(int rank, int ncta, int warp) { return warp * ncta + rank; }
+
 // --------------------------------------------------------- fused step (K1) --
 // Work units come from a team-wide counter: first whole tiles of CW columns,
 // then the last `nsplit` tiles (one per warp of the team at most) cut into
@@ -514,10 +541,12 @@ __device__ void fused_step(const Ctx<typename AccOf<TA>::type>& x, const UnitDes
   const bool val_lane = (x.lane & ((1 << SH) - 1)) == 0;
   Acc bw = Acc(0), bh = Acc(0);
   int bcol = -1, slot = 0;
-  uint32_t* ctr = x.team->tile_ctr + (t & 1);
-  int unit = 0;
-  if (x.lane == 0) unit = (int)atomicAdd(ctr, 1u);
-  unit = __shfl_sync(0xffffffffu, unit, 0);
+  // units after a warp's first come from the team's counter (in shared memory
+  // for a single CTA)
+  const int W = x.ncta * NW;
+  uint32_t* ctr = (x.ncta == 1 ? x.sctr : x.team->tile_ctr) + (t & 1);
+  const bool more = W < nunits;
+  int unit = first_unit(x.rank, x.ncta, x.warp);
   // short columns (at most 2 KB): a tile's loads are one or two dependent
   // memory round trips, so the warp asks L2 for the columns of its next unit
   // as soon as it draws it (one bulk prefetch per column).  Measured on the
@@ -526,8 +555,8 @@ __device__ void fused_step(const Ctx<typename AccOf<TA>::type>& x, const UnitDes
   // rows) it was 5 % longer, so those are left alone
   const bool pf_next = u.vec_ok && (size_t)m * sizeof(TA) <= 2048 && (size_t)m * sizeof(TA) >= 16;
   while (unit < nunits) {
-    int next = 0;
-    if (x.lane == 0) next = (int)atomicAdd(ctr, 1u);
+    int next = nunits;
+    if (more && x.lane == 0) next = W + (int)atomicAdd(ctr, 1u);
     if (pf_next) {
       const int nx = __shfl_sync(0xffffffffu, next, 0);
       if (nx < nunits && x.lane < CW) {
@@ -613,25 +642,292 @@ __device__ void fused_step(const Ctx<typename AccOf<TA>::type>& x, const UnitDes
     }
     unit = __shfl_sync(0xffffffffu, next, 0);
     if (slot == TPB || unit >= nunits) {
-      if (bcol >= 0) {
-        const int col = bcol;
-        double fi = ld_cg(u.f + col), gi = ld_cg(u.g + col);
-        const double thr = ld_cg(u.thr + col);
-        bool selected = __ldcg(u.selmask + col) != 0;
-        const double w = to_f64(bw), h = to_f64(bh);
-        // Theorem 2 / Theorem 4: f - 2 omega o x + s (omega o omega), g - omega o omega
-        fi = fi - 2.0 * w * h + s * (w * w);
-        gi = gi - w * w;
-        u.f[col] = fi;
-        u.g[col] = gi;
-        if (u.W) u.W[(long long)t * n + col] = w;
-        if (col == p) { u.selmask[col] = 1; selected = true; }
-        if (!selected && gi > thr) {
-          const double sc = u.score_mode ? gi : fmax(fi, 0.0) / gi;
-          const long long sk = score_key(sc);
-          if (better(sk, col, bv, bi)) { bv = sk; bi = col; }
+      if (bcol >= 0) update_column(u, t, p, s, bcol, to_f64(bw), to_f64(bh), bv, bi);
+      slot = 0;
+      bcol = -1;
+    }
+  }
+}
+
+// ------------------------------------------------- fused step, ring form ----
+// The same step with its loads in asynchronous copies: every warp owns
+// kRingSlots slots of shared memory, a slot holds one row step (32 lanes x 16
+// bytes) of a tile's eight columns, and a lane reads back only what it copied
+// itself, so the slots need no barrier.  The copies run kRingSlots steps ahead
+// and across unit boundaries, and the first unit of a warp is fixed, so its
+// first steps are copied before the pivot and wait in shared memory when q and
+// y' arrive.  FP32 only: there the register form exposes its tiles' round trips
+// (1999 x 30011: 69.5 us a step, 3.4 TB/s; here 37.6 us, 6.4 TB/s; 100 picks
+// 13.0 -> 10.4 ms).  In BF16, which takes twice the arithmetic per byte, the
+// shared-memory trip costs more than it hides (4096 x 65536: 78 -> 82 us; the
+// column blocks of 2048 x 262144: 25 -> 33 ms), and FP64 is bound by its
+// arithmetic.
+//
+// Every sum is formed in the order of fused_step, so the results are the same
+// bits; only who forms it and when it is loaded differ.
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, uint64_t pol) {
+  asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "l"(pol) : "memory");
+}
+// `bytes` of a 16-byte vector, the rest zero
+__device__ __forceinline__ void cp_async16_part(uint32_t dst, const void* src, uint32_t bytes) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+__device__ __forceinline__ uint4 lds16(uint32_t a) {
+  uint4 v;
+  asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a) : "memory");
+  return v;
+}
+
+// The units of a step: whole tiles, then the split tiles' row chunks.
+template <typename TA>
+struct StepShape {
+  static constexpr int V = Vec<TA>::V;
+  int nbulk, nunits, rch, m_vec;
+  __device__ __forceinline__ StepShape(const UnitDesc& u, int split_cap) {
+    const int ntiles = (u.n + 7) / 8;
+    const int nsplit = min(ntiles, split_cap);
+    nbulk = ntiles - nsplit;
+    nunits = nbulk + nsplit * kSplitR;
+    rch = ((u.m + kSplitR - 1) / kSplitR + 32 * V - 1) / (32 * V) * (32 * V);
+    m_vec = u.vec_ok ? (u.m / V) * V : 0;
+  }
+  // tile, split index (-1: whole tile) and rows of a unit
+  __device__ __forceinline__ void rows(const UnitDesc& u, int unit, int& tile, int& sidx, int& chunk, int& r_lo,
+                                       int& r_hi) const {
+    tile = unit;
+    sidx = -1;
+    chunk = 0;
+    r_lo = 0;
+    r_hi = u.m;
+    if (unit >= nbulk) {
+      sidx = (unit - nbulk) / kSplitR;
+      chunk = (unit - nbulk) - sidx * kSplitR;
+      tile = nbulk + sidx;
+      r_lo = min(u.m, chunk * rch);
+      r_hi = (chunk == kSplitR - 1) ? u.m : min(u.m, r_lo + rch);
+    }
+  }
+};
+
+// The copies' position: a unit, and the row step within it.
+template <typename TA>
+struct Feed {
+  static constexpr int V = Vec<TA>::V;
+  int unit, step, nsteps, r, v_hi, cols, tail;   // tail: bytes of the column ends past m_vec
+  const TA* src;
+
+  __device__ __forceinline__ void at(const UnitDesc& u, const StepShape<TA>& sh, int unit_, int lane) {
+    unit = unit_;
+    step = 0;
+    if (unit >= sh.nunits) return;
+    int tile, sidx, chunk, r_lo, r_hi;
+    sh.rows(u, unit, tile, sidx, chunk, r_lo, r_hi);
+    v_hi = min(r_hi, sh.m_vec);
+    nsteps = max(1, (v_hi - r_lo + 32 * V - 1) / (32 * V));
+    r = r_lo + lane * V;
+    cols = min(8, u.n - tile * 8);
+    tail = (sh.m_vec > 0 && r_lo <= sh.m_vec && r_hi > sh.m_vec) ? (r_hi - sh.m_vec) * (int)sizeof(TA) : 0;
+    src = reinterpret_cast<const TA*>(u.A) + (long long)(tile * 8) * u.lda;
+  }
+  // copies the next step into `slot` (and after a unit's last one its column
+  // ends); true: that was the unit's last step
+  __device__ __forceinline__ bool copy(const UnitDesc& u, const StepShape<TA>& sh, uint32_t slot, uint32_t tslot,
+                                       int lane, uint64_t pol) {
+    if (r < v_hi) {
+      const TA* p = src + r;
+#pragma unroll
+      for (int c = 0; c < 8; ++c)
+        if (c < cols) cp_async16(slot + c * 512 + lane * 16, p + c * u.lda, pol);
+    }
+    if (step == nsteps - 1 && tail > 0 && lane < cols)
+      cp_async16_part(tslot + lane * 16, src + lane * u.lda + sh.m_vec, (uint32_t)tail);
+    return skip();
+  }
+  __device__ __forceinline__ bool skip() {
+    r += 32 * V;
+    return ++step == nsteps;
+  }
+};
+
+// Copies the first steps of this warp's first unit (at most kRingSlots).
+template <typename TA>
+__device__ __forceinline__ void prime_ring(const Ctx<typename AccOf<TA>::type>& x, const UnitDesc& u, uint64_t pol) {
+  const StepShape<TA> sh(u, x.team->split_cap);
+  Feed<TA> fd;
+  fd.at(u, sh, first_unit(x.rank, x.ncta, x.warp), x.lane);
+  if (fd.unit >= sh.nunits) return;
+#pragma unroll 1
+  for (int i = 0; i < kRingSlots; ++i) {
+    const bool last = fd.copy(u, sh, x.ring + i * kRingSlotBytes, x.tails, x.lane, pol);
+    cp_async_commit();
+    if (last) break;
+  }
+}
+
+template <typename TA>
+__device__ void fused_step_ring(const Ctx<typename AccOf<TA>::type>& x, const UnitDesc& u, int t, int p, double s,
+                                uint64_t pol, long long& bv, int& bi) {
+  using Acc = typename AccOf<TA>::type;
+  constexpr int V = Vec<TA>::V;
+  constexpr int CW = 8, NV = 16, SH = 1;
+  static_assert(kRingSlots == 2, "the queue below holds two steps");
+  const int n = u.n, lane = x.lane;
+  const StepShape<TA> sh(u, x.team->split_cap);
+  Acc* split_part = reinterpret_cast<Acc*>(x.team->split_part);
+  constexpr int SLOT = kSplitR * kSplitVals * 8 / (int)sizeof(Acc);
+  const int my_c = lane % CW;
+  const int src_w = (2 * my_c) << SH, src_h = (2 * my_c + 1) << SH;
+  const int my_slot = lane / CW;
+  const bool val_lane = (lane & 1) == 0;
+  Acc bw = Acc(0), bh = Acc(0);
+  int bcol = -1, slot = 0;
+  // units after the first: from the team's counter (in shared memory for a
+  // single CTA), one drawn ahead; none when every unit is some warp's first
+  const int W = x.ncta * NW;
+  uint32_t* ctr = (x.ncta == 1 ? x.sctr : x.team->tile_ctr) + (t & 1);
+  const bool more = W < sh.nunits;
+  int drawn = sh.nunits;
+  if (more && lane == 0) drawn = W + (int)atomicAdd(ctr, 1u);
+  Feed<TA> fd;
+  fd.at(u, sh, first_unit(x.rank, x.ncta, x.warp), lane);
+  uint32_t tslot = 0;
+  // the step just copied (or skipped: already there) as unit * 2 + last, -1: none
+  auto next_unit = [&]() {
+    const int nu = __shfl_sync(0xffffffffu, drawn, 0);
+    if (more && lane == 0 && nu < sh.nunits) drawn = W + (int)atomicAdd(ctr, 1u);
+    tslot = (tslot + 1) & (kTailSlots - 1);
+    fd.at(u, sh, nu, lane);
+  };
+  auto feed = [&](uint32_t ring_slot, bool primed) -> int {
+    int what = -1;
+    if (fd.unit < sh.nunits) {
+      what = fd.unit * 2;
+      const bool last = primed ? fd.skip()
+                               : fd.copy(u, sh, x.ring + ring_slot * kRingSlotBytes, x.tails + tslot * 128, lane, pol);
+      if (last) {
+        ++what;
+        next_unit();
+      }
+    }
+    if (!primed) cp_async_commit();
+    return what;
+  };
+  const bool has = fd.unit < sh.nunits;
+  int q0 = feed(0, has);
+  int q1 = feed(1, has && !(q0 & 1));
+  int cur = -1, tile = 0, sidx = -1, chunk = 0, r = 0, r_lo = 0, r_hi = 0, v_hi = 0;
+  uint32_t rslot = 0, tread = 0;
+  Acc v[NV];
+  while (q0 >= 0) {
+    const int unit = q0 >> 1;
+    const bool last = q0 & 1;
+    if (unit != cur) {
+      cur = unit;
+      sh.rows(u, unit, tile, sidx, chunk, r_lo, r_hi);
+      v_hi = min(r_hi, sh.m_vec);
+      r = r_lo + lane * V;
+#pragma unroll
+      for (int i = 0; i < NV; ++i) v[i] = Acc(0);
+    }
+    cp_async_wait<kRingSlots - 1>();
+    if (r < v_hi) {
+      Acc qa[V], ya[V];
+      lds_vec<Acc, V>(x.sq + r, qa);
+      lds_vec<Acc, V>(x.sy + r, ya);
+      const uint32_t at = x.ring + rslot * kRingSlotBytes + lane * 16;
+#pragma unroll
+      for (int c = 0; c < CW; ++c) {
+        Acc a[V];
+        Vec<TA>::unpack(lds16(at + c * 512), a);
+        Acc tw = a[0] * qa[0], th = a[0] * ya[0];
+#pragma unroll
+        for (int e = 1; e < V; ++e) { tw = fma(a[e], qa[e], tw); th = fma(a[e], ya[e], th); }
+        v[2 * c] += tw;
+        v[2 * c + 1] += th;
+      }
+    }
+    r += 32 * V;
+    q0 = q1;
+    q1 = feed(rslot, false);
+    rslot ^= 1u;
+    if (!last) continue;
+
+    // ---- the unit's end: rows past the last whole vector
+    const int c0 = tile * CW;
+    const int t_lo = max(r_lo, sh.m_vec);
+    if (sh.m_vec > 0) {
+      if (t_lo < r_hi) {
+        __syncwarp();   // the column ends were copied by lanes 0..7
+        const int rr = t_lo + lane;
+        if (rr < r_hi) {
+          const Acc qa = x.sq[rr], ya = x.sy[rr];
+          const uint32_t at = x.tails + tread * 128 + lane * (uint32_t)sizeof(TA);
+#pragma unroll
+          for (int c = 0; c < CW; ++c) {
+            Acc a;
+            if constexpr (sizeof(TA) == 8) {
+              asm volatile("ld.shared.f64 %0, [%1];" : "=d"(a) : "r"(at + c * 16) : "memory");
+            } else if constexpr (sizeof(TA) == 4) {
+              asm volatile("ld.shared.f32 %0, [%1];" : "=f"(a) : "r"(at + c * 16) : "memory");
+            } else {
+              unsigned short b;
+              asm volatile("ld.shared.u16 %0, [%1];" : "=h"(b) : "r"(at + c * 16) : "memory");
+              a = __uint_as_float((uint32_t)b << 16);
+            }
+            v[2 * c] = fma(a, qa, v[2 * c]);
+            v[2 * c + 1] = fma(a, ya, v[2 * c + 1]);
+          }
         }
       }
+    } else {
+      // a layout that refuses vector copies: element by element
+      const TA* base = reinterpret_cast<const TA*>(u.A);
+      for (int rr = t_lo + lane; rr < r_hi; rr += 32) {
+        const Acc qa = x.sq[rr], ya = x.sy[rr];
+#pragma unroll
+        for (int c = 0; c < CW; ++c) {
+          const Acc a = load_elem<TA>(base + (long long)min(c0 + c, n - 1) * u.lda + rr);
+          v[2 * c] = fma(a, qa, v[2 * c]);
+          v[2 * c + 1] = fma(a, ya, v[2 * c + 1]);
+        }
+      }
+    }
+    tread = (tread + 1) & (kTailSlots - 1);
+    Acc red = transpose_reduce<NV>(v, lane);
+    bool have = true;
+    if (sidx >= 0) {
+      Acc* sp = split_part + (size_t)sidx * SLOT;
+      if (val_lane) __stcg(sp + chunk * kSplitVals + (lane >> SH), red);
+      __syncwarp();
+      uint32_t old = 0;
+      if (lane == 0) old = atom_add_acqrel_u32(x.team->split_done + sidx, 1u);
+      old = __shfl_sync(0xffffffffu, old, 0);
+      have = old == (uint32_t)(kSplitR - 1);
+      if (have) {
+        __syncwarp();   // lane 0's acquire orders the other lanes' loads
+        if (val_lane) {
+          Acc sum = Acc(0);
+#pragma unroll
+          for (int c = 0; c < kSplitR; ++c) sum += ld_cg(sp + c * kSplitVals + (lane >> SH));
+          red = sum;
+        }
+        // every chunk has arrived: the counter is free for the next step
+        if (lane == 0) x.team->split_done[sidx] = 0u;
+      }
+    }
+    if (have) {
+      const Acc wv = __shfl_sync(0xffffffffu, red, src_w);
+      const Acc hv = __shfl_sync(0xffffffffu, red, src_h);
+      if (my_slot == slot && c0 + my_c < n) { bw = wv; bh = hv; bcol = c0 + my_c; }
+      ++slot;
+    }
+    if (slot == 32 / CW || q0 < 0) {
+      if (bcol >= 0) update_column(u, t, p, s, bcol, to_f64(bw), to_f64(bh), bv, bi);
       slot = 0;
       bcol = -1;
     }
@@ -697,8 +993,66 @@ __device__ void init_pass(const Ctx<typename AccOf<TA>::type>& x, const UnitDesc
   }
 }
 
+// y_i = C_i: e for rows too short for sixteen loads in flight: the rows of a
+// warp stream through kRowSlots slots of asynchronous copies of 512 bytes,
+// across row boundaries.  done(i, k, sum) runs in lane 0 for the warp's k-th
+// row i.  The sums are those of the loop for long rows, in its order (one
+// accumulator, then the elements past the last whole vector).
+template <typename Acc, typename Done>
+__device__ __forceinline__ void short_rows(const Ctx<Acc>& x, int m, int m_vec, const Acc* C, long long ldc,
+                                           Done done) {
+  constexpr int VC = 16 / sizeof(Acc);
+  const uint64_t pol = policy_evict_last();
+  const int stride = x.ncta * NW, l0 = x.lane * VC;
+  const int nseg = (m_vec + 32 * VC - 1) / (32 * VC);
+  int li = x.rank * NW + x.warp, ls = 0;   // the copies' row and segment
+  auto feed = [&](uint32_t slot) {
+    if (li < m) {
+      const int l = ls * 32 * VC + l0;
+      if (l < m_vec) cp_async16(x.cring + slot * 512 + x.lane * 16, C + (long long)li * ldc + l, pol);
+      if (++ls == nseg) {
+        ls = 0;
+        li += stride;
+      }
+    }
+    cp_async_commit();
+  };
+#pragma unroll 1
+  for (uint32_t i = 0; i < kRowSlots; ++i) feed(i);
+  const bool tail = x.lane < m - m_vec;   // at most VC - 1 elements
+  const Acc et = tail ? x.seacc[m_vec + x.lane] : Acc(0);
+  int i = x.rank * NW + x.warp;
+  Acc ct = tail && i < m ? __ldg(C + (long long)i * ldc + m_vec + x.lane) : Acc(0);
+  uint32_t slot = 0;
+  for (int kr = 0; i < m; i += stride, ++kr) {
+    Acc next = Acc(0);
+    if (tail && i + stride < m) next = __ldg(C + (long long)(i + stride) * ldc + m_vec + x.lane);
+    Acc acc = Acc(0);
+    for (int sg = 0; sg < nseg; ++sg) {
+      cp_async_wait<kRowSlots - 1>();
+      const int l = sg * 32 * VC + l0;
+      if (l < m_vec) {
+        Acc cv[VC], ev[VC];
+        const uint4 raw = lds16(x.cring + slot * 512 + x.lane * 16);
+        if constexpr (sizeof(Acc) == 4) Vec<float>::unpack(raw, cv);
+        else Vec<double>::unpack(raw, cv);
+        lds_vec<Acc, VC>(x.seacc + l, ev);
+#pragma unroll
+        for (int e = 0; e < VC; ++e) acc = fma(cv[e], ev[e], acc);
+      }
+      feed(slot);
+      slot = (slot + 1) & (kRowSlots - 1);
+    }
+    if (tail) acc = fma(ct, et, acc);
+    acc = warp_sum(acc);
+    if (x.lane == 0) done(i, kr, acc);
+    ct = next;
+  }
+  cp_async_wait<0>();
+}
+
 // --------------------------------------------------------------- the unit ---
-template <typename TA, int CW>
+template <typename TA, int CW, int FEED>
 __device__ void run_unit(const Ctx<typename AccOf<TA>::type>& x, const UnitDesc& u) {
   using Acc = typename AccOf<TA>::type;
   // BF16/FP32 input: Q, Z (CSS), e and the coefficients are held as float
@@ -729,7 +1083,10 @@ __device__ void run_unit(const Ctx<typename AccOf<TA>::type>& x, const UnitDesc&
   if (x.rank == 0 && x.tid == 0) {
     tm.tile_ctr[0] = 0u;
     tm.tile_ctr[1] = 0u;
+    x.sctr[0] = 0u;
+    x.sctr[1] = 0u;
   }
+  if constexpr (FEED == kFeedRing) prime_ring<TA>(x, u, pol_stream);
   const int cb0 = cta_argmax_publish(x, bv, bi);
   if (x.tid == 0) prefetch_column<TA>(u, cb0);
   if (!team_barrier(tm.bar, x.ncta, x.st, 1, x.epoch)) return;
@@ -758,6 +1115,7 @@ __device__ void run_unit(const Ctx<typename AccOf<TA>::type>& x, const UnitDesc&
       // counter of the next iteration's fused step; its last user finished
       // before the previous iteration's final barrier
       tm.tile_ctr[(t + 1) & 1] = 0u;
+      x.sctr[(t + 1) & 1] = 0u;
       if (u.diag_argmax) u.diag_argmax[t] = p_arg;
       u.sel[t] = p;
     }
@@ -849,8 +1207,21 @@ __device__ void run_unit(const Ctx<typename AccOf<TA>::type>& x, const UnitDesc&
       Acc* srow = reinterpret_cast<Acc*>(x.sred);
       const int rows_per_warp = (m + x.ncta * NW - 1) / (x.ncta * NW);
       const bool gather = rows_per_warp * NW <= NS * RB * (int)(sizeof(double) / sizeof(Acc));
+      auto row_done = [&](int i, int kr, Acc acc) {
+        if (gather) {
+          srow[kr * NW + x.warp] = acc;
+        } else {
+          u.y[i] = (double)acc;
+          ey += (kDF ? df_to_f64(se2[i]) : x.se64[i]) * (double)acc;
+        }
+      };
       int kr = 0;
-      for (int i = x.rank * NW + x.warp; i < m; i += x.ncta * NW, ++kr) {
+      bool short_path = false;
+      if constexpr (FEED != kFeedRegs) {
+        short_path = x.cring != 0u && m_vec > 0 && m_vec <= (UC - 1) * 32 * VC;
+        if (short_path) short_rows<Acc>(x, m, m_vec, C, u.ldt, row_done);
+      }
+      for (int i = x.rank * NW + x.warp; !short_path && i < m; i += x.ncta * NW, ++kr) {
         const Acc* cp = C + (long long)i * u.ldt;
         Acc accs[UC];
 #pragma unroll
@@ -883,14 +1254,7 @@ __device__ void run_unit(const Ctx<typename AccOf<TA>::type>& x, const UnitDesc&
         for (int q = 0; q < UC; ++q) acc += accs[q];
         for (int l2 = m_vec + x.lane; l2 < m; l2 += 32) acc = fma(__ldg(cp + l2), x.seacc[l2], acc);
         acc = warp_sum(acc);
-        if (x.lane == 0) {
-          if (gather) {
-            srow[kr * NW + x.warp] = acc;
-          } else {
-            u.y[i] = (double)acc;
-            ey += (kDF ? df_to_f64(se2[i]) : x.se64[i]) * (double)acc;
-          }
-        }
+        if (x.lane == 0) row_done(i, kr, acc);
       }
       if (gather) {
         __syncthreads();
@@ -1011,7 +1375,12 @@ __device__ void run_unit(const Ctx<typename AccOf<TA>::type>& x, const UnitDesc&
       mark(12);
       long long bv2 = -1;
       int bi2 = -1;
-      fused_step<TA, CW>(x, u, t, p, s, pol_stream, bv2, bi2);
+      if constexpr (FEED == kFeedRing) {
+        fused_step_ring<TA>(x, u, t, p, s, pol_stream, bv2, bi2);
+        if (t + 1 < u.k) prime_ring<TA>(x, u, pol_stream);
+      } else {
+        fused_step<TA, CW>(x, u, t, p, s, pol_stream, bv2, bi2);
+      }
       mark(13);
       const int cb = cta_argmax_publish(x, bv2, bi2);
       if (x.tid == 0) prefetch_column<TA>(u, cb);
@@ -1034,7 +1403,7 @@ __device__ void run_unit(const Ctx<typename AccOf<TA>::type>& x, const UnitDesc&
   team_barrier(tm.bar, x.ncta, x.st, 9, x.epoch);
 }
 
-template <typename TA, int CW>
+template <typename TA, int CW, int FEED>
 __global__ void __launch_bounds__(NT, CSS_GREEDY_CTAS_PER_SM) greedy_kernel(GreedyLaunch L) {
   using Acc = typename AccOf<TA>::type;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -1064,29 +1433,41 @@ __global__ void __launch_bounds__(NT, CSS_GREEDY_CTAS_PER_SM) greedy_kernel(Gree
   x.sups = reinterpret_cast<Acc*>(p);
   p += ((size_t)L.r_max * sizeof(Acc) + 15) & ~(size_t)15;
   x.sred = reinterpret_cast<double*>(p);
+  p += (size_t)NS * RB * sizeof(double);
+  {
+    uint32_t base = (uint32_t)__cvta_generic_to_shared(p);
+    x.ring = base + x.warp * (kRingSlots * kRingSlotBytes);
+    x.tails = base + NW * (kRingSlots * kRingSlotBytes) + x.warp * (kTailSlots * 128);
+    if (FEED == kFeedRing) base += NW * (kRingSlots * kRingSlotBytes + kTailSlots * 128);
+    x.cring = L.short_rows ? base + x.warp * (kRowSlots * 512) : 0u;
+  }
+  __shared__ uint32_t s_ctr[2];
+  x.sctr = s_ctr;
   __shared__ uint32_t s_epoch;
   if (threadIdx.x == 0) s_epoch = 0u;   // used by thread 0 only
   x.epoch = &s_epoch;
 
   for (int ui = tm.u_begin; ui < tm.u_end; ++ui) {
     const UnitDesc u = L.units[L.order[ui]];
-    run_unit<TA, CW>(x, u);
+    run_unit<TA, CW, FEED>(x, u);
+    // no copy may outlive the unit's use of its slots, or the CTA
+    if constexpr (FEED != kFeedRegs) cp_async_wait<0>();
     if (ld_volatile_i32(&L.st->code) != 0) return;
   }
 }
 
-template <typename TA, int CW>
-void* kernel_ptr() { return (void*)greedy_kernel<TA, CW>; }
+template <typename TA, int CW, int FEED = kFeedRegs>
+void* kernel_ptr() { return (void*)greedy_kernel<TA, CW, FEED>; }
 
-void* pick_kernel(int dtype, int cw) {
+template <typename TA>
+void* pick_width(int cw) {
+  return cw == 2 ? kernel_ptr<TA, 2>() : cw == 8 ? kernel_ptr<TA, 8>() : kernel_ptr<TA, 4>();
+}
+void* pick_kernel(int dtype, int cw, int feed) {
   switch (dtype) {
-    case CSS_F64:
-      return cw == 2 ? kernel_ptr<double, 2>() : cw == 8 ? kernel_ptr<double, 8>() : kernel_ptr<double, 4>();
-    case CSS_F32:
-      return cw == 2 ? kernel_ptr<float, 2>() : cw == 8 ? kernel_ptr<float, 8>() : kernel_ptr<float, 4>();
-    default:
-      return cw == 2 ? kernel_ptr<__nv_bfloat16, 2>() : cw == 8 ? kernel_ptr<__nv_bfloat16, 8>()
-                     : kernel_ptr<__nv_bfloat16, 4>();
+    case CSS_F64: return pick_width<double>(cw);
+    case CSS_F32: return feed == kFeedRing ? kernel_ptr<float, 8, kFeedRing>() : pick_width<float>(cw);
+    default: return feed == kFeedRows ? kernel_ptr<__nv_bfloat16, 8, kFeedRows>() : pick_width<__nv_bfloat16>(cw);
   }
 }
 
@@ -1105,8 +1486,28 @@ size_t greedy_smem_bytes(int dtype, int m_max, int k_max, int r_max) {
   return b;
 }
 
-int greedy_occupancy(int dtype, int tile_cols, size_t smem) {
-  void* k = pick_kernel(dtype, tile_cols);
+// Shared memory a CTA may take so that CSS_GREEDY_CTAS_PER_SM share an SM.
+constexpr size_t kSmemCta = (size_t)(228 / CSS_GREEDY_CTAS_PER_SM - 1) * 1024;
+
+size_t greedy_feed(int dtype, int tile_cols, size_t smem, size_t cta_bytes, bool solo, int* feed, int* short_rows) {
+  const size_t a = (size_t)NW * (kRingSlots * kRingSlotBytes + kTailSlots * 128), c = (size_t)NW * kRowSlots * 512;
+  *feed = kFeedRegs;
+  *short_rows = 0;
+  if (tile_cols != 8) return smem;
+  if (dtype == CSS_F32 && cta_bytes >= kRingMinBytes && smem + a <= kSmemCta) {
+    *feed = kFeedRing;
+    smem += a;
+  }
+  if (solo && (dtype == CSS_BF16 || *feed == kFeedRing) && smem + c <= kSmemCta) {
+    if (*feed == kFeedRegs) *feed = kFeedRows;
+    *short_rows = 1;
+    smem += c;
+  }
+  return smem;
+}
+
+int greedy_occupancy(int dtype, int tile_cols, int feed, size_t smem) {
+  void* k = pick_kernel(dtype, tile_cols, feed);
   if (smem > 48 * 1024) {
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
       return 0;
@@ -1119,7 +1520,7 @@ int greedy_occupancy(int dtype, int tile_cols, size_t smem) {
 cudaError_t greedy_launch(const GreedyLaunch& L, cudaStream_t stream) {
   // the plan (team sizes, split slots) was made for this shape's CTAs
   if (L.threads != NT) return cudaErrorInvalidConfiguration;
-  void* k = pick_kernel(L.dtype, L.tile_cols);
+  void* k = pick_kernel(L.dtype, L.tile_cols, L.feed);
   if (L.smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.smem);
     if (e != cudaSuccess) return e;

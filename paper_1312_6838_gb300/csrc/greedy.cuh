@@ -68,6 +68,20 @@ constexpr int kSplitR = CSS_SPLIT_ROWS;   // row chunks of a split tile
 constexpr int kSplitVals = 16;      // value slots per chunk (2 x the widest tile)
 constexpr size_t kSplitSlotBytes = (size_t)kSplitR * kSplitVals * 8;
 
+// The fused step's ring of asynchronous copies (per warp): slots of one row
+// step of eight columns, column ends, and slots for short rows of C.
+constexpr int kRingSlots = 2, kRingSlotBytes = 8 * 32 * 16;
+constexpr int kTailSlots = 4;
+constexpr uint32_t kRowSlots = 8;
+// How a launch feeds its products: loads into registers; these, with short
+// rows of C through asynchronous copies; or the fused step's ring as well.
+enum Feed_ { kFeedRegs = 0, kFeedRows = 1, kFeedRing = 2 };
+// The ring pays where a CTA has enough to stream: FP32 selections, us without and
+// with it at bytes of A per CTA: 54 KB (512 x 4096) 1339 and 1380, 105 KB (GCSS
+// 500 x 8000) 1712 and 1803, 220 KB (1024 x 8192) 1750 and 1749, 880 KB
+// (2048 x 16384) 3078 and 2865, 4.6 MB (256 batched problems) 39.8 and 36.6 ms.
+constexpr size_t kRingMinBytes = 256 * 1024;
+
 struct GreedyLaunch {
   const UnitDesc* units;
   const int* order;
@@ -79,6 +93,8 @@ struct GreedyLaunch {
   int m_max, k_max, r_max;
   int grid;        // CTAs
   int threads;
+  int feed;        // Feed_
+  int short_rows;  // rows of C through asynchronous copies
   size_t smem;
 };
 
@@ -92,23 +108,34 @@ constexpr int kGreedyThreadsPaired = 256;
 #define CSS_GREEDY_SHAPE_API                                                     \
   /* Bytes of dynamic shared memory the kernel needs. */                        \
   size_t greedy_smem_bytes(int dtype, int m_max, int k_max, int r_max);         \
+  /* Picks GreedyLaunch::feed and short_rows for CTAs that stream cta_bytes   */ \
+  /* of A a step (solo: one CTA per problem, more problems than CTAs) and     */ \
+  /* returns `smem` with their slots. */                                         \
+  size_t greedy_feed(int dtype, int tile_cols, size_t smem, size_t cta_bytes,   \
+                     bool solo, int* feed, int* short_rows);                    \
   /* Max co-resident CTAs per SM for the given configuration (0 on error). */   \
-  int greedy_occupancy(int dtype, int tile_cols, size_t smem);                  \
+  int greedy_occupancy(int dtype, int tile_cols, int feed, size_t smem);        \
   /* Enqueue the persistent kernel (cooperative launch). */                     \
   cudaError_t greedy_launch(const GreedyLaunch& L, cudaStream_t stream);
 namespace one_per_sm { CSS_GREEDY_SHAPE_API }
 namespace two_per_sm { CSS_GREEDY_SHAPE_API }
 #undef CSS_GREEDY_SHAPE_API
 
-// The same three calls for the shape with `threads` threads per CTA
+// The same four calls for the shape with `threads` threads per CTA
 // (kGreedyThreads or kGreedyThreadsPaired; GreedyLaunch::threads for the launch).
 inline size_t greedy_smem_bytes(int dtype, int m_max, int k_max, int r_max, int threads) {
   return threads == kGreedyThreadsPaired ? two_per_sm::greedy_smem_bytes(dtype, m_max, k_max, r_max)
                                          : one_per_sm::greedy_smem_bytes(dtype, m_max, k_max, r_max);
 }
-inline int greedy_occupancy(int dtype, int tile_cols, size_t smem, int threads) {
-  return threads == kGreedyThreadsPaired ? two_per_sm::greedy_occupancy(dtype, tile_cols, smem)
-                                         : one_per_sm::greedy_occupancy(dtype, tile_cols, smem);
+inline size_t greedy_feed(int dtype, int tile_cols, size_t smem, size_t cta_bytes, bool solo, int* feed,
+                          int* short_rows, int threads) {
+  return threads == kGreedyThreadsPaired
+             ? two_per_sm::greedy_feed(dtype, tile_cols, smem, cta_bytes, solo, feed, short_rows)
+             : one_per_sm::greedy_feed(dtype, tile_cols, smem, cta_bytes, solo, feed, short_rows);
+}
+inline int greedy_occupancy(int dtype, int tile_cols, int feed, size_t smem, int threads) {
+  return threads == kGreedyThreadsPaired ? two_per_sm::greedy_occupancy(dtype, tile_cols, feed, smem)
+                                         : one_per_sm::greedy_occupancy(dtype, tile_cols, feed, smem);
 }
 inline cudaError_t greedy_launch(const GreedyLaunch& L, cudaStream_t stream) {
   return L.threads == kGreedyThreadsPaired ? two_per_sm::greedy_launch(L, stream)
