@@ -456,10 +456,12 @@ struct SelectLayout {
   UnitState s;
   void* C;
   double* partial;
+  void* f64_scratch;   // digits of the FP64 initial scores, or null
   size_t bytes;
 };
 
-SelectLayout select_layout(void* ws, size_t cap, int dt, int64_t m, int64_t n, int32_t k, bool need_W) {
+SelectLayout select_layout(void* ws, size_t cap, int dt, int64_t m, int64_t n, int32_t k, bool need_W,
+                           bool digits) {
   WsCarver c(ws, cap);
   SelectLayout L{};
   carve_header(c, 1, L.h, n);
@@ -473,6 +475,8 @@ SelectLayout select_layout(void* ws, size_t cap, int dt, int64_t m, int64_t n, i
     cbytes = std::max(cbytes, tc::css_f0_scratch_bytes((int)m, (int)n, dt == CSS_F32 ? tc::kF0F32Staged : tc::kF0Bf16Staged));
   L.C = c.take<char>(cbytes);
   L.partial = c.take<double>(css_f0_partial_doubles(dt, (int)m, (int)n));
+  const size_t f64 = digits && dt == CSS_F64 ? css_f0_f64_bytes(m, n) : 0;
+  if (f64) L.f64_scratch = c.take<char>(f64);
   L.bytes = c.off;
   return L;
 }
@@ -558,9 +562,13 @@ cudaError_t gcss_f0(int dt, const void* A, int64_t lda, int64_t m, int64_t n, co
   return gcss_f0_simt(dt, A, lda, (int)m, (int)n, B, ldb, (int)r, partial, f, s);
 }
 
-int team_ctas_for(int64_t n, int64_t m) {
-  // enough CTAs to keep the column stream and the FP64 pivot work spread out
-  int64_t a = (n + 127) / 128;
+int team_ctas_for(int64_t n, int64_t m, int dt = CSS_BF16) {
+  // enough CTAs to keep the column stream and the FP64 pivot work spread out.
+  // Algorithm 1's fused step of FP64 input is bound by each SM's FP64 rate (two lanes a
+  // clock), so it takes an SM per tile of eight columns: 500 x 1000, k = 50,
+  // on 32 CTAs (the FP32 rule) 17.9 us a step, on 64 9.9, on 128 6.2; 50 picks
+  // 2.57 / 2.13 / 1.89 ms
+  int64_t a = dt == CSS_F64 ? (n + 7) / 8 : (n + 127) / 128;
   int64_t b = (m + 15) / 16;
   return (int)std::max<int64_t>(1, std::max(a, b));
 }
@@ -613,7 +621,7 @@ size_t css_workspace_size(css_op op, css_dtype dtype, int64_t m, int64_t n, int6
     case CSS_OP_SELECT:
     case CSS_OP_HOST_SELECT: {
       if (k <= 0) return 0;
-      size_t b = select_layout(nullptr, (size_t)-1, dtype, m, n, k, true).bytes;
+      size_t b = select_layout(nullptr, (size_t)-1, dtype, m, n, k, true, true).bytes;
       return op == CSS_OP_HOST_SELECT ? b + host_out_bytes(k) : b;
     }
     case CSS_OP_GCSS:
@@ -647,6 +655,10 @@ size_t css_workspace_size(css_op op, css_dtype dtype, int64_t m, int64_t n, int6
 
 }  // extern "C"
 
+size_t css::select_least_workspace(int dtype, int64_t m, int64_t n, int32_t k) {
+  return select_layout(nullptr, (size_t)-1, dtype, m, n, k, true, false).bytes;
+}
+
 namespace {
 
 // css_select; pipe: A's columns arrive in chunks (css_select_host).
@@ -661,7 +673,9 @@ css_status select_impl(const void* A, css_dtype dtype, int64_t m, int64_t n, int
   if (o.score_mode != 0 && o.score_mode != 1) return CSS_ERR_INVALID_ARG;
   if (!valid_test_hook(o) || !valid_knobs(o)) return CSS_ERR_INVALID_ARG;
   if (!ws || ((uintptr_t)ws % kWsAlign) != 0) return CSS_ERR_WORKSPACE;
-  SelectLayout L = select_layout(ws, ws_bytes, dtype, m, n, k, W == nullptr);
+  // (FP64: the digits of the initial scores are used where they fit)
+  SelectLayout L = select_layout(ws, ws_bytes, dtype, m, n, k, W == nullptr, true);
+  if (L.bytes > ws_bytes) L = select_layout(ws, ws_bytes, dtype, m, n, k, W == nullptr, false);
   if (L.bytes > ws_bytes) return CSS_ERR_WORKSPACE;
   if (!device_ok()) return CSS_ERR_UNSUPPORTED;
   css_status cs = check_forced(o, (int)n, k, s);
@@ -682,7 +696,10 @@ css_status select_impl(const void* A, css_dtype dtype, int64_t m, int64_t n, int
   } else {
     e = cudaSuccess;
     for (int z = 0; pipe && z < pipe->chunks && e == cudaSuccess; ++z) e = cudaStreamWaitEvent(s, pipe->ready[z], 0);
-    if (e == cudaSuccess)
+    if (e == cudaSuccess && dtype == CSS_F64 && L.f64_scratch && o.init_path != 1)
+      e = css_f0_f64((const double*)A, lda, (int)m, (int)n, (double*)L.C, c_ld(m, 8), L.f64_scratch, L.s.f,
+                     L.h.aux_err, spin, s);
+    else if (e == cudaSuccess)
       e = css_f0_simt(dtype, A, lda, (int)m, (int)n, L.C, c_ld(m, (int)accsize(dtype)), L.partial, L.s.f, s);
   }
   if (e != cudaSuccess) return cuda_status(e);
@@ -690,7 +707,7 @@ css_status select_impl(const void* A, css_dtype dtype, int64_t m, int64_t n, int
   std::vector<UnitDesc> units{make_unit(As, dtype, m, n, ldas, k, 0, L.C, c_ld(m, (int)accsize(dtype)), 0, L.s, W,
                                         sel, trace, n_sel, o)};
   const int tile = pick_tile(o, dtype, m, n);
-  int gmax = o.grid_ctas > 0 ? o.grid_ctas : team_ctas_for(n, m);
+  int gmax = o.grid_ctas > 0 ? o.grid_ctas : team_ctas_for(n, m, dtype);
   cs = launch_units(L.h, units, {1.0}, dtype, gmax, tile, o.spin_budget_ns, s, stall_barrier(o),
                     pick_split_share(o, dtype, m, n));
   if (cs != CSS_OK) return cs;
@@ -818,8 +835,9 @@ css_status css_select_host(const void* A_host, css_dtype dtype, int64_t m, int64
   if (!ws || ((uintptr_t)ws % kWsAlign) != 0 || ws_bytes < kWsAlign) return CSS_ERR_WORKSPACE;
   cudaStream_t s = (cudaStream_t)stream;
   // outputs live in the first 256-byte slot... too small for k; carve after the select workspace
-  const size_t need = select_layout(nullptr, (size_t)-1, dtype, m, n, k, true).bytes;
   const size_t out_bytes = host_out_bytes(k);
+  size_t need = select_layout(nullptr, (size_t)-1, dtype, m, n, k, true, true).bytes;
+  if (ws_bytes < need + out_bytes) need = css::select_least_workspace(dtype, m, n, k);
   if (ws_bytes < need + out_bytes) return CSS_ERR_WORKSPACE;
   char* outs = (char*)ws + need;
   int32_t* d_sel = (int32_t*)outs;

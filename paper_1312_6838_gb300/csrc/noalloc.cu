@@ -10,7 +10,7 @@
 // take from the caller lives in g_css_scratch below.
 #include <mutex>
 
-#include "css_common.cuh"
+#include "init.cuh"
 
 namespace {
 
@@ -54,9 +54,8 @@ extern "C" css_status css_select_noalloc(const void* A, css_dtype dtype, int64_t
   // the device status sits in the library's array, which the caller cannot
   // pass to css_read_status, so the call always synchronises and reports it
   if (o.timing_ms || !o.sync) return CSS_ERR_INVALID_ARG;
-  const size_t need = css_workspace_size(CSS_OP_SELECT, dtype, m, n, 0, k, 0, &o);
-  if (need == 0) return CSS_ERR_INVALID_ARG;
-  if (need > (size_t)CSS_NOALLOC_SCRATCH_BYTES) return CSS_ERR_WORKSPACE;
+  if (css_workspace_size(CSS_OP_SELECT, dtype, m, n, 0, k, 0, &o) == 0) return CSS_ERR_INVALID_ARG;
+  if (css::select_least_workspace(dtype, m, n, k) > (size_t)CSS_NOALLOC_SCRATCH_BYTES) return CSS_ERR_WORKSPACE;
   void* ws = nullptr;
   css_status s = scratch_for_current_device(&ws);
   if (s != CSS_OK) return s;
