@@ -7,7 +7,9 @@
 // Gram matrix G = W W^T = U^(W) (Sigma^(W))^2 U^(W)^T:
 //   1. G on the slice GEMM (slice_gemm.cu): exact digit products, so G is as
 //      accurate as an FP64 product, on the tensor cores.
-//   2. jacobi_kernel: the eigenvalues of G by two-sided cyclic Jacobi
+//   2. From l = 32 on, an estimate X of the eigenvectors (eigvec.cu): the
+//      rounds below then start from X^T G X, and mostly find nothing to rotate.
+//      jacobi_kernel: the eigenvalues of G by two-sided cyclic Jacobi
 //      rotations (Golub and Van Loan, Matrix Computations, Sec. 8.5) in the
 //      parallel round-robin ordering of Brent and Luk (1985): each round
 //      rotates l/2 disjoint index pairs at once.  One cooperative kernel, one
@@ -29,6 +31,7 @@
 #include <vector>
 
 #include "css_common.cuh"
+#include "eigvec.cuh"
 #include "lowrank.cuh"
 #include "slice_gemm.cuh"
 
@@ -59,6 +62,7 @@ struct JacobiArgs {
   int lp;
   int gdim;
   int chunk;          // pairs per chunk
+  float tol2;         // the first check's (see needs_rot); 1e-30 after it
   uint32_t* bar;
   int* flags;         // [kMaxSweeps + 1]: some pair still needs a rotation
   int* info;          // [0] sweeps, [1] buffer holding the final G, [2] rounds
@@ -92,9 +96,9 @@ __device__ __forceinline__ void rot(double c, double s, double a, double b, doub
 // of Demmel and Veselic) or |g_pq| <= 1e-17 trace(G), far below the Gram
 // matrix's own rounding.  Evaluated in FP32 on the entries scaled by
 // 1 / trace(G) (all of magnitude <= 1 for a PSD G).
-__device__ __forceinline__ bool needs_rot(double gpp, double gqq, double gpq, double inv_tr) {
+__device__ __forceinline__ bool needs_rot(double gpp, double gqq, double gpq, double inv_tr, float tol2 = 1e-30f) {
   const float ps = (float)(gpp * inv_tr), qs = (float)(gqq * inv_tr), xs = fabsf((float)(gpq * inv_tr));
-  return xs > 1e-17f && xs * xs > 1e-30f * fabsf(ps * qs);
+  return xs > 1e-17f && xs * xs > tol2 * fabsf(ps * qs);
 }
 
 // The rotation that annihilates g_pq: t = tan(theta), the smaller root of
@@ -173,7 +177,7 @@ __global__ void __launch_bounds__(kJacobiThreads) jacobi_kernel(JacobiArgs A) {
         if (p >= q) continue;
         const double gpq = __ldcg(Gc + idx);
         const double gpp = __ldcg(Gc + (long long)p * lp + p), gqq = __ldcg(Gc + (long long)q * lp + q);
-        bad |= needs_rot(gpp, gqq, gpq, inv_tr) ? 1 : 0;
+        bad |= needs_rot(gpp, gqq, gpq, inv_tr, sweep ? 1e-30f : A.tol2) ? 1 : 0;
       }
       if (__syncthreads_or(bad) && tid == 0) atomicOr(A.flags + sweep, 1);
       if (!team_barrier(A.bar, ncta, A.st, 40, &s_epoch)) return;
@@ -279,8 +283,9 @@ __global__ void __launch_bounds__(kJacobiThreads) jacobi_kernel(JacobiArgs A) {
 __global__ void __launch_bounds__(512) replay_columns_kernel(const double2* __restrict__ rotlog,
                                                              const int* __restrict__ info,
                                                              const int* __restrict__ ord, int l, int lp,
-                                                             double* __restrict__ Uw) {
-  extern __shared__ double col[];
+                                                             const double* __restrict__ X, double* __restrict__ Uw) {
+  extern __shared__ double col_[];
+  double* col = col_;
   __shared__ double s_best[16];
   __shared__ int s_bi[16];
   const int h = lp / 2, j = threadIdx.x;   // blockDim.x: h rounded up to whole warps
@@ -304,6 +309,22 @@ __global__ void __launch_bounds__(512) replay_columns_kernel(const double2* __re
     __syncthreads();
     cs = nxt;
     if (--r < 0) r = lp - 2;
+  }
+  if (X) {
+    // the rounds started from X^T G X: the eigenvector of G is X V e
+    for (int i0 = 0; i0 < l; i0 += blockDim.x) {
+      const int i = i0 + threadIdx.x;
+      double u = 0.0;
+      if (R == 0) {
+        if (i < l) u = X[(long long)c0 * l + i];
+      } else if (i < l) {
+#pragma unroll 8
+        for (int q = 0; q < l; ++q) u = fma(X[(long long)q * l + i], col[q], u);
+      }
+      if (i < l) col[lp + i] = u;
+    }
+    __syncthreads();
+    col += lp;
   }
   // sign rule: block-wide argmax of |v_i| (lowest index on ties)
   double best = -1.0;
@@ -338,16 +359,24 @@ __global__ void __launch_bounds__(1024) order_kernel(const double* __restrict__ 
                                                      double* __restrict__ sigma, double* __restrict__ scale,
                                                      double* __restrict__ tail, int* __restrict__ ord_out) {
   __shared__ double lam[kMaxL];
+  __shared__ long long key[kMaxL];   // orders like lam (zeros of either sign are equal); FP64 compares are slow
   __shared__ int ord[kMaxL];
   __shared__ double red[32];
   const double* G = info[1] ? G1 : G0;
-  for (int i = threadIdx.x; i < l; i += blockDim.x) lam[i] = G[(long long)i * lp + i];
+  for (int i = threadIdx.x; i < l; i += blockDim.x) {
+    const double v = G[(long long)i * lp + i];
+    const long long b = __double_as_longlong(v);
+    lam[i] = v;
+    key[i] = b >= 0 ? b : -(b & 0x7fffffffffffffffll);
+  }
   __syncthreads();
   double tr = 0.0;
   for (int i = threadIdx.x; i < l; i += blockDim.x) {
     const double v = lam[i];
+    const long long kv = key[i];
     int rk = 0;
-    for (int j = 0; j < l; ++j) rk += (lam[j] > v) || (lam[j] == v && j < i);
+#pragma unroll 4
+    for (int j = 0; j < l; ++j) rk += (key[j] > kv) || (key[j] == kv && j < i);
     ord[rk] = i;
     tr += fmax(v, 0.0);
   }
@@ -377,6 +406,7 @@ struct LrLayout {
   int* ord;
   double2* rotlog;
   long long max_rounds;
+  Estimate est;
   sg::Digits DW, DUw;   // W (both ways, one after the other) or Q, and U^(W)_k
   sg::Scratch sc;
   size_t bytes;
@@ -397,6 +427,7 @@ LrLayout lr_layout(void* ws, size_t cap, int64_t n, int32_t l, int32_t k) {
   L.rotlog = c.take<double2>((size_t)L.max_rounds * (lp / 2));
   L.Uw = c.take<double>((size_t)l * k);
   L.scale = c.take<double>(k);
+  L.est = carve_estimate(c, l);
   // the digits of W by rows, of W by columns and of Q (n rows at a time)
   // share their space
   const size_t at = c.off;
@@ -492,14 +523,26 @@ extern "C" css_status css_lowrank(const double* W, int64_t ldw, const double* Q,
   if (lp > l) pad_kernel<<<(lp + 255) / 256, 256, 0, s>>>(L.G0, l, lp);
   if (cudaGetLastError() != cudaSuccess) return CSS_ERR_CUDA;
   if (timed) cudaEventRecord(ev[1], s);
-  JacobiArgs ja{L.G0, L.G1, L.rotlog, L.max_rounds, lp, gdim, chunk, L.bar, L.flags, L.info, L.st};
+  // the rounds start from G itself, or from X^T G X for an estimate X of its
+  // eigenvectors (from kEstimateMinL columns on)
+  const double* X = nullptr;
+  if (estimate_fits(l, sms)) {
+    e = estimate_eigvecs(L.G0, L.G1, l, lp, L.est, L.st, sms, &X, s);
+    if (e != cudaSuccess) return CSS_ERR_CUDA;
+    std::swap(L.G0, L.G1);
+    if (lp > l) pad_kernel<<<(lp + 255) / 256, 256, 0, s>>>(L.G0, l, lp);
+  }
+  // X^T G X comes out of products with a rounding of about 1e-15 of its
+  // diagonal: what is below 4e-15 is not worth a sweep
+  const float tol2 = X ? 1.6e-29f : 1e-30f;
+  JacobiArgs ja{L.G0, L.G1, L.rotlog, L.max_rounds, lp, gdim, chunk, tol2, L.bar, L.flags, L.info, L.st};
   void* args[] = {&ja};
   e = cudaLaunchCooperativeKernel((const void*)jacobi_kernel, dim3(gdim * (gdim + 1) / 2), dim3(kJacobiThreads),
                                   args, 0, s);
   if (e != cudaSuccess) return CSS_ERR_CUDA;
   double* uw = Uw ? Uw : L.Uw;
   order_kernel<<<1, 1024, 0, s>>>(L.G0, L.G1, L.info, l, lp, k, (long long)n, sigma, L.scale, tail, L.ord);
-  replay_columns_kernel<<<k, (h + 31) / 32 * 32, lp * sizeof(double), s>>>(L.rotlog, L.info, L.ord, l, lp, uw);
+  replay_columns_kernel<<<k, (h + 31) / 32 * 32, 2 * lp * sizeof(double), s>>>(L.rotlog, L.info, L.ord, l, lp, X, uw);
   if (timed) cudaEventRecord(ev[2], s);
   sg::Digits& DQ = L.DW;
   const sg::Source us{uw, CSS_F64, l, 1, k, l};
