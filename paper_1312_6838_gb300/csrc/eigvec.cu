@@ -6,8 +6,8 @@
 // grid barrier and FP64 at two lanes per clock and SM), and starting from G
 // they take some twelve sweeps of l - 1 rounds: 11.9 of the 13.1 ms of
 // css_lowrank at l = 256 (here 2.44 in all: 1.5 for part 1 and 0.9 for parts 2
-// and 3, and no sweep is left).  From l = 32 on: 1.15 -> 0.39 ms there, below
-// it the rounds are as fast.  A spectrum that FP32 does not resolve leaves
+// and 3, and no sweep is left).  From l = 17 on (l = 31: 1.15 -> 0.39 ms; at
+// l = 16 the rounds take 0.37).  A spectrum that FP32 does not resolve leaves
 // more sweeps: singular values 1 / i at l = 256 14.2 -> 9.4 ms.  Here:
 //   1. estimate_kernel: block Jacobi in FP32 (the ordering of Brent and Luk
 //      over 32-column blocks; Golub and Van Loan, Matrix Computations,

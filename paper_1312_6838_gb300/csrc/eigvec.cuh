@@ -6,7 +6,7 @@
 
 namespace css {
 
-constexpr int kEstimateMinL = 32;   // see eigvec.cu
+constexpr int kEstimateMinL = 17;   // see eigvec.cu
 
 // Scratch of the estimate; G and H are lp x lp (leading dimension lp, l <= lp).
 struct Estimate {

@@ -7,7 +7,7 @@
 // Gram matrix G = W W^T = U^(W) (Sigma^(W))^2 U^(W)^T:
 //   1. G on the slice GEMM (slice_gemm.cu): exact digit products, so G is as
 //      accurate as an FP64 product, on the tensor cores.
-//   2. From l = 32 on, an estimate X of the eigenvectors (eigvec.cu): the
+//   2. From l = 17 on, an estimate X of the eigenvectors (eigvec.cu): the
 //      rounds below then start from X^T G X, and mostly find nothing to rotate.
 //      jacobi_kernel: the eigenvalues of G by two-sided cyclic Jacobi
 //      rotations (Golub and Van Loan, Matrix Computations, Sec. 8.5) in the
@@ -396,6 +396,35 @@ __global__ void __launch_bounds__(1024) order_kernel(const double* __restrict__ 
   }
 }
 
+// out[i + j ldo] = scale_j sum_q S[i + q lds] U[q + j l] for few multiply-adds
+// (kSmallProduct): eight columns a block, a row a thread, one FP64 pass where
+// the slice GEMM takes five launches (l = 16, n = 8000, k = 8, U and V:
+// 58 -> 10 us).
+constexpr int kSmallL = 64;
+constexpr double kSmallProduct = 1.6e7;   // the FP64 rate's 27 us
+__global__ void __launch_bounds__(128) small_product_kernel(const double* __restrict__ S, long long lds, long long rows,
+                                                            int l, int k, const double* __restrict__ U,
+                                                            const double* __restrict__ scale, double* __restrict__ out,
+                                                            long long ldo) {
+  __shared__ __align__(16) double su[kSmallL][8];
+  const int j0 = blockIdx.y * 8;
+  for (int e = threadIdx.x; e < l * 8; e += 128) su[e >> 3][e & 7] = j0 + (e & 7) < k ? U[(long long)(j0 + (e & 7)) * l + (e >> 3)] : 0.0;
+  __syncthreads();
+  const long long i = (long long)blockIdx.x * 128 + threadIdx.x;
+  if (i >= rows) return;
+  double acc[8] = {};
+#pragma unroll 8
+  for (int q = 0; q < l; ++q) {
+    const double v = __ldg(S + q * lds + i);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) acc[j] = fma(v, su[q][j], acc[j]);
+  }
+#pragma unroll
+  for (int j = 0; j < 8; ++j)
+    if (j0 + j < k) out[(long long)(j0 + j) * ldo + i] = scale ? acc[j] * scale[j0 + j] : acc[j];
+}
+bool small_product(long long rows, int l, int k) { return l <= kSmallL && (double)rows * l * k <= kSmallProduct; }
+
 // ------------------------------------------------------------ host side --
 struct LrLayout {
   DevStatus* st;
@@ -546,15 +575,23 @@ extern "C" css_status css_lowrank(const double* W, int64_t ldw, const double* Q,
   if (timed) cudaEventRecord(ev[2], s);
   sg::Digits& DQ = L.DW;
   const sg::Source us{uw, CSS_F64, l, 1, k, l};
-  e = U || V ? sg::split(us, L.DUw, s) : cudaSuccess;
+  const bool small_u = small_product(m, l, k), small_v = small_product(n, l, k);
+  e = (U && !small_u) || (V && !small_v) ? sg::split(us, L.DUw, s) : cudaSuccess;
   const int rows = ((int)n + 127) / 128 * 128;   // the digits' space holds whole tiles
-  for (int64_t r0 = 0; U && e == cudaSuccess && r0 < m; r0 += rows) {
+  if (U && small_u) {
+    small_product_kernel<<<dim3((unsigned)((m + 127) / 128), (k + 7) / 8), 128, 0, s>>>(Q, ldq, m, l, k, uw, nullptr,
+                                                                                       U, ldu);
+  }
+  for (int64_t r0 = 0; U && !small_u && e == cudaSuccess && r0 < m; r0 += rows) {
     const sg::Source q{Q + r0, CSS_F64, 1, ldq, (int)std::min<int64_t>(rows, m - r0), l};
     e = sg::split(q, DQ, s);
     if (e == cudaSuccess)
       e = sg::gemm(DQ, q, L.DUw, us, sg::Store{U + r0, 1, ldu, 0}, L.sc, err, hs.spin_budget_ns, s);
   }
-  if (V && e == cudaSuccess) {
+  if (V && small_v && e == cudaSuccess) {
+    small_product_kernel<<<dim3((unsigned)((n + 127) / 128), (k + 7) / 8), 128, 0, s>>>(W, ldw, n, l, k, uw, L.scale,
+                                                                                       V, ldv);
+  } else if (V && e == cudaSuccess) {
     e = sg::split(wr, L.DW, s);
     if (e == cudaSuccess)
       e = sg::gemm(L.DW, wr, L.DUw, us, sg::Store{V, 1, ldv, 0, L.scale}, L.sc, err, hs.spin_budget_ns, s);
