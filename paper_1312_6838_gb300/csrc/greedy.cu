@@ -1223,60 +1223,54 @@ __device__ void run_unit(const Ctx<typename AccOf<TA>::type>& x, const UnitDesc&
       }
       for (int i = x.rank * NW + x.warp; !short_path && i < m; i += x.ncta * NW, ++kr) {
         const Acc* cp = C + (long long)i * u.ldt;
-        Acc accs[UC];
-#pragma unroll
-        for (int q = 0; q < UC; ++q) accs[q] = Acc(0);
-        int l = x.lane * VC;
-        for (; l + (UC - 1) * 32 * VC < m_vec; l += UC * 32 * VC) {
-          uint4 raw[UC];
-#pragma unroll
-          for (int q = 0; q < UC; ++q) raw[q] = ldg_stream16(cp + l + q * 32 * VC, pol_keep);
-#pragma unroll
-          for (int q = 0; q < UC; ++q) {
-            Acc cv[VC], ev[VC];
-            if constexpr (sizeof(Acc) == 4) Vec<float>::unpack(raw[q], cv);
-            else Vec<double>::unpack(raw[q], cv);
-            lds_vec<Acc, VC>(x.seacc + l + q * 32 * VC, ev);
-#pragma unroll
-            for (int e = 0; e < VC; ++e) accs[q] = fma(cv[e], ev[e], accs[q]);
-          }
-        }
+        Acc acc = Acc(0);
         if constexpr (sizeof(Acc) == 8) {
-          // eight loads in flight, the same sums (a missing vector adds
-          // nothing): rows below 960 elements took a memory trip per vector
-          // (m = 500: 6.7 us a pivot)
+          // FP64: one accumulator (sixteen end in a chain of sixteen slow
+          // additions, and spill) and eight loads in flight for rows of any
+          // length: m = 500 6.7 -> 3.8 us a pivot
           constexpr int UR = 8;
-          for (; l < m_vec; l += UR * 32 * VC) {
+          for (int l = x.lane * VC; l < m_vec; l += UR * 32 * VC) {
             uint4 raw[UR];
 #pragma unroll
             for (int q = 0; q < UR; ++q)
-              if (l + q * 32 * VC < m_vec) raw[q] = ldg_stream16(cp + l + q * 32 * VC, pol_keep);
+              raw[q] = l + q * 32 * VC < m_vec ? ldg_stream16(cp + l + q * 32 * VC, pol_keep) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
             for (int q = 0; q < UR; ++q) {
-              if (l + q * 32 * VC < m_vec) {
-                Acc cv[VC], ev[VC];
-                Vec<double>::unpack(raw[q], cv);
-                lds_vec<Acc, VC>(x.seacc + l + q * 32 * VC, ev);
+              if (l + q * 32 * VC >= m_vec) break;
+              Acc cv[VC], ev[VC];
+              Vec<double>::unpack(raw[q], cv);
+              lds_vec<Acc, VC>(x.seacc + l + q * 32 * VC, ev);
 #pragma unroll
-                for (int e = 0; e < VC; ++e) accs[0] = fma(cv[e], ev[e], accs[0]);
-              }
+              for (int e = 0; e < VC; ++e) acc = fma(cv[e], ev[e], acc);
             }
           }
-        }
-        for (; l < m_vec; l += 32 * VC) {
-          Acc cv[VC], ev[VC];
-          if constexpr (sizeof(Acc) == 4) Vec<float>::unpack(ldg_stream16(cp + l, pol_keep), cv);
-          else Vec<double>::unpack(ldg_stream16(cp + l, pol_keep), cv);
-          lds_vec<Acc, VC>(x.seacc + l, ev);
+        } else {
+          Acc accs[UC];
 #pragma unroll
-          for (int e = 0; e < VC; ++e) accs[0] = fma(cv[e], ev[e], accs[0]);
-        }
-        Acc acc = Acc(0);
-        if (sizeof(Acc) == 4 || m_vec > (UC - 1) * 32 * VC) {
+          for (int q = 0; q < UC; ++q) accs[q] = Acc(0);
+          int l = x.lane * VC;
+          for (; l + (UC - 1) * 32 * VC < m_vec; l += UC * 32 * VC) {
+            uint4 raw[UC];
+#pragma unroll
+            for (int q = 0; q < UC; ++q) raw[q] = ldg_stream16(cp + l + q * 32 * VC, pol_keep);
+#pragma unroll
+            for (int q = 0; q < UC; ++q) {
+              Acc cv[VC], ev[VC];
+              Vec<float>::unpack(raw[q], cv);
+              lds_vec<Acc, VC>(x.seacc + l + q * 32 * VC, ev);
+#pragma unroll
+              for (int e = 0; e < VC; ++e) accs[q] = fma(cv[e], ev[e], accs[q]);
+            }
+          }
+          for (; l < m_vec; l += 32 * VC) {
+            Acc cv[VC], ev[VC];
+            Vec<float>::unpack(ldg_stream16(cp + l, pol_keep), cv);
+            lds_vec<Acc, VC>(x.seacc + l, ev);
+#pragma unroll
+            for (int e = 0; e < VC; ++e) accs[0] = fma(cv[e], ev[e], accs[0]);
+          }
 #pragma unroll
           for (int q = 0; q < UC; ++q) acc += accs[q];
-        } else {
-          acc = accs[0];   // the others are zero, and an FP64 sum is a chain of sixteen
         }
         for (int l2 = m_vec + x.lane; l2 < m; l2 += 32) acc = fma(__ldg(cp + l2), x.seacc[l2], acc);
         acc = warp_sum(acc);
