@@ -80,17 +80,12 @@ struct Header {
   DevStatus* st;
   DevStatus* st_init;   // the status a launch starts from (copied into st)
   UnitDesc* units;
-  TeamDesc* teams;
-  int* order;
-  int* cta_team;
-  uint32_t* bars;
   double* part;
   double* cand_val;
   int* cand_idx;
-  uint32_t* tile_ctr;
   int* aux_err;   // error flag of the tensor-core initial-score kernel
   void* split_part;
-  uint32_t* split_done;
+  uint32_t *bars, *tile_ctr, *split_done;
   int split_slots;
 };
 
@@ -113,18 +108,21 @@ static_assert(sizeof(DevStatus) <= kAuxErrOffset && kAuxErrOffset + sizeof(int) 
 void carve_header(WsCarver& c, int max_units, Header& h, int64_t split_cols) {
   h.st = c.take<DevStatus>(1);
   h.aux_err = h.st ? reinterpret_cast<int*>(reinterpret_cast<char*>(h.st) + kAuxErrOffset) : nullptr;
+  // the plan, filled by one copy: status, units, teams, order, CTAs' teams
+  // (the last three as long as the plan needs, see prepare_units)
   h.st_init = c.take<DevStatus>(1);
   h.units = c.take<UnitDesc>(max_units);
-  h.teams = c.take<TeamDesc>(kMaxCtas);
-  h.order = c.take<int>(max_units);
-  h.cta_team = c.take<int>(kMaxCtas);
-  h.bars = c.take<uint32_t>(2 * kMaxCtas);
+  c.take<TeamDesc>(kMaxCtas);
+  c.take<int>(max_units);
+  c.take<int>(kMaxCtas);
   h.part = c.take<double>(4 * kMaxCtas);
   h.cand_val = c.take<double>(kMaxCtas);
   h.cand_idx = c.take<int>(kMaxCtas);
-  h.tile_ctr = c.take<uint32_t>(2 * kMaxCtas);
   h.split_slots = split_slots_for(split_cols);
   h.split_part = c.take<char>((size_t)h.split_slots * kSplitSlotBytes);
+  // zeroed by one memset a launch: barriers, tile counters, split arrivals
+  h.bars = c.take<uint32_t>(2 * kMaxCtas);
+  h.tile_ctr = c.take<uint32_t>(2 * kMaxCtas);
   h.split_done = c.take<uint32_t>(h.split_slots);
 }
 
@@ -229,9 +227,7 @@ Plan make_plan(const std::vector<double>& work, int grid) {
 struct LaunchInfo {
   GreedyLaunch L;
   int split_used;
-  uint32_t* bars;
-  uint32_t* tile_ctr;
-  uint32_t* split_done;
+  uint32_t *bars, *split_done;
   DevStatus* st;
   DevStatus* st_init;
   // false: the launch keeps the status an earlier launch of the same call
@@ -291,17 +287,25 @@ css_status prepare_units(const Header& h, std::vector<UnitDesc>& units, const st
   DevStatus st{};
   st.spin_budget_ns = spin_ns ? spin_ns : kDefaultSpinNs;
   st.stall_where = stall_where;
-  cudaError_t e;
-  if ((e = cudaMemcpyAsync(h.st_init, &st, sizeof(st), cudaMemcpyHostToDevice, s)) != cudaSuccess) return cuda_status(e);
-  if ((e = cudaMemcpyAsync(h.units, units.data(), units.size() * sizeof(UnitDesc), cudaMemcpyHostToDevice, s)) != cudaSuccess) return cuda_status(e);
-  if ((e = cudaMemcpyAsync(h.teams, P.teams.data(), P.teams.size() * sizeof(TeamDesc), cudaMemcpyHostToDevice, s)) != cudaSuccess) return cuda_status(e);
-  if ((e = cudaMemcpyAsync(h.order, P.order.data(), P.order.size() * sizeof(int), cudaMemcpyHostToDevice, s)) != cudaSuccess) return cuda_status(e);
-  if ((e = cudaMemcpyAsync(h.cta_team, P.cta_team.data(), P.cta_team.size() * sizeof(int), cudaMemcpyHostToDevice, s)) != cudaSuccess) return cuda_status(e);
+  // one copy for the whole plan: each one more cost a small call about 3 us
+  const size_t at_units = (size_t)((char*)h.units - (char*)h.st_init);
+  const size_t at_teams = at_units + align_up(units.size() * sizeof(UnitDesc));
+  const size_t at_order = at_teams + align_up(P.teams.size() * sizeof(TeamDesc));
+  const size_t at_ctas = at_order + align_up(P.order.size() * sizeof(int));
+  std::vector<char> plan(at_ctas + P.cta_team.size() * sizeof(int));
+  std::memcpy(plan.data(), &st, sizeof(st));
+  std::memcpy(plan.data() + at_units, units.data(), units.size() * sizeof(UnitDesc));
+  std::memcpy(plan.data() + at_teams, P.teams.data(), P.teams.size() * sizeof(TeamDesc));
+  std::memcpy(plan.data() + at_order, P.order.data(), P.order.size() * sizeof(int));
+  std::memcpy(plan.data() + at_ctas, P.cta_team.data(), P.cta_team.size() * sizeof(int));
+  char* const dev = (char*)h.st_init;
+  const cudaError_t e = cudaMemcpyAsync(dev, plan.data(), plan.size(), cudaMemcpyHostToDevice, s);
+  if (e != cudaSuccess) return cuda_status(e);
   GreedyLaunch L{};
   L.units = h.units;
-  L.order = h.order;
-  L.teams = h.teams;
-  L.cta_team = h.cta_team;
+  L.order = (const int*)(dev + at_order);
+  L.teams = (const TeamDesc*)(dev + at_teams);
+  L.cta_team = (const int*)(dev + at_ctas);
   L.st = h.st;
   L.dtype = dt;
   L.tile_cols = tile_cols;
@@ -316,7 +320,6 @@ css_status prepare_units(const Header& h, std::vector<UnitDesc>& units, const st
   info.L = L;
   info.split_used = split_used;
   info.bars = h.bars;
-  info.tile_ctr = h.tile_ctr;
   info.split_done = h.split_done;
   info.st = h.st;
   info.st_init = h.st_init;
@@ -329,12 +332,9 @@ css_status start_units(const LaunchInfo& info, cudaStream_t s) {
   if (info.reset_status &&
       (e = cudaMemcpyAsync(info.st, info.st_init, sizeof(DevStatus), cudaMemcpyDeviceToDevice, s)) != cudaSuccess)
     return cuda_status(e);
-  if ((e = cudaMemsetAsync(info.bars, 0, 2 * sizeof(uint32_t) * info.L.grid, s)) != cudaSuccess) return cuda_status(e);
-  if ((e = cudaMemsetAsync(info.tile_ctr, 0, 2 * sizeof(uint32_t) * info.L.grid, s)) != cudaSuccess)
-    return cuda_status(e);
-  if (info.split_used > 0 &&
-      (e = cudaMemsetAsync(info.split_done, 0, sizeof(uint32_t) * info.split_used, s)) != cudaSuccess)
-    return cuda_status(e);
+  // barriers, tile counters and the used split arrivals lie one after another
+  const size_t used = (size_t)((char*)(info.split_done + info.split_used) - (char*)info.bars);
+  if ((e = cudaMemsetAsync(info.bars, 0, used, s)) != cudaSuccess) return cuda_status(e);
   return cuda_status(greedy_launch(info.L, s));
 }
 
@@ -348,13 +348,22 @@ css_status launch_units(const Header& h, std::vector<UnitDesc>& units, const std
   return start_units(info, s);
 }
 
+// The status slot at the start of a workspace (the DevStatus and the
+// tensor-core kernels' flag), read in one copy.
+cudaError_t read_status_slot(const void* slot, DevStatus& st, int& aux, cudaStream_t s) {
+  char buf[kAuxErrOffset + sizeof(int)] = {};
+  cudaError_t e = cudaMemcpyAsync(buf, slot, sizeof(buf), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  std::memcpy(&st, buf, sizeof(st));
+  std::memcpy(&aux, buf + kAuxErrOffset, sizeof(int));
+  return e;
+}
+
 css_status finish(const Header& h, const css_opts& o, cudaStream_t s) {
   if (!o.sync) return CSS_OK;
   DevStatus st{};
   int aux = 0;
-  cudaError_t e = cudaMemcpyAsync(&st, h.st, sizeof(st), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&aux, h.aux_err, sizeof(int), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  const cudaError_t e = read_status_slot(h.st, st, aux, s);
   if (e != cudaSuccess) return cuda_status(e);
   if (aux != 0) return (css_status)aux;
   if (st.code != 0) return (css_status)st.code;
@@ -816,11 +825,7 @@ css_status css_read_status(const void* ws, css_stream_t stream) {
   if (!ws) return CSS_ERR_WORKSPACE;
   DevStatus st{};
   int aux = 0;
-  cudaError_t e = cudaMemcpyAsync(&st, ws, sizeof(st), cudaMemcpyDeviceToHost, (cudaStream_t)stream);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(&aux, (const char*)ws + kAuxErrOffset, sizeof(int), cudaMemcpyDeviceToHost,
-                        (cudaStream_t)stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize((cudaStream_t)stream);
+  const cudaError_t e = read_status_slot(ws, st, aux, (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_status(e);
   if (aux != 0) return (css_status)aux;
   if (st.code != 0) return (css_status)st.code;
