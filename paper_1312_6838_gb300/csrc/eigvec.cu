@@ -327,7 +327,8 @@ __global__ void __launch_bounds__(kNT, 1) estimate_kernel(EstArgs A) {
     if (blockIdx.x == 0 && tid == 0) set_error(A.st, (int32_t)CSS_ERR_NONFINITE, 0);
     return;
   }
-  const double inv_tr = tr > 0.0 ? 1.0 / tr : 0.0;
+  // (a trace whose inverse overflows: X stays the identity)
+  const double inv_tr = tr > 0.0 && 1.0 / tr < 1e308 ? 1.0 / tr : 0.0;
   for (int e = blockIdx.x * kNT + tid; e < L * L; e += ncta * kNT) {
     const int r = e % L, c = e / L;
     __stcg(A.w.A0 + e, r < A.l && c < A.l ? (float)(A.G[(long long)c * A.lp + r] * inv_tr) : 0.f);
