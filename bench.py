@@ -596,16 +596,15 @@ def run_adjoint(args):
                    "noise": c["noise"], "l2": "A and dA (268 MB each) larger than L2"},
         "roofline": {"bound": "alu", "achieved": tf, "peak": FP32_TFLOPS, "unit": "TFLOP/s",
                      "frac": tf / FP32_TFLOPS, "traffic": None,
-                     "kernel": "the adjoint's three GEMM-shaped kernels (double-float W and R, FP32 R W^T)",
-                     "note": "algorithmic 6 k m n FLOPs; W and R run in double-float (about 12 FP32 operations "
-                             "per multiply-add), so the FP32 pipe does several times the algorithmic count"},
+                     "kernel": "the adjoint's three products on the slice GEMM (W, R, R W^T)",
+                     "note": "algorithmic 6 k m n FLOPs against the FP32 rate; the products run as exact "
+                             "products of 8-bit digits on the BF16 tensor cores"},
         "hbm_bytes_per_call": 3 * m * n * 4, "loss": float(loss.item()), "clocks": clocks,
-        # per call: gather A_S, Gram (2), the Cholesky (one launch for
-        # k <= 128; above, the blocked form: initial diagonal, per 32-column
-        # panel the diagonal block and, but for the last panel, the rows below
-        # and the trailing update), L^-1, Q, W, R with the loss partials, loss
-        # sum, R W^T slices, their sum, dA_S
-        "gpu_launches": (12 if k <= 128 else 10 + 3 * ((k + 31) // 32)) * args.steps,
+        # per call (k <= 128): gather A_S, Gram (2), the initial diagonal, per
+        # 32-column panel the diagonal block, the rows and (but for the last)
+        # the update, Q, the splits of Q (both ways), A, W (both ways) and R
+        # (two launches each), W, R, R W^T with its finish, loss sum, dA_S
+        "gpu_launches": (22 + 3 * ((k + 31) // 32)) * args.steps,
     }
     if not args.no_cpu_baseline:
         from oracle import css_oracle as O
@@ -641,7 +640,7 @@ def run_lowrank(args):
         css.lowrank(W, kr, Q)
     phases = css.lowrank(W, kr, Q, timing=True).timing_ms
     # the embedding of Sec. 3.2 formed from scratch for the same selection
-    # (CholeskyQR2 of A_S, then W = Q^T A in double-float arithmetic)
+    # (CholeskyQR2 of A_S, then W = Q^T A from digit products)
     S = res.indices
     css.embed(A, S)
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -662,7 +661,7 @@ def run_lowrank(args):
     torch.cuda.synchronize()
     clocks = clk.stop()
     ms = ev0.elapsed_time(ev1) / args.steps
-    # the dominant kernel: the Gram matrix W W^T, l (l + 1) / 2 n FP64 FMAs
+    # the Gram matrix W W^T: l (l + 1) / 2 n multiply-adds
     gram_flop = 2.0 * (l * (l + 1) / 2) * n
     gram_tf = gram_flop / (phases[0] * 1e-3) / 1e12
     v_flop = 2.0 * n * l * kr + 2.0 * m * l * kr
@@ -675,17 +674,13 @@ def run_lowrank(args):
         "phases_ms": {"gram": phases[0], "eigendecomposition": phases[1], "products": phases[2]},
         "jacobi_sweeps": int(phases[3]),
         "embed_ms": embed_ms,
-        # algorithmic FLOP rates: the Gram matrix in FP64, the products of
-        # FP64 operands accumulated in double-float on the FP32 pipe
+        # algorithmic FLOP rates; both run as digit products on the tensor cores
         "tflops": {"gram_fp64": gram_tf,
-                   "products_double_float": v_flop / (phases[2] * 1e-3) / 1e12},
-        # traffic: DRAM bytes read + written by one gram_rows_kernel launch on
-        # this workload, from an ncu capture of that kernel (W read once, the
-        # slices' partial tiles written)
-        "roofline": {"bound": "alu", "achieved": gram_tf, "peak": FP64_TFLOPS, "unit": "TFLOP/s",
-                     "frac": gram_tf / FP64_TFLOPS,
-                     "traffic": (134.7e6 + 9.4e6) if (m, n, l) == (4096, 65536, 256) else None,
-                     "kernel": "gram_rows_kernel (FP64)"},
+                   "products_fp64": v_flop / (phases[2] * 1e-3) / 1e12},
+        "roofline": {"bound": "latency", "achieved": gram_tf, "peak": FP64_TFLOPS, "unit": "TFLOP/s",
+                     "frac": gram_tf / FP64_TFLOPS, "traffic": None,
+                     "kernel": "the Gram matrix as digit products, against the FP64 rate; the call's time is the "
+                               "eigendecomposition's dependent rounds"},
         "sigma_1": float(out.sigma[0]), "tail": out.tail, "clocks": clocks,
     }
     if not args.no_cpu_baseline:

@@ -533,9 +533,9 @@ css_status css_autotune_distributed(const void* A, css_dtype dtype, int64_t m, i
  * The k x k factor of A_S^T A_S is recomputed here (FP64 Cholesky); a pivot at or below 1e-12 of its
  * column's squared norm (dependent columns in S) gives CSS_ERR_INVALID_ARG
  * (reported in sync mode), as do out-of-range or repeated indices.
- * FP32/BF16 input: the two products that cancel (Q^T A and A - Q W, with
- * Q = A_S L^-T) run in double-float arithmetic (FP32 pairs, error-free
- * products and sums), R W^T accumulates in FP32, the factorisation and the
+ * Q^T A, Q W and R W^T are sums of exact products of 8-bit digits (what is
+ * dropped is below 2^-64 of the rows' largest products; R W^T of FP32/BF16
+ * input, whose R is held in FP32, keeps 2^-33); the factorisation and the
  * loss are FP64; dA is rounded once to the dtype of A.  k <= 1024.
  */
 css_status css_residual_backward(const void* A, css_dtype dtype, int64_t m,
@@ -583,9 +583,8 @@ css_status css_residual_backward_factors(const void* A, css_dtype dtype,
  * more on Q1), orthonormal to working precision while the condition number of
  * A_S stays below about 1e7.  A pivot at or below 1e-12 of its column's
  * squared norm (dependent columns) gives CSS_ERR_INVALID_ARG (sync mode).
- * W: FP64 products for FP64 input; FP32/BF16 input runs in double-float
- * arithmetic (FP32 pairs with error-free products and sums).  l <= 1024,
- * l <= min(m, n).  Workspace: css_workspace_size(CSS_OP_EMBED, dtype, m, n,
+ * W: sums of exact digit products (dropped: below 2^-64 of the rows' largest
+ * products), rounded to FP64 once.  l <= 1024, l <= min(m, n).  Workspace: css_workspace_size(CSS_OP_EMBED, dtype, m, n,
  * 0, l, 0, opts).
  */
 css_status css_embed(const void* A, css_dtype dtype, int64_t m, int64_t n,
@@ -621,11 +620,11 @@ css_status css_embed(const void* A, css_dtype dtype, int64_t m, int64_t n,
  *             the first term being css_select's final error trace entry.
  * Each singular vector is signed so that the entry of largest magnitude of
  * its U^(W) column (lowest index on ties) is positive.
- * Method: G = W W^T (FP64), its eigendecomposition by cyclic Jacobi
- * rotations in FP64 (parallel round-robin ordering, one cooperative
- * kernel), sigma_i^2 = lambda_i, then U~ and V~ as products of FP64
- * operands accumulated in double-float (48 significant bits; Q's entries,
- * at most 1 for an orthonormal basis, must lie in FP32's range).  The
+ * Method: G = W W^T (sums of exact digit products), its eigendecomposition
+ * by cyclic Jacobi rotations in FP64 (parallel round-robin ordering, one
+ * cooperative kernel), from l = 17 on of X^T G X for an estimate X of the
+ * eigenvectors (FP32 block Jacobi refined in FP64), sigma_i^2 = lambda_i, then
+ * U~ and V~ from digit products (FP64 sums where they are few).  The
  * eigenvalues carry an absolute error of about (n + l) 2^-53 ||W||_F^2 (the
  * Gram matrix's rounding): sigma_i is accurate relative to sigma_1^2 /
  * sigma_i, not to sigma_i.  CSS_ERR_NOT_CONVERGED if the rotations have not

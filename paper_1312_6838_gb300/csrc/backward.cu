@@ -12,10 +12,9 @@
 // of its own forward call):
 //   W = Q^T A,  R = A - Q W,  T = L^-T W,  R T^T = (R W^T) L^-1.
 // R is a small difference of large terms (the part of A outside span(A_S)),
-// so W and R are accumulated in double-float arithmetic (pairs of FP32 values
-// with error-free products and sums: Dekker's product by FMA and Knuth's
-// TwoSum) when A is FP32/BF16; FP64 input uses FP64 throughout.  R W^T has no
-// such cancellation and is accumulated in FP32 (FP64 for FP64 input).
+// so W, Q W and R W^T are sums of exact digit products on the slice GEMM
+// (slice_gemm.cu); R of FP32/BF16 input is formed from pairs of FP32 values
+// and held in FP32, and its product with W^T keeps the digits that matter there.
 #include <algorithm>
 #include <vector>
 
