@@ -539,9 +539,8 @@ def run_relative_accuracy(args):
         "results": rows}), flush=True)
 
 
-FP64_TFLOPS = 1.20   # FP64 FMA throughput of this part, measured with a dependent-free FMA loop
 DIGIT_TFLOPS = 1934.3 / 36   # the BF16 tensor rate over the 36 digit products of an FP64 multiply-add (slice_gemm.cu)
-FP32_TFLOPS = 67.9   # FP32 FMA throughput of this part, measured the same way
+FP32_TFLOPS = 67.9   # FP32 FMA throughput of this part, measured with a dependent-free FMA loop
 
 
 def run_adjoint(args):
