@@ -396,6 +396,33 @@ __device__ __forceinline__ void store(const Store& st, int row, int c, double v)
   else st.out[row * st.rs + c * st.cs] = v;
 }
 
+// sum_i (h_i + l_i)^2 over eight pairs of FP32 values, in FP64's range: the
+// squares are formed at the power of two that takes the largest |h_i| to
+// [1, 2), so that one below 2^-126 of the largest is all that underflows, and
+// summed as a pair.  (Squares in FP64 would cost four FP64 instructions an
+// entry, at two lanes a clock and SM; here half of one.)
+__device__ __forceinline__ double sum_squares(const float (&h)[8], const float (&l)[8]) {
+  int top = 0;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) top = max(top, __float_as_int(h[i]) & 0x7fffffff);
+  if (top == 0) return 0.0;
+  // two factors, because 2^149 leaves FP32's range (an infinity or a NaN stays one)
+  const int e = max(1, top >> 23) - 127, e1 = e / 2;
+  const float f1 = pow2f(-e1), f2 = pow2f(e1 - e);
+  float sh = 0.f, sl = 0.f;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const float x = h[i] * f1 * f2, y = l[i] * f1 * f2;
+    const float p = x * x, pe = fmaf(x, x, -p) + 2.f * x * y;
+    const float ns = sh + p, nb = ns - sh;
+    sl += ((sh - (ns - nb)) + (p - nb)) + pe;
+    sh = ns;
+  }
+  // an infinite square leaves inf - inf in the low part
+  const double s = isfinite(sh) ? to_f64(sh) + to_f64(sl) : to_f64(sh);
+  return s * __longlong_as_double((long long)(2 * e + 1023) << 52);
+}
+
 // 32 columns of this warp's TMEM lanes
 constexpr int kLd = 32;
 __device__ __forceinline__ void tmem_ld(uint32_t taddr, float (&v)[32]) {
@@ -591,7 +618,7 @@ __global__ void __launch_bounds__(kThreads, 1) slice_gemm_kernel(const __grid_co
     const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(ch * 64);
     uint32_t chunk = 0;
     bool ok = true;
-    float lsh = 0.f, lsl = 0.f;   // residual: ||R||^2 of this thread's entries in double-float
+    double loss = 0.0;            // residual: ||R||^2 of this thread's entries
     for (int it = blockIdx.x; ok && it < items; it += gridDim.x) {
       const Item w = item_of(P, it);
       const int row = w.tm * kT + r_tile, col0 = w.tn * kT + ch * 64;
@@ -720,10 +747,12 @@ __global__ void __launch_bounds__(kThreads, 1) slice_gemm_kernel(const __grid_co
                            : load_val((const __nv_bfloat16*)R.A + (long long)c * R.lda + row);
           }
           const int ey = j0 < 32 ? ey2[0] : ey2[1];
+          float rhi[8], rlo[8];
 #pragma unroll
           for (int jj = 0; jj < 8; ++jj) {
             const int c = col0 + j0 + jj;
             const int eyr = __shfl_sync(0xffffffffu, ey, (j0 + jj) & 31);
+            rhi[jj] = rlo[jj] = 0.f;
             if (!row_ok || c >= P.N) continue;
             const int e = ex + scale_exp(eyr, P.ydt);
             const int e1 = max(-126, min(127, e)), e2 = max(-126, min(127, e - e1));
@@ -736,11 +765,8 @@ __global__ void __launch_bounds__(kThreads, 1) slice_gemm_kernel(const __grid_co
             const float s = a - vh, bb = s - a;
             const float t = ((a - (s - bb)) + (-vh - bb)) - vl;
             const float rh = s + t, rl = t - (rh - s);
-            const float p = rh * rh;
-            const float pe = fmaf(rh, rh, -p) + 2.f * rh * rl;
-            const float ns = lsh + p, nb = ns - lsh;
-            lsl += ((lsh - (ns - nb)) + (p - nb)) + pe;
-            lsh = ns;
+            rhi[jj] = rh;
+            rlo[jj] = rl;
             if (R.R) R.R[(long long)c * P.M + row] = rh;
             if (R.dA) {
               float g;
@@ -754,13 +780,14 @@ __global__ void __launch_bounds__(kThreads, 1) slice_gemm_kernel(const __grid_co
               else ((__nv_bfloat16*)R.dA)[(long long)c * R.ldda + row] = __float2bfloat16_rn(g);
             }
           }
+          loss += sum_squares(rhi, rlo);
         }
       }
     }
     if constexpr (EP == kEpResidual) {
       // the CTA's share of ||R||^2, in a fixed order
       __shared__ double s_loss[kEpiWarps];
-      const double t = warp_sum(to_f64(lsh) + to_f64(lsl));
+      const double t = warp_sum(loss);
       if (lane == 0) s_loss[warp - 4] = t;
       asm volatile("bar.sync 1, 256;" ::: "memory");
       if (warp == 4 && lane == 0) {
