@@ -534,9 +534,8 @@ css_status css_autotune_distributed(const void* A, css_dtype dtype, int64_t m, i
  * column's squared norm (dependent columns in S) gives CSS_ERR_INVALID_ARG
  * (reported in sync mode), as do out-of-range or repeated indices.
  * Q^T A, Q W and R W^T are sums of exact products of 8-bit digits (what is
- * dropped is below 2^-64 of the rows' largest products; R W^T of FP32/BF16
- * input, whose R is held in FP32, keeps 2^-33); the factorisation and the
- * loss are FP64; dA is rounded once to the dtype of A.  k <= 1024.
+ * dropped is below 2^-64 of the rows' largest products; R of FP32/BF16 input
+ * is held in FP32); the factorisation and the loss are FP64; dA is rounded once to the dtype of A.  k <= 1024.
  */
 css_status css_residual_backward(const void* A, css_dtype dtype, int64_t m,
                                  int64_t n, int64_t lda, const int32_t* sel,

@@ -171,7 +171,7 @@ __device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) 
 // or a NaN get zero digits (the product restores them from the source).
 template <typename T, typename V, bool KC, bool VEC>
 __global__ void __launch_bounds__(256) split_kernel(const T* __restrict__ p, long long rs, long long ks, int rows,
-                                                    int K, int k64, int dtype, int slices,
+                                                    int K, int k64, int dtype,
                                                     const int* __restrict__ ex, unsigned char* __restrict__ d,
                                                     unsigned char* __restrict__ ns) {
   const int r0 = blockIdx.x * kT, kb = blockIdx.y;
@@ -213,10 +213,10 @@ __global__ void __launch_bounds__(256) split_kernel(const T* __restrict__ p, lon
     }
   }
   int s = 0;
-  for (; s < slices; ++s) {
+  for (; s < kS; ++s) {
     int any = 0;
     if constexpr (sizeof(V) == 4) {
-      const float least = 0.5f * pow2f(-8 * (slices - 1 - s));
+      const float least = 0.5f * pow2f(-8 * (kS - 1 - s));
 #pragma unroll
       for (int q = 0; q < 4; ++q)
 #pragma unroll
@@ -282,7 +282,6 @@ struct Args {
   int tn, tiles;       // tiles along N; tiles in all
   int lower;
   int ksplit, k16_per; // K slices and their 16-k blocks (a multiple of 4)
-  int halves;          // 2, or 1: the high digits alone
   Store st;
   Source sx, sy;
   long long* part;
@@ -486,7 +485,7 @@ __global__ void __launch_bounds__(kThreads, 1) slice_gemm_kernel(const __grid_co
     bool ok = true;
     for (int it = blockIdx.x; ok && it < items; it += gridDim.x) {
       const Item w = item_of(P, it);
-      for (int half = P.halves - 1; ok && half >= 0; --half) {
+      for (int half = 1; ok && half >= 0; --half) {
         const int kps = half ? 1 : 2, cap = half ? kS : 4;
         int cnt = 0;
         for (int k = w.k0; ok && k < w.k1; k += kps, ++st) {
@@ -551,7 +550,7 @@ __global__ void __launch_bounds__(kThreads, 1) slice_gemm_kernel(const __grid_co
     };
     for (int it = blockIdx.x; ok && it < items; it += gridDim.x) {
       const Item w = item_of(P, it);
-      for (int half = P.halves - 1; ok && half >= 0; --half) {
+      for (int half = 1; ok && half >= 0; --half) {
         const int kps = half ? 1 : 2, w0 = half ? 6 : 2;
         int used = 0, budget = 0, ready = 0;   // accumulators written, and waited for, in this chunk
         for (int k = w.k0; k < w.k1; k += kps, ++st) {
@@ -641,7 +640,7 @@ __global__ void __launch_bounds__(kThreads, 1) slice_gemm_kernel(const __grid_co
       // results are formed from there in short loops, because 64 unrolled
       // copies of that code do not stay in the instruction cache
       long long* mine = P.part + (long long)blockIdx.x * (2 * kT * kT) + (long long)(ch * 64) * kT + r_tile;
-      for (int half = P.halves - 1; ok && half >= 0; --half) {
+      for (int half = 1; ok && half >= 0; --half) {
         if constexpr (EP != kEpResidual) {
 #pragma unroll
           for (int j = 0; j < 64; ++j) acc[j] = 0;
@@ -701,14 +700,13 @@ __global__ void __launch_bounds__(kThreads, 1) slice_gemm_kernel(const __grid_co
       if (!ok) break;
       if constexpr (EP == kEpStore) {
         const int ex = scale_exp(exr, P.xdt);
-        const bool two = P.halves > 1;
 #pragma unroll 1
         for (int j0 = 0; j0 < 64; j0 += 8) {
           long long hv[8], lv[8];
 #pragma unroll
           for (int jj = 0; jj < 8; ++jj) {
             hv[jj] = __ldcg(mine + (long long)(j0 + jj) * kT);
-            lv[jj] = two ? __ldcg(mine + (long long)(kT + j0 + jj) * kT) : 0;
+            lv[jj] = __ldcg(mine + (long long)(kT + j0 + jj) * kT);
           }
           const int ey = j0 < 32 ? ey2[0] : ey2[1];
 #pragma unroll
@@ -823,22 +821,22 @@ __global__ void __launch_bounds__(256) finish_kernel(const __grid_constant__ Arg
 int k_blocks(long long K) { return (int)ceil_div(K, kKb); }
 
 template <typename T, typename V, bool KC, bool VEC>
-void launch_split(const Source& src, const Digits& D, int slices, cudaStream_t s) {
+void launch_split(const Source& src, const Digits& D, cudaStream_t s) {
   const int k64 = k_blocks(src.K);
   const unsigned tiles = (unsigned)ceil_div(src.rows, kT);
   const unsigned ky = (unsigned)std::min<long long>(k64, std::max<long long>(1, ceil_div(152 * 8, tiles)));
   row_exp_kernel<T, V, KC, VEC><<<dim3(tiles, ky), 256, 0, s>>>((const T*)src.p, src.rs, src.ks, src.rows, src.K,
                                                                 D.ex);
   split_kernel<T, V, KC, VEC><<<dim3(tiles, (unsigned)k64), 256, 0, s>>>((const T*)src.p, src.rs, src.ks, src.rows,
-                                                                        src.K, k64, src.dtype, slices, D.ex, D.d,
+                                                                        src.K, k64, src.dtype, D.ex, D.d,
                                                                         D.ns);
 }
 template <typename T, typename V>
-void launch_split_of(const Source& src, const Digits& D, int slices, cudaStream_t s) {
+void launch_split_of(const Source& src, const Digits& D, cudaStream_t s) {
   const bool vec = ((uintptr_t)src.p & 15u) == 0 && (src.rs * (long long)sizeof(T)) % 16 == 0;
-  if (src.ks == 1 && vec) launch_split<T, V, true, true>(src, D, slices, s);
-  else if (src.ks == 1) launch_split<T, V, true, false>(src, D, slices, s);
-  else launch_split<T, V, false, false>(src, D, slices, s);
+  if (src.ks == 1 && vec) launch_split<T, V, true, true>(src, D, s);
+  else if (src.ks == 1) launch_split<T, V, true, false>(src, D, s);
+  else launch_split<T, V, false, false>(src, D, s);
 }
 
 Args base_args(const Digits& X, const Digits& Y, int* err, unsigned long long spin_ns) {
@@ -859,7 +857,6 @@ Args base_args(const Digits& X, const Digits& Y, int* err, unsigned long long sp
   P.tn = (int)ceil_div(P.N, kT);
   P.tiles = (int)ceil_div(P.M, kT) * P.tn;
   P.ksplit = 1;
-  P.halves = 2;
   P.k16_per = P.k64 * 4;
   P.err = err;
   P.spin_ns = spin_ns;
@@ -892,16 +889,16 @@ Digits carve_digits(WsCarver& c, long long rows, long long K) {
   return D;
 }
 
-cudaError_t split(const Source& src, Digits& D, cudaStream_t s, Precision prec) {
+cudaError_t split(const Source& src, Digits& D, cudaStream_t s) {
   D.rows = src.rows;
   D.K = src.K;
   D.dtype = src.dtype;
   cudaError_t e = cudaMemsetAsync(D.ex, 0, sizeof(int) * (size_t)src.rows, s);
   if (e != cudaSuccess) return e;
   switch (src.dtype) {
-    case CSS_F64: launch_split_of<double, double>(src, D, prec, s); break;
-    case CSS_F32: launch_split_of<float, float>(src, D, prec, s); break;
-    default: launch_split_of<__nv_bfloat16, float>(src, D, prec, s); break;
+    case CSS_F64: launch_split_of<double, double>(src, D, s); break;
+    case CSS_F32: launch_split_of<float, float>(src, D, s); break;
+    default: launch_split_of<__nv_bfloat16, float>(src, D, s); break;
   }
   return cudaGetLastError();
 }
@@ -920,9 +917,8 @@ Scratch carve_scratch(WsCarver& c, size_t words) {
 }
 
 cudaError_t gemm(const Digits& X, const Source& sx, const Digits& Y, const Source& sy, const Store& st,
-                 const Scratch& w, int* err, unsigned long long spin_ns, cudaStream_t s, Precision prec) {
+                 const Scratch& w, int* err, unsigned long long spin_ns, cudaStream_t s) {
   Args P = base_args(X, Y, err, spin_ns);
-  P.halves = prec == kFull ? 2 : 1;
   P.st = st;
   P.sx = sx;
   P.sy = sy;

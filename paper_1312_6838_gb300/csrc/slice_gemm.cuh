@@ -23,17 +23,12 @@ struct Digits {
   int rows, K, dtype;
 };
 
-// Accuracy of a product: kFull keeps all eight slices (what is dropped is
-// below 2^-64 of the rows' largest products), kSingle four and the digit
-// products down to 2^-33, for results that are held in FP32.
-enum Precision { kFull = 8, kSingle = 4 };
-
 // Carves the digits of a rows x K operand (whole tiles of 128 rows) from a
 // workspace (rows may be the
 // largest of several operands that use the same space one after another).
 Digits carve_digits(WsCarver& c, long long rows, long long K);
 // Splits src into digits (src.rows <= the carved rows).  Three launches.
-cudaError_t split(const Source& src, Digits& D, cudaStream_t s, Precision prec = kFull);
+cudaError_t split(const Source& src, Digits& D, cudaStream_t s);
 
 // Scratch of gemm: per-CTA partial sums, and the integer sums of a product
 // whose inner dimension is cut into slices (taken when they fit).
@@ -57,7 +52,7 @@ struct Store {
   float* out32;
 };
 cudaError_t gemm(const Digits& X, const Source& sx, const Digits& Y, const Source& sy, const Store& st,
-                 const Scratch& w, int* err, unsigned long long spin_ns, cudaStream_t s, Precision prec = kFull);
+                 const Scratch& w, int* err, unsigned long long spin_ns, cudaStream_t s);
 
 // R = A - X Y^T for FP32 or BF16 A (M x N, leading dimension lda): writes R
 // (FP32, leading dimension M) when R != null, dA = g2 R when dA != null, and
