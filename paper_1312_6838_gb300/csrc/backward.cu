@@ -338,10 +338,10 @@ cudaError_t orth(const double* AS, int m, int k, double* Q, OrthSpace& w, unsign
   }
   const sg::Source a{AS, CSS_F64, m, 1, k, m}, ar{AS, CSS_F64, 1, m, m, k}, li{w.Linv, CSS_F64, 1, k, k, k};
   if ((e = sg::split(a, w.DS, s)) != cudaSuccess || (e = sg::split(ar, w.DSr, s)) != cudaSuccess) return e;
-  if ((e = sg::gemm(w.DS, a, w.DS, a, sg::Store{w.G, 1, k, 1}, w.sc, w.status + 1, spin_ns, s)) != cudaSuccess) return e;
+  if ((e = sg::gemm(w.DS, w.DS, sg::Store{w.G, 1, k, 1}, w.sc, w.status + 1, spin_ns, s)) != cudaSuccess) return e;
   chol_inv(w.G, k, w.Linv, w.gpart, w.status, s);
   if ((e = sg::split(li, w.DL, s)) != cudaSuccess) return e;
-  return sg::gemm(w.DSr, ar, w.DL, li, sg::Store{Q, 1, m, 0}, w.sc, w.status + 1, spin_ns, s);
+  return sg::gemm(w.DSr, w.DL, sg::Store{Q, 1, m, 0}, w.sc, w.status + 1, spin_ns, s);
 }
 
 // The call's status once its work is enqueued (opts->sync): [0] A_S is rank
@@ -383,7 +383,7 @@ cudaError_t w_product(const sg::Digits& DQ, const sg::Source& q, const void* A, 
     cudaError_t e = sg::split(a, DA, s);
     if (e != cudaSuccess) return e;
     const sg::Store st{W + c0 * wc, wc, wj, 0};
-    if ((e = sg::gemm(DA, a, DQ, q, st, sc, err, spin_ns, s)) != cudaSuccess) return e;
+    if ((e = sg::gemm(DA, DQ, st, sc, err, spin_ns, s, a, q)) != cudaSuccess) return e;
   }
   return cudaSuccess;
 }
@@ -494,7 +494,7 @@ css_status run_backward(const TA* A, int m, int n, long long lda, const int* sel
   int parts = kLossBlocks;
   if constexpr (dt == CSS_F64) {
     const sg::Store st{(double*)L.R, 1, m, 0};
-    if (sg::gemm(L.DQr, qr, L.DWr, wr, st, L.sc, err, spin, s) != cudaSuccess) return CSS_ERR_CUDA;
+    if (sg::gemm(L.DQr, L.DWr, st, L.sc, err, spin, s, qr, wr) != cudaSuccess) return CSS_ERR_CUDA;
     residual_f64_kernel<<<kLossBlocks, 256, 0, s>>>((const double*)A, lda, m, (long long)m * n, (double*)L.R,
                                                     (double*)dA, ldda, 2.0 * grad_out, L.loss_part);
   } else {
@@ -507,7 +507,7 @@ css_status run_backward(const TA* A, int m, int n, long long lda, const int* sel
     const sg::Source r{L.R, dt == CSS_F64 ? CSS_F64 : CSS_F32, 1, m, m, n};
     const sg::Store st{L.Psum, 1, m, 0};
     if (sg::split(r, L.DR, s) != cudaSuccess || sg::split(w, L.DW, s) != cudaSuccess ||
-        sg::gemm(L.DR, r, L.DW, w, st, L.scp, err, spin, s) != cudaSuccess)
+        sg::gemm(L.DR, L.DW, st, L.scp, err, spin, s) != cudaSuccess)
       return CSS_ERR_CUDA;
     das_kernel<TA><<<(unsigned)((mk + 255) / 256), 256, 0, s>>>(L.Psum, L.o.Linv, m, k, sel, 2.0 * grad_out, dA,
                                                                ldda);

@@ -3,6 +3,7 @@
 // digit products keep 2^-64 of the rows' largest products, so C and C A are
 // as accurate as FP64 sums.  Equal columns get equal bits (each entry is an
 // exact integer sum rounded once, and the columns' dots run in one order).
+// Infinities become NaN: the selection reports either as non-finite data.
 //
 // The FP64 tiles of init_simt.cu are bound by an SM's FP64 rate (two lanes a
 // clock), and a small problem has too few of them: 500 x 1000 took 1.63 ms
@@ -76,7 +77,7 @@ cudaError_t css_f0_f64(const double* A, long long lda, int m, int n, double* C, 
   Layout L = carve(c, m, n);
   const sg::Source rows{A, CSS_F64, 1, lda, m, n}, cs{C, CSS_F64, ldc, 1, m, m};
   cudaError_t e = sg::split(rows, L.rows, s);
-  if (e == cudaSuccess) e = sg::gemm(L.rows, rows, L.rows, rows, sg::Store{C, 1, ldc, 1}, L.sc, err, spin_ns, s);
+  if (e == cudaSuccess) e = sg::gemm(L.rows, L.rows, sg::Store{C, 1, ldc, 1}, L.sc, err, spin_ns, s);
   if (e == cudaSuccess) e = sg::split(cs, L.left, s);
   if (e != cudaSuccess) return e;
   const long long nb = chunk_cols(m, n);
@@ -84,7 +85,7 @@ cudaError_t css_f0_f64(const double* A, long long lda, int m, int n, double* C, 
     const int nc = (int)std::min<long long>(nb, n - c0);
     const sg::Source cols{A + c0 * lda, CSS_F64, lda, 1, nc, m};
     e = sg::split(cols, L.cols, s);
-    if (e == cudaSuccess) e = sg::gemm(L.left, cs, L.cols, cols, sg::Store{L.D, 1, m, 0}, L.sc, err, spin_ns, s);
+    if (e == cudaSuccess) e = sg::gemm(L.left, L.cols, sg::Store{L.D, 1, m, 0}, L.sc, err, spin_ns, s);
     if (e != cudaSuccess) return e;
     column_dots_kernel<<<(nc + 7) / 8, 256, 0, s>>>(L.D, A + c0 * lda, lda, m, nc, f + c0);
   }

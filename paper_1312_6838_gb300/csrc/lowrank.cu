@@ -547,7 +547,7 @@ extern "C" css_status css_lowrank(const double* W, int64_t ldw, const double* Q,
     DG = sg::carve_digits(c, l, n);
   }
   e = sg::split(w, DG, s);
-  if (e == cudaSuccess) e = sg::gemm(DG, w, DG, w, sg::Store{L.G0, 1, lp, 1}, L.sc, err, hs.spin_budget_ns, s);
+  if (e == cudaSuccess) e = sg::gemm(DG, DG, sg::Store{L.G0, 1, lp, 1}, L.sc, err, hs.spin_budget_ns, s);
   if (e != cudaSuccess) return CSS_ERR_CUDA;
   if (lp > l) pad_kernel<<<(lp + 255) / 256, 256, 0, s>>>(L.G0, l, lp);
   if (cudaGetLastError() != cudaSuccess) return CSS_ERR_CUDA;
@@ -586,7 +586,7 @@ extern "C" css_status css_lowrank(const double* W, int64_t ldw, const double* Q,
     const sg::Source q{Q + r0, CSS_F64, 1, ldq, (int)std::min<int64_t>(rows, m - r0), l};
     e = sg::split(q, DQ, s);
     if (e == cudaSuccess)
-      e = sg::gemm(DQ, q, L.DUw, us, sg::Store{U + r0, 1, ldu, 0}, L.sc, err, hs.spin_budget_ns, s);
+      e = sg::gemm(DQ, L.DUw, sg::Store{U + r0, 1, ldu, 0}, L.sc, err, hs.spin_budget_ns, s, q, us);
   }
   if (V && small_v && e == cudaSuccess) {
     small_product_kernel<<<dim3((unsigned)((n + 127) / 128), (k + 7) / 8), 128, 0, s>>>(W, ldw, n, l, k, uw, L.scale,
@@ -594,7 +594,7 @@ extern "C" css_status css_lowrank(const double* W, int64_t ldw, const double* Q,
   } else if (V && e == cudaSuccess) {
     e = sg::split(wr, L.DW, s);
     if (e == cudaSuccess)
-      e = sg::gemm(L.DW, wr, L.DUw, us, sg::Store{V, 1, ldv, 0, L.scale}, L.sc, err, hs.spin_budget_ns, s);
+      e = sg::gemm(L.DW, L.DUw, sg::Store{V, 1, ldv, 0, L.scale}, L.sc, err, hs.spin_budget_ns, s);
   }
   if (e != cudaSuccess) return CSS_ERR_CUDA;
   if (cudaGetLastError() != cudaSuccess) return CSS_ERR_CUDA;

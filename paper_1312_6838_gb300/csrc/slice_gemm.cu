@@ -58,12 +58,19 @@ constexpr int kBudget = 1024;           // digit products per accumulator betwee
 __host__ __device__ inline long long ceil_div(long long a, long long b) { return (a + b - 1) / b; }
 
 __host__ __device__ inline int exp_bias(int dtype) { return dtype == CSS_F64 ? 1023 : 127; }
-__host__ __device__ inline int exp_special(int dtype) { return dtype == CSS_F64 ? 2047 : 255; }
+// in the place of the largest exponent of a row that holds an infinity, a NaN
+constexpr int kExInf = 1 << 20, kExNan = 1 << 21;
 // entries of a row with largest biased exponent e are at most 2^(scale_exp - 1)
 __device__ __forceinline__ int scale_exp(int e, int dtype) { return e - exp_bias(dtype) + 2; }
 
-__device__ __forceinline__ int biased_exp(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
-__device__ __forceinline__ int biased_exp(float v) { return (__float_as_int(v) >> 23) & 0xff; }
+__device__ __forceinline__ int biased_exp(double v) {
+  const int h = __double2hiint(v), e = (h >> 20) & 0x7ff;
+  return e < 0x7ff ? e : (h & 0xfffff) | __double2loint(v) ? kExNan : kExInf;
+}
+__device__ __forceinline__ int biased_exp(float v) {
+  const int b = __float_as_int(v), e = (b >> 23) & 0xff;
+  return e < 0xff ? e : b & 0x7fffff ? kExNan : kExInf;
+}
 __device__ __forceinline__ float load_val(const float* p) { return __ldg(p); }
 __device__ __forceinline__ double load_val(const double* p) { return __ldg(p); }
 __device__ __forceinline__ float load_val(const __nv_bfloat16* p) {
@@ -168,7 +175,7 @@ __device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) 
 
 // Digits of one block of 128 rows x 64 k; slices are written until what is
 // left can give no digit, and their number goes to ns.  Rows with an infinity
-// or a NaN get zero digits (the product restores them from the source).
+// or a NaN get zero digits (see restore_kernel).
 template <typename T, typename V, bool KC, bool VEC>
 __global__ void __launch_bounds__(256) split_kernel(const T* __restrict__ p, long long rs, long long ks, int rows,
                                                     int K, int k64, int dtype,
@@ -186,7 +193,7 @@ __global__ void __launch_bounds__(256) split_kernel(const T* __restrict__ p, lon
     const int kc = KC ? (int)threadIdx.x % 8 : (int)threadIdx.x / 128 + 2 * q;
     out[q] = d + (((long long)blockIdx.x * k64 + kb) * 4 + kc / 2) * (kS * kSliceBytes) + (kc % 2) * (kT * 16) + rl * 16;
     const int e = r0 + rl < rows ? ex[r0 + rl] : 0;
-    const bool dead = e == exp_special(dtype);
+    const bool dead = e >= kExInf;
     if constexpr (sizeof(V) == 4) {
       // two factors, so that neither leaves FP32's range
       const int sh = 8 - scale_exp(e, dtype), h1 = sh / 2;
@@ -327,24 +334,30 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
+// Element (i, j) of the product as FP64 arithmetic gives it, by a warp.
 template <typename TX>
-__device__ double plain_dot_x(const Source& x, const Source& y, int i, int j) {
+__device__ double warp_dot_x(const Source& x, const Source& y, int i, int j) {
   const TX* p = (const TX*)x.p + i * x.rs;
+  const int lane = threadIdx.x & 31;
   double s = 0.0;
-  for (int k = 0; k < x.K; ++k) {
-    const long long o = j * y.rs + k * y.ks;
-    const double b = y.dtype == CSS_F64   ? ((const double*)y.p)[o]
-                     : y.dtype == CSS_F32 ? (double)((const float*)y.p)[o]
-                                          : (double)load_val((const __nv_bfloat16*)y.p + o);
-    s = fma((double)load_val(p + k * x.ks), b, s);
+  for (int k0 = 0; k0 < x.K; k0 += 1024) {
+    const int ke = min(x.K, k0 + 1024);
+#pragma unroll 4
+    for (int k = k0 + lane; k < ke; k += 32) {
+      const long long o = j * y.rs + k * y.ks;
+      const double b = y.dtype == CSS_F64   ? ((const double*)y.p)[o]
+                       : y.dtype == CSS_F32 ? (double)((const float*)y.p)[o]
+                                            : (double)load_val((const __nv_bfloat16*)y.p + o);
+      s = fma((double)load_val(p + k * x.ks), b, s);
+    }
+    if (__any_sync(0xffffffffu, isnan(s))) break;
   }
-  return s;
+  return warp_sum(s);
 }
-// A row with an infinity or a NaN: the product as FP64 arithmetic gives it.
-__device__ __noinline__ double plain_dot(const Source& x, const Source& y, int i, int j) {
-  if (x.dtype == CSS_F64) return plain_dot_x<double>(x, y, i, j);
-  if (x.dtype == CSS_F32) return plain_dot_x<float>(x, y, i, j);
-  return plain_dot_x<__nv_bfloat16>(x, y, i, j);
+__device__ double warp_dot(const Source& x, const Source& y, int i, int j) {
+  if (x.dtype == CSS_F64) return warp_dot_x<double>(x, y, i, j);
+  if (x.dtype == CSS_F32) return warp_dot_x<float>(x, y, i, j);
+  return warp_dot_x<__nv_bfloat16>(x, y, i, j);
 }
 
 // The result from its integer sums, (hi 2^32 + lo) 2^(e - 72), rounded once to
@@ -629,7 +642,6 @@ __global__ void __launch_bounds__(kThreads, 1) slice_gemm_kernel(const __grid_co
         for (int i = 0; i < 2; ++i)
           if (col0 + 32 * i + lane < P.N) ey2[i] = __ldg(P.ye + col0 + 32 * i + lane);
       }
-      const bool dead_r = exr == exp_special(P.xdt);
       long long acc[EP == kEpResidual ? 1 : 64];
       DF df[EP == kEpResidual ? 64 : 1];
       if constexpr (EP == kEpResidual) {
@@ -715,7 +727,7 @@ __global__ void __launch_bounds__(kThreads, 1) slice_gemm_kernel(const __grid_co
             const int eyr = __shfl_sync(0xffffffffu, ey, (j0 + jj) & 31);
             if (row >= P.M || c >= P.N) continue;
             double v = combine(hv[jj], lv[jj], ex + scale_exp(eyr, P.ydt));
-            if (dead_r || eyr == exp_special(P.ydt)) v = plain_dot(P.sx, P.sy, row, c);
+            if (max(exr, eyr) >= kExInf) v = __longlong_as_double(0x7fffffffffffffffll);
             store(P.st, row, c, v);
             if (P.lower && row != c) store(P.st, c, row, v);
           }
@@ -757,7 +769,7 @@ __global__ void __launch_bounds__(kThreads, 1) slice_gemm_kernel(const __grid_co
             const float f1 = pow2f(e1), f2 = pow2f(e2);
             float vh = pv[jj].x * f1 * f2;
             const float vl = pv[jj].y * f1 * f2;
-            if (dead_r || eyr == exp_special(P.ydt)) vh = __int_as_float(0x7fffffff);
+            if (max(exr, eyr) >= kExInf) vh = __int_as_float(0x7fffffff);
             const float a = av[jj];
             // r = a - vh - vl as a normalised pair
             const float s = a - vh, bb = s - a;
@@ -814,8 +826,36 @@ __global__ void __launch_bounds__(256) finish_kernel(const __grid_constant__ Arg
   const int exr = P.xe[row], eyr = P.ye[c];
   double v = combine((long long)P.sums[(long long)P.M * P.N + at], (long long)P.sums[at],
                      scale_exp(exr, P.xdt) + scale_exp(eyr, P.ydt));
-  if (exr == exp_special(P.xdt) || eyr == exp_special(P.ydt)) v = plain_dot(P.sx, P.sy, row, c);
+  if (max(exr, eyr) >= kExInf) v = __longlong_as_double(0x7fffffffffffffffll);
   store(P.st, row, c, v);
+}
+
+// A row (of X or Y) with an infinity or a NaN has no digits, and its results
+// were stored as NaN.  That is what they are beside a NaN; beside infinities
+// they depend on the signs and zeros they meet, so these are formed from the
+// sources, a warp an entry.  Most calls find nothing (3 us).  (Inside the
+// product, one thread walking K while the others' bounded waits ran, it ended
+// FP64 selections of 2304 x 16384 with an infinity in a timeout; called after
+// its loops it cost the kernel spills, css_embed of 4096 x 65536 2 %.)
+__global__ void __launch_bounds__(256) restore_kernel(const __grid_constant__ Args P) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int tn = (P.N + kT - 1) / kT, tiles = (P.M + kT - 1) / kT * tn;
+  for (int it = blockIdx.x; it < tiles; it += gridDim.x) {
+    const int r0 = it / tn * kT, c0 = it % tn * kT;
+    const int at = (threadIdx.x < kT ? r0 : c0) + threadIdx.x % kT;
+    const int ex = at >= (threadIdx.x < kT ? P.M : P.N) ? 0 : threadIdx.x < kT ? P.xe[at] : P.ye[at];
+    if (!__syncthreads_or(ex >= kExInf && ex < kExNan)) continue;
+    for (int row = r0 + warp; row < min(P.M, r0 + kT); row += 8) {
+      for (int cb = c0; cb < min(P.N, c0 + kT); cb += 32) {
+        const int e = cb + lane < P.N ? max(P.xe[row], P.ye[cb + lane]) : 0;
+        for (unsigned todo = __ballot_sync(0xffffffffu, e >= kExInf && e < kExNan); todo; todo &= todo - 1) {
+          const int c = cb + __ffs(todo) - 1;
+          const double v = warp_dot(P.sx, P.sy, row, c);
+          if (lane == 0) store(P.st, row, c, v);
+        }
+      }
+    }
+  }
 }
 
 int k_blocks(long long K) { return (int)ceil_div(K, kKb); }
@@ -871,6 +911,14 @@ cudaError_t launch_gemm(const Args& P, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+// (without sources the results beside infinities stay NaN)
+cudaError_t restore(const Args& P, cudaStream_t s) {
+  if (!P.sx.p || !P.sy.p) return cudaSuccess;
+  const long long tiles = ceil_div(P.M, kT) * ceil_div(P.N, kT);
+  restore_kernel<<<(unsigned)std::min<long long>(8 * kCtas, tiles), 256, 0, s>>>(P);
+  return cudaGetLastError();
+}
+
 // K slices for `tiles` result tiles: enough items for every SM, slices of at
 // least 256 k (a few drains each; below that the atomics of the sums show).
 int k_slices(long long tiles, long long K) {
@@ -916,8 +964,8 @@ Scratch carve_scratch(WsCarver& c, size_t words) {
   return w;
 }
 
-cudaError_t gemm(const Digits& X, const Source& sx, const Digits& Y, const Source& sy, const Store& st,
-                 const Scratch& w, int* err, unsigned long long spin_ns, cudaStream_t s) {
+cudaError_t gemm(const Digits& X, const Digits& Y, const Store& st, const Scratch& w, int* err,
+                 unsigned long long spin_ns, cudaStream_t s, const Source& sx, const Source& sy) {
   Args P = base_args(X, Y, err, spin_ns);
   P.st = st;
   P.sx = sx;
@@ -927,7 +975,10 @@ cudaError_t gemm(const Digits& X, const Source& sx, const Digits& Y, const Sourc
   if (st.lower) P.tiles = P.tn * (P.tn + 1) / 2;
   const size_t words = sum_words(P.M, P.N, P.K, P.lower);
   P.ksplit = words && words <= w.cap ? k_slices(P.tiles, P.K) : 1;
-  if (P.ksplit == 1) return launch_gemm<kEpStore>(P, s);
+  if (P.ksplit == 1) {
+    cudaError_t e = launch_gemm<kEpStore>(P, s);
+    return e == cudaSuccess ? restore(P, s) : e;
+  }
   P.sums = w.sums;
   P.k16_per = (int)ceil_div(ceil_div(P.k16, P.ksplit), 4) * 4;
   P.ksplit = (int)ceil_div(P.k16, P.k16_per);
@@ -936,7 +987,8 @@ cudaError_t gemm(const Digits& X, const Source& sx, const Digits& Y, const Sourc
   if (e != cudaSuccess) return e;
   if ((e = launch_gemm<kEpSplitK>(P, s)) != cudaSuccess) return e;
   finish_kernel<<<(unsigned)((mn + 255) / 256), 256, 0, s>>>(P);
-  return cudaGetLastError();
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  return restore(P, s);
 }
 
 int residual_parts() { return kCtas; }

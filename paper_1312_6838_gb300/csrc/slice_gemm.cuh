@@ -51,8 +51,11 @@ struct Store {
   const double* cscale;
   float* out32;
 };
-cudaError_t gemm(const Digits& X, const Source& sx, const Digits& Y, const Source& sy, const Store& st,
-                 const Scratch& w, int* err, unsigned long long spin_ns, cudaStream_t s);
+// Rows with an infinity or a NaN give NaN; with the operands' sources their
+// results beside infinities are as FP64 arithmetic gives them.
+cudaError_t gemm(const Digits& X, const Digits& Y, const Store& st, const Scratch& w, int* err,
+                 unsigned long long spin_ns, cudaStream_t s, const Source& sx = Source{},
+                 const Source& sy = Source{});
 
 // R = A - X Y^T for FP32 or BF16 A (M x N, leading dimension lda): writes R
 // (FP32, leading dimension M) when R != null, dA = g2 R when dA != null, and
