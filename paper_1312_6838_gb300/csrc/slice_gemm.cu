@@ -181,7 +181,9 @@ __global__ void __launch_bounds__(256) split_kernel(const T* __restrict__ p, lon
                                                     int K, int k64, int dtype,
                                                     const int* __restrict__ ex, unsigned char* __restrict__ d,
                                                     unsigned char* __restrict__ ns) {
-  const int r0 = blockIdx.x * kT, kb = blockIdx.y;
+  // (one grid dimension: K / 64 may exceed the others' 65535)
+  const unsigned tiles = (unsigned)(rows + kT - 1) / kT, tile = blockIdx.x % tiles;
+  const int r0 = (int)tile * kT, kb = (int)(blockIdx.x / tiles);
   V v[4][8];
   load_block<T, V, KC, VEC>(p, rs, ks, rows, K, r0, kb * kKb, v);
   unsigned char* out[4];
@@ -191,7 +193,7 @@ __global__ void __launch_bounds__(256) split_kernel(const T* __restrict__ p, lon
   for (int q = 0; q < 4; ++q) {
     const int rl = KC ? (int)threadIdx.x / 8 + 32 * q : (int)threadIdx.x % 128;
     const int kc = KC ? (int)threadIdx.x % 8 : (int)threadIdx.x / 128 + 2 * q;
-    out[q] = d + (((long long)blockIdx.x * k64 + kb) * 4 + kc / 2) * (kS * kSliceBytes) + (kc % 2) * (kT * 16) + rl * 16;
+    out[q] = d + (((long long)tile * k64 + kb) * 4 + kc / 2) * (kS * kSliceBytes) + (kc % 2) * (kT * 16) + rl * 16;
     const int e = r0 + rl < rows ? ex[r0 + rl] : 0;
     const bool dead = e >= kExInf;
     if constexpr (sizeof(V) == 4) {
@@ -262,7 +264,7 @@ __global__ void __launch_bounds__(256) split_kernel(const T* __restrict__ p, lon
       *reinterpret_cast<uint4*>(out[q] + s * kSliceBytes) = make_uint4(w[0], w[1], w[2], w[3]);
     }
   }
-  if (threadIdx.x == 0) ns[(long long)blockIdx.x * k64 + kb] = (unsigned char)s;
+  if (threadIdx.x == 0) ns[(long long)tile * k64 + kb] = (unsigned char)s;
 }
 
 // ------------------------------------------------------------- product -----
@@ -867,7 +869,7 @@ void launch_split(const Source& src, const Digits& D, cudaStream_t s) {
   const unsigned ky = (unsigned)std::min<long long>(k64, std::max<long long>(1, ceil_div(152 * 8, tiles)));
   row_exp_kernel<T, V, KC, VEC><<<dim3(tiles, ky), 256, 0, s>>>((const T*)src.p, src.rs, src.ks, src.rows, src.K,
                                                                 D.ex);
-  split_kernel<T, V, KC, VEC><<<dim3(tiles, (unsigned)k64), 256, 0, s>>>((const T*)src.p, src.rs, src.ks, src.rows,
+  split_kernel<T, V, KC, VEC><<<tiles * (unsigned)k64, 256, 0, s>>>((const T*)src.p, src.rs, src.ks, src.rows,
                                                                         src.K, k64, src.dtype, D.ex, D.d,
                                                                         D.ns);
 }
