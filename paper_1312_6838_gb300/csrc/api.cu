@@ -623,7 +623,7 @@ size_t css_workspace_size(css_op op, css_dtype dtype, int64_t m, int64_t n, int6
   if (op == CSS_OP_LOWRANK) {
     // m may be 0 here (U not requested); r is the embedding dimension l
     if (n <= 0 || n > (int64_t)INT32_MAX || r < 1 || r > 1024 || k < 1 || k > r) return 0;
-    return lowrank_workspace_bytes(n, (int32_t)r, k);
+    return lowrank_workspace_bytes(m, n, (int32_t)r, k);
   }
   if (!valid_dtype(dtype) || m <= 0 || n <= 0) return 0;
   switch (op) {

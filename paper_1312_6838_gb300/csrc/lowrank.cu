@@ -436,12 +436,14 @@ struct LrLayout {
   double2* rotlog;
   long long max_rounds;
   Estimate est;
-  sg::Digits DW, DUw;   // W (both ways, one after the other) or Q, and U^(W)_k
+  sg::Digits DG, DW, DUw;   // parts of W by rows, of W by columns or of Q (in one space), and U^(W)_k
+  long long part_k, part_rows;
   sg::Scratch sc;
   size_t bytes;
 };
 
-LrLayout lr_layout(void* ws, size_t cap, int64_t n, int32_t l, int32_t k) {
+// rows: of W^T and Q, as many as a part may take (at least n)
+LrLayout lr_layout(void* ws, size_t cap, int64_t rows, int64_t n, int32_t l, int32_t k) {
   WsCarver c(ws, cap);
   LrLayout L{};
   L.st = (DevStatus*)c.take<char>(kStatusBytes);   // first: css_read_status reads it
@@ -457,16 +459,16 @@ LrLayout lr_layout(void* ws, size_t cap, int64_t n, int32_t l, int32_t k) {
   L.Uw = c.take<double>((size_t)l * k);
   L.scale = c.take<double>(k);
   L.est = carve_estimate(c, l);
-  // the digits of W by rows, of W by columns and of Q (n rows at a time)
-  // share their space
+  L.part_k = std::min<long long>(n, sg::part_k(l));
+  L.part_rows = std::min<long long>((rows + 127) / 128 * 128, sg::part_rows(l));
   const size_t at = c.off;
-  sg::carve_digits(c, l, n);
+  L.DG = sg::carve_digits(c, l, L.part_k);
   const size_t end = c.off;
   c.off = at;
-  L.DW = sg::carve_digits(c, n, l);
+  L.DW = sg::carve_digits(c, L.part_rows, l);
   c.off = std::max(c.off, end);
   L.DUw = sg::carve_digits(c, k, l);
-  L.sc = sg::carve_scratch(c, sg::sum_words(l, l, n, 1));
+  L.sc = sg::carve_scratch(c, sg::sum_words(l, l, L.part_k, 1));
   L.bytes = c.off;
   return L;
 }
@@ -480,8 +482,8 @@ int device_sms() {
 
 }  // namespace
 
-size_t lowrank_workspace_bytes(int64_t n, int32_t l, int32_t k) {
-  return lr_layout(nullptr, (size_t)-1, n, l, k).bytes;
+size_t lowrank_workspace_bytes(int64_t m, int64_t n, int32_t l, int32_t k) {
+  return lr_layout(nullptr, (size_t)-1, std::max(m, n), n, l, k).bytes;
 }
 
 extern "C" css_status css_lowrank(const double* W, int64_t ldw, const double* Q, int64_t ldq, int64_t m,
@@ -496,7 +498,9 @@ extern "C" css_status css_lowrank(const double* W, int64_t ldw, const double* Q,
   if (U && (!Q || m < 1 || m > INT32_MAX || ldq < m || ldu < m)) return CSS_ERR_INVALID_ARG;
   if (V && ldv < n) return CSS_ERR_INVALID_ARG;
   if (!ws || ((uintptr_t)ws % kWsAlign) != 0) return CSS_ERR_WORKSPACE;
-  LrLayout L = lr_layout(ws, ws_bytes, n, l, k);
+  // (a workspace sized without U's rows takes them in parts of W's)
+  LrLayout L = lr_layout(ws, ws_bytes, U ? std::max(m, n) : n, n, l, k);
+  if (L.bytes > ws_bytes) L = lr_layout(ws, ws_bytes, n, n, l, k);
   if (L.bytes > ws_bytes) return CSS_ERR_WORKSPACE;
   int dev = 0, major = 0, minor = 0, coop = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return CSS_ERR_CUDA;
@@ -539,15 +543,12 @@ extern "C" css_status css_lowrank(const double* W, int64_t ldw, const double* Q,
   } guard{ev};
   if (timed) cudaEventRecord(ev[0], s);
   int* err = &L.st->code;
-  const sg::Source w{W, CSS_F64, ldw, 1, l, (int)n}, wr{W, CSS_F64, 1, ldw, (int)n, l};
-  sg::Digits DG = L.DW;
-  {
-    // (the same space, carved for l rows of n)
-    WsCarver c(L.DW.d, (size_t)-1);
-    DG = sg::carve_digits(c, l, n);
+  for (int64_t c0 = 0; e == cudaSuccess && c0 < n; c0 += L.part_k) {
+    const sg::Source w{W + c0, CSS_F64, ldw, 1, l, (int)std::min<int64_t>(L.part_k, n - c0)};
+    e = sg::split(w, L.DG, s);
+    if (e == cudaSuccess)
+      e = sg::gemm(L.DG, L.DG, sg::Store{L.G0, 1, lp, 1, nullptr, nullptr, c0 > 0}, L.sc, err, hs.spin_budget_ns, s);
   }
-  e = sg::split(w, DG, s);
-  if (e == cudaSuccess) e = sg::gemm(DG, DG, sg::Store{L.G0, 1, lp, 1}, L.sc, err, hs.spin_budget_ns, s);
   if (e != cudaSuccess) return CSS_ERR_CUDA;
   if (lp > l) pad_kernel<<<(lp + 255) / 256, 256, 0, s>>>(L.G0, l, lp);
   if (cudaGetLastError() != cudaSuccess) return CSS_ERR_CUDA;
@@ -573,28 +574,29 @@ extern "C" css_status css_lowrank(const double* W, int64_t ldw, const double* Q,
   order_kernel<<<1, 1024, 0, s>>>(L.G0, L.G1, L.info, l, lp, k, (long long)n, sigma, L.scale, tail, L.ord);
   replay_columns_kernel<<<k, (h + 31) / 32 * 32, 2 * lp * sizeof(double), s>>>(L.rotlog, L.info, L.ord, l, lp, X, uw);
   if (timed) cudaEventRecord(ev[2], s);
-  sg::Digits& DQ = L.DW;
   const sg::Source us{uw, CSS_F64, l, 1, k, l};
   const bool small_u = small_product(m, l, k), small_v = small_product(n, l, k);
   e = (U && !small_u) || (V && !small_v) ? sg::split(us, L.DUw, s) : cudaSuccess;
-  const int rows = ((int)n + 127) / 128 * 128;   // the digits' space holds whole tiles
   if (U && small_u) {
     small_product_kernel<<<dim3((unsigned)((m + 127) / 128), (k + 7) / 8), 128, 0, s>>>(Q, ldq, m, l, k, uw, nullptr,
                                                                                        U, ldu);
   }
-  for (int64_t r0 = 0; U && !small_u && e == cudaSuccess && r0 < m; r0 += rows) {
-    const sg::Source q{Q + r0, CSS_F64, 1, ldq, (int)std::min<int64_t>(rows, m - r0), l};
-    e = sg::split(q, DQ, s);
+  for (int64_t r0 = 0; U && !small_u && e == cudaSuccess && r0 < m; r0 += L.part_rows) {
+    const sg::Source q{Q + r0, CSS_F64, 1, ldq, (int)std::min<int64_t>(L.part_rows, m - r0), l};
+    e = sg::split(q, L.DW, s);
     if (e == cudaSuccess)
-      e = sg::gemm(DQ, L.DUw, sg::Store{U + r0, 1, ldu, 0}, L.sc, err, hs.spin_budget_ns, s, q, us);
+      e = sg::gemm(L.DW, L.DUw, sg::Store{U + r0, 1, ldu, 0}, L.sc, err, hs.spin_budget_ns, s, q, us);
   }
   if (V && small_v && e == cudaSuccess) {
     small_product_kernel<<<dim3((unsigned)((n + 127) / 128), (k + 7) / 8), 128, 0, s>>>(W, ldw, n, l, k, uw, L.scale,
                                                                                        V, ldv);
-  } else if (V && e == cudaSuccess) {
-    e = sg::split(wr, L.DW, s);
-    if (e == cudaSuccess)
-      e = sg::gemm(L.DW, L.DUw, sg::Store{V, 1, ldv, 0, L.scale}, L.sc, err, hs.spin_budget_ns, s);
+  } else {
+    for (int64_t r0 = 0; V && e == cudaSuccess && r0 < n; r0 += L.part_rows) {
+      const sg::Source wr{W + r0, CSS_F64, 1, ldw, (int)std::min<int64_t>(L.part_rows, n - r0), l};
+      e = sg::split(wr, L.DW, s);
+      if (e == cudaSuccess)
+        e = sg::gemm(L.DW, L.DUw, sg::Store{V + r0, 1, ldv, 0, L.scale}, L.sc, err, hs.spin_budget_ns, s);
+    }
   }
   if (e != cudaSuccess) return CSS_ERR_CUDA;
   if (cudaGetLastError() != cudaSuccess) return CSS_ERR_CUDA;

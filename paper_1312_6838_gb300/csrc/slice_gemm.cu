@@ -406,8 +406,12 @@ __device__ __forceinline__ double combine(long long hi, long long lo, int e) {
 
 __device__ __forceinline__ void store(const Store& st, int row, int c, double v) {
   if (st.cscale) v *= __ldg(st.cscale + c);
-  if (st.out32) st.out32[row * st.rs + c * st.cs] = (float)v;
-  else st.out[row * st.rs + c * st.cs] = v;
+  if (st.out32) {
+    st.out32[row * st.rs + c * st.cs] = (float)v;
+  } else {
+    double* p = st.out + row * st.rs + c * st.cs;
+    *p = st.add ? *p + v : v;
+  }
 }
 
 // sum_i (h_i + l_i)^2 over eight pairs of FP32 values, in FP64's range: the
@@ -731,7 +735,7 @@ __global__ void __launch_bounds__(kThreads, 1) slice_gemm_kernel(const __grid_co
             double v = combine(hv[jj], lv[jj], ex + scale_exp(eyr, P.ydt));
             if (max(exr, eyr) >= kExInf) v = __longlong_as_double(0x7fffffffffffffffll);
             store(P.st, row, c, v);
-            if (P.lower && row != c) store(P.st, c, row, v);
+            if (P.lower && w.tm != w.tn) store(P.st, c, row, v);
           }
         }
       }

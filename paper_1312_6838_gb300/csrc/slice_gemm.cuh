@@ -2,6 +2,8 @@
 // FP32 or BF16 matrices to FP64 accuracy on the BF16 tensor cores.
 #pragma once
 
+#include <algorithm>
+
 #include "css_common.cuh"
 
 namespace css {
@@ -27,6 +29,18 @@ struct Digits {
 // workspace (rows may be the
 // largest of several operands that use the same space one after another).
 Digits carve_digits(WsCarver& c, long long rows, long long K);
+// Digits take 16 bytes an entry of whole 128-row x 64-k blocks.  Operands of
+// more than this many bytes are formed a part at a time: by parts of the inner
+// dimension whose products are added (Store::add; this also keeps the integer
+// sums far inside 64 bits: K is at most 2^20 a part, and 2^25 fit), or by rows.
+constexpr long long kDigitBudget = 1280ll << 20;
+// Inner indices a part that `rows` rows allow, and rows that K allows.
+inline long long part_k(long long rows, long long budget = kDigitBudget) {
+  return std::max<long long>(64, budget / (2048 * ((rows + 127) / 128)) / 64 * 64);
+}
+inline long long part_rows(long long K, long long budget = kDigitBudget) {
+  return std::max<long long>(128, budget / (1024 * ((K + 63) / 64)) / 128 * 128);
+}
 // Splits src into digits (src.rows <= the carved rows).  Three launches.
 cudaError_t split(const Source& src, Digits& D, cudaStream_t s);
 
@@ -43,13 +57,15 @@ Scratch carve_scratch(WsCarver& c, size_t words);
 
 // out[i * rs + j * cs] = cscale[j] sum_k X[i, k] Y[j, k] (FP64, or FP32 to
 // out32; cscale may be null).  lower: X and Y are the same operand; only tiles
-// touching i >= j are computed and both triangles written.
+// touching i >= j are computed and both triangles written.  add: out += that
+// (FP64 only).
 struct Store {
   double* out;
   long long rs, cs;
   int lower;
   const double* cscale;
   float* out32;
+  int add;
 };
 // Rows with an infinity or a NaN give NaN; with the operands' sources their
 // results beside infinities are as FP64 arithmetic gives them.

@@ -1,5 +1,6 @@
 """Products from digits whose inner dimension is beyond a grid's 65535 blocks
-of 64 (4,194,240): the embedding and the residual of tall matrices, the Gram
+of 64 (4,194,240) and beyond what one 64-bit sum holds (2^25 products of the
+largest digits): the embedding and the residual of tall matrices, the Gram
 matrix of long rows, FP64 selections of few rows."""
 import numpy as np
 import pytest
@@ -27,6 +28,35 @@ def test_lowrank_of_long_rows(l, n):
     assert float(err) <= 1e-10
     rec = (r.Uw * r.sigma) @ r.V.t()
     assert float((rec - W).abs().max()) <= 1e-9
+
+
+def test_gram_of_equal_digits():
+    """2^26 products of the largest digit: 2^26 * 2^-6 is the exact sum."""
+    from paper_1312_6838_gb300 import css
+    W = torch.full((1, 1 << 26), 0.125, dtype=torch.float64, device="cuda")
+    assert float(css.lowrank(W, 1, want_V=False).sigma[0]) == 2.0 ** 10
+
+
+def test_lowrank_with_more_rows_of_q_than_columns():
+    """U~ = Q U^(W) takes Q in parts; a workspace sized without Q's rows (m = 0)
+    takes smaller ones, with the same result."""
+    import ctypes as C
+
+    from paper_1312_6838_gb300 import _lib as L, css
+    l, n, m, k = 70, 300, 200001, 70
+    W, Q = _randn(l, n, seed=1), _randn(l, m, seed=2).t()
+    r = css.lowrank(W, k, Q)
+    assert float((r.U - Q @ r.Uw).abs().max()) <= 4 * l * U * float(Q.abs().max()) * l ** 0.5
+    lib, o = L.load(), L.default_opts()
+    size = lib.css_workspace_size(L.CSS_OP_LOWRANK, L.CSS_F64, 0, n, l, k, 0, C.byref(o))
+    ws = torch.empty(size + 256, dtype=torch.uint8, device="cuda")
+    U2 = torch.empty((k, m), dtype=torch.float64, device="cuda").t()
+    sig = torch.empty(k, dtype=torch.float64, device="cuda")
+    p = lambda t: C.c_void_p(t.data_ptr())
+    code = lib.css_lowrank(p(W), n, p(Q), m, m, n, l, k, p(sig), p(U2), m, C.c_void_p(0), n, C.c_void_p(0),
+                           C.c_void_p(0), C.c_void_p((ws.data_ptr() + 255) // 256 * 256), size, C.byref(o),
+                           C.c_void_p(torch.cuda.current_stream().cuda_stream))
+    assert code == 0 and torch.equal(U2, r.U)
 
 
 @pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
