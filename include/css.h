@@ -530,7 +530,8 @@ css_status css_autotune_distributed(const void* A, css_dtype dtype, int64_t m, i
  *   dA        DEVICE, same dtype as A, m x n with leading dimension ldda, or
  *             NULL to compute the loss only.
  *   loss      DEVICE double[1] or NULL.
- * The k x k factor of A_S^T A_S is recomputed here (FP64 Cholesky); a pivot at or below 1e-12 of its
+ * The k x k factor of A_S^T A_S is recomputed here (FP64 Cholesky), not
+ * carried over from a forward pass; a pivot at or below 1e-12 of its
  * column's squared norm (dependent columns in S) gives CSS_ERR_INVALID_ARG
  * (reported in sync mode), as do out-of-range or repeated indices.
  * Q^T A, Q W and R W^T are sums of exact products of 8-bit digits (what is
@@ -543,25 +544,6 @@ css_status css_residual_backward(const void* A, css_dtype dtype, int64_t m,
                                  int64_t ldda, double* loss, void* ws,
                                  size_t ws_bytes, const css_opts* opts,
                                  css_stream_t stream);
-
-/*
- * css_residual_backward that leaves its factors with the caller, so that the
- * gradient at the same A and S needs not form them again.
- *
- *   factors   DEVICE double[k * (m + n + k)] or NULL: Q (m x k), then W = Q^T A
- *             (k x n), then the inverse of the Cholesky factor (k x k), all
- *             column-major.  formed = 0: written; formed != 0: read, as an
- *             earlier call with formed = 0 for the same A and S wrote them.
- */
-css_status css_residual_backward_factors(const void* A, css_dtype dtype,
-                                         int64_t m, int64_t n, int64_t lda,
-                                         const int32_t* sel, int32_t k,
-                                         double grad_out, void* dA,
-                                         int64_t ldda, double* loss,
-                                         double* factors, int32_t formed,
-                                         void* ws, size_t ws_bytes,
-                                         const css_opts* opts,
-                                         css_stream_t stream);
 
 /*
  * Embedding into the span of a selection (Sec. 3.2, Eq. CSS_LowDim):

@@ -128,8 +128,6 @@ _SIGS = {
                           C.POINTER(css_opts), P]),
     "css_residual_backward": (I32, [P, I32, I64, I64, I64, P, I32, DBL, P, I64, P, P, SZ,
                                     C.POINTER(css_opts), P]),
-    "css_residual_backward_factors": (I32, [P, I32, I64, I64, I64, P, I32, DBL, P, I64, P, P, I32, P, SZ,
-                                            C.POINTER(css_opts), P]),
     "css_select_host": (I32, [P, I32, I64, I64, I64, I32, P, P, P, P, P, SZ,
                               C.POINTER(css_opts), P]),
     "css_read_status": (I32, [P, P]),

@@ -8,8 +8,8 @@
 //   dL/dA = 2 R  (columns outside S),  dL/dA_S = -2 R T^T
 //
 // With the Cholesky factor A_S^T A_S = L L^T in FP64 and Q = A_S L^-T
-// (orthonormal; Q, W and L^-1 are formed here unless the caller hands back those
-// of its own forward call):
+// (orthonormal; formed anew by each call, so that nothing of a forward pass is
+// kept for the gradient):
 //   W = Q^T A,  R = A - Q W,  T = L^-T W,  R T^T = (R W^T) L^-1.
 // R is a small difference of large terms (the part of A outside span(A_S)),
 // so W, Q W and R W^T are sums of exact digit products on the slice GEMM
@@ -476,7 +476,7 @@ BwLayout bw_layout(void* ws, size_t cap, int dt, int64_t m, int64_t n, int32_t k
 template <typename TA>
 css_status run_backward(const TA* A, int m, int n, long long lda, const int* sel, int k,
                         double grad_out, TA* dA, long long ldda, double* loss, BwLayout& L,
-                        bool formed, const css_opts& o, cudaStream_t s) {
+                        const css_opts& o, cudaStream_t s) {
   constexpr int dt = sizeof(TA) == 8 ? CSS_F64 : sizeof(TA) == 4 ? CSS_F32 : CSS_BF16;
   const unsigned long long spin = o.spin_budget_ns ? o.spin_budget_ns : 2000000000ull;
   cudaMemsetAsync(L.status, 0, 2 * sizeof(int), s);
@@ -484,12 +484,10 @@ css_status run_backward(const TA* A, int m, int n, long long lda, const int* sel
   const long long mk = (long long)m * k;
   const sg::Source q{L.Q, CSS_F64, m, 1, k, m}, qr{L.Q, CSS_F64, 1, m, m, k};
   const sg::Source w{L.W, CSS_F64, 1, k, k, n}, wr{L.W, CSS_F64, k, 1, n, k};
-  if (!formed) {
-    gather_cols_kernel<TA><<<(unsigned)((mk + 255) / 256), 256, 0, s>>>(A, lda, m, sel, k, L.AS);
-    if (orth(L.AS, m, k, L.Q, L.o, spin, s) != cudaSuccess || sg::split(q, L.DQ, s) != cudaSuccess ||
-        w_product(L.DQ, q, A, dt, lda, m, n, k, L.W, 1, k, L.DA, L.sc, err, spin, s) != cudaSuccess)
-      return CSS_ERR_CUDA;
-  }
+  gather_cols_kernel<TA><<<(unsigned)((mk + 255) / 256), 256, 0, s>>>(A, lda, m, sel, k, L.AS);
+  if (orth(L.AS, m, k, L.Q, L.o, spin, s) != cudaSuccess || sg::split(q, L.DQ, s) != cudaSuccess ||
+      w_product(L.DQ, q, A, dt, lda, m, n, k, L.W, 1, k, L.DA, L.sc, err, spin, s) != cudaSuccess)
+    return CSS_ERR_CUDA;
   if (sg::split(qr, L.DQr, s) != cudaSuccess || sg::split(wr, L.DWr, s) != cudaSuccess) return CSS_ERR_CUDA;
   int parts = kLossBlocks;
   if constexpr (dt == CSS_F64) {
@@ -630,18 +628,15 @@ size_t backward_workspace_bytes(int dtype, int64_t m, int64_t n, int32_t k) {
   return bw_layout(nullptr, (size_t)-1, dtype, m, n, k, true).bytes;
 }
 
-// factors (Q, W, L^-1) stay with the caller between the forward and the
-// gradient call: at 4096 x 16384, k = 128 (FP32) forming them is 0.95 of a
-// call's 2 ms, forward and backward 4.97 -> 3.94 ms.
-extern "C" css_status css_residual_backward_factors(const void* A, css_dtype dtype, int64_t m, int64_t n,
-                                                    int64_t lda, const int32_t* sel, int32_t k, double grad_out,
-                                                    void* dA, int64_t ldda, double* loss, double* factors,
-                                                    int32_t formed, void* ws, size_t ws_bytes,
-                                                    const css_opts* opts, css_stream_t stream) {
+extern "C" css_status css_residual_backward(const void* A, css_dtype dtype, int64_t m, int64_t n,
+                                            int64_t lda, const int32_t* sel, int32_t k,
+                                            double grad_out, void* dA, int64_t ldda, double* loss,
+                                            void* ws, size_t ws_bytes, const css_opts* opts,
+                                            css_stream_t stream) {
   css_opts o;
   css_opts_default(&o);
   if (opts) o = *opts;
-  if (!A || !sel || (!dA && !loss) || (formed && !factors)) return CSS_ERR_INVALID_ARG;
+  if (!A || !sel || (!dA && !loss)) return CSS_ERR_INVALID_ARG;
   if (dtype != CSS_F64 && dtype != CSS_F32 && dtype != CSS_BF16) return CSS_ERR_INVALID_ARG;
   if (m < 1 || n < 1 || lda < m || k < 1 || k > 1024 || k > m || k > n) return CSS_ERR_INVALID_ARG;
   if (dA && ldda < m) return CSS_ERR_INVALID_ARG;
@@ -649,11 +644,6 @@ extern "C" css_status css_residual_backward_factors(const void* A, css_dtype dty
   if (!ws || ((uintptr_t)ws % kWsAlign) != 0) return CSS_ERR_WORKSPACE;
   BwLayout L = bw_layout(ws, ws_bytes, dtype, m, n, k, dA != nullptr);
   if (L.bytes > ws_bytes) return CSS_ERR_WORKSPACE;
-  if (factors) {
-    L.Q = factors;
-    L.W = L.Q + (size_t)m * k;
-    L.o.Linv = L.W + (size_t)k * n;
-  }
   // the selected indices: in range and distinct (a small stream-ordered copy)
   cudaStream_t s = (cudaStream_t)stream;
   const css_status cs = check_selection(sel, k, n, s);
@@ -661,21 +651,12 @@ extern "C" css_status css_residual_backward_factors(const void* A, css_dtype dty
   switch (dtype) {
     case CSS_F64:
       return run_backward<double>((const double*)A, (int)m, (int)n, lda, sel, k, grad_out,
-                                  (double*)dA, ldda, loss, L, formed != 0, o, s);
+                                  (double*)dA, ldda, loss, L, o, s);
     case CSS_F32:
       return run_backward<float>((const float*)A, (int)m, (int)n, lda, sel, k, grad_out,
-                                 (float*)dA, ldda, loss, L, formed != 0, o, s);
+                                 (float*)dA, ldda, loss, L, o, s);
     default:
       return run_backward<__nv_bfloat16>((const __nv_bfloat16*)A, (int)m, (int)n, lda, sel, k,
-                                         grad_out, (__nv_bfloat16*)dA, ldda, loss, L, formed != 0, o, s);
+                                         grad_out, (__nv_bfloat16*)dA, ldda, loss, L, o, s);
   }
-}
-
-extern "C" css_status css_residual_backward(const void* A, css_dtype dtype, int64_t m, int64_t n,
-                                            int64_t lda, const int32_t* sel, int32_t k,
-                                            double grad_out, void* dA, int64_t ldda, double* loss,
-                                            void* ws, size_t ws_bytes, const css_opts* opts,
-                                            css_stream_t stream) {
-  return css_residual_backward_factors(A, dtype, m, n, lda, sel, k, grad_out, dA, ldda, loss, nullptr, 0, ws, ws_bytes,
-                                       opts, stream);
 }

@@ -672,20 +672,16 @@ class _Residual(torch.autograd.Function):
         k = int(sel.numel())
         nbytes = lib.css_workspace_size(L.CSS_OP_BACKWARD, dt, m, n, 0, k, 0, C.byref(o))
         _keep, ws = _workspace(nbytes, A.device)
-        # Q, W = Q^T A and L^-1, which the gradient needs again
-        factors = None
-        if ctx.needs_input_grad[0]:
-            factors = torch.empty(k * (m + n + k), dtype=torch.float64, device=A.device)
-        code = lib.css_residual_backward_factors(_ptr(A), dt, m, n, lda, _ptr(sel), k, 1.0,
-                                                 C.c_void_p(0), 0, _ptr(loss), _ptr(factors), 0, _ptr(ws),
-                                                 nbytes, C.byref(o), _stream(None))
+        code = lib.css_residual_backward(_ptr(A), dt, m, n, lda, _ptr(sel), k, 1.0,
+                                         C.c_void_p(0), 0, _ptr(loss), _ptr(ws), nbytes,
+                                         C.byref(o), _stream(None))
         _check(code, "css_residual_backward(loss)")
-        ctx.save_for_backward(A, sel, factors)
+        ctx.save_for_backward(A, sel)
         return loss[0].to(A.dtype if A.dtype != torch.bfloat16 else torch.float32)
 
     @staticmethod
     def backward(ctx, grad):
-        A, sel, factors = ctx.saved_tensors
+        A, sel = ctx.saved_tensors
         m, n, lda = _colmajor(A)
         dt = _DT[A.dtype]
         lib = L.load()
@@ -695,10 +691,9 @@ class _Residual(torch.autograd.Function):
         k = int(sel.numel())
         nbytes = lib.css_workspace_size(L.CSS_OP_BACKWARD, dt, m, n, 0, k, 0, C.byref(o))
         _keep, ws = _workspace(nbytes, A.device)
-        code = lib.css_residual_backward_factors(_ptr(A), dt, m, n, lda, _ptr(sel), k, float(grad.item()),
-                                                 _ptr(dA), ldd, C.c_void_p(0), _ptr(factors),
-                                                 int(factors is not None), _ptr(ws), nbytes,
-                                                 C.byref(o), _stream(None))
+        code = lib.css_residual_backward(_ptr(A), dt, m, n, lda, _ptr(sel), k, float(grad.item()),
+                                         _ptr(dA), ldd, C.c_void_p(0), _ptr(ws), nbytes,
+                                         C.byref(o), _stream(None))
         _check(code, "css_residual_backward")
         return dA, None
 
