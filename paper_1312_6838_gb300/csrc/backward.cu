@@ -308,7 +308,8 @@ constexpr int kSliceK = 128;
 // A_S's orthonormal basis by Cholesky: G = A_S^T A_S = L L^T, Q = A_S L^-T.
 struct OrthSpace {
   double *G, *gpart, *Linv;
-  sg::Digits DS, DSr, DL;   // A_S both ways, L^-1
+  sg::Digits DS, DSr, DL;   // parts of A_S both ways (in one space), L^-1
+  long long part_k, part_rows;
   sg::Scratch sc;
   int* status;              // [0] rank deficient, [1] error of the products
 };
@@ -318,13 +319,20 @@ OrthSpace carve_orth(WsCarver& c, int* status, long long m, int k) {
   w.G = c.take<double>((size_t)k * k);
   w.gpart = c.take<double>(gram_part_doubles((int)m, k));
   w.Linv = c.take<double>((size_t)k * k);
-  if (k > kSliceK) {
-    w.DS = sg::carve_digits(c, k, m);
-    w.DSr = sg::carve_digits(c, m, k);
-    w.DL = sg::carve_digits(c, k, k);
-    w.sc = sg::carve_scratch(c, std::max(sg::sum_words(k, k, m, 1), sg::sum_words(m, k, k, 0)));
-  }
   return w;
+}
+void carve_orth_digits(WsCarver& c, long long m, int k, OrthSpace& w) {
+  if (k <= kSliceK) return;
+  w.part_k = std::min<long long>(m, sg::part_k(k));
+  w.part_rows = std::min<long long>((m + 127) / 128 * 128, sg::part_rows(k));
+  const size_t at = c.off;
+  w.DS = sg::carve_digits(c, k, w.part_k);
+  const size_t end = c.off;
+  c.off = at;
+  w.DSr = sg::carve_digits(c, w.part_rows, k);
+  c.off = std::max(c.off, end);
+  w.DL = sg::carve_digits(c, k, k);
+  w.sc = sg::carve_scratch(c, std::max(sg::sum_words(k, k, w.part_k, 1), sg::sum_words(w.part_rows, k, k, 0)));
 }
 cudaError_t orth(const double* AS, int m, int k, double* Q, OrthSpace& w, unsigned long long spin_ns,
                  cudaStream_t s) {
@@ -336,12 +344,21 @@ cudaError_t orth(const double* AS, int m, int k, double* Q, OrthSpace& w, unsign
     q_kernel<<<(unsigned)((mk + 255) / 256), 256, 0, s>>>(AS, w.Linv, m, k, Q);
     return cudaGetLastError();
   }
-  const sg::Source a{AS, CSS_F64, m, 1, k, m}, ar{AS, CSS_F64, 1, m, m, k}, li{w.Linv, CSS_F64, 1, k, k, k};
-  if ((e = sg::split(a, w.DS, s)) != cudaSuccess || (e = sg::split(ar, w.DSr, s)) != cudaSuccess) return e;
-  if ((e = sg::gemm(w.DS, w.DS, sg::Store{w.G, 1, k, 1}, w.sc, w.status + 1, spin_ns, s)) != cudaSuccess) return e;
+  for (long long r0 = 0; r0 < m; r0 += w.part_k) {
+    const sg::Source a{AS + r0, CSS_F64, m, 1, k, (int)std::min(w.part_k, m - r0)};
+    if ((e = sg::split(a, w.DS, s)) != cudaSuccess) return e;
+    const sg::Store st{w.G, 1, k, 1, nullptr, nullptr, r0 > 0};
+    if ((e = sg::gemm(w.DS, w.DS, st, w.sc, w.status + 1, spin_ns, s)) != cudaSuccess) return e;
+  }
   chol_inv(w.G, k, w.Linv, w.gpart, w.status, s);
+  const sg::Source li{w.Linv, CSS_F64, 1, k, k, k};
   if ((e = sg::split(li, w.DL, s)) != cudaSuccess) return e;
-  return sg::gemm(w.DSr, w.DL, sg::Store{Q, 1, m, 0}, w.sc, w.status + 1, spin_ns, s);
+  for (long long r0 = 0; r0 < m; r0 += w.part_rows) {
+    const sg::Source ar{AS + r0, CSS_F64, 1, m, (int)std::min(w.part_rows, m - r0), k};
+    if ((e = sg::split(ar, w.DSr, s)) != cudaSuccess) return e;
+    if ((e = sg::gemm(w.DSr, w.DL, sg::Store{Q + r0, 1, m, 0}, w.sc, w.status + 1, spin_ns, s)) != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 // The call's status once its work is enqueued (opts->sync): [0] A_S is rank
@@ -357,39 +374,49 @@ css_status finish(const int* status, const css_opts& o, cudaStream_t s) {
 }
 
 // -------------------------------------------------- products in digits -----
-// W = Q^T A, R = A - Q W and P = R W^T run on the slice GEMM (slice_gemm.cu).
-// W's operand A is split a range of columns at a time, which bounds the
-// workspace: as many tiles of 128 columns as 1.25 GB of digits hold, cut to a
-// whole number of rounds over the 152 SMs.
-constexpr long long kDigitBudget = 1280ll << 20;
+// W = Q^T A, R = A - Q W and P = R W^T run on the slice GEMM (slice_gemm.cu),
+// a range of columns of A at a time, which bounds the workspace: as many tiles
+// of 128 columns as kDigitBudget of A's digits hold, cut to a whole number of
+// rounds over the 152 SMs.  Where not even one tile's do (m above 655360) the
+// rows are taken in parts as well.
 constexpr int kRound = 152;
+
+// Rows a part of W = Q^T A.
+long long w_rows(long long m, int k) { return std::min(m, sg::part_k(std::max(k, 128))); }
 
 long long chunk_cols(long long m, long long n, int k) {
   const long long tiles = (n + 127) / 128, tn = (k + 127) / 128;
-  const long long per_tile = 128 * 16 * ((m + 63) / 64 * 64);
-  long long c = std::max<long long>(1, kDigitBudget / per_tile);
+  const long long per_tile = 128 * 16 * ((w_rows(m, k) + 63) / 64 * 64);
+  long long c = std::max<long long>(1, sg::kDigitBudget / per_tile);
   if (c * tn > kRound) c = c * tn / kRound * kRound / tn;
   return std::min(c, tiles) * 128;
 }
 
-// W = Q^T A: element (j, c) to W[j * wj + c * wc].  Q's digits are in DQ.
-cudaError_t w_product(const sg::Digits& DQ, const sg::Source& q, const void* A, int dtype, long long lda, int m, int n,
-                      int k, double* W, long long wj, long long wc, sg::Digits& DA, const sg::Scratch& sc, int* err,
-                      unsigned long long spin_ns, cudaStream_t s) {
-  const long long cols = chunk_cols(m, n, k);
+// W = Q^T A: element (j, c) to W[j * wj + c * wc].  DQ: whether the digits of
+// the whole of Q are already there.
+cudaError_t w_product(const double* Q, const void* A, int dtype, long long lda, int m, int n, int k, double* W,
+                      long long wj, long long wc, sg::Digits& DQ, bool have_q, sg::Digits& DA, const sg::Scratch& sc,
+                      int* err, unsigned long long spin_ns, cudaStream_t s) {
+  const long long cols = chunk_cols(m, n, k), rows = w_rows(m, k);
   const long long esz = dtype == CSS_F64 ? 8 : dtype == CSS_F32 ? 4 : 2;
   for (long long c0 = 0; c0 < n; c0 += cols) {
-    const sg::Source a{(const char*)A + c0 * lda * esz, dtype, lda, 1, (int)std::min(cols, n - c0), m};
-    cudaError_t e = sg::split(a, DA, s);
-    if (e != cudaSuccess) return e;
-    const sg::Store st{W + c0 * wc, wc, wj, 0};
-    if ((e = sg::gemm(DA, DQ, st, sc, err, spin_ns, s, a, q)) != cudaSuccess) return e;
+    for (long long r0 = 0; r0 < m; r0 += rows) {
+      const int mm = (int)std::min(rows, m - r0);
+      const sg::Source q{Q + r0, CSS_F64, m, 1, k, mm};
+      const sg::Source a{(const char*)A + (c0 * lda + r0) * esz, dtype, lda, 1, (int)std::min(cols, n - c0), mm};
+      cudaError_t e = cudaSuccess;
+      if (rows < m || (c0 == 0 && !have_q)) e = sg::split(q, DQ, s);
+      if (e == cudaSuccess) e = sg::split(a, DA, s);
+      if (e != cudaSuccess) return e;
+      const sg::Store st{W + c0 * wc, wc, wj, 0, nullptr, nullptr, r0 > 0};
+      if ((e = sg::gemm(DA, DQ, st, sc, err, spin_ns, s, a, q)) != cudaSuccess) return e;
+    }
   }
   return cudaSuccess;
 }
 
 // FP64 input: V = Q W on entry, R = A - V on return (in place), dA = g2 R when
-// dA != null, and one partial of ||R||^2 per block.
+// dA != null, and each block's share of ||R||^2 added to its partial sum.
 constexpr int kLossBlocks = 152 * 8;
 __global__ void __launch_bounds__(256) residual_f64_kernel(const double* __restrict__ A, long long lda, int m,
                                                            long long mn, double* __restrict__ R,
@@ -405,7 +432,7 @@ __global__ void __launch_bounds__(256) residual_f64_kernel(const double* __restr
     sq = fma(r, r, sq);
   }
   sq = block_sum(sq, red);
-  if (threadIdx.x == 0) loss_part[blockIdx.x] = sq;
+  if (threadIdx.x == 0) loss_part[blockIdx.x] += sq;
 }
 
 __global__ void sum_kernel(const double* __restrict__ part, long long cnt, double scale,
@@ -431,13 +458,13 @@ __global__ void das_kernel(const double* __restrict__ P, const double* __restric
 
 struct BwLayout {
   int* status;   // [0] A_S is rank deficient, [1] error of the products
-  double *AS, *Q, *W;
+  double *AS, *Q, *Psum, *loss_part;
   OrthSpace o;
-  void* R;       // residual: FP32, FP64 for FP64 input
-  double* Psum;
-  double* loss_part;
-  sg::Digits DQ, DQr, DW, DWr, DA, DR;   // operands of the products (r: the other way round)
-  sg::Scratch sc, scp;
+  long long cols, rows;   // of a part
+  double* W;     // a part's columns
+  void* R;       // a part of the residual: FP32, FP64 for FP64 input
+  sg::Digits DQ, DQr, DW, DWr, DA, DR;   // operands of a part's products (r: the other way round)
+  sg::Scratch sc;
   size_t bytes;
 };
 
@@ -448,28 +475,33 @@ BwLayout bw_layout(void* ws, size_t cap, int dt, int64_t m, int64_t n, int32_t k
   L.AS = c.take<double>((size_t)m * k);
   L.o = carve_orth(c, L.status, m, k);
   L.Q = c.take<double>((size_t)m * k);
-  L.W = c.take<double>((size_t)k * n);
-  const size_t rs = dt == CSS_F64 ? 8 : 4;
-  L.R = grad || dt == CSS_F64 ? (void*)c.take<char>((size_t)m * n * rs) : nullptr;
   L.Psum = grad ? c.take<double>((size_t)m * k) : nullptr;
   L.loss_part = c.take<double>((size_t)std::max(kLossBlocks, sg::residual_parts()));
-  L.DQ = sg::carve_digits(c, k, m);
-  L.DQr = sg::carve_digits(c, m, k);
-  L.DWr = sg::carve_digits(c, n, k);
-  const long long cols = chunk_cols(m, n, k);
-  L.sc = sg::carve_scratch(c, std::max(sg::sum_words(cols, k, m, 0), sg::sum_words(128, k, m, 0)));
-  L.DW = sg::carve_digits(c, k, n);
-  // A's digits are done with when R's are formed
+  // the basis is formed before the first part's digits
   const size_t at = c.off;
-  L.DA = sg::carve_digits(c, cols, m);
-  if (grad) {
-    const size_t end = c.off;
-    c.off = at;
-    L.DR = sg::carve_digits(c, m, n);
-    c.off = std::max(c.off, end);
-    L.scp = sg::carve_scratch(c, sg::sum_words(m, k, n, 0));
-  }
-  L.bytes = c.off;
+  carve_orth_digits(c, m, k, L.o);
+  const size_t end = c.off;
+  c.off = at;
+  L.cols = chunk_cols(m, n, k);
+  L.rows = std::min<long long>((m + 127) / 128 * 128, sg::part_rows(std::max<long long>(L.cols, k)));
+  const long long cols = std::min<long long>(L.cols, n), rows = std::min<long long>(L.rows, m);
+  L.W = c.take<double>((size_t)k * cols);
+  const size_t rs = dt == CSS_F64 ? 8 : 4;
+  L.R = grad || dt == CSS_F64 ? (void*)c.take<char>((size_t)rows * cols * rs) : nullptr;
+  L.DQ = sg::carve_digits(c, k, w_rows(m, k));
+  L.DQr = sg::carve_digits(c, rows, k);
+  L.DWr = sg::carve_digits(c, cols, k);
+  L.DW = grad ? sg::carve_digits(c, k, cols) : sg::Digits{};
+  size_t words = std::max(sg::sum_words(cols, k, w_rows(m, k), 0), sg::sum_words(128, k, w_rows(m, k), 0));
+  if (grad) words = std::max(words, sg::sum_words(rows, k, cols, 0));
+  L.sc = sg::carve_scratch(c, words);
+  // A's digits are done with when R's are formed
+  const size_t da = c.off;
+  L.DA = sg::carve_digits(c, cols, w_rows(m, k));
+  const size_t da_end = c.off;
+  c.off = da;
+  if (grad) L.DR = sg::carve_digits(c, rows, cols);
+  L.bytes = std::max({c.off, da_end, end});
   return L;
 }
 
@@ -479,37 +511,45 @@ css_status run_backward(const TA* A, int m, int n, long long lda, const int* sel
                         const css_opts& o, cudaStream_t s) {
   constexpr int dt = sizeof(TA) == 8 ? CSS_F64 : sizeof(TA) == 4 ? CSS_F32 : CSS_BF16;
   const unsigned long long spin = o.spin_budget_ns ? o.spin_budget_ns : 2000000000ull;
+  const int parts = dt == CSS_F64 ? kLossBlocks : sg::residual_parts();
   cudaMemsetAsync(L.status, 0, 2 * sizeof(int), s);
+  cudaMemsetAsync(L.loss_part, 0, parts * sizeof(double), s);
   int* err = L.status + 1;
   const long long mk = (long long)m * k;
-  const sg::Source q{L.Q, CSS_F64, m, 1, k, m}, qr{L.Q, CSS_F64, 1, m, m, k};
-  const sg::Source w{L.W, CSS_F64, 1, k, k, n}, wr{L.W, CSS_F64, k, 1, n, k};
   gather_cols_kernel<TA><<<(unsigned)((mk + 255) / 256), 256, 0, s>>>(A, lda, m, sel, k, L.AS);
-  if (orth(L.AS, m, k, L.Q, L.o, spin, s) != cudaSuccess || sg::split(q, L.DQ, s) != cudaSuccess ||
-      w_product(L.DQ, q, A, dt, lda, m, n, k, L.W, 1, k, L.DA, L.sc, err, spin, s) != cudaSuccess)
-    return CSS_ERR_CUDA;
-  if (sg::split(qr, L.DQr, s) != cudaSuccess || sg::split(wr, L.DWr, s) != cudaSuccess) return CSS_ERR_CUDA;
-  int parts = kLossBlocks;
-  if constexpr (dt == CSS_F64) {
-    const sg::Store st{(double*)L.R, 1, m, 0};
-    if (sg::gemm(L.DQr, L.DWr, st, L.sc, err, spin, s, qr, wr) != cudaSuccess) return CSS_ERR_CUDA;
-    residual_f64_kernel<<<kLossBlocks, 256, 0, s>>>((const double*)A, lda, m, (long long)m * n, (double*)L.R,
-                                                    (double*)dA, ldda, 2.0 * grad_out, L.loss_part);
-  } else {
-    const sg::Residual r{A, dt, lda, dA ? (float*)L.R : nullptr, dA, ldda, 2.0 * grad_out, L.loss_part};
-    parts = sg::residual_parts();
-    if (sg::gemm_residual(L.DQr, L.DWr, r, L.sc, err, spin, s) != cudaSuccess) return CSS_ERR_CUDA;
+  if (orth(L.AS, m, k, L.Q, L.o, spin, s) != cudaSuccess) return CSS_ERR_CUDA;
+  for (long long c0 = 0; c0 < n; c0 += L.cols) {
+    const int nc = (int)std::min(L.cols, n - c0);
+    const TA* Ac = A + c0 * lda;
+    const sg::Source w{L.W, CSS_F64, 1, k, k, nc}, wr{L.W, CSS_F64, k, 1, nc, k};
+    if (w_product(L.Q, Ac, dt, lda, m, nc, k, L.W, 1, k, L.DQ, c0 > 0, L.DA, L.sc, err, spin, s) != cudaSuccess ||
+        sg::split(wr, L.DWr, s) != cudaSuccess || (dA && sg::split(w, L.DW, s) != cudaSuccess))
+      return CSS_ERR_CUDA;
+    for (long long r0 = 0; r0 < m; r0 += L.rows) {
+      const int mr = (int)std::min<long long>(L.rows, m - r0);
+      const sg::Source qr{L.Q + r0, CSS_F64, 1, m, mr, k};
+      TA* const dAc = dA ? dA + c0 * ldda + r0 : nullptr;
+      if ((c0 == 0 || L.rows < m) && sg::split(qr, L.DQr, s) != cudaSuccess) return CSS_ERR_CUDA;
+      if constexpr (dt == CSS_F64) {
+        const sg::Store st{(double*)L.R, 1, mr, 0};
+        if (sg::gemm(L.DQr, L.DWr, st, L.sc, err, spin, s, qr, wr) != cudaSuccess) return CSS_ERR_CUDA;
+        residual_f64_kernel<<<kLossBlocks, 256, 0, s>>>(Ac + r0, lda, mr, (long long)mr * nc, (double*)L.R, dAc, ldda,
+                                                        2.0 * grad_out, L.loss_part);
+      } else {
+        const sg::Residual r{Ac + r0, dt, lda, dA ? (float*)L.R : nullptr, dAc, ldda, 2.0 * grad_out, L.loss_part};
+        if (sg::gemm_residual(L.DQr, L.DWr, r, L.sc, err, spin, s) != cudaSuccess) return CSS_ERR_CUDA;
+      }
+      if (!dA) continue;
+      const sg::Source r{L.R, dt == CSS_F64 ? CSS_F64 : CSS_F32, 1, mr, mr, nc};
+      const sg::Store st{L.Psum + r0, 1, m, 0, nullptr, nullptr, c0 > 0};
+      if (sg::split(r, L.DR, s) != cudaSuccess || sg::gemm(L.DR, L.DW, st, L.sc, err, spin, s) != cudaSuccess)
+        return CSS_ERR_CUDA;
+    }
   }
   if (loss) sum_kernel<<<1, 512, 0, s>>>(L.loss_part, parts, 1.0, loss);
-  if (dA) {
-    const sg::Source r{L.R, dt == CSS_F64 ? CSS_F64 : CSS_F32, 1, m, m, n};
-    const sg::Store st{L.Psum, 1, m, 0};
-    if (sg::split(r, L.DR, s) != cudaSuccess || sg::split(w, L.DW, s) != cudaSuccess ||
-        sg::gemm(L.DR, L.DW, st, L.scp, err, spin, s) != cudaSuccess)
-      return CSS_ERR_CUDA;
+  if (dA)
     das_kernel<TA><<<(unsigned)((mk + 255) / 256), 256, 0, s>>>(L.Psum, L.o.Linv, m, k, sel, 2.0 * grad_out, dA,
                                                                ldda);
-  }
   if (cudaGetLastError() != cudaSuccess) return CSS_ERR_CUDA;
   return finish(L.status, o, s);
 }
@@ -541,11 +581,16 @@ EmbLayout emb_layout(void* ws, size_t cap, int64_t m, int64_t n, int32_t l) {
   L.o = carve_orth(c, L.status, m, l);
   L.Q1 = c.take<double>((size_t)m * l);
   L.Q = c.take<double>((size_t)m * l);
-  const long long cols = chunk_cols(m, n, l);
-  L.DQ = sg::carve_digits(c, l, m);
-  L.DA = sg::carve_digits(c, cols, m);
-  L.sc = sg::carve_scratch(c, std::max(sg::sum_words(cols, l, m, 0), sg::sum_words(128, l, m, 0)));
-  L.bytes = c.off;
+  // the basis is formed before W's digits
+  const size_t at = c.off;
+  carve_orth_digits(c, m, l, L.o);
+  const size_t end = c.off;
+  c.off = at;
+  const long long cols = chunk_cols(m, n, l), rows = w_rows(m, l);
+  L.DQ = sg::carve_digits(c, l, rows);
+  L.DA = sg::carve_digits(c, std::min<long long>(cols, n), rows);
+  L.sc = sg::carve_scratch(c, std::max(sg::sum_words(cols, l, rows, 0), sg::sum_words(128, l, rows, 0)));
+  L.bytes = std::max(c.off, end);
   return L;
 }
 
@@ -563,12 +608,8 @@ css_status run_embed(const TA* A, int m, int n, long long lda, const int* sel, i
   const unsigned long long spin = o.spin_budget_ns ? o.spin_budget_ns : 2000000000ull;
   if (orth(L.AS, m, l, L.Q1, L.o, spin, s) != cudaSuccess || orth(L.Q1, m, l, L.Q, L.o, spin, s) != cudaSuccess)
     return CSS_ERR_CUDA;
-  if (W) {
-    const sg::Source q{L.Q, CSS_F64, m, 1, l, m};
-    if (sg::split(q, L.DQ, s) != cudaSuccess ||
-        w_product(L.DQ, q, A, dt, lda, m, n, l, W, ldw, 1, L.DA, L.sc, L.status + 1, spin, s) != cudaSuccess)
-      return CSS_ERR_CUDA;
-  }
+  if (W && w_product(L.Q, A, dt, lda, m, n, l, W, ldw, 1, L.DQ, false, L.DA, L.sc, L.status + 1, spin, s) != cudaSuccess)
+    return CSS_ERR_CUDA;
   if (Qout) copy_cols_kernel<<<gb, 256, 0, s>>>(L.Q, m, l, Qout, ldq);
   if (cudaGetLastError() != cudaSuccess) return CSS_ERR_CUDA;
   return finish(L.status, o, s);

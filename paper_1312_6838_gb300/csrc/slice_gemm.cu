@@ -404,6 +404,12 @@ __device__ __forceinline__ double combine(long long hi, long long lo, int e) {
   return neg ? -v : v;
 }
 
+// What stands for an entry without digits: NaN, or nothing where restore_kernel
+// will add to what is there.
+__device__ __forceinline__ double unformed(const Args& P, int ex) {
+  return ex < kExNan && P.st.add && P.sx.p ? 0.0 : __longlong_as_double(0x7fffffffffffffffll);
+}
+
 __device__ __forceinline__ void store(const Store& st, int row, int c, double v) {
   if (st.cscale) v *= __ldg(st.cscale + c);
   if (st.out32) {
@@ -733,7 +739,7 @@ __global__ void __launch_bounds__(kThreads, 1) slice_gemm_kernel(const __grid_co
             const int eyr = __shfl_sync(0xffffffffu, ey, (j0 + jj) & 31);
             if (row >= P.M || c >= P.N) continue;
             double v = combine(hv[jj], lv[jj], ex + scale_exp(eyr, P.ydt));
-            if (max(exr, eyr) >= kExInf) v = __longlong_as_double(0x7fffffffffffffffll);
+            if (max(exr, eyr) >= kExInf) v = unformed(P, max(exr, eyr));
             store(P.st, row, c, v);
             if (P.lower && w.tm != w.tn) store(P.st, c, row, v);
           }
@@ -809,7 +815,7 @@ __global__ void __launch_bounds__(kThreads, 1) slice_gemm_kernel(const __grid_co
       if (warp == 4 && lane == 0) {
         double sum = 0.0;
         for (int i = 0; i < kEpiWarps; ++i) sum += s_loss[i];
-        P.r.loss_part[blockIdx.x] = sum;
+        P.r.loss_part[blockIdx.x] += sum;
       }
     }
     fence_before();
@@ -832,7 +838,7 @@ __global__ void __launch_bounds__(256) finish_kernel(const __grid_constant__ Arg
   const int exr = P.xe[row], eyr = P.ye[c];
   double v = combine((long long)P.sums[(long long)P.M * P.N + at], (long long)P.sums[at],
                      scale_exp(exr, P.xdt) + scale_exp(eyr, P.ydt));
-  if (max(exr, eyr) >= kExInf) v = __longlong_as_double(0x7fffffffffffffffll);
+  if (max(exr, eyr) >= kExInf) v = unformed(P, max(exr, eyr));
   store(P.st, row, c, v);
 }
 
@@ -1004,11 +1010,6 @@ cudaError_t gemm_residual(const Digits& X, const Digits& Y, const Residual& r, c
   Args P = base_args(X, Y, err, spin_ns);
   P.part = w.part;
   P.r = r;
-  const int ctas = std::min(kCtas, P.tiles);
-  if (ctas < kCtas) {
-    cudaError_t e = cudaMemsetAsync(r.loss_part, 0, sizeof(double) * kCtas, s);
-    if (e != cudaSuccess) return e;
-  }
   return launch_gemm<kEpResidual>(P, s);
 }
 

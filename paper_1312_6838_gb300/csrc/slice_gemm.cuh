@@ -75,7 +75,7 @@ cudaError_t gemm(const Digits& X, const Digits& Y, const Store& st, const Scratc
 
 // R = A - X Y^T for FP32 or BF16 A (M x N, leading dimension lda): writes R
 // (FP32, leading dimension M) when R != null, dA = g2 R when dA != null, and
-// one partial of ||R||^2 per CTA of the launch (residual_parts of them).
+// adds its share of ||R||^2 to a partial sum per CTA (residual_parts of them).
 struct Residual {
   const void* A;
   int dtype;

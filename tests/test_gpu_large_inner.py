@@ -60,7 +60,7 @@ def test_lowrank_with_more_rows_of_q_than_columns():
 
 
 @pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
-@pytest.mark.parametrize("m,n,l", [(4194241, 5, 2), (4300001, 9, 4)])
+@pytest.mark.parametrize("m,n,l", [(4194241, 5, 2), (4300001, 9, 4), (40000, 3000, 20), (700000, 300, 130)])
 def test_embedding_and_residual_of_tall_columns(dtype, m, n, l):
     from paper_1312_6838_gb300 import css
     A = _randn(n, m, seed=m, dtype=dtype).t()
@@ -82,9 +82,19 @@ def test_embedding_and_residual_of_tall_columns(dtype, m, n, l):
     u = 2.0 ** -53 if dtype == torch.float64 else 2.0 ** -24
     ref = float(E.square().sum())
     assert abs(float(loss.detach()) - ref) <= (1e-10 + 2 * u) * ref
+    # (the last two sizes: columns, and columns and rows, in several parts)
     G = 2 * E
     G[:, S] = -2 * (E @ torch.linalg.solve_triangular(R, W, upper=True).t())
     assert float((Ag.grad.double() - G).abs().max()) <= (1e-10 + 8 * u) * float(G.abs().max())
+
+
+def test_embedding_of_equal_digits():
+    """A column of 2^26 ones: Q is 2^-13 throughout and W 2^13, exactly."""
+    from paper_1312_6838_gb300 import css
+    A = torch.ones(1, 1 << 26, dtype=torch.bfloat16, device="cuda").t()
+    emb = css.embed(A, [0])
+    assert float(emb.W[0, 0]) == 2.0 ** 13
+    assert float(emb.Q.min()) == float(emb.Q.max()) == 2.0 ** -13
 
 
 @pytest.mark.parametrize("m,n", [(5, 4194241), (3, 20000000)])
