@@ -41,8 +41,8 @@ cudaError_t gcss_f0_simt(int dtype, const void* A, long long lda, int m, int n, 
                          long long ldb, int r, double* partial, double* f, cudaStream_t s);
 
 // css_f0_simt's results for FP64 input on the slice GEMM (init_f64.cu).  The
-// scratch size is 0 where the digits would exceed the scratch bound: the
-// kernels above run then.
+// scratch size is 0 for matrices beyond 2^30 entries: the kernels above run
+// then.
 size_t css_f0_f64_bytes(int64_t m, int64_t n);
 // Least workspace that css_select takes (css_workspace_size's holds the FP64
 // digits too, without which FP64 runs the kernels above).

@@ -17,41 +17,41 @@
 namespace css {
 namespace {
 
-constexpr long long kChunk = 16384;               // columns whose products are held at a time
-constexpr size_t kMaxDigits = (size_t)1 << 34;    // scratch bound: beyond it the FP64 tiles run
-
-// Columns per chunk: digits of at most 1 GB.
-long long chunk_cols(long long m, long long n) {
-  const long long fit = std::max<long long>(128, ((1ll << 30) / (16 * std::max<long long>(m, 64))) / 128 * 128);
-  return std::min(std::min(kChunk, fit), n);
-}
+constexpr long long kChunk = 16384;                // most columns whose products are held at a time
+// Digits of a part of A by rows; of one by columns, and of a part of C's rows.
+constexpr long long kRowBytes = 256ll << 20, kPartBytes = 1ll << 30;
+constexpr size_t kMaxEntries = (size_t)1 << 30;   // of A; beyond it the FP64 tiles run (not measured there)
 
 struct Layout {
-  sg::Digits rows, cols, left;   // A by rows, A's chunk by columns (in the same space), C
+  sg::Digits rows, cols, left;   // parts of A by rows and by columns (in one space), and of C
+  long long part_k, part_cols, part_left;
   double* D;
   sg::Scratch sc;
 };
 
 Layout carve(WsCarver& c, long long m, long long n) {
   Layout L{};
-  const long long nb = chunk_cols(m, n);
+  L.part_k = std::min(n, sg::part_k(m, kRowBytes));
+  L.part_cols = std::min(std::min(n, kChunk), sg::part_rows(m, kPartBytes));
+  L.part_left = std::min(m, sg::part_rows(m, kPartBytes));
   const size_t at = c.off;
-  L.rows = sg::carve_digits(c, m, n);
+  L.rows = sg::carve_digits(c, m, L.part_k);
   const size_t end = c.off;
   c.off = at;
-  L.cols = sg::carve_digits(c, nb, m);
+  L.cols = sg::carve_digits(c, L.part_cols, m);
   c.off = std::max(c.off, end);
-  L.left = sg::carve_digits(c, m, m);
-  L.D = c.take<double>((size_t)m * nb);
-  size_t words = std::max(sg::sum_words(m, m, n, 1), sg::sum_words(m, nb, m, 0));
-  if (n % nb) words = std::max(words, sg::sum_words(m, n % nb, m, 0));
+  L.left = sg::carve_digits(c, L.part_left, m);
+  L.D = c.take<double>((size_t)(L.part_left * L.part_cols));
+  size_t words = std::max(sg::sum_words(m, m, L.part_k, 1), sg::sum_words(L.part_left, L.part_cols, m, 0));
+  if (n % L.part_cols) words = std::max(words, sg::sum_words(L.part_left, n % L.part_cols, m, 0));
   L.sc = sg::carve_scratch(c, words);
   return L;
 }
 
-// f[i] = sum_r D[r, i] A[r, i]: one warp a column, memory-bound.
+// f[i] = sum_r D[r, i] A[r, i], or f[i] += that: one warp a column, memory-bound.
 __global__ void __launch_bounds__(256) column_dots_kernel(const double* __restrict__ D, const double* __restrict__ A,
-                                                          long long lda, int m, int n, double* __restrict__ f) {
+                                                          long long lda, int m, int n, double* __restrict__ f,
+                                                          bool add) {
   const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (i >= n) return;
   const double *d = D + (long long)i * m, *a = A + (long long)i * lda;
@@ -59,14 +59,14 @@ __global__ void __launch_bounds__(256) column_dots_kernel(const double* __restri
 #pragma unroll 4
   for (int r = lane; r < m; r += 32) s = fma(d[r], a[r], s);
   s = warp_sum(s);
-  if (lane == 0) f[i] = s;
+  if (lane == 0) f[i] = add ? f[i] + s : s;
 }
 
 }  // namespace
 
 size_t css_f0_f64_bytes(int64_t m, int64_t n) {
   WsCarver c(nullptr, (size_t)-1);
-  if ((size_t)m * (size_t)n > kMaxDigits / 16) return 0;
+  if ((size_t)m * (size_t)n > kMaxEntries) return 0;
   carve(c, m, n);
   return c.off;
 }
@@ -75,20 +75,26 @@ cudaError_t css_f0_f64(const double* A, long long lda, int m, int n, double* C, 
                        double* f, int* err, unsigned long long spin_ns, cudaStream_t s) {
   WsCarver c(scratch, (size_t)-1);
   Layout L = carve(c, m, n);
-  const sg::Source rows{A, CSS_F64, 1, lda, m, n}, cs{C, CSS_F64, ldc, 1, m, m};
-  cudaError_t e = sg::split(rows, L.rows, s);
-  if (e == cudaSuccess) e = sg::gemm(L.rows, L.rows, sg::Store{C, 1, ldc, 1}, L.sc, err, spin_ns, s);
-  if (e == cudaSuccess) e = sg::split(cs, L.left, s);
-  if (e != cudaSuccess) return e;
-  const long long nb = chunk_cols(m, n);
-  for (long long c0 = 0; c0 < n; c0 += nb) {
-    const int nc = (int)std::min<long long>(nb, n - c0);
+  cudaError_t e = cudaSuccess;
+  for (long long c0 = 0; e == cudaSuccess && c0 < n; c0 += L.part_k) {
+    const sg::Source rows{A + c0 * lda, CSS_F64, 1, lda, m, (int)std::min(L.part_k, n - c0)};
+    e = sg::split(rows, L.rows, s);
+    const sg::Store st{C, 1, ldc, 1, nullptr, nullptr, c0 > 0};
+    if (e == cudaSuccess) e = sg::gemm(L.rows, L.rows, st, L.sc, err, spin_ns, s);
+  }
+  for (long long c0 = 0; e == cudaSuccess && c0 < n; c0 += L.part_cols) {
+    const int nc = (int)std::min(L.part_cols, n - c0);
     const sg::Source cols{A + c0 * lda, CSS_F64, lda, 1, nc, m};
     e = sg::split(cols, L.cols, s);
-    if (e == cudaSuccess) e = sg::gemm(L.left, L.cols, sg::Store{L.D, 1, m, 0}, L.sc, err, spin_ns, s);
-    if (e != cudaSuccess) return e;
-    column_dots_kernel<<<(nc + 7) / 8, 256, 0, s>>>(L.D, A + c0 * lda, lda, m, nc, f + c0);
+    for (long long r0 = 0; e == cudaSuccess && r0 < m; r0 += L.part_left) {
+      const int mr = (int)std::min<long long>(L.part_left, m - r0);
+      const sg::Source cs{C + r0 * ldc, CSS_F64, ldc, 1, mr, m};
+      if (c0 == 0 || L.part_left < m) e = sg::split(cs, L.left, s);
+      if (e == cudaSuccess) e = sg::gemm(L.left, L.cols, sg::Store{L.D, 1, mr, 0}, L.sc, err, spin_ns, s);
+      column_dots_kernel<<<(nc + 7) / 8, 256, 0, s>>>(L.D, A + c0 * lda + r0, lda, mr, nc, f + c0, r0 > 0);
+    }
   }
+  if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
 

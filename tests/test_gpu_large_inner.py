@@ -97,8 +97,9 @@ def test_embedding_of_equal_digits():
     assert float(emb.Q.min()) == float(emb.Q.max()) == 2.0 ** -13
 
 
-@pytest.mark.parametrize("m,n", [(5, 4194241), (3, 20000000)])
+@pytest.mark.parametrize("m,n", [(5, 4194241), (3, 20000000), (9001, 300)])
 def test_fp64_selection_of_few_long_rows(m, n):
+    """(9001 rows: C's digits in two parts)"""
     from paper_1312_6838_gb300 import css
     A = _randn(n, m, seed=m).t()
     a, b = css.select(A, 2), css.select(A, 2, init_path=1)

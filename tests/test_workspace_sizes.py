@@ -39,3 +39,10 @@ def test_embedding(L, m, n, l):
 @pytest.mark.parametrize("m,n,l", [(4096, 65536, 256), (4096, 8000000, 1024), (8000000, 1000, 100), (10, 1 << 30, 1)])
 def test_lowrank(L, m, n, l):
     assert 0 < _size(L, L.CSS_OP_LOWRANK, L.CSS_F64, m, n, l, l) <= 4 * GB
+
+
+@pytest.mark.parametrize("m,n", [(8, 4190000), (8, 16000000), (100, 10000000), (1000, 1000000), (100000, 10000)])
+def test_fp64_selection(L, m, n):
+    # C, its digits and C A of a part, the score state, and the digits of a part of A
+    size = _size(L, L.CSS_OP_SELECT, L.CSS_F64, m, n, 0, 4)
+    assert 0 < size <= 8 * m * m + 100 * n + min(32 * (m + 128) ** 2, 17 * GB) + 2 * GB
