@@ -7,8 +7,7 @@
 //
 // The FP64 tiles of init_simt.cu are bound by an SM's FP64 rate (two lanes a
 // clock), and a small problem has too few of them: 500 x 1000 took 1.63 ms
-// with 36 blocks in C = A A^T; here
-// 0.23 ms; 1024 x 8192: 23.4 -> 1.03 ms.
+// with 36 blocks in C = A A^T; here 0.23 ms; 1024 x 8192: 23.4 -> 1.03 ms.
 #include <algorithm>
 
 #include "init.cuh"
@@ -26,6 +25,7 @@ struct Layout {
   sg::Digits rows, cols, left;   // parts of A by rows and by columns (in one space), and of C
   long long part_k, part_cols, part_left;
   double* D;
+  int* kexp;   // of the sizes of A's rows
   sg::Scratch sc;
 };
 
@@ -42,6 +42,7 @@ Layout carve(WsCarver& c, long long m, long long n) {
   c.off = std::max(c.off, end);
   L.left = sg::carve_digits(c, L.part_left, m);
   L.D = c.take<double>((size_t)(L.part_left * L.part_cols));
+  L.kexp = c.take<int>((size_t)m);
   size_t words = std::max(sg::sum_words(m, m, L.part_k, 1), sg::sum_words(L.part_left, L.part_cols, m, 0));
   if (n % L.part_cols) words = std::max(words, sg::sum_words(L.part_left, n % L.part_cols, m, 0));
   L.sc = sg::carve_scratch(c, words);
@@ -82,13 +83,15 @@ cudaError_t css_f0_f64(const double* A, long long lda, int m, int n, double* C, 
     const sg::Store st{C, 1, ldc, 1, nullptr, nullptr, c0 > 0};
     if (e == cudaSuccess) e = sg::gemm(L.rows, L.rows, st, L.sc, err, spin_ns, s);
   }
+  // C A with A's rows at one size: (C S^-1)(S A), S^2 the diagonal of C
+  if (e == cudaSuccess) sg::gram_exponents(C, ldc, m, L.kexp, s);
   for (long long c0 = 0; e == cudaSuccess && c0 < n; c0 += L.part_cols) {
     const int nc = (int)std::min(L.part_cols, n - c0);
-    const sg::Source cols{A + c0 * lda, CSS_F64, lda, 1, nc, m};
+    const sg::Source cols{A + c0 * lda, CSS_F64, lda, 1, nc, m, L.kexp, 1};
     e = sg::split(cols, L.cols, s);
     for (long long r0 = 0; e == cudaSuccess && r0 < m; r0 += L.part_left) {
       const int mr = (int)std::min<long long>(L.part_left, m - r0);
-      const sg::Source cs{C + r0 * ldc, CSS_F64, ldc, 1, mr, m};
+      const sg::Source cs{C + r0 * ldc, CSS_F64, ldc, 1, mr, m, L.kexp, -1};
       if (c0 == 0 || L.part_left < m) e = sg::split(cs, L.left, s);
       if (e == cudaSuccess) e = sg::gemm(L.left, L.cols, sg::Store{L.D, 1, mr, 0}, L.sc, err, spin_ns, s);
       column_dots_kernel<<<(nc + 7) / 8, 256, 0, s>>>(L.D, A + c0 * lda + r0, lda, mr, nc, f + c0, r0 > 0);

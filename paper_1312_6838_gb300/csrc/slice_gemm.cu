@@ -71,6 +71,11 @@ __device__ __forceinline__ int biased_exp(float v) {
   const int b = __float_as_int(v), e = (b >> 23) & 0xff;
   return e < 0xff ? e : b & 0x7fffff ? kExNan : kExInf;
 }
+// with 2^ke applied: zeros have none, subnormals that of their range
+__device__ __forceinline__ int scaled_exp(double v, int ke) {
+  const int e = biased_exp(v);
+  return e >= kExInf ? e : v == 0.0 ? 0 : max(e, 1) + ke;
+}
 __device__ __forceinline__ float load_val(const float* p) { return __ldg(p); }
 __device__ __forceinline__ double load_val(const double* p) { return __ldg(p); }
 __device__ __forceinline__ float load_val(const __nv_bfloat16* p) {
@@ -142,11 +147,21 @@ __device__ __forceinline__ void load_block(const T* p, long long rs, long long k
   }
 }
 
+// First k of this thread's chunk q, and the exponent applied at k.
+template <bool KC>
+__device__ __forceinline__ int k_of(int k0, int q) {
+  return k0 + 8 * (KC ? (int)threadIdx.x % 8 : (int)threadIdx.x / 128 + 2 * q);
+}
+__device__ __forceinline__ int k_exp(const int* kexp, int sign, int k, int K) {
+  return k < K ? sign * __ldg(kexp + k) : 0;
+}
+
 // Largest biased exponent of every row (ex zeroed before): a block takes 128
 // rows and every gridDim.y-th 64 k of them.  Memory-bound.
-template <typename T, typename V, bool KC, bool VEC>
+template <typename T, typename V, bool KC, bool VEC, bool SC>
 __global__ void __launch_bounds__(256) row_exp_kernel(const T* __restrict__ p, long long rs, long long ks, int rows,
-                                                      int K, int* __restrict__ ex) {
+                                                      int K, const int* __restrict__ kexp, int sign,
+                                                      int* __restrict__ ex) {
   const int r0 = blockIdx.x * kT;
   int best[4] = {0, 0, 0, 0};
   for (int k0 = blockIdx.y * kKb; k0 < K; k0 += gridDim.y * kKb) {
@@ -155,7 +170,10 @@ __global__ void __launch_bounds__(256) row_exp_kernel(const T* __restrict__ p, l
 #pragma unroll
     for (int q = 0; q < 4; ++q)
 #pragma unroll
-      for (int e = 0; e < 8; ++e) best[q] = max(best[q], biased_exp(v[q][e]));
+      for (int e = 0; e < 8; ++e) {
+        if constexpr (SC) best[q] = max(best[q], scaled_exp(v[q][e], k_exp(kexp, sign, k_of<KC>(k0, q) + e, K)));
+        else best[q] = max(best[q], biased_exp(v[q][e]));
+      }
   }
   if (KC) {
 #pragma unroll
@@ -176,9 +194,9 @@ __device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) 
 // Digits of one block of 128 rows x 64 k; slices are written until what is
 // left can give no digit, and their number goes to ns.  Rows with an infinity
 // or a NaN get zero digits (see restore_kernel).
-template <typename T, typename V, bool KC, bool VEC>
+template <typename T, typename V, bool KC, bool VEC, bool SC>
 __global__ void __launch_bounds__(256) split_kernel(const T* __restrict__ p, long long rs, long long ks, int rows,
-                                                    int K, int k64, int dtype,
+                                                    int K, int k64, int dtype, const int* __restrict__ kexp, int sign,
                                                     const int* __restrict__ ex, unsigned char* __restrict__ d,
                                                     unsigned char* __restrict__ ns) {
   // (one grid dimension: K / 64 may exceed the others' 65535)
@@ -210,7 +228,8 @@ __global__ void __launch_bounds__(256) split_kernel(const T* __restrict__ p, lon
         unsigned long long mant = b & 0xfffffffffffffull;
         if (be > 0) mant |= 1ull << 52;
         // |x| 2^(64 - scale), rounded to an integer below 2^63
-        const int sh = max(be, 1) - e + 10;
+        const int ke = SC ? k_exp(kexp, sign, k_of<KC>(kb * kKb, q) + i, K) : 0;
+        const int sh = max(be, 1) + ke - e + 10;
         unsigned long long F = 0;
         if (!dead) {
           if (sh >= 0) F = mant << sh;
@@ -872,20 +891,29 @@ __global__ void __launch_bounds__(256) restore_kernel(const __grid_constant__ Ar
 
 int k_blocks(long long K) { return (int)ceil_div(K, kKb); }
 
-template <typename T, typename V, bool KC, bool VEC>
+template <typename T, typename V, bool KC, bool VEC, bool SC = false>
 void launch_split(const Source& src, const Digits& D, cudaStream_t s) {
   const int k64 = k_blocks(src.K);
   const unsigned tiles = (unsigned)ceil_div(src.rows, kT);
   const unsigned ky = (unsigned)std::min<long long>(k64, std::max<long long>(1, ceil_div(152 * 8, tiles)));
-  row_exp_kernel<T, V, KC, VEC><<<dim3(tiles, ky), 256, 0, s>>>((const T*)src.p, src.rs, src.ks, src.rows, src.K,
-                                                                D.ex);
-  split_kernel<T, V, KC, VEC><<<tiles * (unsigned)k64, 256, 0, s>>>((const T*)src.p, src.rs, src.ks, src.rows,
-                                                                        src.K, k64, src.dtype, D.ex, D.d,
+  const T* p = (const T*)src.p;
+  row_exp_kernel<T, V, KC, VEC, SC><<<dim3(tiles, ky), 256, 0, s>>>(p, src.rs, src.ks, src.rows, src.K, src.kexp,
+                                                                    src.kexp_sign, D.ex);
+  split_kernel<T, V, KC, VEC, SC><<<tiles * (unsigned)k64, 256, 0, s>>>(p, src.rs, src.ks, src.rows, src.K, k64,
+                                                                        src.dtype, src.kexp, src.kexp_sign, D.ex, D.d,
                                                                         D.ns);
 }
 template <typename T, typename V>
 void launch_split_of(const Source& src, const Digits& D, cudaStream_t s) {
   const bool vec = ((uintptr_t)src.p & 15u) == 0 && (src.rs * (long long)sizeof(T)) % 16 == 0;
+  if constexpr (sizeof(T) == 8) {
+    if (src.kexp) {
+      if (src.ks == 1 && vec) launch_split<T, V, true, true, true>(src, D, s);
+      else if (src.ks == 1) launch_split<T, V, true, false, true>(src, D, s);
+      else launch_split<T, V, false, false, true>(src, D, s);
+      return;
+    }
+  }
   if (src.ks == 1 && vec) launch_split<T, V, true, true>(src, D, s);
   else if (src.ks == 1) launch_split<T, V, true, false>(src, D, s);
   else launch_split<T, V, false, false>(src, D, s);
@@ -961,6 +989,17 @@ cudaError_t split(const Source& src, Digits& D, cudaStream_t s) {
     default: launch_split_of<__nv_bfloat16, float>(src, D, s); break;
   }
   return cudaGetLastError();
+}
+
+__global__ void gram_exponents_kernel(const double* __restrict__ G, long long ld, int K, int* __restrict__ e) {
+  const int k = blockIdx.x * 256 + threadIdx.x;
+  if (k >= K) return;
+  const int b = biased_exp(G[k * ld + k]);
+  // (a zero, an infinity or a NaN: nothing to balance)
+  e[k] = b > 0 && b < kExInf ? (b - 1023) >> 1 : 0;
+}
+void gram_exponents(const double* G, long long ld, int K, int* e, cudaStream_t s) {
+  gram_exponents_kernel<<<(K + 255) / 256, 256, 0, s>>>(G, ld, K, e);
 }
 
 size_t sum_words(long long M, long long N, long long K, int lower) {

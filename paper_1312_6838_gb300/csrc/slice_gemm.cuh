@@ -9,13 +9,23 @@
 namespace css {
 namespace sg {
 
-// A rows x K operand in its own type: element (row, k) at p[row * rs + k * ks].
+// A rows x K operand in its own type: element (row, k) at p[row * rs + k * ks],
+// times 2^(kexp_sign kexp[k]) where kexp is given (FP64 only).
 struct Source {
   const void* p;
   int dtype;            // css_dtype
   long long rs, ks;
   int rows, K;
+  const int* kexp;
+  int kexp_sign;
 };
+// Balances operands whose inner index runs over very different sizes: digits
+// hold a row's entries relative to its largest one, so where a few inner
+// indices are by far the largest in X and a row of Y is zero there, what is
+// left of X's rows would be too coarse for it.  e[k] = the exponent of
+// sqrt(G_kk) of a Gram matrix over the inner index: X 2^e and Y 2^-e (or the
+// reverse) have the same product.
+void gram_exponents(const double* G, long long ld, int K, int* e, cudaStream_t s);
 
 // The operand as digits (see slice_gemm.cu).
 struct Digits {
