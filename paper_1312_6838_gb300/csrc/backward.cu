@@ -310,6 +310,7 @@ struct OrthSpace {
   double *G, *gpart, *Linv;
   sg::Digits DS, DSr, DL;   // parts of A_S both ways (in one space), L^-1
   long long part_k, part_rows;
+  int* kexp;                // of the sizes of A_S's columns
   sg::Scratch sc;
   int* status;              // [0] rank deficient, [1] error of the products
 };
@@ -332,6 +333,7 @@ void carve_orth_digits(WsCarver& c, long long m, int k, OrthSpace& w) {
   w.DSr = sg::carve_digits(c, w.part_rows, k);
   c.off = std::max(c.off, end);
   w.DL = sg::carve_digits(c, k, k);
+  w.kexp = c.take<int>(k);
   w.sc = sg::carve_scratch(c, std::max(sg::sum_words(k, k, w.part_k, 1), sg::sum_words(w.part_rows, k, k, 0)));
 }
 cudaError_t orth(const double* AS, int m, int k, double* Q, OrthSpace& w, unsigned long long spin_ns,
@@ -350,11 +352,14 @@ cudaError_t orth(const double* AS, int m, int k, double* Q, OrthSpace& w, unsign
     const sg::Store st{w.G, 1, k, 1, nullptr, nullptr, r0 > 0};
     if ((e = sg::gemm(w.DS, w.DS, st, w.sc, w.status + 1, spin_ns, s)) != cudaSuccess) return e;
   }
+  // Q = (A_S D^-1)(D L^-T), D^2 the diagonal of G: columns of very different
+  // sizes (a greedy choice on graded data) at one size
+  sg::gram_exponents(w.G, k, k, w.kexp, s);
   chol_inv(w.G, k, w.Linv, w.gpart, w.status, s);
-  const sg::Source li{w.Linv, CSS_F64, 1, k, k, k};
+  const sg::Source li{w.Linv, CSS_F64, 1, k, k, k, w.kexp, 1};
   if ((e = sg::split(li, w.DL, s)) != cudaSuccess) return e;
   for (long long r0 = 0; r0 < m; r0 += w.part_rows) {
-    const sg::Source ar{AS + r0, CSS_F64, 1, m, (int)std::min(w.part_rows, m - r0), k};
+    const sg::Source ar{AS + r0, CSS_F64, 1, m, (int)std::min(w.part_rows, m - r0), k, w.kexp, -1};
     if ((e = sg::split(ar, w.DSr, s)) != cudaSuccess) return e;
     if ((e = sg::gemm(w.DSr, w.DL, sg::Store{Q + r0, 1, m, 0}, w.sc, w.status + 1, spin_ns, s)) != cudaSuccess) return e;
   }

@@ -32,3 +32,25 @@ def test_fp64_scores_beside_an_outlying_row(m, n, big):
     worst = np.max(np.abs(a - b) / tol)
     print(f"f beside {big:g}: {worst:.3g} of the tolerance")
     assert worst <= 1.0, worst
+
+
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+@pytest.mark.parametrize("l", [128, 129, 200])
+def test_basis_of_graded_columns(dtype, l):
+    """A_S with columns over eight decades: Q = orth(A_S) does not depend on
+    their sizes.  Against Householder QR of the columns at one scale; both
+    within 8 l u cond^2 (the normal equations square the condition of the
+    scaled columns, which is all that counts), entrywise."""
+    from paper_1312_6838_gb300 import css
+    rng = np.random.default_rng(l)
+    X = rng.standard_normal((400, l)) * np.exp2(np.rint(-26.0 * rng.permutation(l) / (l - 1)))
+    A = css.to_colmajor(torch.from_numpy(X).to(dtype).cuda())
+    X = A.double().cpu().numpy()
+    X = X / np.exp2(np.rint(np.log2(np.abs(X).max(0))))
+    Q, R = np.linalg.qr(X)
+    Q *= np.sign(np.diag(R))
+    got = css.embed(A, list(range(l))).Q.cpu().numpy()
+    tol = 8 * l * U * np.linalg.cond(X) ** 2
+    worst = np.abs(got - Q).max()
+    print(f"Q of graded columns, l = {l}: {worst:.3g}, tolerance {tol:.3g}")
+    assert worst <= tol
