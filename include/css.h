@@ -158,11 +158,13 @@ typedef struct {
     int32_t init_path;
     /* Test hook for the bounded device waits (0 = off, the default).
        1: one team barrier of the persistent greedy kernel (the first of
-       the first iteration) waits for an arrival that no CTA makes; 2: the
-       tensor-core initial-score kernels wait on an mbarrier phase that
-       nothing completes.  The wait runs out after spin_budget_ns, the call
-       reports CSS_ERR_TIMEOUT, nothing faults and the context stays usable
-       for the next call.  css_select and gcss_select. */
+       the first iteration) waits for an arrival that no CTA makes, in
+       css_lowrank (l >= 17) the eigenvector estimate's wait for rotations;
+       2: the tensor-core kernels (initial scores; digit products) wait on an
+       mbarrier phase that nothing completes.  The wait runs out after
+       spin_budget_ns, the call reports CSS_ERR_TIMEOUT, nothing faults and
+       the context stays usable for the next call.  css_select, gcss_select,
+       css_embed, css_residual_backward and css_lowrank. */
     int32_t test_unmet_wait;
     /* Plan knobs (0 = the value the tuning table holds for this device and
        shape, else the default).  split_share: the fused step splits the
@@ -683,8 +685,9 @@ css_status css_select_noalloc(const void* A, css_dtype dtype, int64_t m,
    of css_select, gcss_select, gcss_distributed, css_select_randomized or
    css_select_batched(_run): synchronises `stream`, then returns CSS_OK,
    CSS_RANK_EXHAUSTED or the device error -- that of the greedy kernel, or
-   that of the tensor-core initial-score kernel that ran before it (a
-   bounded wait there that ran out reads as CSS_ERR_TIMEOUT). */
+   that of the tensor-core kernels that ran before it (a bounded wait there
+   that ran out reads as CSS_ERR_TIMEOUT, also after css_embed,
+   css_residual_backward and css_lowrank). */
 css_status css_read_status(const void* ws, css_stream_t stream);
 
 #ifdef __cplusplus

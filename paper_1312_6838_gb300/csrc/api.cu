@@ -97,14 +97,6 @@ int split_slots_for(int64_t split_cols) {
   return (int)std::min<int64_t>(per_grid, (split_cols + 1) / 2 + 1);
 }
 
-// Byte offset, inside the 256-byte status slot at the start of every
-// workspace, of the tensor-core initial-score kernel's error flag.  The
-// greedy launch resets only the DevStatus at offset 0, so the flag survives
-// until css_read_status or finish() reads it.
-constexpr size_t kAuxErrOffset = 128;
-static_assert(sizeof(DevStatus) <= kAuxErrOffset && kAuxErrOffset + sizeof(int) <= kStatusBytes,
-              "the flag sits in the status slot, after the DevStatus");
-
 void carve_header(WsCarver& c, int max_units, Header& h, int64_t split_cols) {
   h.st = c.take<DevStatus>(1);
   h.aux_err = h.st ? reinterpret_cast<int*>(reinterpret_cast<char*>(h.st) + kAuxErrOffset) : nullptr;
@@ -707,7 +699,7 @@ css_status select_impl(const void* A, css_dtype dtype, int64_t m, int64_t n, int
     for (int z = 0; pipe && z < pipe->chunks && e == cudaSuccess; ++z) e = cudaStreamWaitEvent(s, pipe->ready[z], 0);
     if (e == cudaSuccess && dtype == CSS_F64 && L.f64_scratch && o.init_path != 1)
       e = css_f0_f64((const double*)A, lda, (int)m, (int)n, (double*)L.C, c_ld(m, 8), L.f64_scratch, L.s.f,
-                     L.h.aux_err, spin, s);
+                     L.h.aux_err, spin, s, stall_mbarrier(o));
     else if (e == cudaSuccess)
       e = css_f0_simt(dtype, A, lda, (int)m, (int)n, L.C, c_ld(m, (int)accsize(dtype)), L.partial, L.s.f, s);
   }

@@ -306,13 +306,15 @@ __global__ void q_kernel(const double* __restrict__ AS, const double* __restrict
 constexpr int kSliceK = 128;
 
 // A_S's orthonormal basis by Cholesky: G = A_S^T A_S = L L^T, Q = A_S L^-T.
+constexpr int kErr = kAuxErrOffset / sizeof(int);
+
 struct OrthSpace {
   double *G, *gpart, *Linv;
   sg::Digits DS, DSr, DL;   // parts of A_S both ways (in one space), L^-1
   long long part_k, part_rows;
   int* kexp;                // of the sizes of A_S's columns
   sg::Scratch sc;
-  int* status;              // [0] rank deficient, [1] error of the products
+  int* status;              // [0] rank deficient, [kErr] error of the products
 };
 OrthSpace carve_orth(WsCarver& c, int* status, long long m, int k) {
   OrthSpace w{};
@@ -350,7 +352,7 @@ cudaError_t orth(const double* AS, int m, int k, double* Q, OrthSpace& w, unsign
     const sg::Source a{AS + r0, CSS_F64, m, 1, k, (int)std::min(w.part_k, m - r0)};
     if ((e = sg::split(a, w.DS, s)) != cudaSuccess) return e;
     const sg::Store st{w.G, 1, k, 1, nullptr, nullptr, r0 > 0};
-    if ((e = sg::gemm(w.DS, w.DS, st, w.sc, w.status + 1, spin_ns, s)) != cudaSuccess) return e;
+    if ((e = sg::gemm(w.DS, w.DS, st, w.sc, w.status + kErr, spin_ns, s)) != cudaSuccess) return e;
   }
   // Q = (A_S D^-1)(D L^-T), D^2 the diagonal of G: columns of very different
   // sizes (a greedy choice on graded data) at one size
@@ -361,20 +363,20 @@ cudaError_t orth(const double* AS, int m, int k, double* Q, OrthSpace& w, unsign
   for (long long r0 = 0; r0 < m; r0 += w.part_rows) {
     const sg::Source ar{AS + r0, CSS_F64, 1, m, (int)std::min(w.part_rows, m - r0), k, w.kexp, -1};
     if ((e = sg::split(ar, w.DSr, s)) != cudaSuccess) return e;
-    if ((e = sg::gemm(w.DSr, w.DL, sg::Store{Q + r0, 1, m, 0}, w.sc, w.status + 1, spin_ns, s)) != cudaSuccess) return e;
+    if ((e = sg::gemm(w.DSr, w.DL, sg::Store{Q + r0, 1, m, 0}, w.sc, w.status + kErr, spin_ns, s)) != cudaSuccess) return e;
   }
   return cudaSuccess;
 }
 
 // The call's status once its work is enqueued (opts->sync): [0] A_S is rank
-// deficient, [1] a product's wait ran out.
+// deficient, [kErr] a product's wait ran out (where css_read_status looks).
 css_status finish(const int* status, const css_opts& o, cudaStream_t s) {
   if (!o.sync) return CSS_OK;
-  int st[2] = {0, 0};
+  int st[kErr + 1] = {};
   if (cudaMemcpyAsync(st, status, sizeof(st), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess)
     return CSS_ERR_CUDA;
-  if (st[1]) return (css_status)st[1];
+  if (st[kErr]) return (css_status)st[kErr];
   return st[0] ? CSS_ERR_INVALID_ARG : CSS_OK;   // A_S is rank deficient
 }
 
@@ -462,7 +464,7 @@ __global__ void das_kernel(const double* __restrict__ P, const double* __restric
 }
 
 struct BwLayout {
-  int* status;   // [0] A_S is rank deficient, [1] error of the products
+  int* status;   // [0] A_S is rank deficient, [kErr] error of the products
   double *AS, *Q, *Psum, *loss_part;
   OrthSpace o;
   long long cols, rows;   // of a part
@@ -517,9 +519,10 @@ css_status run_backward(const TA* A, int m, int n, long long lda, const int* sel
   constexpr int dt = sizeof(TA) == 8 ? CSS_F64 : sizeof(TA) == 4 ? CSS_F32 : CSS_BF16;
   const unsigned long long spin = o.spin_budget_ns ? o.spin_budget_ns : 2000000000ull;
   const int parts = dt == CSS_F64 ? kLossBlocks : sg::residual_parts();
-  cudaMemsetAsync(L.status, 0, 2 * sizeof(int), s);
+  cudaMemsetAsync(L.status, 0, (kErr + 1) * sizeof(int), s);
+  L.sc.stall = L.o.sc.stall = o.test_unmet_wait == 2;
   cudaMemsetAsync(L.loss_part, 0, parts * sizeof(double), s);
-  int* err = L.status + 1;
+  int* err = L.status + kErr;
   const long long mk = (long long)m * k;
   gather_cols_kernel<TA><<<(unsigned)((mk + 255) / 256), 256, 0, s>>>(A, lda, m, sel, k, L.AS);
   if (orth(L.AS, m, k, L.Q, L.o, spin, s) != cudaSuccess) return CSS_ERR_CUDA;
@@ -606,14 +609,15 @@ css_status run_embed(const TA* A, int m, int n, long long lda, const int* sel, i
                      long long ldq, double* W, long long ldw, EmbLayout& L, const css_opts& o,
                      cudaStream_t s) {
   constexpr int dt = sizeof(TA) == 8 ? CSS_F64 : sizeof(TA) == 4 ? CSS_F32 : CSS_BF16;
-  cudaMemsetAsync(L.status, 0, 2 * sizeof(int), s);
+  cudaMemsetAsync(L.status, 0, (kErr + 1) * sizeof(int), s);
+  L.sc.stall = L.o.sc.stall = o.test_unmet_wait == 2;
   const long long ml = (long long)m * l;
   const unsigned gb = (unsigned)((ml + 255) / 256);
   gather_cols_kernel<TA><<<gb, 256, 0, s>>>(A, lda, m, sel, l, L.AS);
   const unsigned long long spin = o.spin_budget_ns ? o.spin_budget_ns : 2000000000ull;
   if (orth(L.AS, m, l, L.Q1, L.o, spin, s) != cudaSuccess || orth(L.Q1, m, l, L.Q, L.o, spin, s) != cudaSuccess)
     return CSS_ERR_CUDA;
-  if (W && w_product(L.Q, A, dt, lda, m, n, l, W, ldw, 1, L.DQ, false, L.DA, L.sc, L.status + 1, spin, s) != cudaSuccess)
+  if (W && w_product(L.Q, A, dt, lda, m, n, l, W, ldw, 1, L.DQ, false, L.DA, L.sc, L.status + kErr, spin, s) != cudaSuccess)
     return CSS_ERR_CUDA;
   if (Qout) copy_cols_kernel<<<gb, 256, 0, s>>>(L.Q, m, l, Qout, ldq);
   if (cudaGetLastError() != cudaSuccess) return CSS_ERR_CUDA;

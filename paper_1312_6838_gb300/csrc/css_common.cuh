@@ -16,12 +16,19 @@ struct DevStatus {
   int32_t code;            // 0 = ok, else a css_status error value
   int32_t rank_exhausted;  // number of units that stopped early
   int32_t where;           // id of the wait that timed out (diagnostic)
-  int32_t stall_where;     // test hook: this barrier id waits for one arrival too many (0 = none)
+  int32_t stall_where;     // test hook: the wait of this id waits for what never comes (0 = none)
   uint64_t spin_budget_ns;
 };
 
 constexpr size_t kWsAlign = 256;
 constexpr size_t kStatusBytes = 256;
+// Byte offset, inside the 256-byte status slot at the start of every
+// workspace, of the tensor-core kernels' error flag.  A greedy launch resets
+// only the DevStatus at offset 0, so the flag survives until css_read_status
+// or the end of the call reads it.
+constexpr size_t kAuxErrOffset = 128;
+static_assert(sizeof(DevStatus) <= kAuxErrOffset && kAuxErrOffset + sizeof(int) <= kStatusBytes,
+              "the flag sits in the status slot, after the DevStatus");
 
 inline size_t align_up(size_t x, size_t a = kWsAlign) { return (x + a - 1) / a * a; }
 

@@ -115,6 +115,7 @@ __device__ void build_q(const EstArgs& A, unsigned long long* log, float* Qg) {
       xb[q] = b == warp * 4 + q ? 1.f : 0.f;
     }
     const uint64_t t0 = globaltimer_ns();
+    const bool stall = A.st->stall_where == kRotationWait;   // test hook
     bool stop = false;   // every warp still meets the others below
     for (int r0 = 0; r0 < kR && !stop; r0 += kBatch) {
       float2 v[kBatch];
@@ -124,12 +125,13 @@ __device__ void build_q(const EstArgs& A, unsigned long long* log, float* Qg) {
         for (int i = 0; i < kBatch; ++i) v[i] = get_rotation(log + (r0 + i) * kB + lane);
 #pragma unroll
         for (int i = 0; i < kBatch; ++i) have &= v[i].x != 0.f;
+        if (stall) have = false;
         if (__all_sync(0xffffffffu, have)) break;
         if ((spins & 63u) == 0u) {
           if (ld_volatile_i32(&A.st->code) != 0) {
             stop = true;
           } else if (globaltimer_ns() - t0 > A.st->spin_budget_ns) {
-            set_error(A.st, (int32_t)CSS_ERR_TIMEOUT, 46);
+            set_error(A.st, (int32_t)CSS_ERR_TIMEOUT, kRotationWait);
             stop = true;
           }
         }

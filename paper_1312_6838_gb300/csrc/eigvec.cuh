@@ -15,6 +15,7 @@ struct Estimate {
   unsigned long long* log;     // the rotations of every block pair's sweep
   uint32_t *bar, *most;        // zeroed before the launch (kEstimateZeroed words from bar)
 };
+constexpr int kRotationWait = 46;   // id of the wait for a sweep's rotations
 constexpr int kEstimateSweeps = 12;
 constexpr int kEstimateZeroed = 32 + 2 * kEstimateSweeps;
 

@@ -48,6 +48,6 @@ size_t css_f0_f64_bytes(int64_t m, int64_t n);
 // digits too, without which FP64 runs the kernels above).
 size_t select_least_workspace(int dtype, int64_t m, int64_t n, int32_t k);
 cudaError_t css_f0_f64(const double* A, long long lda, int m, int n, double* C, long long ldc, void* scratch,
-                       double* f, int* err, unsigned long long spin_ns, cudaStream_t s);
+                       double* f, int* err, unsigned long long spin_ns, cudaStream_t s, int stall);
 
 }  // namespace css

@@ -73,9 +73,10 @@ size_t css_f0_f64_bytes(int64_t m, int64_t n) {
 }
 
 cudaError_t css_f0_f64(const double* A, long long lda, int m, int n, double* C, long long ldc, void* scratch,
-                       double* f, int* err, unsigned long long spin_ns, cudaStream_t s) {
+                       double* f, int* err, unsigned long long spin_ns, cudaStream_t s, int stall) {
   WsCarver c(scratch, (size_t)-1);
   Layout L = carve(c, m, n);
+  L.sc.stall = stall;
   cudaError_t e = cudaSuccess;
   for (long long c0 = 0; e == cudaSuccess && c0 < n; c0 += L.part_k) {
     const sg::Source rows{A + c0 * lda, CSS_F64, 1, lda, m, (int)std::min(L.part_k, n - c0)};

@@ -28,6 +28,7 @@
 // of FP64 arithmetic (two lanes per clock and SM) and a grid barrier each.
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <vector>
 
 #include "css_common.cuh"
@@ -523,7 +524,12 @@ extern "C" css_status css_lowrank(const double* W, int64_t ldw, const double* Q,
 
   DevStatus hs{};
   hs.spin_budget_ns = o.spin_budget_ns ? o.spin_budget_ns : 2000000000ull;
-  cudaError_t e = cudaMemcpyAsync(L.st, &hs, sizeof(hs), cudaMemcpyHostToDevice, s);
+  hs.stall_where = o.test_unmet_wait == 1 ? kRotationWait : 0;
+  L.sc.stall = o.test_unmet_wait == 2;
+  // (the whole status slot: css_read_status also looks at kAuxErrOffset)
+  char slot[kStatusBytes] = {};
+  std::memcpy(slot, &hs, sizeof(hs));
+  cudaError_t e = cudaMemcpyAsync(L.st, slot, sizeof(slot), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(L.flags, 0, sizeof(int) * (kMaxSweeps + 4), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(L.bar, 0, sizeof(uint32_t) * 64, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(L.info, 0, sizeof(int) * 64, s);

@@ -317,6 +317,7 @@ struct Args {
   Residual r;
   int* err;
   unsigned long long spin_ns;
+  int stall;           // test hook: the epilogue first waits on a phase nothing completes
 };
 
 struct Item {
@@ -492,7 +493,8 @@ __global__ void __launch_bounds__(kThreads, 1) slice_gemm_kernel(const __grid_co
   uint64_t* acc_full = empty + kStages;
   uint64_t* acc_empty = acc_full + 1;      // one per accumulator
   uint64_t* done = acc_empty + 4;
-  uint32_t* s_tmem = (uint32_t*)(done + 1);
+  uint64_t* never = done + 1;
+  uint32_t* s_tmem = (uint32_t*)(never + 1);
   int* s_chunk = (int*)(s_tmem + 1);       // accumulators in use | last chunk of the half << 4
   int* s_ns = s_chunk + 1;                 // per stage: slices of X | of Y << 8
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -506,6 +508,7 @@ __global__ void __launch_bounds__(kThreads, 1) slice_gemm_kernel(const __grid_co
     mbar_init(smem_u32(acc_full), 2);      // the MMAs' commit, and the issuer's own arrival
     for (int g = 0; g < 4; ++g) mbar_init(smem_u32(&acc_empty[g]), kEpiWarps);
     mbar_init(smem_u32(done), 1);
+    mbar_init(smem_u32(never), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
@@ -661,6 +664,7 @@ __global__ void __launch_bounds__(kThreads, 1) slice_gemm_kernel(const __grid_co
     const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(ch * 64);
     uint32_t chunk = 0;
     bool ok = true;
+    if (P.stall) ok = mbar_wait_warp(smem_u32(never), 0u, P.err, P.spin_ns);
     double loss = 0.0;            // residual: ||R||^2 of this thread's entries
     for (int it = blockIdx.x; ok && it < items; it += gridDim.x) {
       const Item w = item_of(P, it);
@@ -1022,6 +1026,7 @@ cudaError_t gemm(const Digits& X, const Digits& Y, const Store& st, const Scratc
   P.sx = sx;
   P.sy = sy;
   P.part = w.part;
+  P.stall = w.stall;
   P.lower = st.lower;
   if (st.lower) P.tiles = P.tn * (P.tn + 1) / 2;
   const size_t words = sum_words(P.M, P.N, P.K, P.lower);
@@ -1048,6 +1053,7 @@ cudaError_t gemm_residual(const Digits& X, const Digits& Y, const Residual& r, c
                           unsigned long long spin_ns, cudaStream_t s) {
   Args P = base_args(X, Y, err, spin_ns);
   P.part = w.part;
+  P.stall = w.stall;
   P.r = r;
   return launch_gemm<kEpResidual>(P, s);
 }

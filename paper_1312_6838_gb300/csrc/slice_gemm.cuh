@@ -60,6 +60,7 @@ struct Scratch {
   long long* part;
   unsigned long long* sums;
   size_t cap;           // 8-byte words of sums
+  int stall;            // test hook: the products also wait on a phase nothing completes
 };
 // Words of integer sums that an M x N product over K can use (0: none).
 size_t sum_words(long long M, long long N, long long K, int lower);
