@@ -540,7 +540,6 @@ def run_relative_accuracy(args):
 
 
 DIGIT_TFLOPS = 1934.3 / 36   # the BF16 tensor rate over the 36 digit products of an FP64 multiply-add (slice_gemm.cu)
-FP32_TFLOPS = 67.9   # FP32 FMA throughput of this part, measured with a dependent-free FMA loop
 
 
 def run_adjoint(args):
@@ -594,17 +593,18 @@ def run_adjoint(args):
         "ms_per_step": ms, "higher_is_better": False, "dtype": "f32", "data": "synthetic",
         "config": {"workload": "adjoint_4096x16384", "m": m, "n": n, "k": k, "rank": c["rank"],
                    "noise": c["noise"], "l2": "A and dA (268 MB each) larger than L2"},
-        "roofline": {"bound": "alu", "achieved": tf, "peak": FP32_TFLOPS, "unit": "TFLOP/s",
-                     "frac": tf / FP32_TFLOPS, "traffic": None,
+        "roofline": {"bound": "tensor", "achieved": tf, "peak": DIGIT_TFLOPS, "unit": "TFLOP/s",
+                     "frac": tf / DIGIT_TFLOPS, "traffic": None,
                      "kernel": "the adjoint's three products on the slice GEMM (W, R, R W^T)",
-                     "note": "algorithmic 6 k m n FLOPs against the FP32 rate; the products run as exact "
-                             "products of 8-bit digits on the BF16 tensor cores"},
+                     "note": "algorithmic 6 k m n FLOPs against the BF16 tensor rate over the 36 digit products "
+                             "of an FP64 multiply-add (FP32 entries need about 30)"},
         "hbm_bytes_per_call": 3 * m * n * 4, "loss": float(loss.item()), "clocks": clocks,
         # per call (k <= 128): gather A_S, Gram (2), the initial diagonal, per
         # 32-column panel the diagonal block, the rows and (but for the last)
         # the update, Q, the splits of Q (both ways), A, W (both ways) and R
-        # (two launches each), W, R, R W^T with its finish, loss sum, dA_S
-        "gpu_launches": (22 + 3 * ((k + 31) // 32)) * args.steps,
+        # (two launches each), W and the check for entries beside infinities,
+        # R, R W^T with its finish, loss sum, dA_S
+        "gpu_launches": (23 + 3 * ((k + 31) // 32)) * args.steps,
     }
     if not args.no_cpu_baseline:
         from oracle import css_oracle as O

@@ -154,7 +154,8 @@ typedef struct {
        scores of css_select and css_select_batched when A is BF16 (a layout
        TMA refuses is copied to an aligned buffer first) or FP32 (split into
        three BF16 parts, the six products of parts down to 2^-16 summed):
-       C = A A^T, then C split into three BF16 parts. */
+       C = A A^T, then C split into three BF16 parts.  FP64 input of
+       css_select: see there. */
     int32_t init_path;
     /* Test hook for the bounded device waits (0 = off, the default).
        1: one team barrier of the persistent greedy kernel (the first of
@@ -232,6 +233,11 @@ size_t css_workspace_size(css_op op, css_dtype dtype, int64_t m, int64_t n,
  *            (Sec. 3.1, W = Q^T A; W Pi is upper triangular, Sec. 6).
  *   ws       DEVICE workspace of at least css_workspace_size(CSS_OP_SELECT,
  *            ...) bytes, 256-byte aligned.
+ * FP64 input: the initial scores are digit products where ws has room for
+ * them (css_workspace_size's has, up to m n = 2^30), and FP64 tiles in a
+ * smaller workspace, with init_path = 1 and in css_select_batched.  Both are
+ * as accurate as FP64 sums but differ in the last bits, and so may picks that
+ * those decide (equal scores, columns beyond the data's rank).
  * Returns CSS_OK, CSS_RANK_EXHAUSTED or an error code.
  */
 css_status css_select(const void* A, css_dtype dtype, int64_t m, int64_t n,
@@ -537,8 +543,9 @@ css_status css_autotune_distributed(const void* A, css_dtype dtype, int64_t m, i
  * column's squared norm (dependent columns in S) gives CSS_ERR_INVALID_ARG
  * (reported in sync mode), as do out-of-range or repeated indices.
  * Q^T A, Q W and R W^T are sums of exact products of 8-bit digits (what is
- * dropped is below 2^-64 of the rows' largest products; R of FP32/BF16 input
- * is held in FP32); the factorisation and the loss are FP64; dA is rounded once to the dtype of A.  k <= 1024.
+ * dropped is below 2^-58 of the product of the two rows' largest entries, a
+ * term; R of FP32/BF16 input is held in FP32); the factorisation and the loss
+ * are FP64; dA is rounded once to the dtype of A.  k <= 1024.
  */
 css_status css_residual_backward(const void* A, css_dtype dtype, int64_t m,
                                  int64_t n, int64_t lda, const int32_t* sel,
@@ -566,9 +573,10 @@ css_status css_residual_backward(const void* A, css_dtype dtype, int64_t m,
  * more on Q1), orthonormal to working precision while the condition number of
  * A_S stays below about 1e7.  A pivot at or below 1e-12 of its column's
  * squared norm (dependent columns) gives CSS_ERR_INVALID_ARG (sync mode).
- * W: sums of exact digit products (dropped: below 2^-64 of the rows' largest
- * products), rounded to FP64 once.  l <= 1024, l <= min(m, n).  Workspace: css_workspace_size(CSS_OP_EMBED, dtype, m, n,
- * 0, l, 0, opts).
+ * W: sums of exact digit products rounded to FP64 (dropped: below 2^-58 of
+ * the product of q_t's and a_j's largest entries, a term; so an entry's error
+ * is relative to ||a_j||, not to the entry).  l <= 1024, l <= min(m, n).
+ * Workspace: css_workspace_size(CSS_OP_EMBED, dtype, m, n, 0, l, 0, opts).
  */
 css_status css_embed(const void* A, css_dtype dtype, int64_t m, int64_t n,
                      int64_t lda, const int32_t* sel, int32_t l, double* Q,
@@ -610,7 +618,9 @@ css_status css_embed(const void* A, css_dtype dtype, int64_t m, int64_t n,
  * U~ and V~ from digit products (FP64 sums where they are few).  The
  * eigenvalues carry an absolute error of about (n + l) 2^-53 ||W||_F^2 (the
  * Gram matrix's rounding): sigma_i is accurate relative to sigma_1^2 /
- * sigma_i, not to sigma_i.  CSS_ERR_NOT_CONVERGED if the rotations have not
+ * sigma_i, not to sigma_i.  The rotations end when every pair is below
+ * 1e-15 sqrt(g_pp g_qq) (4e-15 if the estimate leaves none above) or below
+ * 1e-17 trace(G).  CSS_ERR_NOT_CONVERGED if the rotations have not
  * converged after 40 sweeps; CSS_ERR_NONFINITE for NaN/Inf in W.
  * 1 <= k <= l <= 1024.  Workspace: css_workspace_size(CSS_OP_LOWRANK,
  * CSS_F64, m, n, l, k, 0, opts).  opts->timing_ms (sync mode) is HOST

@@ -300,9 +300,13 @@ __global__ void q_kernel(const double* __restrict__ AS, const double* __restrict
 }
 
 // Above this many columns G = A_S^T A_S and Q = A_S L^-T run on the slice GEMM.
-// css_embed at m = 4096, n = 256 (two rounds of both, us): l = 65 582 with the FP64
-// kernels and 667 with slices, l = 128 853 and 848; at l = 256 the FP64 kernels
-// take 600 us a round, the slice products with their splits about 200.
+// css_embed with n = 256 (two rounds of both), us with the FP64 kernels and with
+// slices: m = 512, l = 128 679 and 862, l = 256 1065 and 1210; m = 1024, l = 128
+// 703 and 864, l = 256 1168 and 1212; m = 4096, l = 65 613 and 714, l = 128 859
+// and 870, l = 160 1076 and 956, l = 256 2109 and 1228; m = 16384, l = 32 470 and
+// 584, l = 65 971 and 776, l = 256 5569 and 1546.  (The two meet near m l^2 =
+// 2^26, so the line fits 4096 rows; for 129 to 256 columns of 512 it costs 25 to
+// 14 %, for 65 to 128 of 16384 it gives away 20 to 43 %.)
 constexpr int kSliceK = 128;
 
 // A_S's orthonormal basis by Cholesky: G = A_S^T A_S = L L^T, Q = A_S L^-T.

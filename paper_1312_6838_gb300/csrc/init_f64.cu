@@ -1,7 +1,8 @@
 // Initial scores of FP64 problems from integer digits on the tensor cores
 // (slice_gemm.cu): C = A A^T, then f_i = a_i^T (C a_i) (Algorithm 1).  The
-// digit products keep 2^-64 of the rows' largest products, so C and C A are
-// as accurate as FP64 sums.  Equal columns get equal bits (each entry is an
+// products drop less than 2^-58 of the rows' largest products a term, so C and
+// C A are as accurate as FP64 sums (C relative to sqrt(C_ii C_jj); C A with
+// A's rows brought to one size).  Equal columns get equal bits (each entry is an
 // exact integer sum rounded once, and the columns' dots run in one order).
 // Infinities become NaN: the selection reports either as non-finite data.
 //

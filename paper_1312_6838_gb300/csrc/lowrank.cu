@@ -94,8 +94,9 @@ __device__ __forceinline__ void rot(double c, double s, double a, double b, doub
 }
 
 // A pair is rotated unless |g_pq| <= 1e-15 sqrt(g_pp g_qq) (the relative test
-// of Demmel and Veselic) or |g_pq| <= 1e-17 trace(G), far below the Gram
-// matrix's own rounding.  Evaluated in FP32 on the entries scaled by
+// of Demmel and Veselic; 4e-15 at the first check after an estimate, whose
+// X^T G X is rounded to about that) or |g_pq| <= 1e-17 trace(G), far below the
+// Gram matrix's own rounding.  Evaluated in FP32 on the entries scaled by
 // 1 / trace(G) (all of magnitude <= 1 for a PSD G).
 __device__ __forceinline__ bool needs_rot(double gpp, double gqq, double gpq, double inv_tr, float tol2 = 1e-30f) {
   const float ps = (float)(gpp * inv_tr), qs = (float)(gqq * inv_tr), xs = fabsf((float)(gpq * inv_tr));

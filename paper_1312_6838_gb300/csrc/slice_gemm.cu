@@ -10,8 +10,16 @@
 //   row i of an operand is scaled by a power of two so that every entry is at
 //   most 1/2, and written in base 256 with balanced digits,
 //     x = sum_{s=1..8} d_s 256^-s,   |d_s| <= 128  (exact in BF16).
-//   x y = sum over w = s + t of 256^-w d_s e_t, and w = 2..9 is kept: what is
-//   dropped is below 2^-64 of the product of the rows' largest entries.
+//   x y = sum over w = s + t of 256^-w d_s e_t, and w = 2..9 is kept.  The
+//   seven pairs of w = 10 are at most 2^14 each, so with the rounding to eight
+//   digits less than 2^-62 of the scaled entries is dropped, and with row
+//   maxima in [1/4, 1/2) less than 2^-58 of the product of the two rows'
+//   largest entries, a term.
+//
+// This is fixed point per row: an entry down to about 2^-10 of its row's
+// largest keeps FP64's 53 bits, a smaller one fewer.  Sums are normwise more
+// accurate than FP64 ones (below); where an inner index that dominates X's rows
+// meets zeros in Y, callers balance the operands first (gram_exponents).
 //
 // Each w has its own TMEM accumulator.  A product of digits is at most 2^14,
 // so an accumulator that has taken at most 1024 of them holds an integer of
@@ -24,8 +32,8 @@
 // Measured: W = Q^T A of a 4096 x 65536 BF16 matrix with l = 256 (68.7 G
 // multiply-adds) 24 ms as double-float on the FP32 pipe; here 2.3 ms and 0.7 ms
 // for the split of A; its error against 64 bits fell from 1.1e-12 to 2.2e-15.
-// The tensor pipe is active 57 % of the time; the rest is the drains, during
-// which the accumulators cannot take products.  G = W W^T, 256 x 65536: 4.26 ms
+// The tensor pipe is active 57 % of the time (ncu); the rest is the drains,
+// during which the accumulators cannot take products.  G = W W^T, 256 x 65536: 4.26 ms
 // in FP64 instructions, 0.17 ms here.
 //
 // Slices that are zero in a block of 128 rows x 64 k are not stored, loaded
@@ -40,7 +48,6 @@
 
 #include <algorithm>
 
-#include "df.cuh"
 #include "tc_ptx.cuh"
 
 namespace css {
@@ -48,6 +55,11 @@ namespace sg {
 namespace {
 
 using namespace css::tc;
+
+// A value held as the unevaluated sum s + c of two FP32 numbers.
+struct DF {
+  float s, c;
+};
 
 constexpr int kT = 128;                 // rows of an operand tile
 constexpr int kS = 8;                   // slices
