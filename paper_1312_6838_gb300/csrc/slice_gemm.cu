@@ -821,17 +821,27 @@ __global__ void __launch_bounds__(kThreads, 1) slice_gemm_kernel(const __grid_co
             // r = a - vh - vl as a normalised pair
             const float s = a - vh, bb = s - a;
             const float t = ((a - (s - bb)) + (-vh - bb)) - vl;
-            const float rh = s + t, rl = t - (rh - s);
-            rhi[jj] = rh;
-            rlo[jj] = rl;
+            float rh = s + t;
+            const float rl = t - (rh - s);
+            const bool pair = fabsf(s) < 0x1p126f;   // else near or beyond FP32's limit, or a NaN
+            const auto wide = [&] { return pair ? (double)rh + (double)rl : ((double)a - (double)vh) - (double)vl; };
+            if (pair) {
+              rhi[jj] = rh;
+              rlo[jj] = rl;
+            } else {
+              const double r = wide();
+              loss = fma(r, r, loss);
+              rh = (float)r;
+            }
             if (R.R) R.R[(long long)c * P.M + row] = rh;
             if (R.dA) {
               float g;
-              if (g_plain) {
-                const float gp = gh * rh;
-                g = gp + (fmaf(gh, rh, -gp) + (gh * rl + gl * rh));
+              if (g_plain && pair) {
+                g = gh * rh;
+                // (an infinite product would meet its negative in the low part)
+                if (fabsf(g) < __int_as_float(0x7f800000)) g += fmaf(gh, rh, -g) + (gh * rl + gl * rh);
               } else {
-                g = (float)(R.g2 * ((double)rh + (double)rl));
+                g = (float)(R.g2 * wide());
               }
               if (f32) ((float*)R.dA)[(long long)c * R.ldda + row] = g;
               else ((__nv_bfloat16*)R.dA)[(long long)c * R.ldda + row] = __float2bfloat16_rn(g);
