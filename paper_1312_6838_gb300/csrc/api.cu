@@ -567,8 +567,12 @@ int team_ctas_for(int64_t n, int64_t m, int dt = CSS_BF16) {
   // enough CTAs to keep the column stream and the FP64 pivot work spread out.
   // Algorithm 1's fused step of FP64 input is bound by each SM's FP64 rate (two lanes a
   // clock), so it takes an SM per tile of eight columns: 500 x 1000, k = 50,
-  // on 32 CTAs (the FP32 rule) 17.9 us a step, on 64 9.9, on 128 6.2; 50 picks
-  // 2.57 / 2.13 / 1.89 ms
+  // on 32 CTAs (the FP32 rule) 17.9 us a step, on 64 9.9, on 128 6.2.  Whole
+  // calls, us by the FP32 rule and by this one (CTAs): 32 x 64, k = 8 553 and
+  // 493 (2, 8); 64 x 128, k = 8 605 and 519 (4, 16); 300 x 600, k = 50 2446 and
+  // 2034 (19, 75); 500 x 1000 2761 and 2152; 200 x 2000, k = 32 2791 and 1376
+  // (16, 152); 1000 x 8000, k = 64 12882 and 9329 (63, 152); numbers between
+  // the two were between them
   int64_t a = dt == CSS_F64 ? (n + 7) / 8 : (n + 127) / 128;
   int64_t b = (m + 15) / 16;
   return (int)std::max<int64_t>(1, std::max(a, b));

@@ -9,6 +9,9 @@
 // The FP64 tiles of init_simt.cu are bound by an SM's FP64 rate (two lanes a
 // clock), and a small problem has too few of them: 500 x 1000 took 1.63 ms
 // with 36 blocks in C = A A^T; here 0.23 ms; 1024 x 8192: 23.4 -> 1.03 ms.
+// Whole selections, us with the tiles and here: 64 x 128, k = 8 587 and 519;
+// 1000 x 500, k = 50 4114 and 2782; 64 x 20000, k = 16 21955 and 1215; the tiles
+// only win at a single tile (32 x 64, k = 8: 468 and 493).
 #include <algorithm>
 
 #include "init.cuh"

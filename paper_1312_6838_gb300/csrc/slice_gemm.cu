@@ -32,8 +32,10 @@
 // Measured: W = Q^T A of a 4096 x 65536 BF16 matrix with l = 256 (68.7 G
 // multiply-adds) 24 ms as double-float on the FP32 pipe; here 2.3 ms and 0.7 ms
 // for the split of A; its error against 64 bits fell from 1.1e-12 to 2.2e-15.
-// The tensor pipe is active 57 % of the time (ncu); the rest is the drains,
-// during which the accumulators cannot take products.  G = W W^T, 256 x 65536: 4.26 ms
+// The tensor pipe is active 57 % of the time there (ncu; 61 to 66 % with k = 128
+// and in Gram matrices), and 27 % in the residual's product, whose epilogue reads
+// A and writes R and dA; the rest is the drains, during which the accumulators
+// cannot take products.  G = W W^T, 256 x 65536: 4.26 ms
 // in FP64 instructions, 0.17 ms here.
 //
 // Slices that are zero in a block of 128 rows x 64 k are not stored, loaded
