@@ -266,9 +266,15 @@ css_status prepare_units(const Header& h, std::vector<UnitDesc>& units, const st
     d.cand_idx = h.cand_idx + d.cta0;
     d.tile_ctr = h.tile_ctr + 2 * d.cta0;
     // split the last tiles of each fused step: at most one per warp of the team
-    int widest = 0;
-    for (int q = d.u_begin; q < d.u_end; ++q)
+    int widest = 0, tallest = 0;
+    for (int q = d.u_begin; q < d.u_end; ++q) {
       widest = std::max(widest, (units[P.order[q]].n + tile_cols - 1) / tile_cols);
+      tallest = std::max(tallest, units[P.order[q]].m);
+    }
+    // rows of a chunk: a multiple of a warp's step of 16-byte vectors
+    const int step = 32 * 16 / (dt == CSS_F64 ? 8 : dt == CSS_F32 ? 4 : 2);
+    const int rch = ((tallest + kSplitR - 1) / kSplitR + step - 1) / step * step;
+    d.turn = tallest <= (kSplitR - 1) * rch;
     const int cap = std::min({widest, d.ncta * (threads / 32) / std::max(1, split_share),
                               h.split_slots - split_used});
     d.split_cap = std::max(cap, 0);

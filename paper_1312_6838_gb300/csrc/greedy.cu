@@ -497,8 +497,16 @@ __device__ __forceinline__ void update_column(const UnitDesc& u, int t, int p, d
   }
 }
 
-// A warp's first unit of work in a fused step.
-__device__ __forceinline__ int first_unit(int rank, int ncta, int warp) { return warp * ncta + rank; }
+// A warp's first unit of work in a fused step: a bijection onto the first
+// ncta x NW units.  Where columns are so short that a split tile's last chunk is
+// empty, they are turned by one CTA from warp to warp (`turn`, 0 or 1): a team
+// whose size is a multiple of kSplitR would have all chunks with rows on a few of
+// its CTAs (FP64 GCSS of 64 x 128, k = 32, on four: 1.57 ms with drawn first
+// units, 1.73 fixed, 1.53 with the turn).  Elsewhere it gains nothing (FP64 GCSS
+// of 1000 x 1000: 4.80 without and 5.13 with it).
+__device__ __forceinline__ int first_unit(int rank, int ncta, int warp, int turn) {
+  return warp * ncta + (rank + turn * warp) % ncta;
+}
 
 // --------------------------------------------------------- fused step (K1) --
 // Work units come from a team-wide counter: first whole tiles of CW columns,
@@ -546,7 +554,7 @@ __device__ void fused_step(const Ctx<typename AccOf<TA>::type>& x, const UnitDes
   const int W = x.ncta * NW;
   uint32_t* ctr = (x.ncta == 1 ? x.sctr : x.team->tile_ctr) + (t & 1);
   const bool more = W < nunits;
-  int unit = first_unit(x.rank, x.ncta, x.warp);
+  int unit = first_unit(x.rank, x.ncta, x.warp, x.team->turn);
   // short columns (at most 2 KB): a tile's loads are one or two dependent
   // memory round trips, so the warp asks L2 for the columns of its next unit
   // as soon as it draws it (one bulk prefetch per column).  Measured on the
@@ -759,7 +767,7 @@ template <typename TA>
 __device__ __forceinline__ void prime_ring(const Ctx<typename AccOf<TA>::type>& x, const UnitDesc& u, uint64_t pol) {
   const StepShape<TA> sh(u, x.team->split_cap);
   Feed<TA> fd;
-  fd.at(u, sh, first_unit(x.rank, x.ncta, x.warp), x.lane);
+  fd.at(u, sh, first_unit(x.rank, x.ncta, x.warp, x.team->turn), x.lane);
   if (fd.unit >= sh.nunits) return;
 #pragma unroll 1
   for (int i = 0; i < kRingSlots; ++i) {
@@ -794,7 +802,7 @@ __device__ void fused_step_ring(const Ctx<typename AccOf<TA>::type>& x, const Un
   int drawn = sh.nunits;
   if (more && lane == 0) drawn = W + (int)atomicAdd(ctr, 1u);
   Feed<TA> fd;
-  fd.at(u, sh, first_unit(x.rank, x.ncta, x.warp), lane);
+  fd.at(u, sh, first_unit(x.rank, x.ncta, x.warp, x.team->turn), lane);
   uint32_t tslot = 0;
   // the step just copied (or skipped: already there) as unit * 2 + last, -1: none
   auto next_unit = [&]() {

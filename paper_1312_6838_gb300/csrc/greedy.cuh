@@ -57,7 +57,7 @@ struct TeamDesc {
   void* split_part;
   uint32_t* split_done;             // split_cap arrival counters (zero between uses)
   int split_cap;
-  int pad_;
+  int turn;                         // see first_unit
 };
 
 #ifndef CSS_SPLIT_ROWS
