@@ -601,10 +601,10 @@ def run_adjoint(args):
         "hbm_bytes_per_call": 3 * m * n * 4, "loss": float(loss.item()), "clocks": clocks,
         # per call (k <= 128): gather A_S, Gram (2), the initial diagonal, per
         # 32-column panel the diagonal block, the rows and (but for the last)
-        # the update, Q, the splits of Q (both ways), A, W (both ways) and R
-        # (two launches each), W and the check for entries beside infinities,
-        # R, R W^T with its finish, loss sum, dA_S
-        "gpu_launches": (23 + 3 * ((k + 31) // 32)) * args.steps,
+        # the update, Q, the splits of Q, A, W and R (two launches each), those
+        # of Q and W by rows of k <= 128 entries (one each), W and the check
+        # for entries beside infinities, R, R W^T with its finish, loss sum, dA_S
+        "gpu_launches": (21 + 3 * ((k + 31) // 32)) * args.steps,
     }
     if not args.no_cpu_baseline:
         from oracle import css_oracle as O

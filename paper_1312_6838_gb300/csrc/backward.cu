@@ -169,7 +169,9 @@ __global__ void __launch_bounds__(256) chol_diag_kernel(double* __restrict__ G, 
     D[r][c] = r < b && c <= r ? G[(long long)(j0 + c) * k + j0 + r] : 0.0;
     V[r][c] = r == c ? 1.0 : 0.0;
   }
-  const double least = t < b ? 1e-12 * diag0[j0 + t] : 0.0;
+  __syncthreads();
+  // (a single panel's initial diagonal is its own)
+  const double least = t < b ? 1e-12 * (diag0 ? diag0[j0 + t] : D[t][t]) : 0.0;
   __syncthreads();
   bool bad = false;
   for (int c = 0; c < b; ++c) {
@@ -203,10 +205,8 @@ __global__ void __launch_bounds__(256) chol_diag_kernel(double* __restrict__ G, 
   if (t == 0 && bad) status[0] = 1;
   for (int e = t; e < kCb * kCb; e += 256) {
     const int r = e % kCb, c = e / kCb;
-    if (r < b && c <= r) {
-      G[(long long)(j0 + c) * k + j0 + r] = D[r][c];
-      X[(long long)(j0 + c) * k + j0 + r] = V[r][c];
-    }
+    if (r < b && c <= r) G[(long long)(j0 + c) * k + j0 + r] = D[r][c];
+    if (r < b && c < b) X[(long long)(j0 + c) * k + j0 + r] = V[r][c];   // (zero above the diagonal)
   }
 }
 
@@ -274,8 +274,12 @@ __global__ void __launch_bounds__(256) chol_update_kernel(double* __restrict__ G
 // Cholesky of the k x k matrix in G (overwritten by L) and L^-1 into Linv
 // (status[0] = 1 for a rank-deficient G).  diag0: k doubles of scratch.
 void chol_inv(double* G, int k, double* Linv, double* diag0, int* status, cudaStream_t s) {
-  cudaMemsetAsync(Linv, 0, (size_t)k * k * sizeof(double), s);
-  chol_save_kernel<<<(k + 255) / 256, 256, 0, s>>>(G, k, diag0);
+  if (k > kCb) {
+    cudaMemsetAsync(Linv, 0, (size_t)k * k * sizeof(double), s);
+    chol_save_kernel<<<(k + 255) / 256, 256, 0, s>>>(G, k, diag0);
+  } else {
+    diag0 = nullptr;
+  }
   for (int j0 = 0; j0 < k; j0 += kCb) {
     const int below = std::max(0, k - j0 - kCb);
     chol_diag_kernel<<<1, 256, 0, s>>>(G, Linv, k, j0, diag0, status);

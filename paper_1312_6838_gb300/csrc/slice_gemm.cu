@@ -170,6 +170,18 @@ __device__ __forceinline__ int k_exp(const int* kexp, int sign, int k, int K) {
   return k < K ? sign * __ldg(kexp + k) : 0;
 }
 
+// Largest biased exponents of this thread's entries of a block, by chunk.
+template <bool KC, bool SC, typename V>
+__device__ __forceinline__ void block_exps(const V (&v)[4][8], const int* kexp, int sign, int k0, int K, int (&best)[4]) {
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      if constexpr (SC) best[q] = max(best[q], scaled_exp(v[q][e], k_exp(kexp, sign, k_of<KC>(k0, q) + e, K)));
+      else best[q] = max(best[q], biased_exp(v[q][e]));
+    }
+}
+
 // Largest biased exponent of every row (ex zeroed before): a block takes 128
 // rows and every gridDim.y-th 64 k of them.  Memory-bound.
 template <typename T, typename V, bool KC, bool VEC, bool SC>
@@ -181,13 +193,7 @@ __global__ void __launch_bounds__(256) row_exp_kernel(const T* __restrict__ p, l
   for (int k0 = blockIdx.y * kKb; k0 < K; k0 += gridDim.y * kKb) {
     V v[4][8];
     load_block<T, V, KC, VEC>(p, rs, ks, rows, K, r0, k0, v);
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        if constexpr (SC) best[q] = max(best[q], scaled_exp(v[q][e], k_exp(kexp, sign, k_of<KC>(k0, q) + e, K)));
-        else best[q] = max(best[q], biased_exp(v[q][e]));
-      }
+    block_exps<KC, SC>(v, kexp, sign, k0, K, best);
   }
   if (KC) {
 #pragma unroll
@@ -207,97 +213,127 @@ __device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) 
 
 // Digits of one block of 128 rows x 64 k; slices are written until what is
 // left can give no digit, and their number goes to ns.  Rows with an infinity
-// or a NaN get zero digits (see restore_kernel).
-template <typename T, typename V, bool KC, bool VEC, bool SC>
+// or a NaN get zero digits (see restore_kernel).  WHOLE: of all k of 128 rows,
+// whose exponents are formed here too (see kWholeK).
+template <typename T, typename V, bool KC, bool VEC, bool SC, bool WHOLE>
 __global__ void __launch_bounds__(256) split_kernel(const T* __restrict__ p, long long rs, long long ks, int rows,
                                                     int K, int k64, int dtype, const int* __restrict__ kexp, int sign,
-                                                    const int* __restrict__ ex, unsigned char* __restrict__ d,
+                                                    int* __restrict__ ex, unsigned char* __restrict__ d,
                                                     unsigned char* __restrict__ ns) {
   // (one grid dimension: K / 64 may exceed the others' 65535)
   const unsigned tiles = (unsigned)(rows + kT - 1) / kT, tile = blockIdx.x % tiles;
-  const int r0 = (int)tile * kT, kb = (int)(blockIdx.x / tiles);
-  V v[4][8];
-  load_block<T, V, KC, VEC>(p, rs, ks, rows, K, r0, kb * kKb, v);
-  unsigned char* out[4];
-  unsigned long long G[4][8];   // FP64: the balanced digits of |x|, biased by 128 but for the first
-  uint32_t neg[4] = {0, 0, 0, 0};
+  const int r0 = (int)tile * kT;
+  int es[4] = {0, 0, 0, 0};
+  if constexpr (WHOLE) {
+    int best[4] = {0, 0, 0, 0};
+    for (int k0 = 0; k0 < K; k0 += kKb) {
+      V v[4][8];
+      load_block<T, V, KC, VEC>(p, rs, ks, rows, K, r0, k0, v);
+      block_exps<KC, SC>(v, kexp, sign, k0, K, best);
+    }
+    if (KC) {
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int rl = KC ? (int)threadIdx.x / 8 + 32 * q : (int)threadIdx.x % 128;
-    const int kc = KC ? (int)threadIdx.x % 8 : (int)threadIdx.x / 128 + 2 * q;
-    out[q] = d + (((long long)tile * k64 + kb) * 4 + kc / 2) * (kS * kSliceBytes) + (kc % 2) * (kT * 16) + rl * 16;
-    const int e = r0 + rl < rows ? ex[r0 + rl] : 0;
-    const bool dead = e >= kExInf;
-    if constexpr (sizeof(V) == 4) {
-      // two factors, so that neither leaves FP32's range
-      const int sh = 8 - scale_exp(e, dtype), h1 = sh / 2;
-      const float f1 = pow2f(h1), f2 = pow2f(sh - h1);
+      for (int q = 0; q < 4; ++q) {
 #pragma unroll
-      for (int i = 0; i < 8; ++i) v[q][i] = dead ? 0.f : v[q][i] * f1 * f2;
-    } else {
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const unsigned long long b = (unsigned long long)__double_as_longlong(v[q][i]);
-        const int be = (int)(b >> 52) & 0x7ff;
-        unsigned long long mant = b & 0xfffffffffffffull;
-        if (be > 0) mant |= 1ull << 52;
-        // |x| 2^(64 - scale), rounded to an integer below 2^63
-        const int ke = SC ? k_exp(kexp, sign, k_of<KC>(kb * kKb, q) + i, K) : 0;
-        const int sh = max(be, 1) + ke - e + 10;
-        unsigned long long F = 0;
-        if (!dead) {
-          if (sh >= 0) F = mant << sh;
-          else if (sh > -64) F = (mant + (1ull << (-sh - 1))) >> -sh;
-        }
-        if (b >> 63) neg[q] |= 1u << i;
-        G[q][i] = F;
+        for (int o = 4; o > 0; o >>= 1) best[q] = max(best[q], __shfl_xor_sync(0xffffffffu, best[q], o));
+        es[q] = best[q];
+        const int row = r0 + threadIdx.x / 8 + 32 * q;
+        if (threadIdx.x % 8 == 0 && row < rows) ex[row] = best[q];
       }
+    } else {
+      __shared__ int s_best[2][kT];
+      s_best[threadIdx.x / kT][threadIdx.x % kT] = max(max(best[0], best[1]), max(best[2], best[3]));
+      __syncthreads();
+      const int row = threadIdx.x % kT, b = max(s_best[0][row], s_best[1][row]);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) es[q] = b;
+      if (threadIdx.x < kT && r0 + row < rows) ex[r0 + row] = b;
     }
   }
-  int s = 0;
-  for (; s < kS; ++s) {
-    int any = 0;
-    if constexpr (sizeof(V) == 4) {
-      const float least = 0.5f * pow2f(-8 * (kS - 1 - s));
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-#pragma unroll
-        for (int i = 0; i < 8; ++i) any |= fabsf(v[q][i]) >= least;
-    } else {
-      const unsigned long long mask = s == 0 ? ~0ull : (1ull << (64 - 8 * s)) - 1;
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-#pragma unroll
-        for (int i = 0; i < 8; ++i) any |= (G[q][i] & mask) != 0;
-    }
-    if (!__syncthreads_or(any)) break;
+  for (int kb = WHOLE ? 0 : (int)(blockIdx.x / tiles), kend = WHOLE ? k64 : kb + 1; kb < kend; ++kb) {
+    V v[4][8];
+    load_block<T, V, KC, VEC>(p, rs, ks, rows, K, r0, kb * kKb, v);
+    unsigned char* out[4];
+    unsigned long long G[4][8];   // FP64: the balanced digits of |x|, biased by 128 but for the first
+    uint32_t neg[4] = {0, 0, 0, 0};
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      uint32_t w[4];
+      const int rl = KC ? (int)threadIdx.x / 8 + 32 * q : (int)threadIdx.x % 128;
+      const int kc = KC ? (int)threadIdx.x % 8 : (int)threadIdx.x / 128 + 2 * q;
+      out[q] = d + (((long long)tile * k64 + kb) * 4 + kc / 2) * (kS * kSliceBytes) + (kc % 2) * (kT * 16) + rl * 16;
+      const int e = WHOLE ? es[q] : r0 + rl < rows ? ex[r0 + rl] : 0;
+      const bool dead = e >= kExInf;
+      if constexpr (sizeof(V) == 4) {
+        // two factors, so that neither leaves FP32's range
+        const int sh = 8 - scale_exp(e, dtype), h1 = sh / 2;
+        const float f1 = pow2f(h1), f2 = pow2f(sh - h1);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        float dg[2];
+        for (int i = 0; i < 8; ++i) v[q][i] = dead ? 0.f : v[q][i] * f1 * f2;
+      } else {
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          const int x = 2 * i + j;
-          if constexpr (sizeof(V) == 4) {
-            const float f = (v[q][x] + 12582912.f) - 12582912.f;   // round to nearest integer
-            v[q][x] = (v[q][x] - f) * 256.f;
-            dg[j] = f;
-          } else {
-            const unsigned long long b = G[q][x] + 0x0080808080808080ull;
-            const uint32_t byte = (uint32_t)(b >> (56 - 8 * s)) & 0xffu;
-            float f = __uint_as_float(0x4b000000u | byte) - (s == 0 ? 8388608.f : 8388736.f);
-            dg[j] = (neg[q] >> x) & 1u ? -f : f;
+        for (int i = 0; i < 8; ++i) {
+          const unsigned long long b = (unsigned long long)__double_as_longlong(v[q][i]);
+          const int be = (int)(b >> 52) & 0x7ff;
+          unsigned long long mant = b & 0xfffffffffffffull;
+          if (be > 0) mant |= 1ull << 52;
+          // |x| 2^(64 - scale), rounded to an integer below 2^63
+          const int ke = SC ? k_exp(kexp, sign, k_of<KC>(kb * kKb, q) + i, K) : 0;
+          const int sh = max(be, 1) + ke - e + 10;
+          unsigned long long F = 0;
+          if (!dead) {
+            if (sh >= 0) F = mant << sh;
+            else if (sh > -64) F = (mant + (1ull << (-sh - 1))) >> -sh;
           }
+          if (b >> 63) neg[q] |= 1u << i;
+          G[q][i] = F;
         }
-        // digits have at most 8 bits, so their upper halves are their BF16
-        w[i] = __byte_perm(__float_as_uint(dg[0]), __float_as_uint(dg[1]), 0x7632);
       }
-      *reinterpret_cast<uint4*>(out[q] + s * kSliceBytes) = make_uint4(w[0], w[1], w[2], w[3]);
     }
+    int s = 0;
+    for (; s < kS; ++s) {
+      int any = 0;
+      if constexpr (sizeof(V) == 4) {
+        const float least = 0.5f * pow2f(-8 * (kS - 1 - s));
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+          for (int i = 0; i < 8; ++i) any |= fabsf(v[q][i]) >= least;
+      } else {
+        const unsigned long long mask = s == 0 ? ~0ull : (1ull << (64 - 8 * s)) - 1;
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+          for (int i = 0; i < 8; ++i) any |= (G[q][i] & mask) != 0;
+      }
+      if (!__syncthreads_or(any)) break;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        uint32_t w[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          float dg[2];
+#pragma unroll
+          for (int j = 0; j < 2; ++j) {
+            const int x = 2 * i + j;
+            if constexpr (sizeof(V) == 4) {
+              const float f = (v[q][x] + 12582912.f) - 12582912.f;   // round to nearest integer
+              v[q][x] = (v[q][x] - f) * 256.f;
+              dg[j] = f;
+            } else {
+              const unsigned long long b = G[q][x] + 0x0080808080808080ull;
+              const uint32_t byte = (uint32_t)(b >> (56 - 8 * s)) & 0xffu;
+              float f = __uint_as_float(0x4b000000u | byte) - (s == 0 ? 8388608.f : 8388736.f);
+              dg[j] = (neg[q] >> x) & 1u ? -f : f;
+            }
+          }
+          // digits have at most 8 bits, so their upper halves are their BF16
+          w[i] = __byte_perm(__float_as_uint(dg[0]), __float_as_uint(dg[1]), 0x7632);
+        }
+        *reinterpret_cast<uint4*>(out[q] + s * kSliceBytes) = make_uint4(w[0], w[1], w[2], w[3]);
+      }
+    }
+    if (threadIdx.x == 0) ns[(long long)tile * k64 + kb] = (unsigned char)s;
   }
-  if (threadIdx.x == 0) ns[(long long)tile * k64 + kb] = (unsigned char)s;
 }
 
 // ------------------------------------------------------------- product -----
@@ -937,17 +973,28 @@ __global__ void __launch_bounds__(256) restore_kernel(const __grid_constant__ Ar
 
 int k_blocks(long long K) { return (int)ceil_div(K, kKb); }
 
+// Up to this many k a block forms a row tile's exponents and digits: one launch
+// instead of three, which is what small calls wait for (css.embed of 64 x 128,
+// l = 8, FP32 229 -> 212 us; css.residual of it 300 -> 267, a launch less of the
+// Cholesky panel in it).
+constexpr int kWholeK = 128;
+
 template <typename T, typename V, bool KC, bool VEC, bool SC = false>
 void launch_split(const Source& src, const Digits& D, cudaStream_t s) {
   const int k64 = k_blocks(src.K);
   const unsigned tiles = (unsigned)ceil_div(src.rows, kT);
   const unsigned ky = (unsigned)std::min<long long>(k64, std::max<long long>(1, ceil_div(152 * 8, tiles)));
   const T* p = (const T*)src.p;
+  if (src.K <= kWholeK) {
+    split_kernel<T, V, KC, VEC, SC, true><<<tiles, 256, 0, s>>>(p, src.rs, src.ks, src.rows, src.K, k64, src.dtype,
+                                                                src.kexp, src.kexp_sign, D.ex, D.d, D.ns);
+    return;
+  }
+  cudaMemsetAsync(D.ex, 0, sizeof(int) * (size_t)src.rows, s);
   row_exp_kernel<T, V, KC, VEC, SC><<<dim3(tiles, ky), 256, 0, s>>>(p, src.rs, src.ks, src.rows, src.K, src.kexp,
                                                                     src.kexp_sign, D.ex);
-  split_kernel<T, V, KC, VEC, SC><<<tiles * (unsigned)k64, 256, 0, s>>>(p, src.rs, src.ks, src.rows, src.K, k64,
-                                                                        src.dtype, src.kexp, src.kexp_sign, D.ex, D.d,
-                                                                        D.ns);
+  split_kernel<T, V, KC, VEC, SC, false><<<tiles * (unsigned)k64, 256, 0, s>>>(
+      p, src.rs, src.ks, src.rows, src.K, k64, src.dtype, src.kexp, src.kexp_sign, D.ex, D.d, D.ns);
 }
 template <typename T, typename V>
 void launch_split_of(const Source& src, const Digits& D, cudaStream_t s) {
@@ -1027,8 +1074,6 @@ cudaError_t split(const Source& src, Digits& D, cudaStream_t s) {
   D.rows = src.rows;
   D.K = src.K;
   D.dtype = src.dtype;
-  cudaError_t e = cudaMemsetAsync(D.ex, 0, sizeof(int) * (size_t)src.rows, s);
-  if (e != cudaSuccess) return e;
   switch (src.dtype) {
     case CSS_F64: launch_split_of<double, double>(src, D, s); break;
     case CSS_F32: launch_split_of<float, float>(src, D, s); break;

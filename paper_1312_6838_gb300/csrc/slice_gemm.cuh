@@ -51,7 +51,7 @@ inline long long part_k(long long rows, long long budget = kDigitBudget) {
 inline long long part_rows(long long K, long long budget = kDigitBudget) {
   return std::max<long long>(128, budget / (1024 * ((K + 63) / 64)) / 128 * 128);
 }
-// Splits src into digits (src.rows <= the carved rows).  Three launches.
+// Splits src into digits (src.rows <= the carved rows).
 cudaError_t split(const Source& src, Digits& D, cudaStream_t s);
 
 // Scratch of gemm: per-CTA partial sums, and the integer sums of a product
