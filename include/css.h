@@ -544,8 +544,9 @@ css_status css_autotune_distributed(const void* A, css_dtype dtype, int64_t m, i
  * (reported in sync mode), as do out-of-range or repeated indices.
  * Q^T A, Q W and R W^T are sums of exact products of 8-bit digits (what is
  * dropped is below 2^-58 of the product of the two rows' largest entries, a
- * term; R of FP32/BF16 input is held in FP32); the factorisation and the loss
- * are FP64; dA is rounded once to the dtype of A.  k <= 1024.
+ * term; R of FP32/BF16 input is held in FP32), in small calls (m n k up to 1e7,
+ * FP64 input 2^19) FP64 sums, compensated for FP64 input; the factorisation and
+ * the loss are FP64; dA is rounded once to the dtype of A.  k <= 1024.
  */
 css_status css_residual_backward(const void* A, css_dtype dtype, int64_t m,
                                  int64_t n, int64_t lda, const int32_t* sel,

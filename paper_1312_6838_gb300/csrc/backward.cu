@@ -430,20 +430,98 @@ cudaError_t w_product(const double* Q, const void* A, int dtype, long long lda, 
   return cudaSuccess;
 }
 
-// FP64 input: V = Q W on entry, R = A - V on return (in place), dA = g2 R when
-// dA != null, and each block's share of ||R||^2 added to its partial sum.
+// ------------------------------------------ products of small calls in FP64 --
+// out(i, j) = sum_q x(i, q) y(j, q) in FP64: 8 x 8 outputs a block, four threads
+// an output (q mod 4), the next 32 q in registers.  COMP: products and sums with
+// their rounding errors (Ogita, Rump and Oishi, SIAM J. Sci. Comput. 26, 2005),
+// so that FP64 input loses nothing against digits; FP32 and BF16 input has its
+// results rounded to FP32 anyway.  Digits take five launches a product, which is
+// what a small call waits for; FP64's two lanes a clock and SM set the other side.
+constexpr int kSo = 8, kSq = 32, kSp = kSq + 4;   // (rows padded: no bank conflicts)
+template <typename TX, bool COMP>
+__global__ void __launch_bounds__(256) small_sums_kernel(const TX* __restrict__ x, long long xr, long long xq,
+                                                         const double* __restrict__ y, long long yr, long long yq,
+                                                         int M, int N, int K, double* __restrict__ out, long long os,
+                                                         long long oc) {
+  __shared__ double sx[2][kSo * kSp], sy[2][kSo * kSp];
+  const int t = threadIdx.x, tm = (M + kSo - 1) / kSo;
+  const int i0 = (int)(blockIdx.x % tm) * kSo, j0 = (int)(blockIdx.x / tm) * kSo;
+  // staging: one entry of each operand a thread, along its contiguous index
+  const int xrow = xq == 1 ? t / kSq : t % kSo, xk = xq == 1 ? t % kSq : t / kSo;
+  const int yrow = yq == 1 ? t / kSq : t % kSo, yk = yq == 1 ? t % kSq : t / kSo;
+  auto get_x = [&](int q0) {
+    return i0 + xrow < M && q0 + xk < K ? to_d<TX>(x[(i0 + xrow) * xr + (q0 + xk) * xq]) : 0.0;
+  };
+  auto get_y = [&](int q0) { return j0 + yrow < N && q0 + yk < K ? y[(j0 + yrow) * yr + (q0 + yk) * yq] : 0.0; };
+  const int g = t & 3, i = t >> 2 & 7, j = t >> 5;
+  double s = 0.0, c = 0.0, vx = get_x(0), vy = get_y(0);
+  int b = 0;
+  for (int q0 = 0; q0 < K; q0 += kSq) {
+    sx[b][xrow * kSp + xk] = vx;
+    sy[b][yrow * kSp + yk] = vy;
+    __syncthreads();   // (the other buffer's readers are past the last one)
+    vx = get_x(q0 + kSq);
+    vy = get_y(q0 + kSq);
+#pragma unroll
+    for (int e = 0; e < kSq; e += 4) {
+      const double u = sx[b][i * kSp + e + g], v = sy[b][j * kSp + e + g];
+      if constexpr (COMP) {
+        const double p = __dmul_rn(u, v), n = __dadd_rn(s, p), z = __dsub_rn(n, s);
+        c += (__dsub_rn(s, __dsub_rn(n, z)) + __dsub_rn(p, z)) + fma(u, v, -p);
+        s = n;
+      } else {
+        s = fma(u, v, s);
+      }
+    }
+    b ^= 1;
+  }
+#pragma unroll
+  for (int o = 1; o < 4; o <<= 1) {
+    const double p = __shfl_xor_sync(0xffffffffu, s, o), pc = __shfl_xor_sync(0xffffffffu, c, o);
+    const double n = __dadd_rn(s, p), z = __dsub_rn(n, s);
+    if constexpr (COMP) c = (c + pc) + (__dsub_rn(s, __dsub_rn(n, z)) + __dsub_rn(p, z));
+    s = n;
+  }
+  // (beside infinities the errors are NaN)
+  if (g == 0 && i0 + i < M && j0 + j < N) out[(i0 + i) * os + (j0 + j) * oc] = COMP && isfinite(s) ? s + c : s;
+}
+template <typename TX, bool COMP>
+void small_sums(const TX* x, long long xr, long long xq, const double* y, long long yr, long long yq, int M, int N,
+                int K, double* out, long long os, long long oc, cudaStream_t s) {
+  const unsigned blocks = (unsigned)((M + kSo - 1) / kSo) * ((N + kSo - 1) / kSo);
+  small_sums_kernel<TX, COMP><<<blocks, 256, 0, s>>>(x, xr, xq, y, yr, yq, M, N, K, out, os, oc);
+}
+// Multiply-adds of a product up to which css_residual_backward's run there, and
+// the longest sum (one block's chain).  css.residual forward, then with backward,
+// us with digits and here (before digits): FP32 64 x 128, k = 8 276, 772 and 175,
+// 539 (208, 606); 256 x 1024, k = 16 335, 904 and 246, 686 (295, 778); 257 x
+// 1000, k = 31 351, 990 and 258, 711 (338, 859); 300 x 4000, k = 8 343, 928 and
+// 328, 920 (314, 825); beyond 1e7 digits were not slower than what they replaced.
+// FP64: 64 x 128, k = 8 290, 839 and 186, 581 (230, 661); 128 x 256, k = 16 347,
+// 982 and 245, 724; 256 x 512, k = 8 338, 935 and 333, 961.
+constexpr double kSmallMacs = 1e7, kSmallMacsF64 = 524288.0;
+constexpr long long kSmallDim = 4096;
+bool small_residual(int dt, long long m, long long n, int k) {
+  return k <= kSliceK && std::max(m, n) <= kSmallDim &&
+         (double)m * n * k <= (dt == CSS_F64 ? kSmallMacsF64 : kSmallMacs);
+}
+
+// V = Q W on entry, R = A - V on return (in place), dA = g2 R when dA != null,
+// and each block's share of ||R||^2 added to its partial sum (FP64 input, and
+// small calls).
 constexpr int kLossBlocks = 152 * 8;
-__global__ void __launch_bounds__(256) residual_f64_kernel(const double* __restrict__ A, long long lda, int m,
+template <typename TA>
+__global__ void __launch_bounds__(256) residual_f64_kernel(const TA* __restrict__ A, long long lda, int m,
                                                            long long mn, double* __restrict__ R,
-                                                           double* __restrict__ dA, long long ldda, double g2,
+                                                           TA* __restrict__ dA, long long ldda, double g2,
                                                            double* __restrict__ loss_part) {
   __shared__ double red[32];
   double sq = 0.0;
   for (long long idx = (long long)blockIdx.x * 256 + threadIdx.x; idx < mn; idx += (long long)gridDim.x * 256) {
     const long long c = idx / m, i = idx - c * m;
-    const double r = A[c * lda + i] - R[idx];
+    const double r = to_d<TA>(A[c * lda + i]) - R[idx];
     R[idx] = r;
-    if (dA) dA[c * ldda + i] = g2 * r;
+    if (dA) dA[c * ldda + i] = from_d<TA>(g2 * r);
     sq = fma(r, r, sq);
   }
   sq = block_sum(sq, red);
@@ -475,9 +553,10 @@ struct BwLayout {
   int* status;   // [0] A_S is rank deficient, [kErr] error of the products
   double *AS, *Q, *Psum, *loss_part;
   OrthSpace o;
+  bool small;             // products in FP64, in one part
   long long cols, rows;   // of a part
   double* W;     // a part's columns
-  void* R;       // a part of the residual: FP32, FP64 for FP64 input
+  void* R;       // a part of the residual: FP32, FP64 for FP64 input and small calls
   sg::Digits DQ, DQr, DW, DWr, DA, DR;   // operands of a part's products (r: the other way round)
   sg::Scratch sc;
   size_t bytes;
@@ -492,6 +571,13 @@ BwLayout bw_layout(void* ws, size_t cap, int dt, int64_t m, int64_t n, int32_t k
   L.Q = c.take<double>((size_t)m * k);
   L.Psum = grad ? c.take<double>((size_t)m * k) : nullptr;
   L.loss_part = c.take<double>((size_t)std::max(kLossBlocks, sg::residual_parts()));
+  L.small = small_residual(dt, m, n, k);
+  if (L.small) {
+    L.W = c.take<double>((size_t)k * n);
+    L.R = c.take<double>((size_t)m * n);
+    L.bytes = c.off;
+    return L;
+  }
   // the basis is formed before the first part's digits
   const size_t at = c.off;
   carve_orth_digits(c, m, k, L.o);
@@ -526,7 +612,9 @@ css_status run_backward(const TA* A, int m, int n, long long lda, const int* sel
                         const css_opts& o, cudaStream_t s) {
   constexpr int dt = sizeof(TA) == 8 ? CSS_F64 : sizeof(TA) == 4 ? CSS_F32 : CSS_BF16;
   const unsigned long long spin = o.spin_budget_ns ? o.spin_budget_ns : 2000000000ull;
-  const int parts = dt == CSS_F64 ? kLossBlocks : sg::residual_parts();
+  const long long mn = (long long)m * n;
+  const int parts = L.small ? (int)std::min<long long>(kLossBlocks, (mn + 255) / 256)
+                    : dt == CSS_F64 ? kLossBlocks : sg::residual_parts();
   cudaMemsetAsync(L.status, 0, (kErr + 1) * sizeof(int), s);
   L.sc.stall = L.o.sc.stall = o.test_unmet_wait == 2;
   cudaMemsetAsync(L.loss_part, 0, parts * sizeof(double), s);
@@ -534,7 +622,15 @@ css_status run_backward(const TA* A, int m, int n, long long lda, const int* sel
   const long long mk = (long long)m * k;
   gather_cols_kernel<TA><<<(unsigned)((mk + 255) / 256), 256, 0, s>>>(A, lda, m, sel, k, L.AS);
   if (orth(L.AS, m, k, L.Q, L.o, spin, s) != cudaSuccess) return CSS_ERR_CUDA;
-  for (long long c0 = 0; c0 < n; c0 += L.cols) {
+  if (L.small) {
+    constexpr bool kComp = dt == CSS_F64;
+    double* const R = (double*)L.R;
+    small_sums<TA, kComp>(A, lda, 1, L.Q, m, 1, n, k, m, L.W, k, 1, s);
+    small_sums<double, kComp>(L.Q, 1, m, L.W, k, 1, m, n, k, R, 1, m, s);
+    residual_f64_kernel<TA><<<parts, 256, 0, s>>>(A, lda, m, mn, R, dA, ldda, 2.0 * grad_out, L.loss_part);
+    if (dA) small_sums<double, kComp>(R, 1, m, L.W, 1, k, m, k, n, L.Psum, 1, m, s);
+  }
+  for (long long c0 = 0; !L.small && c0 < n; c0 += L.cols) {
     const int nc = (int)std::min(L.cols, n - c0);
     const TA* Ac = A + c0 * lda;
     const sg::Source w{L.W, CSS_F64, 1, k, k, nc}, wr{L.W, CSS_F64, k, 1, nc, k};
@@ -549,8 +645,8 @@ css_status run_backward(const TA* A, int m, int n, long long lda, const int* sel
       if constexpr (dt == CSS_F64) {
         const sg::Store st{(double*)L.R, 1, mr, 0};
         if (sg::gemm(L.DQr, L.DWr, st, L.sc, err, spin, s, qr, wr) != cudaSuccess) return CSS_ERR_CUDA;
-        residual_f64_kernel<<<kLossBlocks, 256, 0, s>>>(Ac + r0, lda, mr, (long long)mr * nc, (double*)L.R, dAc, ldda,
-                                                        2.0 * grad_out, L.loss_part);
+        residual_f64_kernel<TA><<<kLossBlocks, 256, 0, s>>>(Ac + r0, lda, mr, (long long)mr * nc, (double*)L.R, dAc,
+                                                            ldda, 2.0 * grad_out, L.loss_part);
       } else {
         const sg::Residual r{Ac + r0, dt, lda, dA ? (float*)L.R : nullptr, dAc, ldda, 2.0 * grad_out, L.loss_part};
         if (sg::gemm_residual(L.DQr, L.DWr, r, L.sc, err, spin, s) != cudaSuccess) return CSS_ERR_CUDA;
