@@ -165,7 +165,8 @@ typedef struct {
        mbarrier phase that nothing completes.  The wait runs out after
        spin_budget_ns, the call reports CSS_ERR_TIMEOUT, nothing faults and
        the context stays usable for the next call.  css_select, gcss_select,
-       css_embed, css_residual_backward and css_lowrank. */
+       css_embed, css_residual_backward (but for small calls, which run
+       neither) and css_lowrank. */
     int32_t test_unmet_wait;
     /* Plan knobs (0 = the value the tuning table holds for this device and
        shape, else the default).  split_share: the fused step splits the
